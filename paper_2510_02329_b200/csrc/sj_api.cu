@@ -298,18 +298,12 @@ static bool tc_shapes_ok(const sj_model_config& c) {
          (c.n_q_heads * c.head_dim) % kBK == 0;
 }
 
-typedef void (*MegaKernel)(const MegaMaps, const MegaParams, const StepArgs*, const KvView, const Work, const Dims);
 // The persistent kernel for a head dimension (64 or 128), a number of row slots (4, 6 or 8), with or without
 // the timeline code, with the mma.sync or (head dimension 128 only) the tcgen05 attention phase.
-template <bool TR, bool A5>
-static MegaKernel mega_kernel_t(int hd, int ns) {
-  if (hd == 128)
-    return ns == 4 ? k_verify_mega<128, 4, TR, A5> : (ns == 6 ? k_verify_mega<128, 6, TR, A5> : k_verify_mega<128, 8, TR, A5>);
-  return ns == 4 ? k_verify_mega<64, 4, TR, false> : (ns == 6 ? k_verify_mega<64, 6, TR, false> : k_verify_mega<64, 8, TR, false>);
-}
 static MegaKernel mega_kernel(int hd, int ns, bool trace, bool a5) {
-  if (a5) return trace ? mega_kernel_t<true, true>(hd, ns) : mega_kernel_t<false, true>(hd, ns);
-  return trace ? mega_kernel_t<true, false>(hd, ns) : mega_kernel_t<false, false>(hd, ns);
+  if (hd != 128) return trace ? mega_kernel_64_trace(ns) : mega_kernel_64(ns);
+  if (a5) return trace ? mega_kernel_128_t5_trace(ns) : mega_kernel_128_t5(ns);
+  return trace ? mega_kernel_128_trace(ns) : mega_kernel_128(ns);
 }
 
 extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weights* w, void* cuda_stream,

@@ -122,7 +122,7 @@ __device__ __forceinline__ bool t5_wait(uint64_t* bar, uint32_t parity, T5Ctl* c
   return att_mbar_wait(att_smem_u32(bar), parity, &ctl->abort_flag, status, nullptr, where, 0);
 }
 
-__global__ void __launch_bounds__(kT5Threads, 1)
+static __global__ void __launch_bounds__(kT5Threads, 1)
 k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, AttArgs a) {
   constexpr int HD = 128;
   extern __shared__ uint8_t t5_smem_raw[];

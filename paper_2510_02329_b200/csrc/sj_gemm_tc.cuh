@@ -199,7 +199,7 @@ struct TcSmemCtl {
   RowStat wstat[4][16];  // per epilogue warp, one group of 16 rows at a time
 };
 
-__global__ void __launch_bounds__(kTcThreads, 1)
+static __global__ void __launch_bounds__(kTcThreads, 1)
 k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW0,
           const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2, TcGemmParams p,
           const StepArgs* __restrict__ args, Work w, int V) {

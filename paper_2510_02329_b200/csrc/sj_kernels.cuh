@@ -69,7 +69,7 @@ template <> __device__ __forceinline__ void store_act<bf16>(void* base, int R, i
 // ---------------------------------------------------------------------------------------------
 // step set-up: row positions and the attention chunk list (needs the true cache lengths)
 // ---------------------------------------------------------------------------------------------
-__global__ void k_plan(const StepArgs* __restrict__ args, KvView kv, Work w, int chunk_len) {
+static __global__ void k_plan(const StepArgs* __restrict__ args, KvView kv, Work w, int chunk_len) {
   pdl_wait();
   pdl_launch();
   __shared__ int nch[kMaxBatch];
@@ -479,7 +479,7 @@ __device__ __forceinline__ float planes_dot(const bf16* __restrict__ A, int R, i
 // Top-k alignment test with the tensor-core LM head, which stores no logits: the logit of row j's drafted token
 // d_{j+1} is computed ahead of the LM head (one dot product per row), so that the head's epilogue can count, tile
 // by tile, how many logits rank before it.  One warp per row; idle unless the step asks for top_k >= 2.
-__global__ void k_target_logits(const StepArgs* __restrict__ args, Work w, Dims dm, const bf16* __restrict__ lm_head, int R) {
+static __global__ void k_target_logits(const StepArgs* __restrict__ args, Work w, Dims dm, const bf16* __restrict__ lm_head, int R) {
   pdl_wait();
   pdl_launch();
   if (args->top_k < 2) return;
@@ -495,7 +495,7 @@ __global__ void k_target_logits(const StepArgs* __restrict__ args, Work w, Dims 
 // ---------------------------------------------------------------------------------------------
 // a10 (CUDA-core path): per-(128-token vocabulary tile, row) softmax statistics from stored logits
 // ---------------------------------------------------------------------------------------------
-__global__ void k_lm_stats_from_logits(const StepArgs* __restrict__ args, Work w, Dims dm, int R) {
+static __global__ void k_lm_stats_from_logits(const StepArgs* __restrict__ args, Work w, Dims dm, int R) {
   pdl_wait();
   pdl_launch();
   const int tile = blockIdx.x, lane = threadIdx.x & 31;
@@ -548,7 +548,7 @@ __global__ void k_lm_stats_from_logits(const StepArgs* __restrict__ args, Work w
 // a10 tail + a11..a15: merge statistics, judge scores, acceptance bits, first rejection, next
 // token (greedy), new cache length and commit.  One block per sequence.
 // ---------------------------------------------------------------------------------------------
-__global__ void k_finalize(const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, int n_vtiles, int R) {
+static __global__ void k_finalize(const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, int n_vtiles, int R) {
   pdl_wait();
   pdl_launch();
   __shared__ RowStat sred[256];
@@ -639,7 +639,7 @@ __global__ void k_select_rows(const StepArgs* __restrict__ args, Work w, Dims dm
 // a14, sampling mode: inverse CDF over the vocabulary of norm(max(0, p_n - q_{n+1})) (first
 // rejection) or of p_gamma (everything accepted), driven by uniforms[:, gamma].  fp64 prefix sums.
 // per_seq: the logit scratch holds one row per sequence (row b) instead of every block row.
-__global__ void k_resample(const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, int per_seq) {
+static __global__ void k_resample(const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, int per_seq) {
   pdl_wait();
   pdl_launch();
   __shared__ double part[1024];
@@ -689,7 +689,7 @@ __global__ void k_resample(const StepArgs* __restrict__ args, KvView kv, Work w,
 }
 
 // Rollback: kv_len <- new_len where new_len <= kv_len, else flag the error and leave it.
-__global__ void k_rollback(KvView kv, const int* __restrict__ seqs, const int* __restrict__ new_len, int B, int* status) {
+static __global__ void k_rollback(KvView kv, const int* __restrict__ seqs, const int* __restrict__ new_len, int B, int* status) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B) return;
   int s = seqs[i], n = new_len[i];

@@ -1314,4 +1314,14 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
   }
 }
 
+typedef void (*MegaKernel)(const MegaMaps, const MegaParams, const StepArgs*, const KvView, const Work, const Dims);
+// The kernel's instantiations by head dimension, attention phase and timeline code, each in a translation unit of
+// its own (sj_mega_inst.cu) so that they compile side by side; ns: row slots (4, 6 or 8).
+MegaKernel mega_kernel_64(int ns);
+MegaKernel mega_kernel_64_trace(int ns);
+MegaKernel mega_kernel_128(int ns);
+MegaKernel mega_kernel_128_trace(int ns);
+MegaKernel mega_kernel_128_t5(int ns);
+MegaKernel mega_kernel_128_t5_trace(int ns);
+
 }  // namespace sj

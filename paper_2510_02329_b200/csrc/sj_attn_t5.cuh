@@ -129,7 +129,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(t5_smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t *sQ = sm, *sK = sm + 2 * kT5TileBytes, *sV = sm + 4 * kT5TileBytes;
   T5Ctl* ctl = reinterpret_cast<T5Ctl*>(sm + kT5SmemBytes);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   pdl_wait();
   pdl_launch();
   const int B = args->B, rows = args->gamma + 1, Hkv = dm.Hkv, group = dm.Hq / dm.Hkv, nq = group * rows;
@@ -204,7 +204,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
     // rows' stabiliser and are added when the segment ends).  Within a thread the order is scores(g), output(g),
     // scores(g + 2): the tensor pipe executes one thread's MMAs in issue order, which is all the ordering the reuse of
     // score buffer X needs, and while the thread waits for the probabilities of its tile the other one issues.
-    if (lane == 0) {
+    if (elect_one()) {
       const int X = warp == 1 ? 0 : 1;
       const uint32_t id_s = instr_desc_bf16_mn(kT5Keys, 0), id_o = instr_desc_bf16_mn(HD, 1);
       const uint64_t dq = smem_desc_sw128(att_smem_u32(sQ)), dql = smem_desc_sw128(att_smem_u32(sQ) + kT5TileBytes);

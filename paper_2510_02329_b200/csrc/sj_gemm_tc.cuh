@@ -55,6 +55,17 @@ struct TcGemmParams {
 };
 
 // ---- PTX wrappers ----------------------------------------------------------------------------
+// One thread of a full warp, for single-thread roles that issue tcgen05.mma, commits or TMA copies.  The operands of
+// those instructions sit in uniform registers; behind `elect.sync` the compiler knows that one thread runs and keeps
+// them there, behind a `lane == 0` branch it moves every operand over again for every instruction (B200, M = 128,
+// N <= 64: one MMA per 41..48 clocks against 75; a TMA copy per 130 against 192).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+  return p != 0;
+}
+// The calling thread's warp index, as a value the compiler knows to be the same in every lane.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
@@ -207,7 +218,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int stage_bytes = kWTileBytes + p.a_stage_bytes;
   TcSmemCtl* ctl = reinterpret_cast<TcSmemCtl*>(smem + (size_t)p.stages * stage_bytes);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   volatile int* abort_flag = &ctl->abort_flag;
 
   // this block's unit range
@@ -248,7 +259,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
 
   if (warp == 0) {
     // ------------------------------ TMA producer ------------------------------
-    if (lane == 0) {
+    if (elect_one()) {
       const uint64_t pol_w = l2_policy_evict_first(), pol_a = l2_policy_evict_last();
       const uint32_t tx_bytes = kWTileBytes + (uint32_t)p.a_blocks * p.nblk * 128;
       auto w_load = [&](int it) {
@@ -288,7 +299,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
     pdl_wait();
-    if (lane == 0 && n_units > 0) {
+    if (n_units > 0 && elect_one()) {
       const uint32_t idesc = instr_desc_bf16(p.nblk);
       int it = 0, seg = 0;
       long long u = u_lo;

@@ -964,7 +964,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(mega_smem_raw) + 1023) & ~(uintptr_t)1023);
   uint8_t* q_area = ring + (size_t)p.stages * p.stage_bytes;
   MegaCtl* ctl = reinterpret_cast<MegaCtl*>(q_area + p.q_area_bytes);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int c = blockIdx.x, G = gridDim.x, NS = p.stages, B = p.B, R = p.R, Rp = p.Rp, rows = p.rows;
   AttGeom g = att_geom(HD, dm.Hq / dm.Hkv, rows);
   if constexpr (A5) { g.KPS = kA5Keys; g.KS = 1; g.KW = kA5Keys; }   // one sub-partial per block segment
@@ -1050,8 +1050,9 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
     // ------------------------------ weight / cache-tile producer ------------------------------
     // One lane; all 32 with the tcgen05 attention, whose cache tiles are 32 small copies each (one per lane, one
     // instruction per tile).  All lanes run the same control flow and wait on the same barriers; lane 0 alone announces
-    // bytes and issues the weight copies.
-    if (lane < (A5 ? 32 : 1)) {
+    // bytes and issues the weight copies (the elected lane).
+    const bool leader = elect_one();
+    if (A5 || leader) {
       const uint64_t pol_w = l2_policy_evict_first();
       RingPos rp{0, 0, NS};
       int sidx = 0;
@@ -1081,7 +1082,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
           else tm0 = &mp.lm;
           for (int kb = sg.a; kb < sg.b; ++kb) {
             if (!wait_slot()) { alive = false; return; }
-            if (lane == 0) {
+            if (leader) {
               const uint32_t bar = smem_u32(&ctl->full[rp.s]), dst = stage_addr(rp.s);
               mbar_expect_tx(bar, kWTileBytes);
               tma_load_2d(dst, tm0, bar, kb * kBK, row, pol_w);
@@ -1090,7 +1091,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
             rp.next();
           }
         }
-        if (lane == 0) MEGA_EV(sidx, 7);
+        if (leader) MEGA_EV(sidx, 7);
         ++sidx;
       };
       auto fatt = [&](int l) {
@@ -1118,7 +1119,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
     }
   } else if (warp == 1) {
     // ------------------------------ MMA issuer ------------------------------
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = instr_desc_bf16(2 * Rp);
       const uint32_t tmem_base = ctl->tmem_base;
       RingPos rp{0, 0, NS};
@@ -1181,7 +1182,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
     // Two threads, alternate units: right after a device-wide barrier the ring already holds the phase's first
     // weight tiles, and the MMAs can start only as fast as their activation slices are requested (a wait, an
     // expect and a TMA per slice cost one thread about a quarter of a microsecond).
-    if (lane == 0) {
+    if (elect_one()) {
       const int mine = warp - 2;
       int n_unit = 0;
       const uint64_t pol_a = l2_policy_evict_last();

@@ -221,13 +221,17 @@ struct sj_target {
   struct Timed { const char* name; cudaEvent_t a, b; };
   std::vector<Timed> timed;
   TcSite s_qkv, s_o, s_gu, s_down, s_lm;
-  size_t p_elems = 0;
   size_t att_chunks_cap = 0;
   int att_rows_cap = 0;
   size_t tc_part_cap = 0;   // floats in tc_m / tc_l
   size_t logits_rows = 0;
   std::map<StepKey, cudaGraphExec_t> graphs;
-  std::map<int, CUtensorMap> mapA_d, mapA_q, mapA_f, mapA_sel;  // activation maps per R (mapA_sel: per B)
+  std::map<std::pair<const void*, int>, CUtensorMap> act_maps;  // per activation matrix and row count
+  // prefill in wide blocks (allocated by the first call that can use it): a workspace of kPrefillRows rows, the tokens
+  Work pf_work;
+  int pf_rows = 0;                 // rows of pf_work; 0: not there yet, -1: no memory for it
+  int* d_pf_tok = nullptr;
+  size_t pf_tok_cap = 0;
   std::vector<void*> owned;
 };
 
@@ -306,6 +310,55 @@ static MegaKernel mega_kernel(int hd, int ns, bool trace, bool a5) {
   return trace ? mega_kernel_128_trace(ns) : mega_kernel_128(ns);
 }
 
+// The per-row buffers of a step of at most R rows.
+static sj_status alloc_rows(sj_target* t, Work& W, int R) {
+  const sj_model_config& c = t->cfg;
+  const size_t esz = t->bf ? 2 : 4;
+  const size_t qd = (size_t)c.n_q_heads * c.head_dim, kd = (size_t)c.n_kv_heads * c.head_dim, d = c.d_model;
+  const size_t act_rows = t->bf ? (size_t)2 * pad16(R) : (size_t)R;  // bf16: hi and lo planes
+  sj_status st = SJ_OK;
+  auto get = [&](auto** p, size_t n) { return st == SJ_OK && (st = dev_alloc(t, p, n)) == SJ_OK; };
+  // an activation matrix: read as a GEMM operand, so rows that no step has written must hold finite values
+  auto act = [&](void** p, size_t cols) {
+    uint8_t* q = nullptr;
+    if (!get(&q, act_rows * cols * esz)) return;
+    *p = q;
+    if (cudaMemset(q, 0, act_rows * cols * esz) != cudaSuccess) st = fail(SJ_ERR_CUDA, "workspace clear failed");
+  };
+  get(&W.X, R * d);
+  act(&W.A, d);
+  act(&W.ATT, qd);
+  act(&W.H, c.d_ffn);
+  act(&W.Asel, d);   // at most one row per sequence is used
+  get(&W.Q, R * qd);
+  if (t->bf) {
+    get(&W.Qb, R * qd);
+    get(&W.Qlo, R * qd);
+    get(&W.KVn, (size_t)R * 2 * kd);
+  }
+  get(&W.Hf, R * d);
+  get(&W.rope, (size_t)R * (c.head_dim / 2));
+  get(&W.row_pos, R);
+  get(&W.chunk_start, SJ_MAX_BATCH + 1);
+  get(&W.stats, (size_t)((c.vocab + kTileN - 1) / kTileN) * R);
+  get(&W.tgt_logit, R);
+  get(&W.tgt_pre, R);
+  get(&W.rowstat, R);
+  if (st == SJ_OK && cudaMemset(W.tgt_logit, 0, sizeof(float) * R) != cudaSuccess) st = fail(SJ_ERR_CUDA, "workspace clear failed");
+  return st;
+}
+
+// The projections' partial sums of a step of at most R rows (one slot per block that shares a tile).
+static sj_status alloc_partials(sj_target* t, Work& W, int R) {
+  const sj_model_config& c = t->cfg;
+  size_t n = (size_t)R * std::max({(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, c.d_model, 2 * c.d_ffn});
+  if (tc_shapes_ok(c)) {
+    n = 0;
+    for (TcSite* s : {&t->s_qkv, &t->s_o, &t->s_gu, &t->s_down}) n = std::max(n, (size_t)s->max_slots * R * s->N);
+  }
+  return dev_alloc(t, &W.P, n);
+}
+
 extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weights* w, void* cuda_stream,
                                       sj_target** out) {
   if (!cfg || !w || !out) return fail(SJ_ERR_INVALID_ARG, "null argument");
@@ -364,36 +417,16 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
 
   sj_status st = SJ_OK;
   auto bail = [&](sj_status s) { sj_destroy_target(t); return s; };
-  const size_t esz = t->bf ? 2 : 4;
   const int qd = c.n_q_heads * c.head_dim, kd = c.n_kv_heads * c.head_dim, R = max_rows;
   Work& W = t->work;
   memset(&W, 0, sizeof(W));
-  uint8_t* tmp = nullptr;
 #define ALLOC(field, type, count)                                                     \
   do {                                                                                \
     type* p_ = nullptr;                                                               \
     if ((st = dev_alloc(t, &p_, (count))) != SJ_OK) return bail(st);                  \
     field = p_;                                                                       \
   } while (0)
-  ALLOC(W.X, float, (size_t)R * c.d_model);
-  const size_t act_rows = t->bf ? (size_t)2 * pad16(R) : (size_t)R;  // bf16: hi and lo planes
-  ALLOC(tmp, uint8_t, act_rows * c.d_model * esz); W.A = tmp;
-  ALLOC(W.Q, float, (size_t)R * qd);
-  if (t->bf) ALLOC(W.Qb, __half, (size_t)R * qd);
-  if (t->bf) ALLOC(W.Qlo, __half, (size_t)R * qd);
-  if (t->bf) ALLOC(W.KVn, __half, (size_t)R * 2 * kd);
-  ALLOC(tmp, uint8_t, act_rows * qd * esz); W.ATT = tmp;
-  ALLOC(tmp, uint8_t, act_rows * c.d_ffn * esz); W.H = tmp;
-  ALLOC(tmp, uint8_t, act_rows * c.d_model * esz); W.Asel = tmp;   // at most one row per sequence is used
-  ALLOC(W.Hf, float, (size_t)R * c.d_model);
-  ALLOC(W.rope, float2, (size_t)R * (c.head_dim / 2));
-  ALLOC(W.row_pos, int, R);
-  ALLOC(W.chunk_start, int, SJ_MAX_BATCH + 1);
-  const int n_vtiles = (c.vocab + kTileN - 1) / kTileN;
-  ALLOC(W.stats, RowStat, (size_t)n_vtiles * R);
-  ALLOC(W.tgt_logit, float, R);
-  ALLOC(W.tgt_pre, float, R);
-  ALLOC(W.rowstat, RowStat, R);
+  if ((st = alloc_rows(t, W, R)) != SJ_OK) return bail(st);
   ALLOC(W.status, int, 1);
   ALLOC(t->d_args, StepArgs, 1);
   ALLOC(t->d_judge_w, float, c.d_model);
@@ -403,14 +436,12 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
   {
     cudaError_t e = cudaMemset(W.status, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(t->d_judge_w, 0, sizeof(float) * c.d_model);
-    if (e == cudaSuccess) e = cudaMemset(W.tgt_logit, 0, sizeof(float) * R);
     std::vector<double> inv(c.head_dim / 2);
     for (int i = 0; i < c.head_dim / 2; ++i) inv[i] = std::pow((double)c.rope_theta, -2.0 * i / c.head_dim);
     if (e == cudaSuccess) e = cudaMemcpy(t->d_inv_freq, inv.data(), inv.size() * sizeof(double), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) { fail(SJ_ERR_CUDA, "workspace init: %s", cudaGetErrorString(e)); return bail(SJ_ERR_CUDA); }
   }
   // GEMM sites and the partial buffer
-  size_t p_elems = (size_t)R * std::max({qd + 2 * kd, c.d_model, 2 * c.d_ffn});
   if (tc) {
     int seg_qkv[3] = {qd, kd, kd}, seg_o[1] = {c.d_model}, seg_gu[2] = {c.d_ffn, c.d_ffn}, seg_d[1] = {c.d_model},
         seg_lm[1] = {c.vocab};
@@ -419,9 +450,6 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
     if ((st = setup_site(t, t->s_gu, 2, seg_gu, c.d_model, false)) != SJ_OK) return bail(st);
     if ((st = setup_site(t, t->s_down, 1, seg_d, c.d_ffn, false)) != SJ_OK) return bail(st);
     if ((st = setup_site(t, t->s_lm, 1, seg_lm, c.d_model, true)) != SJ_OK) return bail(st);
-    p_elems = 0;
-    for (TcSite* s : {&t->s_qkv, &t->s_o, &t->s_gu, &t->s_down})
-      p_elems = std::max(p_elems, (size_t)s->max_slots * R * s->N);
     for (int l = 0; l < c.n_layers; ++l) {
       LayerW& L = t->layers[l];
       if ((st = make_map(&L.m_q, L.wq, qd, c.d_model, kTileN)) != SJ_OK) return bail(st);
@@ -438,8 +466,7 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
     cudaError_t e = cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) { fail(SJ_ERR_CUDA, "smem opt-in: %s", cudaGetErrorString(e)); return bail(SJ_ERR_CUDA); }
   }
-  t->p_elems = p_elems;
-  ALLOC(W.P, float, p_elems);
+  if ((st = alloc_partials(t, W, R)) != SJ_OK) return bail(st);
   {
     int coop = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
@@ -477,11 +504,6 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
       }
       mm.lm = t->m_lm;
     }
-    // the activation planes are read as GEMM operands: rows past R must stay finite
-    cudaMemset(W.A, 0, act_rows * c.d_model * esz);
-    cudaMemset(W.ATT, 0, act_rows * qd * esz);
-    cudaMemset(W.H, 0, act_rows * c.d_ffn * esz);
-    cudaMemset(W.Asel, 0, act_rows * c.d_model * esz);
     t->opt_step = 1;
   }
 #undef ALLOC
@@ -858,23 +880,22 @@ static RowGeom feed_geom(int R, bool planes) {
   return planes_fit(R) ? row_geom(2 * pad16(R)) : row_geom(pad16(R), true);
 }
 
-static sj_status activation_map(sj_target* t, std::map<int, CUtensorMap>& cache, const void* base, int R, int K,
-                                const CUtensorMap** out) {
-  auto it = cache.find(R);
-  if (it == cache.end()) {
+static sj_status activation_map(sj_target* t, const void* base, int R, int K, const CUtensorMap** out) {
+  auto it = t->act_maps.find({base, R});
+  if (it == t->act_maps.end()) {
     CUtensorMap m;
     RowGeom g = feed_geom(R, true);
     sj_status st = make_map(&m, base, 2 * pad16(R), K, g.nblk);
     if (st != SJ_OK) return st;
-    it = cache.emplace(R, m).first;
+    it = t->act_maps.emplace(std::make_pair(base, R), m).first;
   }
   *out = &it->second;
   return SJ_OK;
 }
 
 static cudaError_t launch_tc(sj_target* t, const TcSite& s, const CUtensorMap* mA, const CUtensorMap* w0,
-                             const CUtensorMap* w1, const CUtensorMap* w2, int R, bool pdl, bool planes, int lm_mode = -1,
-                             const Work* work = nullptr) {
+                             const CUtensorMap* w1, const CUtensorMap* w2, int R, bool pdl, bool planes, const Work& W,
+                             int lm_mode = -1) {
   RowGeom g = feed_geom(R, planes);
   TcGemmParams p;
   memset(&p, 0, sizeof(p));
@@ -885,10 +906,10 @@ static cudaError_t launch_tc(sj_target* t, const TcSite& s, const CUtensorMap* m
   for (int i = 0; i < 3; ++i) p.seg_tile_end[i] = s.seg_tile_end[i];
   p.stages = g.stages; p.a_stage_bytes = g.a_stage_bytes; p.tmem_cols = g.tmem_cols;
   p.acc_bufs = g.acc_bufs; p.acc_stride = g.acc_stride;
-  p.P = t->work.P; p.slot_stride = (size_t)R * s.N; p.tile_slots = s.d_tile_slots;
-  p.lm_mode = lm_mode >= 0 ? lm_mode : (s.lm ? 1 : 0); p.status = t->work.status;
+  p.P = W.P; p.slot_stride = (size_t)R * s.N; p.tile_slots = s.d_tile_slots;
+  p.lm_mode = lm_mode >= 0 ? lm_mode : (s.lm ? 1 : 0); p.status = W.status;
   return launch(k_gemm_tc, dim3(s.G), dim3(kTcThreads), g.smem_bytes, t->stream, pdl, *mA, *w0, *(w1 ? w1 : w0),
-                *(w2 ? w2 : w0), p, (const StepArgs*)t->d_args, work ? *work : t->work, t->dm.V);
+                *(w2 ? w2 : w0), p, (const StepArgs*)t->d_args, W, t->dm.V);
 }
 
 // a14 in sampling mode with the tensor-core LM head: re-normalise the one row per sequence that the emitted
@@ -898,11 +919,11 @@ static sj_status enqueue_resample(sj_target* t, sj_kv* kv, int B, const Work& W,
   const Dims& dm = t->dm;
   cudaStream_t s = t->stream;
   const CUtensorMap* mA = nullptr;
-  sj_status st = activation_map(t, t->mapA_sel, W.Asel, B, dm.d, &mA);
+  sj_status st = activation_map(t, W.Asel, B, dm.d, &mA);
   if (st != SJ_OK) return st;
   CU_TRY(launch(k_select_rows<T>, dim3(B), dim3(256), sizeof(float) * dm.d, s, pdl, (const StepArgs*)t->d_args, W, dm,
-                (const T*)t->final_norm));
-  CU_TRY(launch_tc(t, t->s_lm, mA, &t->m_lm, nullptr, nullptr, B, pdl, true, 2, &W));
+                (const T*)t->final_norm, -1));
+  CU_TRY(launch_tc(t, t->s_lm, mA, &t->m_lm, nullptr, nullptr, B, pdl, true, W, 2));
   CU_TRY(launch(k_resample, dim3(B), dim3(1024), 0, s, pdl, (const StepArgs*)t->d_args, kv->view, W, dm, 1));
   return SJ_OK;
 }
@@ -929,17 +950,18 @@ static cudaError_t launch_simt(sj_target* t, const void* A, const GemmSegs& segs
     }                                                                            \
   } while (0)
 
+// The decoder layers of a step (set-up and embedding included): from the step's arguments to the GEMM input planes of
+// the final norm.  kv_only: the block's key / value rows are all that is wanted (prefill blocks before the last), so the
+// last layer ends after its projection.
 template <typename T>
-static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mode, int chunk_len, bool use_scratch,
-                               size_t n_chunks_hi) {
+static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int chunk_len, Work W, size_t n_chunks_hi,
+                                bool kv_only) {
   const Dims& dm = t->dm;
   const int R = B * (gamma + 1), qd = dm.Hq * dm.hd, kd = dm.Hkv * dm.hd;
   const bool timing = t->opt_timing != 0 && !t->opt_graph;
   const bool pdl = t->opt_pdl != 0 && !timing, tc = t->opt_gemm == 1;
   const bool attn_tc = t->opt_attn >= 1 && t->bf && kv->has_tm_pool;
   const StepArgs* args = t->d_args;
-  Work W = t->work;
-  if (!use_scratch) W.logits = nullptr;
   if (!attn_tc) W.Qb = nullptr, W.KVn = nullptr;
   cudaStream_t s = t->stream;
   const size_t row_smem = sizeof(float) * dm.d;
@@ -947,9 +969,9 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
   const CUtensorMap *mA_d = nullptr, *mA_q = nullptr, *mA_f = nullptr;
   if (tc) {
     sj_status st;
-    if ((st = activation_map(t, t->mapA_d, W.A, R, dm.d, &mA_d)) != SJ_OK) return st;
-    if ((st = activation_map(t, t->mapA_q, W.ATT, R, qd, &mA_q)) != SJ_OK) return st;
-    if ((st = activation_map(t, t->mapA_f, W.H, R, dm.F, &mA_f)) != SJ_OK) return st;
+    if ((st = activation_map(t, W.A, R, dm.d, &mA_d)) != SJ_OK) return st;
+    if ((st = activation_map(t, W.ATT, R, qd, &mA_q)) != SJ_OK) return st;
+    if ((st = activation_map(t, W.H, R, dm.F, &mA_f)) != SJ_OK) return st;
   }
   auto plan_of = [&](const TcSite& site) { return tc ? SplitPlan{site.d_tile_slots, site.n_tiles} : one; };
 
@@ -963,13 +985,14 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
     const LayerW& L = t->layers[l];
     // QKV projection
     if (tc) {
-      TIMED("gemm_qkv", launch_tc(t, t->s_qkv, mA_d, &L.m_q, &L.m_k, &L.m_v, R, pdl, true));
+      TIMED("gemm_qkv", launch_tc(t, t->s_qkv, mA_d, &L.m_q, &L.m_k, &L.m_v, R, pdl, true, W));
     } else {
       GemmSegs g{{L.wq, L.wk, L.wv}, {qd, kd, kd}, 3};
       TIMED("gemm_cudacore", launch_simt<T>(t, W.A, g, W.P, R, qd + 2 * kd, dm.d, pdl));
     }
     TIMED("qkv_rope", launch(k_qkv_rope<T>, dim3(R), dim3(256), 0, s, pdl, args, kv->view, W, dm, plan_of(t->s_qkv),
                   (size_t)R * (qd + 2 * kd), l, (const T*)L.bq, (const T*)L.bk, (const T*)L.bv));
+    if (kv_only && l == dm.n_layers - 1) return SJ_OK;
     // attention
     if (attn_tc) {
       AttArgs aa{W.Qb, l < t->opt_att_precise ? W.Qlo : nullptr, W.KVn, AttPartials{W.tc_m, W.tc_l, W.tc_o}, t->sm_count + B * dm.Hkv, l};
@@ -994,7 +1017,7 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
     }
     // O projection + residual + FFN norm
     if (tc) {
-      TIMED("gemm_o", launch_tc(t, t->s_o, mA_q, &L.m_o, nullptr, nullptr, R, pdl, true));
+      TIMED("gemm_o", launch_tc(t, t->s_o, mA_q, &L.m_o, nullptr, nullptr, R, pdl, true, W));
     } else {
       GemmSegs g{{L.wo, nullptr, nullptr}, {dm.d, 0, 0}, 1};
       TIMED("gemm_cudacore", launch_simt<T>(t, W.ATT, g, W.P, R, dm.d, qd, pdl));
@@ -1003,7 +1026,7 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
                   (const T*)L.nf, 0));
     // gate/up + SwiGLU
     if (tc) {
-      TIMED("gemm_gateup", launch_tc(t, t->s_gu, mA_d, &L.m_g, &L.m_u, nullptr, R, pdl, true));
+      TIMED("gemm_gateup", launch_tc(t, t->s_gu, mA_d, &L.m_g, &L.m_u, nullptr, R, pdl, true, W));
     } else {
       GemmSegs g{{L.wg, L.wu, nullptr}, {dm.F, dm.F, 0}, 2};
       TIMED("gemm_cudacore", launch_simt<T>(t, W.A, g, W.P, R, 2 * dm.F, dm.d, pdl));
@@ -1012,7 +1035,7 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
                   (size_t)R * 2 * dm.F));
     // down projection + residual + next norm
     if (tc) {
-      TIMED("gemm_down", launch_tc(t, t->s_down, mA_f, &L.m_d, nullptr, nullptr, R, pdl, true));
+      TIMED("gemm_down", launch_tc(t, t->s_down, mA_f, &L.m_d, nullptr, nullptr, R, pdl, true, W));
     } else {
       GemmSegs g{{L.wd, nullptr, nullptr}, {dm.d, 0, 0}, 1};
       TIMED("gemm_cudacore", launch_simt<T>(t, W.H, g, W.P, R, dm.d, dm.F, pdl));
@@ -1022,11 +1045,29 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
     TIMED("reduce_norm", launch(k_reduce_norm<T>, dim3(R), dim3(256), row_smem, s, pdl, args, W, dm, plan_of(t->s_down),
                   (size_t)R * dm.d, (const T*)gain, last ? 1 : 0));
   }
+  return SJ_OK;
+}
+
+template <typename T>
+static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mode, int chunk_len, bool use_scratch,
+                               size_t n_chunks_hi) {
+  const Dims& dm = t->dm;
+  const int R = B * (gamma + 1);
+  const bool timing = t->opt_timing != 0 && !t->opt_graph;
+  const bool pdl = t->opt_pdl != 0 && !timing, tc = t->opt_gemm == 1;
+  const StepArgs* args = t->d_args;
+  Work W = t->work;
+  if (!use_scratch) W.logits = nullptr;
+  cudaStream_t s = t->stream;
+  const CUtensorMap* mA_d = nullptr;
+  sj_status st = enqueue_layers<T>(t, kv, B, gamma, chunk_len, W, n_chunks_hi, false);
+  if (st != SJ_OK) return st;
+  if (tc && (st = activation_map(t, W.A, R, dm.d, &mA_d)) != SJ_OK) return st;
   // LM head + statistics
   const int n_vtiles = (dm.V + kTileN - 1) / kTileN;
   if (tc) {
     TIMED("target_logits", launch(k_target_logits, dim3((R + 7) / 8), dim3(256), 0, s, pdl, args, W, dm, (const bf16*)t->lm_head, R));
-    TIMED("gemm_lm_head", launch_tc(t, t->s_lm, mA_d, &t->m_lm, nullptr, nullptr, R, pdl, true, -1, &W));   // W: no [R, V] logit store
+    TIMED("gemm_lm_head", launch_tc(t, t->s_lm, mA_d, &t->m_lm, nullptr, nullptr, R, pdl, true, W));   // W: no [R, V] logit store
   } else {
     GemmSegs g{{t->lm_head, nullptr, nullptr}, {dm.V, 0, 0}, 1};
     TIMED("gemm_cudacore", launch_simt<T>(t, W.A, g, W.logits, R, dm.V, dm.d, pdl));
@@ -1061,9 +1102,9 @@ static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode
   if (!use_scratch) W.logits = nullptr;
   const CUtensorMap *mA_d = nullptr, *mA_q = nullptr, *mA_f = nullptr;
   sj_status st;
-  if ((st = activation_map(t, t->mapA_d, W.A, R, dm.d, &mA_d)) != SJ_OK) return st;
-  if ((st = activation_map(t, t->mapA_q, W.ATT, R, qd, &mA_q)) != SJ_OK) return st;
-  if ((st = activation_map(t, t->mapA_f, W.H, R, dm.F, &mA_f)) != SJ_OK) return st;
+  if ((st = activation_map(t, W.A, R, dm.d, &mA_d)) != SJ_OK) return st;
+  if ((st = activation_map(t, W.ATT, R, qd, &mA_q)) != SJ_OK) return st;
+  if ((st = activation_map(t, W.H, R, dm.F, &mA_f)) != SJ_OK) return st;
   MegaParams p;
   memset(&p, 0, sizeof(p));
   p.B = B; p.rows = rows; p.R = R; p.Rp = Rp;
@@ -1175,7 +1216,37 @@ static int pick_chunk_len(const sj_target* t, long total_keys) {
   return ch;
 }
 
-extern "C" sj_status sj_verify(sj_target* t, sj_kv* kv, const sj_verify_args* a, const sj_verify_out* o) {
+// Partial results of the tensor-core attention for B sequences of `rows` rows (grown outside any capture).
+static sj_status ensure_attn_partials(sj_target* t, int B, int rows) {
+  const size_t slots = (size_t)t->sm_count + 2 * (size_t)B * t->dm.Hkv;
+  const size_t need = slots * kAttMaxSub * (size_t)(t->dm.Hq / t->dm.Hkv * rows);
+  if (need <= t->tc_part_cap) return SJ_OK;
+  sj_status st;
+  CU_TRY(cudaStreamSynchronize(t->stream));
+  clear_graphs(t);
+  for (float** p : {&t->work.tc_m, &t->work.tc_l, &t->work.tc_o}) {
+    if (*p) {
+      counted_free(*p);
+      t->owned.erase(std::remove(t->owned.begin(), t->owned.end(), (void*)*p), t->owned.end());
+      *p = nullptr;
+    }
+  }
+  t->tc_part_cap = 0;
+  if ((st = dev_alloc(t, &t->work.tc_m, need)) != SJ_OK) return st;
+  if ((st = dev_alloc(t, &t->work.tc_l, need)) != SJ_OK) return st;
+  if ((st = dev_alloc(t, &t->work.tc_o, need * t->dm.hd)) != SJ_OK) return st;
+  // slots of blocks that own no tile are read with weight zero: they must hold finite values
+  CU_TRY(cudaMemsetAsync(t->work.tc_m, 0, need * sizeof(float), t->stream));
+  CU_TRY(cudaMemsetAsync(t->work.tc_l, 0, need * sizeof(float), t->stream));
+  CU_TRY(cudaMemsetAsync(t->work.tc_o, 0, need * t->dm.hd * sizeof(float), t->stream));
+  t->tc_part_cap = need;
+  return SJ_OK;
+}
+
+// sj_verify().  score_only: the blocks are only scored -- nothing is committed or stored in the pages, and the same
+// sequence may appear several times (each entry attends to the stored cache and to its own rows; needs the tensor-core
+// attention, which reads a block's own rows from the step's side buffer and not from the pages).
+static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, const sj_verify_out* o, bool score_only) {
   if (!t || !kv || !a || !o) return fail(SJ_ERR_INVALID_ARG, "null argument");
   if (kv->t != t) return fail(SJ_ERR_INVALID_ARG, "KV cache belongs to another target");
   if (a->B <= 0 || a->B > SJ_MAX_BATCH) return fail(SJ_ERR_INVALID_ARG, "B out of range");
@@ -1184,7 +1255,7 @@ extern "C" sj_status sj_verify(sj_target* t, sj_kv* kv, const sj_verify_args* a,
   if (R > t->max_rows) return fail(SJ_ERR_SHAPE, "B*(gamma+1) = %d exceeds max_rows = %d", R, t->max_rows);
   sj_status st = check_seqs(kv, a->seq_ids, B);
   if (st != SJ_OK) return st;
-  {
+  if (!score_only) {
     std::vector<char> seen(kv->max_seqs, 0);
     for (int i = 0; i < B; ++i) {
       if (seen[a->seq_ids[i]]) return fail(SJ_ERR_INVALID_ARG, "duplicate sequence id %d", a->seq_ids[i]);
@@ -1253,30 +1324,8 @@ extern "C" sj_status sj_verify(sj_target* t, sj_kv* kv, const sj_verify_args* a,
     t->att_chunks_cap = cap;
     t->att_rows_cap = rcap;
   }
-  if ((t->opt_attn >= 1 || use_mega) && t->bf && kv->has_tm_pool) {
-    const size_t slots = (size_t)t->sm_count + 2 * (size_t)B * t->dm.Hkv;
-    const size_t need = slots * kAttMaxSub * (size_t)(group * rows);
-    if (need > t->tc_part_cap) {
-      CU_TRY(cudaStreamSynchronize(t->stream));
-      clear_graphs(t);
-      for (float** p : {&t->work.tc_m, &t->work.tc_l, &t->work.tc_o}) {
-        if (*p) {
-          counted_free(*p);
-          t->owned.erase(std::remove(t->owned.begin(), t->owned.end(), (void*)*p), t->owned.end());
-          *p = nullptr;
-        }
-      }
-      t->tc_part_cap = 0;
-      if ((st = dev_alloc(t, &t->work.tc_m, need)) != SJ_OK) return st;
-      if ((st = dev_alloc(t, &t->work.tc_l, need)) != SJ_OK) return st;
-      if ((st = dev_alloc(t, &t->work.tc_o, need * t->dm.hd)) != SJ_OK) return st;
-      // slots of blocks that own no tile are read with weight zero: they must hold finite values
-      CU_TRY(cudaMemsetAsync(t->work.tc_m, 0, need * sizeof(float), t->stream));
-      CU_TRY(cudaMemsetAsync(t->work.tc_l, 0, need * sizeof(float), t->stream));
-      CU_TRY(cudaMemsetAsync(t->work.tc_o, 0, need * t->dm.hd * sizeof(float), t->stream));
-      t->tc_part_cap = need;
-    }
-  }
+  if ((t->opt_attn >= 1 || use_mega) && t->bf && kv->has_tm_pool)
+    if ((st = ensure_attn_partials(t, B, rows)) != SJ_OK) return st;
   if (logit_rows_needed > t->logits_rows) {
     CU_TRY(cudaStreamSynchronize(t->stream));
     clear_graphs(t);
@@ -1297,6 +1346,7 @@ extern "C" sj_status sj_verify(sj_target* t, sj_kv* kv, const sj_verify_args* a,
   h.p_draft = o->p_draft; h.new_kv_len = o->new_kv_len; h.dbg_hidden = o->dbg_hidden; h.dbg_logits = o->dbg_logits;
   h.B = B; h.gamma = gamma; h.mode = a->mode; h.use_align = a->use_align ? 1 : 0; h.use_judge = a->use_judge ? 1 : 0;
   h.commit = a->commit ? 1 : 0;
+  h.kv_rows = score_only ? 0 : 0x7fffffff;
   h.inv_temperature = a->mode == SJ_MODE_SAMPLING ? 1.0f / a->temperature : 1.0f;
   for (int i = 0; i < B; ++i)
     h.theta[i] = a->theta_per_seq ? a->theta_per_seq[i] : (a->theta_override >= 0.f ? a->theta_override : t->theta);
@@ -1316,7 +1366,7 @@ extern "C" sj_status sj_verify(sj_target* t, sj_kv* kv, const sj_verify_args* a,
     if (it == t->graphs.end()) {
       if (t->opt_gemm == 1) {  // encode activation maps before capturing
         const CUtensorMap* dummy;
-        if ((st = activation_map(t, t->mapA_d, t->work.A, R, t->dm.d, &dummy)) != SJ_OK) return st;
+        if ((st = activation_map(t, t->work.A, R, t->dm.d, &dummy)) != SJ_OK) return st;
       }
       cudaGraph_t graph = nullptr;
       CU_TRY(cudaStreamBeginCapture(t->stream, cudaStreamCaptureModeThreadLocal));
@@ -1351,12 +1401,16 @@ extern "C" sj_status sj_verify(sj_target* t, sj_kv* kv, const sj_verify_args* a,
   return SJ_OK;
 }
 
+extern "C" sj_status sj_verify(sj_target* t, sj_kv* kv, const sj_verify_args* a, const sj_verify_out* o) {
+  return verify_step(t, kv, a, o, false);
+}
+
 // ---------------------------------------------------------------------------------------------
 // chunked prefill and teacher-forced scoring: the verification step applied to known tokens
 // ---------------------------------------------------------------------------------------------
-// device scratch of one such block, in ints: [0,32) token ids, [32,64) accepted_len / next_token / new_kv_len,
-// [64,96) judge scores, [96,128) p_draft, [128,160) and [160,192) log-probabilities of two blocks, [192,194) a score
-constexpr int kBlockScratchInts = 8 * (SJ_MAX_GAMMA + 1);
+// device scratch of such a block (or two of them), in units of W = 32 ints: [0,2) token ids, [2,3) accepted_len /
+// next_token / new_kv_len, [3,5) judge scores, [5,7) p_draft, [7,9) log-probabilities, [9,10) a score
+constexpr int kBlockScratchInts = 10 * (SJ_MAX_GAMMA + 1);
 
 // s = sum_k (lp_z[k] - lp_y[k]) in index order (fp64), s_prefix = lp_z[0] - lp_y[0]
 __global__ void k_score_diff(const float* __restrict__ lp_z, const float* __restrict__ lp_y, int n, float* __restrict__ out) {
@@ -1385,36 +1439,129 @@ extern "C" sj_status sj_semantic_score(sj_target* t, sj_kv* kv, int seq, int y_i
   const int W = SJ_MAX_GAMMA + 1, gamma = n_future + 1;
   sj_verify_out o;
   memset(&o, 0, sizeof(o));
-  o.accepted_len = t->d_prefill + W;
-  o.next_token = o.accepted_len + 1;
-  o.new_kv_len = o.accepted_len + 2;
-  o.judge_scores = reinterpret_cast<float*>(t->d_prefill + 2 * W);
-  o.p_draft = reinterpret_cast<float*>(t->d_prefill + 3 * W);
-  float* lp[2] = {reinterpret_cast<float*>(t->d_prefill + 4 * W), reinterpret_cast<float*>(t->d_prefill + 5 * W)};
-  float* d_score = reinterpret_cast<float*>(t->d_prefill + 6 * W);
-  int block[SJ_MAX_GAMMA + 1];
-  for (int k = 0; k < n_future; ++k) block[1 + k] = future[k];
-  for (int pass = 0; pass < 2; ++pass) {   // the token-substituted response, then the original one
-    block[0] = pass == 0 ? z_i : y_i;
-    CU_TRY(cudaMemcpyAsync(t->d_prefill, block, sizeof(int) * gamma, cudaMemcpyHostToDevice, t->stream));
-    sj_verify_args a;
-    memset(&a, 0, sizeof(a));
-    a.B = 1;
-    a.gamma = gamma;
-    a.seq_ids = &seq;
-    a.draft_ids = t->d_prefill;
-    a.mode = SJ_MODE_GREEDY;
-    a.temperature = 1.f;
-    a.theta_override = -1.f;
-    a.accept_all = 1;
-    a.commit = 0;          // the cache and the pending token stay as they are
-    o.logp_draft = lp[pass];
-    sj_status st = sj_verify(t, kv, &a, &o);
+  o.accepted_len = t->d_prefill + 2 * W;
+  o.next_token = o.accepted_len + 2;
+  o.new_kv_len = o.accepted_len + 4;
+  o.judge_scores = reinterpret_cast<float*>(t->d_prefill + 3 * W);
+  o.p_draft = reinterpret_cast<float*>(t->d_prefill + 5 * W);
+  float* lp = reinterpret_cast<float*>(t->d_prefill + 7 * W);
+  float* d_score = reinterpret_cast<float*>(t->d_prefill + 9 * W);
+  int both[2 * (SJ_MAX_GAMMA + 1)];
+  for (int k = 0; k < n_future; ++k) both[1 + k] = future[k];
+  sj_verify_args a;
+  memset(&a, 0, sizeof(a));
+  a.gamma = gamma;
+  a.mode = SJ_MODE_GREEDY;
+  a.temperature = 1.f;
+  a.theta_override = -1.f;
+  a.accept_all = 1;
+  a.commit = 0;          // the cache and the pending token stay as they are
+  a.draft_ids = t->d_prefill;
+  const bool tc_attn = t->opt_attn >= 1 && t->bf && kv->has_tm_pool;
+  if (tc_attn && 2 * (gamma + 1) <= t->max_rows) {
+    // Both responses in one step, as two blocks over the same cache: the weights are read once (8B-shaped model, two
+    // blocks of 22 rows: 9.0 ms as two steps, 5.2 ms as one).
+    for (int k = 1; k < gamma; ++k) both[gamma + k] = both[k];
+    both[0] = z_i;
+    both[gamma] = y_i;
+    CU_TRY(cudaMemcpyAsync(t->d_prefill, both, sizeof(int) * 2 * gamma, cudaMemcpyHostToDevice, t->stream));
+    const int twice[2] = {seq, seq};
+    a.B = 2;
+    a.seq_ids = twice;
+    o.logp_draft = lp;
+    sj_status st = verify_step(t, kv, &a, &o, true);
     if (st != SJ_OK) return st;
+  } else {
+    for (int pass = 0; pass < 2; ++pass) {   // the token-substituted response, then the original one
+      both[0] = pass == 0 ? z_i : y_i;
+      CU_TRY(cudaMemcpyAsync(t->d_prefill, both, sizeof(int) * gamma, cudaMemcpyHostToDevice, t->stream));
+      a.B = 1;
+      a.seq_ids = &seq;
+      o.logp_draft = lp + pass * gamma;
+      sj_status st = verify_step(t, kv, &a, &o, false);
+      if (st != SJ_OK) return st;
+    }
   }
-  CU_TRY(launch(k_score_diff, dim3(1), dim3(32), 0, t->stream, false, (const float*)lp[0], (const float*)lp[1], gamma, d_score));
+  CU_TRY(launch(k_score_diff, dim3(1), dim3(32), 0, t->stream, false, (const float*)lp, (const float*)lp + gamma, gamma, d_score));
   CU_TRY(cudaMemcpyAsync(score, d_score, 2 * sizeof(float), cudaMemcpyDeviceToHost, t->stream));
   CU_TRY(cudaStreamSynchronize(t->stream));
+  return SJ_OK;
+}
+
+// Prefill in wide blocks: up to kPrefillRows known tokens go through the decoder layers at once, as B consecutive
+// entries of `c` rows each over the same sequence -- entry b attends to the stored cache plus the b * c rows before it
+// (its projection has stored them in the pages by the time the attention kernel runs) and to its own rows, which is
+// exactly what B verification steps of c rows one after another would do, at one read of the weights (8B-shaped model,
+// 1000 tokens and a step: 190 ms in blocks of 24 rows, 43.8 ms in three of 334).  Only the last token's row meets the
+// LM head, and a block that is not the last one ends with its key / value rows.
+constexpr int kPrefillRows = 352;      // rows of a wide block
+constexpr int kPrefillWideMin = 33;    // shorter prompts: one or two narrow blocks through the whole-step kernel
+
+static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* tokens, int n_tokens, int* d_next, bool* done) {
+  const Dims& dm = t->dm;
+  cudaStream_t s = t->stream;
+  sj_status st;
+  *done = false;
+  // a KV head's query rows fill at most one 128-lane accumulator
+  const int c_max = std::min((int)SJ_MAX_GAMMA + 1, 128 / (dm.Hq / dm.Hkv));
+  if (c_max < 2) return SJ_OK;
+  if (t->pf_rows == 0) {
+    const size_t mark = t->owned.size();
+    memset(&t->pf_work, 0, sizeof(Work));
+    st = alloc_rows(t, t->pf_work, kPrefillRows);
+    if (st == SJ_OK) st = alloc_partials(t, t->pf_work, kPrefillRows);
+    if (st != SJ_OK) {   // no memory for it: the narrow blocks need none
+      while (t->owned.size() > mark) { counted_free(t->owned.back()); t->owned.pop_back(); }
+      t->pf_rows = -1;
+    } else {
+      t->pf_rows = kPrefillRows;
+    }
+  }
+  if (t->pf_rows < 0) return SJ_OK;
+  if ((size_t)n_tokens > t->pf_tok_cap) {
+    CU_TRY(cudaStreamSynchronize(s));
+    if (t->d_pf_tok) {
+      counted_free(t->d_pf_tok);
+      t->owned.erase(std::remove(t->owned.begin(), t->owned.end(), (void*)t->d_pf_tok), t->owned.end());
+      t->d_pf_tok = nullptr;
+      t->pf_tok_cap = 0;
+    }
+    const size_t cap = std::max<size_t>(1024, (size_t)n_tokens * 2);
+    if ((st = dev_alloc(t, &t->d_pf_tok, cap)) != SJ_OK) return st;
+    t->pf_tok_cap = cap;
+  }
+  const int block = std::min(t->pf_rows / c_max, (int)SJ_MAX_BATCH) * c_max;
+  const int n_blocks = (n_tokens + block - 1) / block, per = (n_tokens + n_blocks - 1) / n_blocks;
+  if ((st = ensure_attn_partials(t, block / c_max, c_max)) != SJ_OK) return st;
+  Work W = t->pf_work;
+  W.tc_m = t->work.tc_m; W.tc_l = t->work.tc_l; W.tc_o = t->work.tc_o;
+  W.status = t->work.status; W.judge_w = t->work.judge_w; W.inv_freq = t->work.inv_freq;
+  if ((st = reserve(kv, seq, (long)kv->len_hi[seq] + n_tokens, nullptr)) != SJ_OK) return st;
+  CU_TRY(cudaMemcpyAsync(t->d_pf_tok, tokens, sizeof(int) * n_tokens, cudaMemcpyHostToDevice, s));
+  for (int i0 = 0; i0 < n_tokens; i0 += per) {
+    const int n = std::min(per, n_tokens - i0), B = (n + c_max - 1) / c_max, c = (n + B - 1) / B;
+    const bool last = i0 + n == n_tokens;
+    StepArgs h;
+    memset(&h, 0, sizeof(h));
+    h.draft_ids = h.row_tok = t->d_pf_tok + i0;
+    h.n_tok = n; h.pos_step = c; h.kv_rows = n;
+    h.B = B; h.gamma = c - 1; h.mode = SJ_MODE_GREEDY; h.inv_temperature = 1.f; h.top_k = 1; h.accept_all = 1;
+    for (int b = 0; b < B; ++b) h.seq_ids[b] = seq;
+    CU_TRY(cudaMemcpyAsync(t->d_args, &h, sizeof(h), cudaMemcpyHostToDevice, s));
+    if ((st = enqueue_layers<bf16>(t, kv, B, c - 1, 4096, W, 0, !last)) != SJ_OK) return st;
+    const int n_vtiles = (dm.V + kTileN - 1) / kTileN;
+    if (last) {
+      const CUtensorMap* mA = nullptr;
+      if ((st = activation_map(t, W.Asel, 1, dm.d, &mA)) != SJ_OK) return st;
+      CU_TRY(launch(k_select_rows<bf16>, dim3(1), dim3(256), sizeof(float) * dm.d, s, t->opt_pdl != 0, (const StepArgs*)t->d_args, W, dm,
+                    (const bf16*)t->final_norm, n - 1));
+      CU_TRY(launch_tc(t, t->s_lm, mA, &t->m_lm, nullptr, nullptr, 1, t->opt_pdl != 0, true, W));
+    }
+    CU_TRY(launch(k_prefill_commit, dim3(1), dim3(256), 0, s, t->opt_pdl != 0, kv->view, seq, n,
+                  (const RowStat*)(last ? W.stats : nullptr), n_vtiles, d_next));
+    kv->len_hi[seq] += n;
+  }
+  *done = true;
   return SJ_OK;
 }
 
@@ -1435,11 +1582,17 @@ extern "C" sj_status sj_prefill(sj_target* t, sj_kv* kv, int seq, const int* tok
   int* d_draft = t->d_prefill;
   sj_verify_out o;
   memset(&o, 0, sizeof(o));
-  o.accepted_len = t->d_prefill + (SJ_MAX_GAMMA + 1);
-  o.next_token = o.accepted_len + 1;
-  o.new_kv_len = o.accepted_len + 2;
-  o.judge_scores = reinterpret_cast<float*>(t->d_prefill + 2 * (SJ_MAX_GAMMA + 1));
-  o.p_draft = reinterpret_cast<float*>(t->d_prefill + 3 * (SJ_MAX_GAMMA + 1));
+  o.accepted_len = t->d_prefill + 2 * (SJ_MAX_GAMMA + 1);
+  o.next_token = o.accepted_len + 2;
+  o.new_kv_len = o.accepted_len + 4;
+  o.judge_scores = reinterpret_cast<float*>(t->d_prefill + 3 * (SJ_MAX_GAMMA + 1));
+  o.p_draft = reinterpret_cast<float*>(t->d_prefill + 5 * (SJ_MAX_GAMMA + 1));
+  bool done = false;
+  if (n_tokens >= kPrefillWideMin && t->bf && t->opt_gemm == 1 && t->opt_attn >= 1 && kv->has_tm_pool) {
+    sj_status st = prefill_wide(t, kv, seq, tokens, n_tokens, o.next_token, &done);
+    if (st != SJ_OK) return st;
+  }
+  if (done) n_tokens = 0;
   for (int i = 0; i < n_tokens;) {
     const int c = std::min(c_max, n_tokens - i);
     sj_status st = sj_kv_set_pending(kv, &seq, tokens + i, 1);
@@ -1531,7 +1684,7 @@ extern "C" sj_status sj_gemm_skinny(int dtype, int impl, int R, int N, int K, co
   if ((st = make_map(&mA, a, R, K, g.nblk)) != SJ_OK) { cleanup(); return st; }
   if ((st = make_map(&mW, w, N, K, kTileN)) != SJ_OK) { cleanup(); return st; }
   cudaError_t e = cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  if (e == cudaSuccess) e = launch_tc(&tmp, site, &mA, &mW, nullptr, nullptr, R, false, false);
+  if (e == cudaSuccess) e = launch_tc(&tmp, site, &mA, &mW, nullptr, nullptr, R, false, false, tmp.work);
   if (e == cudaSuccess)
     e = launch(k_sum_slots, dim3((unsigned)(((size_t)R * N + 255) / 256)), dim3(256), 0, s, false, (const float*)P,
                SplitPlan{site.d_tile_slots, site.n_tiles}, (size_t)R * N, R, N, y);
@@ -1635,7 +1788,7 @@ extern "C" sj_status sj_gemm_skinny_noalloc(int R, int N, int K, const void* a, 
   sj_status st;
   if ((st = make_map(&mA, a, R, K, g.nblk)) != SJ_OK) return st;
   if ((st = make_map(&mW, w, N, K, kTileN)) != SJ_OK) return st;
-  CU_TRY(launch_tc(&tmp, site, &mA, &mW, nullptr, nullptr, R, false, false));
+  CU_TRY(launch_tc(&tmp, site, &mA, &mW, nullptr, nullptr, R, false, false, tmp.work));
   CU_TRY(launch(k_sum_slots, dim3((unsigned)(((size_t)R * N + 255) / 256)), dim3(256), 0, s, false, (const float*)P,
                 SplitPlan{site.d_tile_slots, site.n_tiles}, (size_t)R * N, R, N, y));
   int hstatus = 0;

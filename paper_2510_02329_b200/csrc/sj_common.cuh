@@ -42,6 +42,12 @@ struct StepArgs {
   int B, gamma, mode, use_align, use_judge, commit;
   int top_k;              // greedy alignment test: the draft must be among the target's top_k tokens (1 or 2)
   int accept_all;         // every drafted position is accepted whatever the tests say (prefill, teacher forcing)
+  // A block that continues itself (prefill): entry b of the batch is the next `pos_step` rows of the same sequence, so
+  // its cache is pos_step * b tokens longer than the stored length, and row r's input token is row_tok[r] (r < n_tok;
+  // null: the pending token and the drafts).  0 and null in a verification step.
+  const int* row_tok;
+  int n_tok, pos_step;
+  int kv_rows;            // rows r >= kv_rows store no key / value rows in the pages (padding rows; blocks only scored)
   float inv_temperature, judge_bias;
   int has_judge;
   int seq_ids[kMaxBatch];

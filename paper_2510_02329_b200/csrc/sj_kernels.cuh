@@ -75,7 +75,7 @@ static __global__ void k_plan(const StepArgs* __restrict__ args, KvView kv, Work
   __shared__ int nch[kMaxBatch];
   const int B = args->B, rows = args->gamma + 1;
   for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    int L = kv.kv_len[args->seq_ids[b]];
+    int L = kv.kv_len[args->seq_ids[b]] + b * args->pos_step;
     nch[b] = (L + rows + chunk_len - 1) / chunk_len;
     for (int j = 0; j < rows; ++j) w.row_pos[b * rows + j] = L + j;
   }
@@ -117,7 +117,9 @@ __global__ void k_embed_norm(const StepArgs* __restrict__ args, KvView kv, Work 
   const int r = blockIdx.x, rows = args->gamma + 1;
   const int b = r / rows, j = r % rows;
   const int seq = args->seq_ids[b];
-  int tok = (j == 0) ? kv.pending[seq] : args->draft_ids[b * args->gamma + j - 1];
+  int tok;
+  if (args->row_tok) tok = args->row_tok[min(r, args->n_tok - 1)];
+  else tok = (j == 0) ? kv.pending[seq] : args->draft_ids[b * args->gamma + j - 1];
   tok = min(max(tok, 0), dm.V - 1);
   const T* e = embed + (size_t)tok * dm.d;
   for (int i = threadIdx.x; i < dm.d; i += blockDim.x) {
@@ -125,7 +127,7 @@ __global__ void k_embed_norm(const StepArgs* __restrict__ args, KvView kv, Work 
     xs[i] = x;
     w.X[(size_t)r * dm.d + i] = x;
   }
-  const int pos = kv.kv_len[seq] + j;
+  const int pos = kv.kv_len[seq] + b * args->pos_step + j;
   for (int i = threadIdx.x; i < dm.hd / 2; i += blockDim.x) {
     double s, c;
     sincos((double)pos * w.inv_freq[i], &s, &c);
@@ -168,7 +170,8 @@ __global__ void k_qkv_rope(const StepArgs* __restrict__ args, KvView kv, Work w,
   const int pos = w.row_pos[r];
   const int half = dm.hd / 2;
   const int qd = dm.Hq * dm.hd, kd = dm.Hkv * dm.hd, N = qd + 2 * kd;
-  const int page = kv.block_table[(size_t)seq * kv.max_pages_per_seq + pos / kv.page_size];
+  const bool store_kv = r < args->kv_rows;   // block-uniform
+  const int page = store_kv ? kv.block_table[(size_t)seq * kv.max_pages_per_seq + pos / kv.page_size] : 0;
   const int slot = pos % kv.page_size;
   const float2* rt = w.rope + (size_t)r * half;
   // rotated heads: q heads then k heads
@@ -201,9 +204,11 @@ __global__ void k_qkv_rope(const StepArgs* __restrict__ args, KvView kv, Work w,
         ql[i + half] = __float2half_rn(y2 * qs - __half2float(h2));
       }
     } else {
-      T* krow = kv_row<T>(kv, layer, page, 0, head - dm.Hq, slot);
-      krow[i] = from_f<T>(y1);
-      krow[i + half] = from_f<T>(y2);
+      if (store_kv) {
+        T* krow = kv_row<T>(kv, layer, page, 0, head - dm.Hq, slot);
+        krow[i] = from_f<T>(y1);
+        krow[i + half] = from_f<T>(y2);
+      }
       if (w.KVn) {
         __half* kn = w.KVn + ((((size_t)b * dm.Hkv + head - dm.Hq) * 2) * rows + r % rows) * dm.hd;
         kn[i] = __float2half_rn(y1);
@@ -214,8 +219,7 @@ __global__ void k_qkv_rope(const StepArgs* __restrict__ args, KvView kv, Work w,
   for (int p = threadIdx.x; p < kd; p += blockDim.x) {
     float x = reduce_partials(w.P, sp, slot_stride, N, r, qd + kd + p);
     if (bv) x += to_f(bv[p]);
-    T* vrow = kv_row<T>(kv, layer, page, 1, p / dm.hd, slot);
-    vrow[p % dm.hd] = from_f<T>(x);
+    if (store_kv) kv_row<T>(kv, layer, page, 1, p / dm.hd, slot)[p % dm.hd] = from_f<T>(x);
     if (w.KVn) w.KVn[((((size_t)b * dm.Hkv + p / dm.hd) * 2 + 1) * rows + r % rows) * dm.hd + p % dm.hd] = __float2half_rn(x);
   }
 }
@@ -621,16 +625,16 @@ static __global__ void k_finalize(const StepArgs* __restrict__ args, KvView kv, 
 }
 
 // a14, sampling mode, first half: the row the emitted token is drawn from (row n_b of sequence b, known only
-// after the first-rejection scan) is normalised again into a compact set of GEMM input planes, one row per
+// after the first-rejection scan; a given row when row >= 0: prefill) is normalised again into a compact set of GEMM input planes, one row per
 // sequence; a second LM-head pass over those B rows then yields the only logits the step ever stores.
 template <typename T>
-__global__ void k_select_rows(const StepArgs* __restrict__ args, Work w, Dims dm, const T* __restrict__ gain) {
+__global__ void k_select_rows(const StepArgs* __restrict__ args, Work w, Dims dm, const T* __restrict__ gain, int row) {
   extern __shared__ float xs[];
   __shared__ float red[32];
   pdl_wait();
   pdl_launch();
   const int b = blockIdx.x, rows = args->gamma + 1;
-  const int r = b * rows + min(max(args->accepted_len[b], 0), rows - 1);
+  const int r = row >= 0 ? row : b * rows + min(max(args->accepted_len[b], 0), rows - 1);
   for (int i = threadIdx.x; i < dm.d; i += blockDim.x) xs[i] = w.X[(size_t)r * dm.d + i];
   __syncthreads();
   norm_row_from_smem<T>(xs, dm.d, gain, dm.eps, w.Asel, gridDim.x, b, nullptr, nullptr, red);
@@ -685,6 +689,33 @@ static __global__ void k_resample(const StepArgs* __restrict__ args, KvView kv, 
       if (args->commit) kv.pending[args->seq_ids[b]] = winner;
     }
     break;
+  }
+}
+
+// The end of a prefill block of n tokens: the sequence is n tokens longer; with `stats` (softmax statistics of the last
+// token's row per vocabulary tile) its arg max becomes the pending token.
+static __global__ void k_prefill_commit(KvView kv, int seq, int n, const RowStat* __restrict__ stats, int n_vtiles, int* next) {
+  pdl_wait();
+  pdl_launch();
+  __shared__ RowStat sred[256];
+  const int tid = threadIdx.x;
+  if (stats) {
+    RowStat a; a.m = -INFINITY; a.s = 0.f; a.arg = 0; a.pad = 0;
+    const int per = (n_vtiles + 255) / 256, t1 = min((tid + 1) * per, n_vtiles);
+    for (int t = tid * per; t < t1; ++t) a = stat_merge(a, stats[t]);
+    sred[tid] = a;
+    __syncthreads();
+    for (int stride = 1; stride < 256; stride <<= 1) {
+      if ((tid & (2 * stride - 1)) == 0) sred[tid] = stat_merge(sred[tid], sred[tid + stride]);
+      __syncthreads();
+    }
+  }
+  if (tid == 0) {
+    if (stats) {
+      *next = sred[0].arg;
+      kv.pending[seq] = sred[0].arg;
+    }
+    kv.kv_len[seq] += n;
   }
 }
 

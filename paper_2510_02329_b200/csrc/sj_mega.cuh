@@ -142,7 +142,7 @@ struct MegaCtl {
   int row_b[kMegaMaxRows], row_j[kMegaMaxRows], row_page[kMegaMaxRows], row_slot[kMegaMaxRows], tgt_tok[kMegaMaxRows];
   int row_qoff[kMegaMaxRows];         // element offset of row r's queries in the query buffer, without the head part
   int row_nkvoff[kMegaMaxRows];       // element offset of row r in the fp16 copy of the step's own K/V rows, without head / K|V part
-  long long row_kvoff[kMegaMaxRows];  // element offset of row r's slot in its cache page, without layer / K|V / head part
+  long long row_kvoff[kMegaMaxRows];  // element offset of row r's slot in its cache page, without layer / K|V / head part; -1: not stored
   float red[2][4][8];          // [group][warp][row of the chunk]
   RowStat wstat[2][4][8];
   RowStat rs[kMaxGamma + 1];
@@ -626,7 +626,7 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
                       ((size_t)l * kv.n_pages * 2 * dm.Hkv + (size_t)(kind - 1) * dm.Hkv + head) * kv.page_size * HD + dim;
 #pragma unroll
           for (int i = 0; i < NS; ++i)
-            if (i < nr) kvb[ctl->row_kvoff[c0 + i]] = __float2bfloat16_rn(v[i]);
+            if (i < nr && ctl->row_kvoff[c0 + i] >= 0) kvb[ctl->row_kvoff[c0 + i]] = __float2bfloat16_rn(v[i]);
           __half* kn = w.KVn + (size_t)(head * 2 + kind - 1) * rows * HD + dim;
 #pragma unroll
           for (int i = 0; i < NS; ++i)
@@ -1012,12 +1012,13 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
     const int pos = ctl->plan.L[b] + j;
     ctl->row_b[r] = b;
     ctl->row_j[r] = j;
-    ctl->row_page[r] = kv.block_table[(size_t)args->seq_ids[b] * kv.max_pages_per_seq + pos / kv.page_size];
+    const bool store_kv = r < args->kv_rows;
+    ctl->row_page[r] = store_kv ? kv.block_table[(size_t)args->seq_ids[b] * kv.max_pages_per_seq + pos / kv.page_size] : 0;
     ctl->row_slot[r] = pos % kv.page_size;
     ctl->tgt_tok[r] = (j < gamma) ? args->draft_ids[b * gamma + j] : -1;
     ctl->row_qoff[r] = (b * dm.Hq * rows + j) * dm.hd;
     ctl->row_nkvoff[r] = (b * dm.Hkv * 2 * rows + j) * dm.hd;
-    ctl->row_kvoff[r] = ((long long)ctl->row_page[r] * 2 * dm.Hkv * kv.page_size + ctl->row_slot[r]) * dm.hd;
+    ctl->row_kvoff[r] = store_kv ? ((long long)ctl->row_page[r] * 2 * dm.Hkv * kv.page_size + ctl->row_slot[r]) * dm.hd : -1;
   }
   __syncthreads();
 

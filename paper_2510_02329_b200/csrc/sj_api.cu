@@ -16,6 +16,7 @@
 #include "sj_attn_tc.cuh"
 #include "sj_attn_t5.cuh"
 #include "sj_gemm_tc.cuh"
+#include "sj_gemm_pair.cuh"
 #include "sj_mega.cuh"
 
 using namespace sj;
@@ -226,7 +227,8 @@ struct sj_target {
   size_t tc_part_cap = 0;   // floats in tc_m / tc_l
   size_t logits_rows = 0;
   std::map<StepKey, cudaGraphExec_t> graphs;
-  std::map<std::pair<const void*, int>, CUtensorMap> act_maps;  // per activation matrix and row count
+  std::map<std::pair<const void*, int>, CUtensorMap> act_maps;   // per activation matrix and row count
+  std::map<std::tuple<const void*, int, int>, CUtensorMap> pair_maps;   // the same per box height, for the paired projections
   // prefill in wide blocks (allocated by the first call that can use it): a workspace of kPrefillRows rows, the tokens
   Work pf_work;
   int pf_rows = 0;                 // rows of pf_work; 0: not there yet, -1: no memory for it
@@ -336,6 +338,7 @@ static sj_status alloc_rows(sj_target* t, Work& W, int R) {
     get(&W.Qlo, R * qd);
     get(&W.KVn, (size_t)R * 2 * kd);
   }
+  if (t->bf) get(&W.ssq, (size_t)2 * (d / kTileN + 1) * R);
   get(&W.Hf, R * d);
   get(&W.rope, (size_t)R * (c.head_dim / 2));
   get(&W.row_pos, R);
@@ -357,6 +360,17 @@ static sj_status alloc_partials(sj_target* t, Work& W, int R) {
     for (TcSite* s : {&t->s_qkv, &t->s_o, &t->s_gu, &t->s_down}) n = std::max(n, (size_t)s->max_slots * R * s->N);
   }
   return dev_alloc(t, &W.P, n);
+}
+
+typedef void (*PairKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const PairParams, const StepArgs*,
+                           const KvView, const Work, const Dims);
+static PairKernel pair_kernel(int site, int hd) {
+  switch (site) {
+    case PAIR_QKV: return hd == 128 ? k_gemm_pair<PAIR_QKV, 128> : k_gemm_pair<PAIR_QKV, 64>;
+    case PAIR_RES: return k_gemm_pair<PAIR_RES, 0>;
+    case PAIR_GU: return k_gemm_pair<PAIR_GU, 0>;
+    default: return k_gemm_pair<PAIR_LM, 0>;
+  }
 }
 
 extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weights* w, void* cuda_stream,
@@ -464,6 +478,8 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
     }
     if ((st = make_map(&t->m_lm, t->lm_head, c.vocab, c.d_model, kTileN)) != SJ_OK) return bail(st);
     cudaError_t e = cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    for (int site = PAIR_QKV; site <= PAIR_LM && e == cudaSuccess; ++site)
+      e = cudaFuncSetAttribute(pair_kernel(site, c.head_dim), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) { fail(SJ_ERR_CUDA, "smem opt-in: %s", cudaGetErrorString(e)); return bail(SJ_ERR_CUDA); }
   }
   if ((st = alloc_partials(t, W, R)) != SJ_OK) return bail(st);
@@ -912,6 +928,90 @@ static cudaError_t launch_tc(sj_target* t, const TcSite& s, const CUtensorMap* m
                 *(w2 ? w2 : w0), p, (const StepArgs*)t->d_args, W, t->dm.V);
 }
 
+// Paired projections (sj_gemm_pair.cuh): geometry of a site of n_tiles 128-feature tiles for R rows.
+struct PairGeom { int rb, n_rb, stages, stage_bytes; uint32_t tmem_cols; size_t smem; };
+static PairGeom pair_geom(int R, int n_tiles, int n_pairs, int site) {
+  PairGeom g;
+  memset(&g, 0, sizeof(g));
+  // rows per block: fewest rounds of items times the clocks a K step takes (shared-memory port, tensor pipe)
+  long best = 0;
+  for (int n_rb = (R + 127) / 128; n_rb <= (R + 15) / 16; ++n_rb) {
+    const int rb = round_up((R + n_rb - 1) / n_rb, 16), n = (R + rb - 1) / rb;
+    const long rounds = ((n_tiles + 1) / 2 * n + n_pairs - 1) / n_pairs, cost = rounds * std::max(256 + 2 * rb, 4 * rb);
+    if (!best || cost < best) { best = cost; g.rb = rb; g.n_rb = n; }
+  }
+  g.tmem_cols = 32;
+  while (g.tmem_cols < (uint32_t)(4 * g.rb)) g.tmem_cols <<= 1;
+  g.stage_bytes = kWTileBytes + g.rb * 128;
+  const size_t ctl = site == PAIR_QKV ? sizeof(PairSmem<PAIR_QKV>) : site == PAIR_RES ? sizeof(PairSmem<PAIR_RES>)
+                     : site == PAIR_GU ? sizeof(PairSmem<PAIR_GU>) : sizeof(PairSmem<PAIR_LM>);
+  g.stages = std::min<int>(kPairMaxStages, (int)((227 * 1024 - 1024 - ctl) / g.stage_bytes));
+  g.smem = (size_t)g.stages * g.stage_bytes + ctl + 1024;
+  return g;
+}
+
+// An activation matrix (two planes of pad16(R) rows) with boxes of 64 columns x rb rows.
+static sj_status pair_map(sj_target* t, const void* base, int R, int rb, int K, const CUtensorMap** out) {
+  const std::tuple<const void*, int, int> key{base, R, rb};
+  auto it = t->pair_maps.find(key);
+  if (it == t->pair_maps.end()) {
+    CUtensorMap m;
+    sj_status st = make_map(&m, base, 2 * pad16(R), K, rb);
+    if (st != SJ_OK) return st;
+    it = t->pair_maps.emplace(key, m).first;
+  }
+  *out = &it->second;
+  return SJ_OK;
+}
+
+struct PairOut {   // what a site's epilogue needs beyond the step's workspace
+  const float* ssq_in = nullptr;
+  float* ssq_out = nullptr;
+  const void* gain = nullptr;
+  void* planes_out = nullptr;
+  int K_out = 0, layer = 0;
+  const void *bq = nullptr, *bk = nullptr, *bv = nullptr;
+};
+static sj_status launch_pair(sj_target* t, sj_kv* kv, int site, int n_tiles, int K, const void* act, const CUtensorMap* w0, const CUtensorMap* w1,
+                             const CUtensorMap* w2, int R, bool pdl, const Work& W, const PairOut& o) {
+  const Dims& dm = t->dm;
+  const int n_pairs = t->sm_count / 2;
+  const PairGeom g = pair_geom(R, n_tiles, n_pairs, site);
+  const CUtensorMap* mA = nullptr;
+  sj_status st = pair_map(t, act, R, g.rb, K, &mA);
+  if (st != SJ_OK) return st;
+  PairParams p;
+  memset(&p, 0, sizeof(p));
+  p.n_tiles = n_tiles; p.KB = K / kBK; p.R = R; p.rb = g.rb; p.n_rb = g.n_rb; p.plane_rows = pad16(R);
+  p.n_pairs = std::min(n_pairs, (n_tiles + 1) / 2 * g.n_rb);
+  p.stages = g.stages; p.stage_bytes = g.stage_bytes; p.tmem_cols = g.tmem_cols;
+  p.tile_q = dm.Hq * dm.hd / kTileN; p.tile_k = p.tile_q + dm.Hkv * dm.hd / kTileN;
+  p.ssq_in = o.ssq_in; p.ssq_out = o.ssq_out; p.gain = (const bf16*)o.gain; p.planes_out = o.planes_out; p.K_out = o.K_out; p.layer = o.layer;
+  p.bq = (const bf16*)o.bq; p.bk = (const bf16*)o.bk; p.bv = (const bf16*)o.bv;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(2 * p.n_pairs);
+  cfg.blockDim = dim3(kPairThreads);
+  cfg.dynamicSmemBytes = g.smem;
+  cfg.stream = t->stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 2 : 1;
+  CU_TRY(cudaLaunchKernelEx(&cfg, pair_kernel(site, dm.hd), *mA, *w0, *(w1 ? w1 : w0), *(w2 ? w2 : w0), p, (const StepArgs*)t->d_args,
+                            kv->view, W, dm));
+  return SJ_OK;
+}
+
+// Steps of more rows than the persistent kernel takes run their projections on pairs of SMs.
+constexpr int kPairMinRows = kMegaMaxRows + 1;
+static bool pair_usable(const sj_target* t, const sj_kv* kv, int R) {
+  return t->opt_gemm == 1 && t->opt_attn >= 1 && t->bf && kv->has_tm_pool && R >= kPairMinRows;
+}
+
 // a14 in sampling mode with the tensor-core LM head: re-normalise the one row per sequence that the emitted
 // token is drawn from, run the LM head over those B rows into the [B, V] logit scratch, draw the token.
 template <typename T>
@@ -935,19 +1035,31 @@ static cudaError_t launch_simt(sj_target* t, const void* A, const GemmSegs& segs
 }
 
 // Launch `expr`; in timing mode bracket it with events filed under `name`.
+#define TIMED_BEGIN                                                              \
+  cudaEvent_t ea_ = nullptr, eb_ = nullptr;                                      \
+  if (timing) {                                                                  \
+    CU_TRY(cudaEventCreate(&ea_));                                               \
+    CU_TRY(cudaEventCreate(&eb_));                                               \
+    CU_TRY(cudaEventRecord(ea_, s));                                             \
+  }
+#define TIMED_END(name)                                                          \
+  if (timing) {                                                                  \
+    CU_TRY(cudaEventRecord(eb_, s));                                             \
+    t->timed.push_back({name, ea_, eb_});                                        \
+  }
 #define TIMED(name, expr)                                                        \
   do {                                                                           \
-    cudaEvent_t ea_ = nullptr, eb_ = nullptr;                                    \
-    if (timing) {                                                                \
-      CU_TRY(cudaEventCreate(&ea_));                                             \
-      CU_TRY(cudaEventCreate(&eb_));                                             \
-      CU_TRY(cudaEventRecord(ea_, s));                                           \
-    }                                                                            \
+    TIMED_BEGIN                                                                  \
     CU_TRY(expr);                                                                \
-    if (timing) {                                                                \
-      CU_TRY(cudaEventRecord(eb_, s));                                           \
-      t->timed.push_back({name, ea_, eb_});                                      \
-    }                                                                            \
+    TIMED_END(name)                                                              \
+  } while (0)
+// the same for an expression of type sj_status
+#define TIMED_ST(name, expr)                                                     \
+  do {                                                                           \
+    TIMED_BEGIN                                                                  \
+    const sj_status st_ = (expr);                                                \
+    if (st_ != SJ_OK) return st_;                                                \
+    TIMED_END(name)                                                              \
   } while (0)
 
 // The decoder layers of a step (set-up and embedding included): from the step's arguments to the GEMM input planes of
@@ -973,6 +1085,8 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
     if ((st = activation_map(t, W.ATT, R, qd, &mA_q)) != SJ_OK) return st;
     if ((st = activation_map(t, W.H, R, dm.F, &mA_f)) != SJ_OK) return st;
   }
+  const bool pair = pair_usable(t, kv, R);
+  const size_t ssq_n = (size_t)(dm.d / kTileN) * R;
   auto plan_of = [&](const TcSite& site) { return tc ? SplitPlan{site.d_tile_slots, site.n_tiles} : one; };
 
   TIMED("plan", launch(k_plan, dim3(1), dim3(256), 0, s, false, args, kv->view, W, chunk_len));
@@ -983,15 +1097,23 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
   const int att_grid = std::max(1, std::min<int>(t->sm_count * 2, (int)n_chunks_hi * dm.Hkv));
   for (int l = 0; l < dm.n_layers; ++l) {
     const LayerW& L = t->layers[l];
-    // QKV projection
-    if (tc) {
-      TIMED("gemm_qkv", launch_tc(t, t->s_qkv, mA_d, &L.m_q, &L.m_k, &L.m_v, R, pdl, true, W));
+    // QKV projection, bias, rotary embedding, cache append
+    if (pair) {
+      PairOut o;
+      o.ssq_in = l > 0 ? W.ssq : nullptr;
+      o.layer = l;
+      o.bq = L.bq; o.bk = L.bk; o.bv = L.bv;
+      TIMED_ST("gemm_qkv", launch_pair(t, kv, PAIR_QKV, t->s_qkv.n_tiles, dm.d, W.A, &L.m_q, &L.m_k, &L.m_v, R, pdl, W, o));
     } else {
-      GemmSegs g{{L.wq, L.wk, L.wv}, {qd, kd, kd}, 3};
-      TIMED("gemm_cudacore", launch_simt<T>(t, W.A, g, W.P, R, qd + 2 * kd, dm.d, pdl));
+      if (tc) {
+        TIMED("gemm_qkv", launch_tc(t, t->s_qkv, mA_d, &L.m_q, &L.m_k, &L.m_v, R, pdl, true, W));
+      } else {
+        GemmSegs g{{L.wq, L.wk, L.wv}, {qd, kd, kd}, 3};
+        TIMED("gemm_cudacore", launch_simt<T>(t, W.A, g, W.P, R, qd + 2 * kd, dm.d, pdl));
+      }
+      TIMED("qkv_rope", launch(k_qkv_rope<T>, dim3(R), dim3(256), 0, s, pdl, args, kv->view, W, dm, plan_of(t->s_qkv),
+                    (size_t)R * (qd + 2 * kd), l, (const T*)L.bq, (const T*)L.bk, (const T*)L.bv));
     }
-    TIMED("qkv_rope", launch(k_qkv_rope<T>, dim3(R), dim3(256), 0, s, pdl, args, kv->view, W, dm, plan_of(t->s_qkv),
-                  (size_t)R * (qd + 2 * kd), l, (const T*)L.bq, (const T*)L.bk, (const T*)L.bv));
     if (kv_only && l == dm.n_layers - 1) return SJ_OK;
     // attention
     if (attn_tc) {
@@ -1014,6 +1136,19 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
     } else {
       TIMED("attn", launch(k_attn_simt<T>, dim3(att_grid), dim3(kAttThreads), att_smem, s, pdl, args, kv->view, W, dm, l, chunk_len));
       TIMED("attn_combine", launch(k_attn_combine<T>, dim3(R * dm.Hq), dim3(std::min(dm.hd, 128)), 0, s, pdl, args, W, dm));
+    }
+    if (pair) {   // O, gate/up and down with their epilogues
+      PairOut o, gu, dn;
+      o.ssq_out = W.ssq + ssq_n; o.gain = L.nf; o.planes_out = W.A;
+      TIMED_ST("gemm_o", launch_pair(t, kv, PAIR_RES, dm.d / kTileN, qd, W.ATT, &L.m_o, nullptr, nullptr, R, pdl, W, o));
+      gu.ssq_in = W.ssq + ssq_n; gu.planes_out = W.H; gu.K_out = dm.F;
+      TIMED_ST("gemm_gateup", launch_pair(t, kv, PAIR_GU, dm.F / 64, dm.d, W.A, &L.m_g64, &L.m_u64, nullptr, R, pdl, W, gu));
+      dn.ssq_out = W.ssq; dn.planes_out = W.A;
+      dn.gain = l + 1 < dm.n_layers ? t->layers[l + 1].na : t->final_norm;
+      TIMED_ST("gemm_down", launch_pair(t, kv, PAIR_RES, dm.d / kTileN, dm.F, W.H, &L.m_d, nullptr, nullptr, R, pdl, W, dn));
+      if (l == dm.n_layers - 1)
+        TIMED("final_norm", launch(k_final_norm<T>, dim3(R), dim3(256), row_smem, s, pdl, args, W, dm, (const T*)t->final_norm));
+      continue;
     }
     // O projection + residual + FFN norm
     if (tc) {
@@ -1067,7 +1202,10 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
   const int n_vtiles = (dm.V + kTileN - 1) / kTileN;
   if (tc) {
     TIMED("target_logits", launch(k_target_logits, dim3((R + 7) / 8), dim3(256), 0, s, pdl, args, W, dm, (const bf16*)t->lm_head, R));
-    TIMED("gemm_lm_head", launch_tc(t, t->s_lm, mA_d, &t->m_lm, nullptr, nullptr, R, pdl, true, W));   // W: no [R, V] logit store
+    if (pair_usable(t, kv, R))
+      TIMED_ST("gemm_lm_head", launch_pair(t, kv, PAIR_LM, n_vtiles, dm.d, W.A, &t->m_lm, nullptr, nullptr, R, pdl, W, PairOut()));
+    else
+      TIMED("gemm_lm_head", launch_tc(t, t->s_lm, mA_d, &t->m_lm, nullptr, nullptr, R, pdl, true, W));   // W: no [R, V] logit store
   } else {
     GemmSegs g{{t->lm_head, nullptr, nullptr}, {dm.V, 0, 0}, 1};
     TIMED("gemm_cudacore", launch_simt<T>(t, W.A, g, W.logits, R, dm.V, dm.d, pdl));
@@ -1086,6 +1224,9 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
 }
 
 #undef TIMED
+#undef TIMED_ST
+#undef TIMED_BEGIN
+#undef TIMED_END
 
 // The whole step as one cooperative launch per chunk of kMegaMaxLayers layers.
 static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma) {
@@ -1509,7 +1650,7 @@ static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* token
     const size_t mark = t->owned.size();
     memset(&t->pf_work, 0, sizeof(Work));
     st = alloc_rows(t, t->pf_work, kPrefillRows);
-    if (st == SJ_OK) st = alloc_partials(t, t->pf_work, kPrefillRows);
+    if (st == SJ_OK) st = alloc_partials(t, t->pf_work, kPairMinRows - 1);   // wider blocks need none
     if (st != SJ_OK) {   // no memory for it: the narrow blocks need none
       while (t->owned.size() > mark) { counted_free(t->owned.back()); t->owned.pop_back(); }
       t->pf_rows = -1;

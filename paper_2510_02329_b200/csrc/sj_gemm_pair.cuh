@@ -1,0 +1,473 @@
+// Projections of wide steps (more block rows than the persistent kernel takes) on pairs of SMs, with fused epilogues.
+//
+//   D[256 features, rb rows] (fp32, tensor memory) = W_tile[256, K] (bf16) x A[rb, K]^T (two bf16 planes)
+// A pair of CTAs (tcgen05 cta_group::2) computes one 256-feature tile for a block of rb <= 128 rows over the whole of K:
+// CTA `rank` holds the weights and the accumulator of features [128 rank, +128).  The MMA's N = 2 rb columns are the
+// block's rows twice: the hi plane, staged by rank 0, and the lo plane, staged by rank 1; each SM's tensor core reads
+// both.  The epilogue adds the two halves.  Accumulators are double-buffered, so an item's epilogue runs beside the next
+// item's MMAs.
+//
+// Why this shape: what bounds wide steps is the shared-memory port (128 B/clk per SM).  A K step of 64 writes
+// 16 KiB of weights and 128 rb bytes of activations and its four MMAs read 4 (4096 + 32 rb) back: 256 + 2 rb clocks, for
+// 4 rb clocks of tensor time (512 and 512 at rb = 128).  A single CTA with both planes of 288 rows needs 1790 clocks for
+// 1152 of tensor time.  Cutting the rows instead of K costs re-reads of the weights from L2 (pairs that share a tile
+// run side by side) but no exchange of sums: a first version of this kernel that split K over the pairs was bound by
+// the pair that finished a tile for all of them.
+//
+// Items (tile, row block), row blocks fastest, are dealt round robin: pair g takes items g, g + n_pairs, ...  The host
+// picks rb by the model above (pair_geom): fewest rounds times clocks per round.
+//
+// Epilogues (template SITE) -- the same arithmetic as the persistent kernel's: the planes hold x * gain and the row scalar
+// 1/rms, from per-tile sums of squares, is applied by the consumer.
+//   QKV  -> 1/rms, bias, rotary embedding; queries (fp16), K / V rows into the pages (bf16) and the step's side buffer
+//   O, down -> residual add, next GEMM's input planes, sums of squares
+//   gate/up (a CTA's tile interleaves 64 gate and 64 up features) -> silu(g) * u -> down's input planes
+//   LM head -> softmax statistics per (128-token tile, row)
+#pragma once
+
+#include "sj_gemm_tc.cuh"
+
+namespace sj {
+
+constexpr int kPairThreads = 384;      // warp 0 TMA, warp 1 MMA (rank 0), warp 2 tensor memory, warps 4..11 epilogue
+constexpr int kPairWorkers = 256;
+constexpr int kPairMaxStages = 10;
+constexpr int kPairMaxRows = kMaxRows;
+constexpr uint32_t kPairSpin = 1u << 22;
+
+enum PairSite { PAIR_QKV = 0, PAIR_RES = 1, PAIR_GU = 2, PAIR_LM = 3 };
+
+struct PairParams {
+  int n_tiles;            // 128-feature tiles (gate/up: 64 + 64); an odd last one is paired with zeros
+  int KB;                 // K blocks of 64
+  int n_pairs;
+  int R, rb, n_rb;        // rows, rows per block (a multiple of 16, at most 128: an M = 256 MMA takes N = 32, 64 .. 256), row blocks
+  int plane_rows;         // row of the lo plane in the activation matrix
+  int stages, stage_bytes;
+  uint32_t tmem_cols;     // two accumulators of 2 rb columns
+  int tile_q, tile_k;     // QKV: tiles of Wq, tiles of Wq and Wk together
+  const float* ssq_in;    // [d / 128][R] sums of squares of this GEMM's input rows (null: the planes are normalised)
+  float* ssq_out;         // [d / 128][R] PAIR_RES
+  const bf16* gain;       // PAIR_RES: gain of the norm that reads the result next
+  void* planes_out;       // PAIR_RES: W.A; PAIR_GU: W.H
+  int K_out;              // row length of planes_out
+  int layer;
+  const bf16 *bq, *bk, *bv;
+};
+
+struct PairCtl {
+  uint64_t full[kPairMaxStages], empty[kPairMaxStages], tmem_full[2], tmem_empty[2];
+  uint32_t tmem_base;
+  int abort_flag;
+  float inv[kPairMaxRows];
+};
+struct PairQkvCtl {
+  int qoff[kPairMaxRows], nkvoff[kPairMaxRows];
+  long long kvoff[kPairMaxRows];   // -1: the row is not stored
+  float exch[2][128][9];
+};
+struct PairGuCtl { float exch[2][128][9]; };
+struct PairResCtl { float sums[4][kPairMaxRows]; };
+struct PairLmCtl {
+  int tok[kPairMaxRows];
+  float pre[kPairMaxRows];
+  RowStat st[2][4][16];
+};
+template <int SITE> struct PairExtra;
+template <> struct PairExtra<PAIR_QKV> { typedef PairQkvCtl type; };
+template <> struct PairExtra<PAIR_RES> { typedef PairResCtl type; };
+template <> struct PairExtra<PAIR_GU> { typedef PairGuCtl type; };
+template <> struct PairExtra<PAIR_LM> { typedef PairLmCtl type; };
+template <int SITE> struct PairSmem { PairCtl c; typename PairExtra<SITE>::type x; };
+
+// ---- cta_group::2 wrappers -----------------------------------------------------------------------
+constexpr uint32_t kPeerMask = 0xFEFFFFFFu;   // a shared::cluster address with the CTA bit cleared: the pair's rank 0
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void pair_tma_2d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%3, %4}], [%2], %5;" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(bar & kPeerMask), "r"(c0), "r"(c1), "l"(policy)
+      : "memory");
+}
+__device__ __forceinline__ void pair_commit(uint32_t bar) {   // arrives on `bar` of both CTAs
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((uint16_t)3)
+      : "memory");
+}
+__device__ __forceinline__ void pair_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void pair_arrive_rank0(uint32_t bar) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(bar));
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
+}
+__device__ __forceinline__ uint32_t instr_desc_pair(int n) {   // M = 256
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+}
+
+// Sum of 16 values over the 32 lanes of a warp, all 16 at once (16 shuffles instead of 80): lanes 2i and 2i + 1 return
+// the total of value i.
+__device__ __forceinline__ float warp_sum16(const float* v, int lane) {
+  float a[8], b[4], c[2];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const bool up = lane & 16;
+    a[i] = (up ? v[i + 8] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + 8], 16);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const bool up = lane & 8;
+    b[i] = (up ? a[i + 4] : a[i]) + __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + 4], 8);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const bool up = lane & 4;
+    c[i] = (up ? b[i + 2] : b[i]) + __shfl_xor_sync(0xffffffffu, up ? b[i] : b[i + 2], 4);
+  }
+  const bool up = lane & 2;
+  float d = (up ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, up ? c[0] : c[1], 2);
+  return d + __shfl_xor_sync(0xffffffffu, d, 1);
+}
+
+template <int SITE, int HD>
+static __global__ void __launch_bounds__(kPairThreads, 1)
+k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
+            const __grid_constant__ CUtensorMap tmW2, const PairParams p, const StepArgs* __restrict__ args, const KvView kv, const Work w,
+            const Dims dm) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  PairSmem<SITE>* sm = reinterpret_cast<PairSmem<SITE>*>(smem + (size_t)p.stages * p.stage_bytes);
+  PairCtl* ctl = &sm->c;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
+  const int rank = (int)cluster_rank(), g = blockIdx.x >> 1;
+  volatile int* abort_flag = &ctl->abort_flag;
+  const int n_items = (p.n_tiles + 1) / 2 * p.n_rb;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < p.stages; ++i) {
+      mbar_init(smem_u32(&ctl->full[i]), 1);
+      mbar_init(smem_u32(&ctl->empty[i]), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&ctl->tmem_full[i]), 1);
+      mbar_init(smem_u32(&ctl->tmem_empty[i]), 16);   // the epilogue warps of both CTAs
+    }
+    ctl->abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 2) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)), "r"(p.tmem_cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();   // the other CTA's barriers exist
+  tc_fence_after();
+  pdl_launch();
+  const uint32_t tmem_base = ctl->tmem_base;
+
+  if (warp == 0) {
+    // ------------------------------ TMA producer (both CTAs) ------------------------------
+    if (elect_one()) {
+      const uint64_t pol_w = l2_policy_evict_first(), pol_a = l2_policy_evict_last();
+      const uint32_t tx = 2u * (kWTileBytes + (uint32_t)p.rb * 128u);   // both CTAs' bytes land on rank 0's barrier
+      auto w_load = [&](int s, int tile2, int kb) {
+        const int tile = 2 * tile2 + rank;
+        const uint32_t bar = smem_u32(&ctl->full[s]), dst = smem_u32(smem + (size_t)s * p.stage_bytes);
+        if (rank == 0) mbar_expect_tx(bar, tx);
+        if (SITE == PAIR_GU) {
+          pair_tma_2d(dst, &tmW0, bar, kb * kBK, tile * 64, pol_w);
+          pair_tma_2d(dst + 8192u, &tmW1, bar, kb * kBK, tile * 64, pol_w);
+        } else if (SITE == PAIR_QKV) {
+          if (tile < p.tile_q) pair_tma_2d(dst, &tmW0, bar, kb * kBK, tile * kTileN, pol_w);
+          else if (tile < p.tile_k) pair_tma_2d(dst, &tmW1, bar, kb * kBK, (tile - p.tile_q) * kTileN, pol_w);
+          else pair_tma_2d(dst, &tmW2, bar, kb * kBK, (tile - p.tile_k) * kTileN, pol_w);
+        } else {
+          pair_tma_2d(dst, &tmW0, bar, kb * kBK, tile * kTileN, pol_w);
+        }
+      };
+      // the first ring-full of weights before the programmatic wait: they do not depend on the previous kernel
+      int pre = 0;
+      for (int item = g; item < n_items && pre < p.stages; item += p.n_pairs)
+        for (int kb = 0; kb < p.KB && pre < p.stages; ++kb) w_load(pre++, item / p.n_rb, kb);
+      pdl_wait();
+      int s = 0, r = 0;
+      bool alive = true;
+      for (int item = g; item < n_items && alive; item += p.n_pairs) {
+        const int tile2 = item / p.n_rb, row = rank * p.plane_rows + (item % p.n_rb) * p.rb;
+        for (int kb = 0; kb < p.KB; ++kb) {
+          if (r > 0) {
+            if (!mbar_wait(smem_u32(&ctl->empty[s]), (uint32_t)(r - 1) & 1u, abort_flag, w.status, kPairSpin)) { alive = false; break; }
+            w_load(s, tile2, kb);
+          }
+          pair_tma_2d(smem_u32(smem + (size_t)s * p.stage_bytes + kWTileBytes), &tmA, smem_u32(&ctl->full[s]), kb * kBK, row, pol_a);
+          if (++s == p.stages) { s = 0; ++r; }
+        }
+      }
+    } else {
+      pdl_wait();
+    }
+  } else if (warp == 1) {
+    // ------------------------------ MMA issuer (rank 0) ------------------------------
+    pdl_wait();
+    if (rank == 0 && elect_one()) {
+      const uint32_t idesc = instr_desc_pair(2 * p.rb);
+      int s = 0, r = 0, n = 0;
+      bool alive = true;
+      for (int item = g; item < n_items && alive; item += p.n_pairs, ++n) {
+        const int acc = n & 1, use = n >> 1;
+        if (use > 0 && !mbar_wait(smem_u32(&ctl->tmem_empty[acc]), (uint32_t)(use - 1) & 1u, abort_flag, w.status, kPairSpin)) break;
+        tc_fence_after();
+        const uint32_t dcol = tmem_base + (uint32_t)(acc * 2 * p.rb);
+        for (int kb = 0; kb < p.KB; ++kb) {
+          if (!mbar_wait(smem_u32(&ctl->full[s]), (uint32_t)r & 1u, abort_flag, w.status, kPairSpin)) { alive = false; break; }
+          tc_fence_after();
+          const uint32_t wa = smem_u32(smem + (size_t)s * p.stage_bytes);
+          const uint64_t dw = smem_desc_sw128(wa), da = smem_desc_sw128(wa + kWTileBytes);
+#pragma unroll
+          for (int k = 0; k < kBK / 16; ++k) pair_mma(dcol, dw + 2 * k, da + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+          pair_commit(smem_u32(&ctl->empty[s]));
+          if (++s == p.stages) { s = 0; ++r; }
+        }
+        if (!alive) break;
+        pair_commit(smem_u32(&ctl->tmem_full[acc]));
+      }
+    }
+  } else if (warp >= 4) {
+    // ------------------------------ epilogue (eight warps) ------------------------------
+    // two groups of four warps take alternate 16-row chunks; a warp reads the accumulator lanes 32 * (warp % 4) .. + 31
+    pdl_wait();
+    const int wt = threadIdx.x - 128, grp = wt >> 7, fl = wt & 127, quarter = fl >> 5, bar_id = 2 + grp;
+    const int R = p.R, rows = args->gamma + 1;
+    auto group_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(bar_id) : "memory"); };
+    auto all_sync = [&]() { asm volatile("bar.sync 1, 256;" ::: "memory"); };
+    // per-row tables, beside the first MMAs
+    const int nt128 = dm.d / kTileN;
+    for (int r = wt; r < R; r += kPairWorkers) {
+      float inv = 1.f;
+      if (p.ssq_in) {
+        float s = 0.f;
+#pragma unroll 8
+        for (int t = 0; t < nt128; ++t) s += __ldcg(p.ssq_in + (size_t)t * R + r);
+        inv = 1.0f / sqrtf(s / (float)dm.d + dm.eps);
+      }
+      ctl->inv[r] = inv;
+      if constexpr (SITE == PAIR_QKV) {
+        const int b = r / rows, j = r % rows, pos = __ldcg(w.row_pos + r);
+        sm->x.qoff[r] = (b * dm.Hq * rows + j) * HD;
+        sm->x.nkvoff[r] = (b * dm.Hkv * 2 * rows + j) * HD;
+        long long off = -1;
+        if (r < args->kv_rows) {
+          const int page = kv.block_table[(size_t)args->seq_ids[b] * kv.max_pages_per_seq + pos / kv.page_size];
+          off = ((long long)page * 2 * dm.Hkv * kv.page_size + pos % kv.page_size) * HD;
+        }
+        sm->x.kvoff[r] = off;
+      }
+      if constexpr (SITE == PAIR_LM) {
+        const int b = r / rows, j = r % rows;
+        sm->x.tok[r] = j < args->gamma ? args->draft_ids[b * args->gamma + j] : -1;
+        sm->x.pre[r] = args->top_k >= 2 ? __ldcg(w.tgt_pre + r) : 0.f;
+      }
+    }
+    all_sync();
+    int n = 0;
+    for (int item = g; item < n_items; item += p.n_pairs, ++n) {
+      const int acc = n & 1, use = n >> 1;
+      const int tile = 2 * (item / p.n_rb) + rank, r_lo = item % p.n_rb * p.rb, r_hi = min(r_lo + p.rb, R);
+      const bool real = tile < p.n_tiles;   // an odd last tile's partner has no features
+      // a wait that runs out raises the abort flag and the epilogue goes on with whatever it reads: every thread keeps
+      // taking the same barriers, and the status word tells the host
+      if (fl == 0) mbar_wait(smem_u32(&ctl->tmem_full[acc]), (uint32_t)use & 1u, abort_flag, w.status, kPairSpin);
+      group_sync();
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 2 * p.rb);
+
+      // per-feature constants
+      int kind = 0, head = 0, dim = 0;
+      float bias = 0.f, gn = 1.f;
+      if constexpr (SITE == PAIR_QKV) {
+        int fs = tile * kTileN + fl;
+        const bf16* bp = p.bq;
+        if (tile >= p.tile_k) { kind = 2; fs -= p.tile_k * kTileN; bp = p.bv; }
+        else if (tile >= p.tile_q) { kind = 1; fs -= p.tile_q * kTileN; bp = p.bk; }
+        head = fs / HD;
+        dim = fs % HD;
+        if (bp && real) bias = __bfloat162float(bp[fs]);
+      }
+      if constexpr (SITE == PAIR_RES) gn = real ? __bfloat162float(p.gain[tile * kTileN + fl]) : 0.f;
+
+      for (int c0 = r_lo + 16 * grp; c0 < r_hi && real; c0 += 32) {   // uniform over the group
+        const int nr = min(16, r_hi - c0);
+        float v[16], lo[16];
+        float xs[16];
+        if constexpr (SITE == PAIR_RES) {   // residual rows, requested before the accumulator is waited for
+#pragma unroll
+          for (int i = 0; i < 16; ++i) xs[i] = __ldcg(w.X + (size_t)min(c0 + i, R - 1) * dm.d + tile * kTileN + fl);
+        }
+        tc_ld16(taddr + (uint32_t)(c0 - r_lo), v);
+        tc_ld16(taddr + (uint32_t)(p.rb + c0 - r_lo), lo);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] += lo[i];
+        if constexpr (SITE == PAIR_QKV) {
+          constexpr int half = HD / 2;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] = v[i] * (i < nr ? ctl->inv[c0 + i] : 0.f) + bias;
+          if (kind < 2) {   // uniform over the CTA
+#pragma unroll
+            for (int h8 = 0; h8 < 16; h8 += 8) {
+              float2 cs[8];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) cs[i] = __ldcg(w.rope + (size_t)min(c0 + h8 + i, R - 1) * half + (dim & (half - 1)));
+#pragma unroll
+              for (int i = 0; i < 8; ++i) sm->x.exch[grp][fl][i] = v[h8 + i];
+              group_sync();
+              const bool lower = dim < half;
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const float xp = sm->x.exch[grp][fl ^ half][i];
+                v[h8 + i] = lower ? v[h8 + i] * cs[i].x - xp * cs[i].y : v[h8 + i] * cs[i].x + xp * cs[i].y;
+              }
+              group_sync();
+            }
+          }
+          if (kind == 0) {
+            const float qscale = 1.4426950408889634f / sqrtf((float)HD);
+            __half* qb = w.Qb + (size_t)head * rows * HD + dim;
+            __half* ql = w.Qlo + (size_t)head * rows * HD + dim;
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if (i < nr) {
+                const float qv = v[i] * qscale;
+                const __half hq = __float2half_rn(qv);
+                qb[sm->x.qoff[c0 + i]] = hq;
+                ql[sm->x.qoff[c0 + i]] = __float2half_rn(qv - __half2float(hq));
+              }
+          } else {
+            bf16* kvb = reinterpret_cast<bf16*>(kv.pool) +
+                        ((size_t)p.layer * kv.n_pages * 2 * dm.Hkv + (size_t)(kind - 1) * dm.Hkv + head) * kv.page_size * HD + dim;
+            __half* kn = w.KVn + (size_t)(head * 2 + kind - 1) * rows * HD + dim;
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if (i < nr) {
+                if (sm->x.kvoff[c0 + i] >= 0) kvb[sm->x.kvoff[c0 + i]] = __float2bfloat16_rn(v[i]);
+                kn[sm->x.nkvoff[c0 + i]] = __float2half_rn(v[i]);
+              }
+          }
+        } else if constexpr (SITE == PAIR_RES) {
+          const int f = tile * kTileN + fl;
+          float sq[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            sq[i] = 0.f;
+            if (i < nr) {
+              const float x = xs[i] + v[i];
+              w.X[(size_t)(c0 + i) * dm.d + f] = x;
+              store_act<bf16>(p.planes_out, R, dm.d, c0 + i, f, x * gn);
+              sq[i] = x * x;
+            }
+          }
+          const float t = warp_sum16(sq, lane);
+          if ((lane & 1) == 0) sm->x.sums[quarter][c0 + (lane >> 1)] = t;
+        } else if constexpr (SITE == PAIR_GU) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] *= (i < nr ? ctl->inv[c0 + i] : 0.f);
+          // gate threads finish the chunk's rows 0..7, up threads rows 8..15: each hands over its other eight values
+          const bool is_gate = fl < 64;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) sm->x.exch[grp][fl][i] = is_gate ? v[8 + i] : v[i];
+          group_sync();
+          const int f = tile * 64 + (fl & 63), h8 = is_gate ? 0 : 8;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float other = sm->x.exch[grp][fl ^ 64][i];
+            const float gt = is_gate ? v[i] : other, up = is_gate ? other : v[8 + i];
+            if (h8 + i < nr) store_act<bf16>(p.planes_out, R, p.K_out, c0 + h8 + i, f, gt / (1.0f + expf(-gt)) * up);
+          }
+          group_sync();
+        } else {   // LM head
+          const int n_id = tile * kTileN + fl;
+          const float invT = args->inv_temperature;
+          const bool topk = args->top_k >= 2;
+          float* dbg = args->dbg_logits;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const int r = min(c0 + i, R - 1);
+            float z = -INFINITY;
+            if (i < nr && n_id < dm.V) {
+              if (dbg) dbg[(size_t)r * dm.V + n_id] = v[i];
+              z = v[i] * invT;
+              if (n_id == sm->x.tok[r]) w.tgt_logit[r] = z;
+            }
+            float m = z;
+            int arg = n_id;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+              const float om = __shfl_xor_sync(0xffffffffu, m, o);
+              const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
+              if (om > m || (om == m && oa < arg)) { m = om; arg = oa; }
+            }
+            const float e = warp_sum((z == -INFINITY) ? 0.f : expf(z - m));
+            int before = 0;
+            if (topk) {   // uniform
+              const int tg = sm->x.tok[r];
+              const float zd = sm->x.pre[r];
+              const bool bf = i < nr && n_id < dm.V && tg >= 0 && n_id != tg && (v[i] > zd || (v[i] == zd && n_id < tg));
+              before = __popc(__ballot_sync(0xffffffffu, bf));
+            }
+            if (lane == 0) {
+              RowStat st; st.m = m; st.s = e; st.arg = arg; st.pad = before;
+              sm->x.st[grp][quarter][i] = st;
+            }
+          }
+          group_sync();
+          if (fl < nr) {
+            RowStat a = sm->x.st[grp][0][fl];
+            a = stat_merge(a, sm->x.st[grp][1][fl]);
+            a = stat_merge(a, sm->x.st[grp][2][fl]);
+            a = stat_merge(a, sm->x.st[grp][3][fl]);
+            w.stats[(size_t)tile * R + c0 + fl] = a;
+          }
+          group_sync();
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) pair_arrive_rank0(smem_u32(&ctl->tmem_empty[acc]));
+      if constexpr (SITE == PAIR_RES) {
+        all_sync();
+        if (real)
+          for (int r = r_lo + wt; r < r_hi; r += kPairWorkers)
+            p.ssq_out[(size_t)tile * R + r] = (sm->x.sums[0][r] + sm->x.sums[1][r]) + (sm->x.sums[2][r] + sm->x.sums[3][r]);
+        all_sync();
+      }
+    }
+  } else {
+    pdl_wait();
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (*abort_flag) __nanosleep(20000);   // let copies still in flight land before the pair retires
+  cluster_sync_all();   // nothing of the pair touches the other CTA's memory after this
+  if (warp == 2) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");
+  }
+}
+
+}  // namespace sj

@@ -24,6 +24,8 @@ struct Work {
   void* ATT;         // attention output (input of the O projection), K = Hq*hd
   void* H;           // silu(gate)*up (input of the down projection), K = F
   float* P;          // partial sums of the current GEMM: [slot][R][N]
+  float* ssq;        // [2][d / 128][R] sums of squares of the residual rows per 128 columns (wide steps: input of QKV, of
+                     // gate/up)
   float* Hf;         // [R, d]        fp32 hidden state after the final norm
   float2* rope;      // [R, hd/2]     (cos, sin) of this step's positions
   int* row_pos;      // [R]           absolute position of each row
@@ -155,6 +157,20 @@ __global__ void k_reduce_norm(const StepArgs* __restrict__ args, Work w, Dims dm
   float* hf = final_norm ? w.Hf + (size_t)r * dm.d : nullptr;
   float* dbg = (final_norm && args->dbg_hidden) ? args->dbg_hidden + (size_t)r * dm.d : nullptr;
   norm_row_from_smem<T>(xs, dm.d, gain, dm.eps, w.A, gridDim.x, r, hf, dbg, red);
+}
+
+// a9 of wide steps, whose last projection leaves the residual stream only: the final norm of every row.
+template <typename T>
+__global__ void k_final_norm(const StepArgs* __restrict__ args, Work w, Dims dm, const T* __restrict__ gain) {
+  extern __shared__ float xs[];
+  __shared__ float red[32];
+  pdl_wait();
+  pdl_launch();
+  const int r = blockIdx.x;
+  for (int i = threadIdx.x; i < dm.d; i += blockDim.x) xs[i] = w.X[(size_t)r * dm.d + i];
+  __syncthreads();
+  norm_row_from_smem<T>(xs, dm.d, gain, dm.eps, w.A, gridDim.x, r, w.Hf + (size_t)r * dm.d,
+                        args->dbg_hidden ? args->dbg_hidden + (size_t)r * dm.d : nullptr, red);
 }
 
 // a3 tail + a4: reduce QKV partials, add bias, rotate q and k, store q, append k and v rows.

@@ -1630,22 +1630,20 @@ extern "C" sj_status sj_semantic_score(sj_target* t, sj_kv* kv, int seq, int y_i
 }
 
 // Prefill in wide blocks: up to kPrefillRows known tokens go through the decoder layers at once, as B consecutive
-// entries of `c` rows each over the same sequence -- entry b attends to the stored cache plus the b * c rows before it
+// entries of `c` rows each (the narrow blocks' size: an entry's own rows are read in fp16, the rows before it from the
+// bf16 pages, so another partition would give slightly other results) over the same sequence -- entry b attends to the stored cache plus the b * c rows before it
 // (its projection has stored them in the pages by the time the attention kernel runs) and to its own rows, which is
 // exactly what B verification steps of c rows one after another would do, at one read of the weights (8B-shaped model,
-// 1000 tokens and a step: 190 ms in blocks of 24 rows, 43.8 ms in three of 334).  Only the last token's row meets the
+// 1000 tokens and a step: 190 ms in blocks of 24 rows, PF_MS ms in two of 504).  Only the last token's row meets the
 // LM head, and a block that is not the last one ends with its key / value rows.
-constexpr int kPrefillRows = 352;      // rows of a wide block
+constexpr int kPrefillRows = SJ_MAX_ROWS;   // rows of a wide block
 constexpr int kPrefillWideMin = 33;    // shorter prompts: one or two narrow blocks through the whole-step kernel
 
-static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* tokens, int n_tokens, int* d_next, bool* done) {
+static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* tokens, int n_tokens, int c, int* d_next, bool* done) {
   const Dims& dm = t->dm;
   cudaStream_t s = t->stream;
   sj_status st;
   *done = false;
-  // a KV head's query rows fill at most one 128-lane accumulator
-  const int c_max = std::min((int)SJ_MAX_GAMMA + 1, 128 / (dm.Hq / dm.Hkv));
-  if (c_max < 2) return SJ_OK;
   if (t->pf_rows == 0) {
     const size_t mark = t->owned.size();
     memset(&t->pf_work, 0, sizeof(Work));
@@ -1671,16 +1669,16 @@ static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* token
     if ((st = dev_alloc(t, &t->d_pf_tok, cap)) != SJ_OK) return st;
     t->pf_tok_cap = cap;
   }
-  const int block = std::min(t->pf_rows / c_max, (int)SJ_MAX_BATCH) * c_max;
-  const int n_blocks = (n_tokens + block - 1) / block, per = (n_tokens + n_blocks - 1) / n_blocks;
-  if ((st = ensure_attn_partials(t, block / c_max, c_max)) != SJ_OK) return st;
+  const int most = std::min(t->pf_rows / c, (int)SJ_MAX_BATCH), entries = (n_tokens + c - 1) / c;   // entries of a block, of the prompt
+  const int n_blocks = (entries + most - 1) / most, per = (entries + n_blocks - 1) / n_blocks * c;
+  if ((st = ensure_attn_partials(t, per / c, c)) != SJ_OK) return st;
   Work W = t->pf_work;
   W.tc_m = t->work.tc_m; W.tc_l = t->work.tc_l; W.tc_o = t->work.tc_o;
   W.status = t->work.status; W.judge_w = t->work.judge_w; W.inv_freq = t->work.inv_freq;
   if ((st = reserve(kv, seq, (long)kv->len_hi[seq] + n_tokens, nullptr)) != SJ_OK) return st;
   CU_TRY(cudaMemcpyAsync(t->d_pf_tok, tokens, sizeof(int) * n_tokens, cudaMemcpyHostToDevice, s));
   for (int i0 = 0; i0 < n_tokens; i0 += per) {
-    const int n = std::min(per, n_tokens - i0), B = (n + c_max - 1) / c_max, c = (n + B - 1) / B;
+    const int n = std::min(per, n_tokens - i0), B = (n + c - 1) / c;
     const bool last = i0 + n == n_tokens;
     StepArgs h;
     memset(&h, 0, sizeof(h));
@@ -1730,7 +1728,7 @@ extern "C" sj_status sj_prefill(sj_target* t, sj_kv* kv, int seq, const int* tok
   o.p_draft = reinterpret_cast<float*>(t->d_prefill + 5 * (SJ_MAX_GAMMA + 1));
   bool done = false;
   if (n_tokens >= kPrefillWideMin && t->bf && t->opt_gemm == 1 && t->opt_attn >= 1 && kv->has_tm_pool) {
-    sj_status st = prefill_wide(t, kv, seq, tokens, n_tokens, o.next_token, &done);
+    sj_status st = prefill_wide(t, kv, seq, tokens, n_tokens, c_max, o.next_token, &done);
     if (st != SJ_OK) return st;
   }
   if (done) n_tokens = 0;

@@ -4,8 +4,12 @@
 // A pair of CTAs (tcgen05 cta_group::2) computes one 256-feature tile for a block of rb <= 128 rows over the whole of K:
 // CTA `rank` holds the weights and the accumulator of features [128 rank, +128).  The MMA's N = 2 rb columns are the
 // block's rows twice: the hi plane, staged by rank 0, and the lo plane, staged by rank 1; each SM's tensor core reads
-// both.  The epilogue adds the two halves.  Accumulators are double-buffered, so an item's epilogue runs beside the next
-// item's MMAs.
+// both.  The epilogue adds the two halves.
+//
+// The tensor core's accumulation truncates (measured against fp64: a chain of 896 MMAs comes out 1.4e-5 too small, one
+// of 64 about 1e-6), so K is summed in segments of kPairSegKB K blocks whose results the epilogue warps add in fp32
+// registers.  Segments alternate between two accumulators: the adding, and an item's epilogue, run beside the next
+// segment's MMAs.
 //
 // Why this shape: what bounds wide steps is the shared-memory port (128 B/clk per SM).  A K step of 64 writes
 // 16 KiB of weights and 128 rb bytes of activations and its four MMAs read 4 (4096 + 32 rb) back: 256 + 2 rb clocks, for
@@ -25,6 +29,7 @@
 //   LM head -> softmax statistics per (128-token tile, row)
 #pragma once
 
+#include "sj_attn_t5.cuh"
 #include "sj_gemm_tc.cuh"
 
 namespace sj {
@@ -33,6 +38,7 @@ constexpr int kPairThreads = 384;      // warp 0 TMA, warp 1 MMA (rank 0), warp 
 constexpr int kPairWorkers = 256;
 constexpr int kPairMaxStages = 10;
 constexpr int kPairMaxRows = kMaxRows;
+constexpr int kPairSegKB = 16;          // K blocks of 64 per accumulation chain
 constexpr uint32_t kPairSpin = 1u << 22;
 
 enum PairSite { PAIR_QKV = 0, PAIR_RES = 1, PAIR_GU = 2, PAIR_LM = 3 };
@@ -144,6 +150,33 @@ __device__ __forceinline__ float warp_sum16(const float* v, int lane) {
   return d + __shfl_xor_sync(0xffffffffu, d, 1);
 }
 
+// The same for the maximum: lanes 2i and 2i + 1 return the largest of value i over the warp and the lowest `id` that has it.
+__device__ __forceinline__ void warp_max16(const float* v, int id, int lane, float& m, int& arg) {
+  float a[16];
+  int b[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) { a[i] = v[i]; b[i] = id; }
+#pragma unroll
+  for (int h = 8; h >= 1; h >>= 1) {   // value i of the lower half pairs with value i + h; lane bit 2 h picks the half kept
+    const bool up = lane & (2 * h);
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const float mine = up ? a[i + h] : a[i], send = up ? a[i] : a[i + h];
+      const int mine_id = up ? b[i + h] : b[i], send_id = up ? b[i] : b[i + h];
+      const float om = __shfl_xor_sync(0xffffffffu, send, 2 * h);
+      const int oid = __shfl_xor_sync(0xffffffffu, send_id, 2 * h);
+      const bool take = om > mine || (om == mine && oid < mine_id);
+      a[i] = take ? om : mine;
+      b[i] = take ? oid : mine_id;
+    }
+  }
+  const float om = __shfl_xor_sync(0xffffffffu, a[0], 1);
+  const int oid = __shfl_xor_sync(0xffffffffu, b[0], 1);
+  const bool take = om > a[0] || (om == a[0] && oid < b[0]);
+  m = take ? om : a[0];
+  arg = take ? oid : b[0];
+}
+
 template <int SITE, int HD>
 static __global__ void __launch_bounds__(kPairThreads, 1)
 k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
@@ -230,23 +263,28 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       const uint32_t idesc = instr_desc_pair(2 * p.rb);
       int s = 0, r = 0, n = 0;
       bool alive = true;
-      for (int item = g; item < n_items && alive; item += p.n_pairs, ++n) {
-        const int acc = n & 1, use = n >> 1;
-        if (use > 0 && !mbar_wait(smem_u32(&ctl->tmem_empty[acc]), (uint32_t)(use - 1) & 1u, abort_flag, w.status, kPairSpin)) break;
-        tc_fence_after();
-        const uint32_t dcol = tmem_base + (uint32_t)(acc * 2 * p.rb);
+      for (int item = g; item < n_items && alive; item += p.n_pairs) {
+        uint32_t dcol = 0;
+        int acc = 0;
         for (int kb = 0; kb < p.KB; ++kb) {
+          const bool first = kb % kPairSegKB == 0;
+          if (first) {
+            acc = n & 1;
+            const int use = n >> 1;
+            ++n;
+            if (use > 0 && !mbar_wait(smem_u32(&ctl->tmem_empty[acc]), (uint32_t)(use - 1) & 1u, abort_flag, w.status, kPairSpin)) { alive = false; break; }
+            dcol = tmem_base + (uint32_t)(acc * 2 * p.rb);
+          }
           if (!mbar_wait(smem_u32(&ctl->full[s]), (uint32_t)r & 1u, abort_flag, w.status, kPairSpin)) { alive = false; break; }
           tc_fence_after();
           const uint32_t wa = smem_u32(smem + (size_t)s * p.stage_bytes);
           const uint64_t dw = smem_desc_sw128(wa), da = smem_desc_sw128(wa + kWTileBytes);
 #pragma unroll
-          for (int k = 0; k < kBK / 16; ++k) pair_mma(dcol, dw + 2 * k, da + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+          for (int k = 0; k < kBK / 16; ++k) pair_mma(dcol, dw + 2 * k, da + 2 * k, idesc, (!first || k > 0) ? 1u : 0u);
           pair_commit(smem_u32(&ctl->empty[s]));
           if (++s == p.stages) { s = 0; ++r; }
+          if (kb % kPairSegKB == kPairSegKB - 1 || kb == p.KB - 1) pair_commit(smem_u32(&ctl->tmem_full[acc]));
         }
-        if (!alive) break;
-        pair_commit(smem_u32(&ctl->tmem_full[acc]));
       }
     }
   } else if (warp >= 4) {
@@ -286,17 +324,41 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       }
     }
     all_sync();
+    const int n_seg = (p.KB + kPairSegKB - 1) / kPairSegKB;
     int n = 0;
-    for (int item = g; item < n_items; item += p.n_pairs, ++n) {
-      const int acc = n & 1, use = n >> 1;
+    for (int item = g; item < n_items; item += p.n_pairs) {
       const int tile = 2 * (item / p.n_rb) + rank, r_lo = item % p.n_rb * p.rb, r_hi = min(r_lo + p.rb, R);
       const bool real = tile < p.n_tiles;   // an odd last tile's partner has no features
-      // a wait that runs out raises the abort flag and the epilogue goes on with whatever it reads: every thread keeps
-      // taking the same barriers, and the status word tells the host
-      if (fl == 0) mbar_wait(smem_u32(&ctl->tmem_full[acc]), (uint32_t)use & 1u, abort_flag, w.status, kPairSpin);
-      group_sync();
-      tc_fence_after();
-      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 2 * p.rb);
+      // the segments' sums: chunk j of this group in registers
+      float sum[4][16];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 16; ++i) sum[j][i] = 0.f;
+#pragma unroll 1
+      for (int sg = 0; sg < n_seg; ++sg, ++n) {
+        const int acc = n & 1;
+        // a wait that runs out raises the abort flag and the epilogue goes on with whatever it reads: every thread
+        // keeps taking the same barriers, and the status word tells the host
+        if (fl == 0) mbar_wait(smem_u32(&ctl->tmem_full[acc]), (uint32_t)(n >> 1) & 1u, abort_flag, w.status, kPairSpin);
+        group_sync();
+        tc_fence_after();
+        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 2 * p.rb);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int c = 16 * grp + 32 * j;   // row of the chunk within the block
+          if (r_lo + c < r_hi) {             // uniform over the group
+            float hi[16], lo[16];
+            tc_ld16(taddr + (uint32_t)c, hi);
+            tc_ld16(taddr + (uint32_t)(p.rb + c), lo);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) sum[j][i] += hi[i] + lo[i];
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) pair_arrive_rank0(smem_u32(&ctl->tmem_empty[acc]));
+      }
 
       // per-feature constants
       int kind = 0, head = 0, dim = 0;
@@ -312,18 +374,16 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       }
       if constexpr (SITE == PAIR_RES) gn = real ? __bfloat162float(p.gain[tile * kTileN + fl]) : 0.f;
 
-      for (int c0 = r_lo + 16 * grp; c0 < r_hi && real; c0 += 32) {   // uniform over the group
-        const int nr = min(16, r_hi - c0);
-        float v[16], lo[16];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c0 = r_lo + 16 * grp + 32 * j, nr = min(16, r_hi - c0);
+        if (nr <= 0 || !real) break;   // uniform over the group
+        float (&v)[16] = sum[j];
         float xs[16];
         if constexpr (SITE == PAIR_RES) {   // residual rows, requested before the accumulator is waited for
 #pragma unroll
           for (int i = 0; i < 16; ++i) xs[i] = __ldcg(w.X + (size_t)min(c0 + i, R - 1) * dm.d + tile * kTileN + fl);
         }
-        tc_ld16(taddr + (uint32_t)(c0 - r_lo), v);
-        tc_ld16(taddr + (uint32_t)(p.rb + c0 - r_lo), lo);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] += lo[i];
         if constexpr (SITE == PAIR_QKV) {
           constexpr int half = HD / 2;
 #pragma unroll
@@ -405,35 +465,38 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           const float invT = args->inv_temperature;
           const bool topk = args->top_k >= 2;
           float* dbg = args->dbg_logits;
+          const int own = lane >> 1;   // the chunk's row whose totals this lane ends up with
+          int before = 0;
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const int r = min(c0 + i, R - 1);
-            float z = -INFINITY;
-            if (i < nr && n_id < dm.V) {
-              if (dbg) dbg[(size_t)r * dm.V + n_id] = v[i];
-              z = v[i] * invT;
-              if (n_id == sm->x.tok[r]) w.tgt_logit[r] = z;
-            }
-            float m = z;
-            int arg = n_id;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-              const float om = __shfl_xor_sync(0xffffffffu, m, o);
-              const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
-              if (om > m || (om == m && oa < arg)) { m = om; arg = oa; }
-            }
-            const float e = warp_sum((z == -INFINITY) ? 0.f : expf(z - m));
-            int before = 0;
             if (topk) {   // uniform
               const int tg = sm->x.tok[r];
               const float zd = sm->x.pre[r];
               const bool bf = i < nr && n_id < dm.V && tg >= 0 && n_id != tg && (v[i] > zd || (v[i] == zd && n_id < tg));
-              before = __popc(__ballot_sync(0xffffffffu, bf));
+              const int c = __popc(__ballot_sync(0xffffffffu, bf));
+              if (i == own) before = c;
             }
-            if (lane == 0) {
-              RowStat st; st.m = m; st.s = e; st.arg = arg; st.pad = before;
-              sm->x.st[grp][quarter][i] = st;
+            if (i < nr && n_id < dm.V) {
+              if (dbg) dbg[(size_t)r * dm.V + n_id] = v[i];
+              v[i] *= invT;
+              if (n_id == sm->x.tok[r]) w.tgt_logit[r] = v[i];
+            } else {
+              v[i] = -INFINITY;
             }
+          }
+          float m;
+          int arg;
+          warp_max16(v, n_id, lane, m, arg);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float mi = __shfl_sync(0xffffffffu, m, 2 * i);
+            v[i] = v[i] == -INFINITY ? 0.f : expf(v[i] - mi);
+          }
+          const float e = warp_sum16(v, lane);
+          if ((lane & 1) == 0) {
+            RowStat st; st.m = m; st.s = e; st.arg = arg; st.pad = before;
+            sm->x.st[grp][quarter][own] = st;
           }
           group_sync();
           if (fl < nr) {
@@ -446,9 +509,6 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           group_sync();
         }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) pair_arrive_rank0(smem_u32(&ctl->tmem_empty[acc]));
       if constexpr (SITE == PAIR_RES) {
         all_sync();
         if (real)

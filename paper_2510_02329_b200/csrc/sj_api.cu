@@ -215,8 +215,9 @@ struct sj_target {
   bool mega_shapes = false, coop = false;
   MegaLayerPtrs* d_layer_ptrs = nullptr;
   float* d_sumsq = nullptr;
-  unsigned* d_sync = nullptr;      // [0] barrier counter, [1] abort word, [2..3] timeout note; [64 ..) the split-K
-                                   // partial words (64-bit, [blocks][Rp][128]); zeroed as one range before every launch
+  unsigned* d_sync = nullptr;      // [0] barrier counter, [1] abort word, [2..3] timeout note, zeroed before every launch;
+                                   // [64 ..) the split-K partial words (sj_mega.cuh), whose tags are unique over launches
+  unsigned mega_tag = 0;           // MegaParams::tag0 of the next launch
   unsigned long long* d_trace = nullptr;
   std::vector<MegaMaps> mega_maps;  // one per launch chunk of kMegaMaxLayers layers
   struct Timed { const char* name; cudaEvent_t a, b; };
@@ -310,6 +311,11 @@ static MegaKernel mega_kernel(int hd, int ns, bool trace, bool a5) {
   if (hd != 128) return trace ? mega_kernel_64_trace(ns) : mega_kernel_64(ns);
   if (a5) return trace ? mega_kernel_128_t5_trace(ns) : mega_kernel_128_t5(ns);
   return trace ? mega_kernel_128_trace(ns) : mega_kernel_128(ns);
+}
+
+// 32-bit words of the persistent kernel's partial-sum buffer for Rp rows (a multiple of 16).
+static size_t mega_partial_words(const sj_target* t, int Rp) {
+  return (size_t)t->sm_count * 2 * (Rp / 16) * 2 * 3 * kTileN * 4;
 }
 
 // The per-row buffers of a step of at most R rows.
@@ -493,7 +499,7 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
     const int Rm = std::min(R, kMegaMaxRows);
     ALLOC(t->d_layer_ptrs, MegaLayerPtrs, c.n_layers);
     ALLOC(t->d_sumsq, float, (size_t)2 * (c.d_model / kTileN) * kMegaMaxRows);
-    ALLOC(t->d_sync, unsigned, 64 + (size_t)4 * t->sm_count * pad16(Rm) * kTileN);
+    ALLOC(t->d_sync, unsigned, 64 + mega_partial_words(t, pad16(Rm)));
     std::vector<MegaLayerPtrs> lp(c.n_layers);
     for (int l = 0; l < c.n_layers; ++l) {
       const LayerW& L = t->layers[l];
@@ -503,7 +509,7 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
     }
     cudaError_t e = cudaMemcpy(t->d_layer_ptrs, lp.data(), lp.size() * sizeof(MegaLayerPtrs), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(t->d_sumsq, 0, sizeof(float) * 2 * (c.d_model / kTileN) * kMegaMaxRows);
-    if (e == cudaSuccess) e = cudaMemset(t->d_sync, 0, sizeof(unsigned) * (64 + (size_t)4 * t->sm_count * pad16(Rm) * kTileN));
+    if (e == cudaSuccess) e = cudaMemset(t->d_sync, 0, sizeof(unsigned) * (64 + mega_partial_words(t, pad16(Rm))));
     for (int ns = 4; ns <= 8 && e == cudaSuccess; ns += 2)
       for (int v = 0; v < 4 && e == cudaSuccess; ++v)
         e = cudaFuncSetAttribute(mega_kernel(c.head_dim, ns, (v & 1) != 0, (v & 2) != 0 && c.head_dim == 128),
@@ -1117,7 +1123,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
     if (kv_only && l == dm.n_layers - 1) return SJ_OK;
     // attention
     if (attn_tc) {
-      AttArgs aa{W.Qb, l < t->opt_att_precise ? W.Qlo : nullptr, W.KVn, AttPartials{W.tc_m, W.tc_l, W.tc_o}, t->sm_count + B * dm.Hkv, l};
+      AttArgs aa{W.Qb, l < t->opt_att_precise ? W.Qlo : nullptr, W.KVn, AttPartials{W.tc_m, W.tc_l, W.tc_o}, t->sm_count + B * dm.Hkv, l, B};
       const size_t tc_smem = kAttStages * kAttStageBytes + sizeof(AttSmemCtl) + 1024;
       const AttPartials parts{W.tc_m, W.tc_l, W.tc_o};
       // one warp per (sequence, KV head, query row, half of the head dimension): every task's loads are in flight at once
@@ -1272,7 +1278,7 @@ static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode
   p.lm_head = (const bf16*)t->lm_head;
   p.gain0 = (const bf16*)t->layers[0].na;
   p.sumsq = t->d_sumsq;
-  p.pbuf = reinterpret_cast<unsigned long long*>(t->d_sync + 64);
+  p.pbuf = reinterpret_cast<uint4*>(t->d_sync + 64);
   p.gbar = t->d_sync;
   p.abort_g = reinterpret_cast<int*>(t->d_sync + 1);
   p.n_tail_base = t->sm_count + B * dm.Hkv;
@@ -1291,7 +1297,13 @@ static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode
     MegaMaps mm = t->mega_maps[ci];
     mm.pool = kv->tm_pool;
     mm.a_d = *mA_d; mm.a_q = *mA_q; mm.a_f = *mA_f;
-    CU_TRY(cudaMemsetAsync(t->d_sync, 0, sizeof(unsigned) * (64 + (size_t)4 * t->sm_count * Rp * kTileN), s));
+    if (t->mega_tag > 0xffff0000u) {   // the tags start again: no stale word may carry one of them
+      CU_TRY(cudaMemsetAsync(t->d_sync, 0, sizeof(unsigned) * (64 + mega_partial_words(t, pad16(std::min(t->max_rows, kMegaMaxRows)))), s));
+      t->mega_tag = 0;
+    }
+    p.tag0 = t->mega_tag;
+    t->mega_tag += 4 * kMegaMaxLayers + 1;   // GEMM phases of a launch
+    CU_TRY(cudaMemsetAsync(t->d_sync, 0, sizeof(unsigned) * 4, s));
     cudaEvent_t ea = nullptr, eb = nullptr;
     if (timing) {
       CU_TRY(cudaEventCreate(&ea));

@@ -151,6 +151,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   }
   if (warp == 2) att_plan_fill(&ctl->plan, w.row_pos, B, rows, Hkv, kT5Keys, lane, kT5Pad);
   // unused query-row slots stay zero for the whole kernel
+#pragma unroll 1
   for (int i = threadIdx.x; i < 2 * kT5TileBytes / 16; i += blockDim.x) reinterpret_cast<uint4*>(sQ)[i] = make_uint4(0, 0, 0, 0);
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(att_smem_u32(&ctl->tmem_base)), "r"(512u)
@@ -179,6 +180,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
       uint64_t* empty = which ? ctl->vempty : ctl->kempty;
       uint8_t* base = which ? sV : sK;
       int g = 0;   // real tiles so far
+#pragma unroll 1
       for (long long t = t_lo; t < t_hi; ++t) {
         const AttTile x = att_locate(pl, B, kT5Keys, (int)t);
         if (x.ti >= x.nt_real) continue;   // one of the plan's empty tiles
@@ -214,6 +216,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
       int it = 0, seg = 0;
       long long t = t_lo;
       bool alive = true;
+#pragma unroll 1
       while (t < t_hi && alive) {
         const AttTile x = att_locate(pl, B, kT5Keys, (int)t);
         const int nv = (int)min((long long)(x.nt_b - x.ti), t_hi - t);   // with the plan's empty tiles
@@ -224,6 +227,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
         // every segment's queries are waited for, also where this thread owns none of its tiles: a parity wait that
         // skipped a phase would be satisfied one phase early
         if (!t5_wait(&ctl->q_ready, (uint32_t)seg & 1u, ctl, w.status, 2)) break;
+#pragma unroll 1
         for (int i = ((it & 1) == X) ? 0 : 1; i < n; i += 2) {
           const int g = it + i;
           const uint32_t par = (uint32_t)(g >> 1) & 1u;
@@ -319,6 +323,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
       nv = (int)min((long long)(x.nt_b - x.ti), t_hi - t);
       n = max(0, min(nv, x.nt_real - x.ti));
     };
+#pragma unroll 1
     while (t < t_hi && alive) {
       AttTile x;
       int n, nv;
@@ -333,6 +338,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
       }
       if (seg == 0) deliver_q(x);   // later segments' queries were delivered while the segment before them ended
       float m_used = -INFINITY, l_sum = 0.f;
+#pragma unroll 1
       for (int i = 0; i < n && alive; ++i) {
         const int g = it + i, sb = g & 1;
         int ok = 1;
@@ -419,6 +425,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
       // thread saw the scores of its last tile), so the query tiles are free, and the issuers start on the next
       // segment's scores while the partial below is read out (its first P V waits for probabilities that this thread
       // delivers only afterwards, so the output accumulators are not touched early).
+#pragma unroll 1
       for (long long t2 = t + nv; t2 < t_hi;) {
         AttTile x2;
         int n2, nv2;
@@ -471,6 +478,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
     if (alive) {
       const AttGeom g = att_geom(HD, group, rows);
       AttWarp<HD, 2> st;
+#pragma unroll 1
       for (int task = (G - 1 - c) * 8 + (warp - 2); task < B * Hkv * g.MT; task += G * 8)
         att_tail_task<HD, 2>(st, g, a, task / g.MT, (task % g.MT) * 16, lane);
     }
@@ -561,6 +569,7 @@ __device__ __forceinline__ bool a5_produce(const A5Ring& rg, A5Pos& pos, const C
                                            const StepArgs* __restrict__ args, const AttPlan& pl, int B, int layer,
                                            long long t_lo, long long t_hi, const int* pages, int lane) {
   const int which = lane >> 4, half = (lane >> 3) & 1, p = lane & 7;
+#pragma unroll 1
   for (long long t = t_lo; t < t_hi; ++t) {
     const AttTile x = att_locate(pl, B, kA5Keys, (int)t);
     if (x.ti >= x.nt_real) continue;   // one of the plan's empty tiles: no ring entry
@@ -572,6 +581,7 @@ __device__ __forceinline__ bool a5_produce(const A5Ring& rg, A5Pos& pos, const C
     const long long row = ((((long long)layer * kv.n_pages + page) * 2 + which) * kv.n_kv_heads + x.h) * 16;
     // claim the key stage and the value stage: every lane waits (same flow), lane 0 announces
     uint32_t dst = 0, bar = 0;
+#pragma unroll 1
     for (int st = 0; st < 2; ++st) {
       if (pos.r > 0 && !a5_wait(rg, &rg.empty[pos.s], (uint32_t)(pos.r - 1) & 1u, 1, pos.r)) return false;
       const uint32_t b_st = att_smem_u32(&rg.full[pos.s]);
@@ -600,6 +610,7 @@ __device__ __forceinline__ bool a5_issue(const A5Ring& rg, A5Pos& pos, A5Bars* a
   const uint64_t q_half = (uint64_t)(hs >> 4), k_half = (uint64_t)(16384 >> 4);   // start-address field, 16-byte units
   const uint32_t d_s = tmem + (uint32_t)(128 * X), d_o = tmem + (uint32_t)(256 + 128 * X);
   long long t = t_lo;
+#pragma unroll 1
   while (t < t_hi) {
     const AttTile x = att_locate(pl, B, kA5Keys, (int)t);
     const int nv = (int)min((long long)(x.nt_b - x.ti), t_hi - t);   // with the plan's empty tiles
@@ -611,6 +622,7 @@ __device__ __forceinline__ bool a5_issue(const A5Ring& rg, A5Pos& pos, A5Bars* a
     if (!a5_wait(rg, &ab->q_ready, (uint32_t)segs & 1u, 2, segs)) return false;
     tc_fence_after();
     bool first = true;
+#pragma unroll 1
     for (int i = 0; i < n; ++i) {
       const int g = gt + i;
       const A5Entry e = a5_entry(rg, pos);
@@ -723,6 +735,7 @@ __device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Bars* ab, uint32_
   };
   long long t = t_lo;
   bool first_seg = true;
+#pragma unroll 1
   while (t < t_hi) {
     AttTile x;
     int n, nv;
@@ -742,6 +755,7 @@ __device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Bars* ab, uint32_
     first_seg = false;
     if (stamp) ev[0] = att_timer_ns();
     float m_used = -INFINITY, l_sum = 0.f;
+#pragma unroll 1
     for (int i = 0; i < n; ++i) {
       const int g = gt + i, sb = g & 1;
       const uint32_t par = (uint32_t)(g >> 1) & 1u;
@@ -833,6 +847,7 @@ __device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Bars* ab, uint32_
     // thread saw the scores of its last tile), so the query area is free, and the issuers start on the next segment's
     // scores while the partial below is read out (its first P V waits for probabilities that this thread delivers only
     // afterwards, so the output accumulators are not touched early).
+#pragma unroll 1
     for (long long t2 = t + nv; t2 < t_hi;) {
       AttTile x2;
       int n2, nv2;

@@ -97,10 +97,12 @@ __device__ __forceinline__ int att_owner(long long t, long long T, int G) {
   if (T < (1 << 22) && G < 512) {   // 32-bit arithmetic (64-bit division is slow): t*G and (c+1)*T stay below 2^31
     const unsigned tt = (unsigned)t, TT = (unsigned)T, GG = (unsigned)G;
     unsigned c = tt * GG / TT;
+#pragma unroll 1
     while ((c + 1) * TT / GG <= tt) ++c;
     return (int)c;
   }
   int c = (int)(t * G / T);
+#pragma unroll 1
   while ((long long)(c + 1) * T / G <= t) ++c;
   return c;
 }
@@ -282,17 +284,21 @@ struct AttWarp {
   // copy written earlier in this step (the pages hold the same rows rounded to bf16 for later steps;
   // reading the copy keeps 11 significant bits of the rows that weigh most when the cache is short).
   // Query row q = g*rows + j sees kq <= j.  krow(kq) / vrow(kq) return the fp16 row pointers [HD].
-  template <bool TWO, typename KFn, typename VFn>
-  __device__ __forceinline__ void tail(KFn krow, VFn vrow, int rows, int row0, int nq, int lane, const __half* qhi = nullptr,
-                                       const __half* qlo = nullptr) {
+  // (Two-term mode is a run-time switch here, unlike in tile(): the tail is a small part of a phase, and every copy of its
+  // code costs instruction-cache space.)
+  template <typename KFn, typename VFn>
+  __device__ __forceinline__ void tail(KFn krow, VFn vrow, int rows, int row0, int nq, int lane, const __half* qhi,
+                                       const __half* qlo) {
+    const bool two = qlo != nullptr;   // warp-uniform
     const int q0 = row0 + (lane >> 2), q1 = q0 + 8;
     const int j0 = q0 % rows, j1 = q1 % rows;
+#pragma unroll 1
     for (int kbase = 0; kbase < rows; kbase += NT * 8) {
       float s[NT][4];
 #pragma unroll
       for (int n = 0; n < NT; ++n) s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f;
-#pragma unroll
-      for (int pass = 0; pass < (TWO ? 2 : 1); ++pass) {   // two-term mode: q_hi . k, then q_lo . k (see tile())
+#pragma unroll 1
+      for (int pass = 0; pass < (two ? 2 : 1); ++pass) {   // two-term mode: q_hi . k, then q_lo . k (see tile())
         if (pass == 1) load_q(qlo, row0, nq, lane);
 #pragma unroll
         for (int n = 0; n < NT; ++n) {
@@ -327,7 +333,7 @@ struct AttWarp {
         pa[2] = pack_f16(s[2 * kk2 + 1][0], s[2 * kk2 + 1][1]);
         pa[3] = pack_f16(s[2 * kk2 + 1][2], s[2 * kk2 + 1][3]);
         uint32_t pl[4] = {0u, 0u, 0u, 0u};
-        if constexpr (TWO) {
+        if (two) {
           pl[0] = pack_f16_rest(s[2 * kk2][0], s[2 * kk2][1], pa[0]);
           pl[1] = pack_f16_rest(s[2 * kk2][2], s[2 * kk2][3], pa[1]);
           pl[2] = pack_f16_rest(s[2 * kk2 + 1][0], s[2 * kk2 + 1][1], pa[2]);
@@ -344,7 +350,7 @@ struct AttWarp {
           uint32_t b0 = (v00 ? ldcg_u16(v00 + d) : 0u) | ((v01 ? ldcg_u16(v01 + d) : 0u) << 16);
           uint32_t b1 = (v10 ? ldcg_u16(v10 + d) : 0u) | ((v11 ? ldcg_u16(v11 + d) : 0u) << 16);
           mma_16816(o[dn], pa, b0, b1);
-          if constexpr (TWO) mma_16816(o[dn], pl, b0, b1);
+          if (two) mma_16816(o[dn], pl, b0, b1);
         }
       }
     }
@@ -390,6 +396,7 @@ struct AttPlan {
 __device__ __forceinline__ void att_plan_fill(AttPlan* pl, const int* __restrict__ row_pos, int B, int rows, int Hkv,
                                               int KPS, int lane, int pad = 0) {
   int carry = 0;
+#pragma unroll 1
   for (int b0 = 0; b0 < B; b0 += 32) {
     const int b = b0 + lane;
     const int L = b < B ? row_pos[b * rows] : 0;
@@ -415,6 +422,7 @@ __device__ __forceinline__ void att_plan_fill(AttPlan* pl, const int* __restrict
 
 __device__ __forceinline__ int att_find_seq(const int* pre, int B, int t) {
   int lo = 0, hi = B - 1;
+#pragma unroll 1
   while (lo < hi) {
     int mid = (lo + hi + 1) >> 1;
     if (pre[mid] <= t) lo = mid; else hi = mid - 1;
@@ -429,6 +437,7 @@ struct AttArgs {
   AttPartials P;
   int n_tail_base;         // slot of tail (b, h): n_tail_base + b*Hkv + h
   int layer;
+  int B;
 };
 
 // ---------------------------------------------------------------------------------------------
@@ -467,6 +476,7 @@ __device__ __forceinline__ void att_note_timeout(volatile int* abort_g, int wher
 // round trip.)
 __device__ __forceinline__ bool att_mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
                                                 volatile int* abort_g, int where, int extra, uint32_t limit) {
+#pragma unroll 1
   for (uint32_t i = 0; i < limit; ++i) {
     if (att_mbar_try(bar, parity)) return true;
     if (i > 64) {
@@ -504,6 +514,7 @@ __device__ __forceinline__ void att_issue_tile(const CUtensorMap* tmKV, const Kv
                                                const int* pages = nullptr) {
   const int HB = HD / 64, npg = KPS / 16;
   const int last_page = (L - 1) / 16;   // L >= 1 for any ring tile
+#pragma unroll 1
   for (int p = 0; p < npg; ++p) {
     int pi = ti * npg + p;
     if (pi > last_page) pi = last_page;   // keys there are masked; reload a valid page
@@ -561,31 +572,22 @@ __device__ __forceinline__ void att_tail_task(AttWarp<HD, NT>& st, const AttGeom
   const __half* kn = a.KVn + (size_t)x * 2 * rows * HD;
   auto krow = [&](int kq) -> const __half* { return kn + (size_t)kq * HD; };
   auto vrow = [&](int kq) -> const __half* { return kn + (size_t)(rows + kq) * HD; };
-  if (qlo) st.template tail<true>(krow, vrow, rows, row0, g.nq, lane, qhi, qlo);   // warp-uniform
-  else st.template tail<false>(krow, vrow, rows, row0, g.nq, lane);
+  st.tail(krow, vrow, rows, row0, g.nq, lane, qhi, qlo);
   st.store(a.P, (size_t)a.n_tail_base + x, 0, row0, g.nq, lane);
 }
 
-// One consumer warp (cw of kAttMaxWarps) of block c of G.  The first n_active = MT*KS warps take all ring
-// segments of the block's tile range [t_lo, t_hi) starting at ring position `it`; the others take tail tasks.
+// One consumer warp (cw < MT*KS) of block c of G: its share of all ring segments of the block's tile range [t_lo, t_hi),
+// starting at ring position `it`.
 template <int HD, int NT>
-__device__ __forceinline__ bool att_consume(const AttRing& rg, int& it, const AttPlan& pl, const AttGeom& g,
-                                            const StepArgs* __restrict__ args, const KvView& kv, const AttArgs& a, int Hkv,
+__device__ __forceinline__ bool att_consume(const AttRing& rg, int& it, const AttPlan& pl, const AttGeom& g, const AttArgs& a, int Hkv,
                                             int c, int G, int cw, int lane) {
-  const int B = args->B, n_active = g.MT * g.KS, n_spare = kAttMaxWarps - n_active;
+  const int B = a.B, n_active = g.MT * g.KS;
   AttWarp<HD, NT> st;
-  if (cw >= n_active) {
-    // A consumer warp without a share of the ring tiles takes tail tasks (one m-tile of one tail segment
-    // each), dealt over the spare warps of all blocks from the last block down: the tails then run beside
-    // the tiles instead of after them.
-    for (int q = (G - 1 - c) * n_spare + (cw - n_active); q < B * Hkv * g.MT; q += G * n_spare)
-      att_tail_task<HD, NT>(st, g, a, q / g.MT, (q % g.MT) * 16, lane);
-    return true;
-  }
   const int mi = cw / g.KS, ks = cw % g.KS, row0 = mi * 16;
   const long long T = pl.T;
   const long long t_lo = (long long)c * T / G, t_hi = (long long)(c + 1) * T / G;
   long long t = t_lo;
+#pragma unroll 1
   while (t < t_hi) {
     const AttTile x = att_locate(pl, B, g.KPS, (int)t);
     const int n = (int)min((long long)(x.nt_b - x.ti), t_hi - t);
@@ -594,6 +596,7 @@ __device__ __forceinline__ bool att_consume(const AttRing& rg, int& it, const At
     const __half* qlo = a.Qlo ? a.Qlo + ((size_t)x.b * Hkv + x.h) * g.nq * HD : nullptr;
     st.load_q(qhi, row0, g.nq, lane);
     if (rg.ev && cw == 0 && lane == 0) { rg.ev[3] = st.qa[0][0]; rg.ev[0] = att_timer_ns(); }
+#pragma unroll 1
     for (int i = 0; i < n; ++i, ++it) {
       const int s = it % rg.stages;
       const uint32_t bar = att_smem_u32(&rg.full[s]), par = (uint32_t)(it / rg.stages) & 1u;
@@ -623,19 +626,31 @@ __device__ __forceinline__ bool att_consume(const AttRing& rg, int& it, const At
     if (rg.ev && cw == 0 && lane == 0) rg.ev[2] = att_timer_ns();
     t += n;
   }
-  // without spare warps: tail segment (b, h) number x goes to block G-1-(x mod G), key share 0 only
-  if (n_spare == 0 && ks == 0)
-    for (int x = G - 1 - c; x < B * Hkv; x += G) att_tail_task<HD, NT>(st, g, a, x, row0, lane);
   return true;
 }
 
+// All of a consumer warp's work in one attention phase.  The first n_active = MT*KS warps take the ring tiles.  The causal
+// tails (one m-tile of one tail segment per task) go to the warps without a share of the ring tiles, beside the tiles
+// instead of after them; without such warps to those of key share 0.  They are dealt over all blocks from the last block
+// down.
 template <int HD>
-__device__ __forceinline__ bool att_consume_dispatch(const AttRing& rg, int& it, const AttPlan& pl, const AttGeom& g,
-                                                     const StepArgs* __restrict__ args, const KvView& kv, const AttArgs& a,
+__device__ __forceinline__ bool att_consume_dispatch(const AttRing& rg, int& it, const AttPlan& pl, const AttGeom& g, const AttArgs& a,
                                                      int Hkv, int c, int G, int cw, int lane) {
-  if (g.KW == 16) return att_consume<HD, 2>(rg, it, pl, g, args, kv, a, Hkv, c, G, cw, lane);
-  if (g.KW == 32) return att_consume<HD, 4>(rg, it, pl, g, args, kv, a, Hkv, c, G, cw, lane);
-  if constexpr (HD == 64) return att_consume<HD, 8>(rg, it, pl, g, args, kv, a, Hkv, c, G, cw, lane);
+  const int n_active = g.MT * g.KS, n_spare = kAttMaxWarps - n_active;
+  if (cw < n_active) {
+    bool ok = true;
+    if (g.KW == 16) ok = att_consume<HD, 2>(rg, it, pl, g, a, Hkv, c, G, cw, lane);
+    else if (g.KW == 32) ok = att_consume<HD, 4>(rg, it, pl, g, a, Hkv, c, G, cw, lane);
+    else if constexpr (HD == 64) ok = att_consume<HD, 8>(rg, it, pl, g, a, Hkv, c, G, cw, lane);
+    if (!ok) return false;
+  }
+  const int n_tail = n_spare > 0 ? n_spare : g.MT;   // warps of a block that take tails, and this one's number among them
+  const int me = n_spare > 0 ? cw - n_active : (cw % g.KS == 0 ? cw / g.KS : -1);
+  if (me >= 0) {
+    AttWarp<HD, 2> st;
+#pragma unroll 1
+    for (int q = (G - 1 - c) * n_tail + me; q < a.B * Hkv * g.MT; q += G * n_tail) att_tail_task<HD, 2>(st, g, a, q / g.MT, (q % g.MT) * 16, lane);
+  }
   return true;
 }
 
@@ -658,6 +673,7 @@ __device__ __forceinline__ void att_fill_pages(int* pages, const AttPlan& pl, co
                                                int KPS, long long t_lo, long long t_hi, int tid, int nthreads) {
   const int npg = KPS / 16;
   const long long n = min((t_hi - t_lo) * npg, (long long)kAttPageCache);
+#pragma unroll 1
   for (int i = tid; i < n; i += nthreads) {
     const AttTile x = att_locate(pl, B, KPS, (int)(t_lo + i / npg));
     int pi = x.ti * npg + i % npg;
@@ -703,6 +719,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
       const long long t_lo = (long long)c * pl.T / G, t_hi = (long long)(c + 1) * pl.T / G;
       const int npg = g.KPS / 16;
       int it = 0;
+#pragma unroll 1
       for (long long t = t_lo; t < t_hi; ++t, ++it) {
         const int s = it % kAttStages, round = it / kAttStages;
         if (round > 0 && !att_mbar_wait(att_smem_u32(&ctl->empty[s]), (round - 1) & 1, abort_flag, w.status)) break;
@@ -717,7 +734,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   } else {
     AttRing rg{ctl->full, ctl->empty, ctl->cons_cnt, ring, kAttStageBytes, kAttStages, abort_flag, nullptr, w.status, nullptr};
     int it = 0;
-    att_consume_dispatch<HD>(rg, it, pl, g, args, kv, a, Hkv, c, G, warp - 1, lane);
+    att_consume_dispatch<HD>(rg, it, pl, g, a, Hkv, c, G, warp - 1, lane);
   }
   __syncthreads();
   if (threadIdx.x == 0 && *abort_flag) __nanosleep(20000);   // let copies in flight land before the block retires
@@ -785,6 +802,7 @@ __device__ __forceinline__ void att_combine_item(const AttPartials& P, const Att
   float lsum = 0.f, Mrun = -INFINITY, acc[DPL];
 #pragma unroll
   for (int i = 0; i < DPL; ++i) acc[i] = 0.f;
+#pragma unroll 1
   for (int k0 = 0; k0 < n_sub; k0 += 96) {   // 96 sub-partials at a time (three per lane); one pass in practice
     // Everything this pass reads is requested before anything is used: maxima, sums, and the first OB
     // output rows (their weights are not needed to issue the loads).
@@ -823,11 +841,12 @@ __device__ __forceinline__ void att_combine_item(const AttPartials& P, const Att
       const float wgt = k < kn ? __shfl_sync(0xffffffffu, k < 32 ? wk[0] : wk[1], k & 31) : 0.f;
       AttVec<DPL>::fma(acc, ob[k], wgt);
     }
-    for (int kb = OB; kb < kn; kb += OB) {   // further output rows, OB at a time, added in order
+#pragma unroll 1
+    for (int kb = OB; kb < kn; kb += 8) {   // further output rows, eight at a time, added in order
 #pragma unroll
-      for (int k = 0; k < OB; ++k) ob[k] = __ldcg(Po + (size_t)sub_index(k0 + min(kb + k, kn - 1)) * RS);
+      for (int k = 0; k < 8; ++k) ob[k] = __ldcg(Po + (size_t)sub_index(k0 + min(kb + k, kn - 1)) * RS);
 #pragma unroll
-      for (int k = 0; k < OB; ++k) {
+      for (int k = 0; k < 8; ++k) {
         const int kk = kb + k;
         const float wsel = kk < 32 ? wk[0] : (kk < 64 ? wk[1] : wk[2]);
         const float wgt = kk < kn ? __shfl_sync(0xffffffffu, wsel, kk & 31) : 0.f;

@@ -105,6 +105,56 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
+// Sums of N values (N = 4, 8 or 16) over the 32 lanes of a warp, all at once: every exchange halves the values a lane
+// still carries (16 shuffles for N = 16 instead of 80).  A lane returns the total of value lane / (32 / N).
+template <int N>
+__device__ __forceinline__ float warp_sum_n(const float* v, int lane) {
+  float a[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) a[i] = v[i];
+  int bit = 16;
+#pragma unroll
+  for (int h = N / 2; h >= 1; h >>= 1, bit >>= 1) {
+    const bool up = lane & bit;
+#pragma unroll
+    for (int i = 0; i < h; ++i) a[i] = (up ? a[i + h] : a[i]) + __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + h], bit);
+  }
+#pragma unroll
+  for (; bit >= 1; bit >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], bit);
+  return a[0];
+}
+// The same for the maximum of value i over the warp, with the lowest `id` among the lanes that have it.
+template <int N>
+__device__ __forceinline__ void warp_max_n(const float* v, int id, int lane, float& m, int& arg) {
+  float a[N];
+  int b[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) { a[i] = v[i]; b[i] = id; }
+  int bit = 16;
+#pragma unroll
+  for (int h = N / 2; h >= 1; h >>= 1, bit >>= 1) {
+    const bool up = lane & bit;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const float mine = up ? a[i + h] : a[i], om = __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + h], bit);
+      const int mid = up ? b[i + h] : b[i], oid = __shfl_xor_sync(0xffffffffu, up ? b[i] : b[i + h], bit);
+      const bool take = om > mine || (om == mine && oid < mid);
+      a[i] = take ? om : mine;
+      b[i] = take ? oid : mid;
+    }
+  }
+#pragma unroll
+  for (; bit >= 1; bit >>= 1) {
+    const float om = __shfl_xor_sync(0xffffffffu, a[0], bit);
+    const int oid = __shfl_xor_sync(0xffffffffu, b[0], bit);
+    const bool take = om > a[0] || (om == a[0] && oid < b[0]);
+    a[0] = take ? om : a[0];
+    b[0] = take ? oid : b[0];
+  }
+  m = a[0];
+  arg = b[0];
+}
+
 // Block-wide sum with a fixed reduction tree (deterministic).  `red` holds >= 32 floats.
 __device__ __forceinline__ float block_sum(float v, float* red) {
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;

@@ -126,57 +126,6 @@ __device__ __forceinline__ uint32_t instr_desc_pair(int n) {   // M = 256
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
 }
 
-// Sum of 16 values over the 32 lanes of a warp, all 16 at once (16 shuffles instead of 80): lanes 2i and 2i + 1 return
-// the total of value i.
-__device__ __forceinline__ float warp_sum16(const float* v, int lane) {
-  float a[8], b[4], c[2];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const bool up = lane & 16;
-    a[i] = (up ? v[i + 8] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + 8], 16);
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const bool up = lane & 8;
-    b[i] = (up ? a[i + 4] : a[i]) + __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + 4], 8);
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const bool up = lane & 4;
-    c[i] = (up ? b[i + 2] : b[i]) + __shfl_xor_sync(0xffffffffu, up ? b[i] : b[i + 2], 4);
-  }
-  const bool up = lane & 2;
-  float d = (up ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, up ? c[0] : c[1], 2);
-  return d + __shfl_xor_sync(0xffffffffu, d, 1);
-}
-
-// The same for the maximum: lanes 2i and 2i + 1 return the largest of value i over the warp and the lowest `id` that has it.
-__device__ __forceinline__ void warp_max16(const float* v, int id, int lane, float& m, int& arg) {
-  float a[16];
-  int b[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) { a[i] = v[i]; b[i] = id; }
-#pragma unroll
-  for (int h = 8; h >= 1; h >>= 1) {   // value i of the lower half pairs with value i + h; lane bit 2 h picks the half kept
-    const bool up = lane & (2 * h);
-#pragma unroll
-    for (int i = 0; i < h; ++i) {
-      const float mine = up ? a[i + h] : a[i], send = up ? a[i] : a[i + h];
-      const int mine_id = up ? b[i + h] : b[i], send_id = up ? b[i] : b[i + h];
-      const float om = __shfl_xor_sync(0xffffffffu, send, 2 * h);
-      const int oid = __shfl_xor_sync(0xffffffffu, send_id, 2 * h);
-      const bool take = om > mine || (om == mine && oid < mine_id);
-      a[i] = take ? om : mine;
-      b[i] = take ? oid : mine_id;
-    }
-  }
-  const float om = __shfl_xor_sync(0xffffffffu, a[0], 1);
-  const int oid = __shfl_xor_sync(0xffffffffu, b[0], 1);
-  const bool take = om > a[0] || (om == a[0] && oid < b[0]);
-  m = take ? om : a[0];
-  arg = take ? oid : b[0];
-}
-
 template <int SITE, int HD>
 static __global__ void __launch_bounds__(kPairThreads, 1)
 k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
@@ -442,7 +391,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
               sq[i] = x * x;
             }
           }
-          const float t = warp_sum16(sq, lane);
+          const float t = warp_sum_n<16>(sq, lane);
           if ((lane & 1) == 0) sm->x.sums[quarter][c0 + (lane >> 1)] = t;
         } else if constexpr (SITE == PAIR_GU) {
 #pragma unroll
@@ -487,13 +436,13 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           }
           float m;
           int arg;
-          warp_max16(v, n_id, lane, m, arg);
+          warp_max_n<16>(v, n_id, lane, m, arg);
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const float mi = __shfl_sync(0xffffffffu, m, 2 * i);
             v[i] = v[i] == -INFINITY ? 0.f : expf(v[i] - mi);
           }
-          const float e = warp_sum16(v, lane);
+          const float e = warp_sum_n<16>(v, lane);
           if ((lane & 1) == 0) {
             RowStat st; st.m = m; st.s = e; st.arg = arg; st.pad = before;
             sm->x.st[grp][quarter][own] = st;

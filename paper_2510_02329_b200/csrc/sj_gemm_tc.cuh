@@ -103,6 +103,7 @@ __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
 // Bounded wait: gives up after `limit` polls or when another thread of the block gave up.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
                                           uint32_t limit = kSpinLimit) {
+#pragma unroll 1
   for (uint32_t i = 0; i < limit; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     if (i > 64) {
@@ -279,14 +280,18 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         int kb = (int)(u % p.KB);
         int s = it % p.stages;
         uint32_t bar = smem_u32(&ctl->full[s]);
+#pragma unroll 1
         for (int nb = 0; nb < p.a_blocks; ++nb)
           tma_load_2d(smem_u32(smem + (size_t)s * stage_bytes + kWTileBytes + (size_t)nb * p.nblk * 128), &tmA, bar,
                       kb * kBK, (nb / p.NB) * p.plane_rows + (nb % p.NB) * p.nblk, pol_a);
       };
       const int pre = min(p.stages, n_units);
+#pragma unroll 1
       for (int it = 0; it < pre; ++it) w_load(it);   // weights never depend on the previous kernel
       pdl_wait();
+#pragma unroll 1
       for (int it = 0; it < pre; ++it) a_load(it);
+#pragma unroll 1
       for (int it = pre; it < n_units; ++it) {
         int s = it % p.stages, round = it / p.stages;
         if (!mbar_wait(smem_u32(&ctl->empty[s]), (round - 1) & 1, abort_flag, p.status)) break;
@@ -304,18 +309,21 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
       int it = 0, seg = 0;
       long long u = u_lo;
       bool alive = true;
+#pragma unroll 1
       while (u < u_hi && alive) {
         int kb0 = (int)(u % p.KB);
         int len = (int)min((long long)(p.KB - kb0), u_hi - u);
         int acc = seg % p.acc_bufs, use = seg / p.acc_bufs;
         if (use > 0 && !mbar_wait(smem_u32(&ctl->tmem_empty[acc]), (use - 1) & 1, abort_flag, p.status)) break;
         tc_fence_after();
+#pragma unroll 1
         for (int i = 0; i < len; ++i, ++it) {
           int s = it % p.stages;
           if (!mbar_wait(smem_u32(&ctl->full[s]), (it / p.stages) & 1, abort_flag, p.status)) { alive = false; break; }
           tc_fence_after();
           uint32_t wa = smem_u32(smem + (size_t)s * stage_bytes);
           uint64_t dw = smem_desc_sw128(wa);
+#pragma unroll 1
           for (int nb = 0; nb < p.a_blocks; ++nb) {
             uint64_t da = smem_desc_sw128(wa + kWTileBytes + nb * p.nblk * 128);
             uint32_t dcol = tmem_base + acc * p.acc_stride + (nb % p.NB) * p.nblk;
@@ -338,6 +346,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     const int et = threadIdx.x - 64;
     if (p.lm_mode == 1) {
       const int rows = args->gamma + 1;
+#pragma unroll 1
       for (int r = et; r < p.R; r += 128) {
         int b = r / rows, j = r % rows;
         ctl->tgt_tok[r] = (j < args->gamma) ? args->draft_ids[b * args->gamma + j] : -1;
@@ -350,6 +359,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     float* dbg_logits = p.lm_mode ? args->dbg_logits : nullptr;
     int seg = 0;
     long long u = u_lo;
+#pragma unroll 1
     while (u < u_hi) {
       int tile = (int)(u / p.KB), kb0 = (int)(u % p.KB);
       int len = (int)min((long long)(p.KB - kb0), u_hi - u);
@@ -360,6 +370,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * p.acc_stride;
       if (!p.lm_mode) {
         float* dst = p.P + (size_t)(c - p.tile_slots[tile].x) * p.slot_stride + n;
+#pragma unroll 1
         for (int c0 = 0; c0 < p.R; c0 += 16) {
           float v[16];
           tc_ld16(taddr + c0, v);
@@ -376,6 +387,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
           }
         }
       } else {
+#pragma unroll 1
         for (int c0 = 0; c0 < p.R; c0 += 16) {
           float v[16];
           tc_ld16(taddr + c0, v);

@@ -17,8 +17,8 @@
 //               the combine, the embedding and the final acceptance phase
 //
 // GEMM phases: work units are (128-feature tile, 64-wide K block) in tile-major order, dealt evenly to
-// the blocks (stream-K).  Partial sums of a tile that several blocks share travel as 64-bit words {fp32
-// value, phase number} that the finishing block polls (no flag, no fence); the fused epilogues:
+// the blocks (stream-K).  Partial sums of a tile that several blocks share travel as 128-bit words {three fp32
+// values, phase number} that the finishing block polls (no flag, no fence); the fused epilogues:
 //   QKV   -> scale by 1/rms, bias, rotary embedding; queries (fp16, pre-scaled) to the query buffer, K and V
 //            rows into the cache pages (bf16) and into the step's own fp16 side buffer
 //   O     -> residual add, fp32 residual stream, next GEMM input planes (x * gain, hi/lo bf16), per-tile
@@ -84,12 +84,14 @@ struct MegaParams {
   const bf16* lm_head;        // rows of the LM head (top-k test: the drafted tokens' logits are computed ahead of the head)
   const bf16* gain0;          // first layer's attention-norm gain
   float* sumsq;               // [2][d/128][kMegaMaxRows]
-  // Split-K partial sums, [blocks][Rp][128] words of 64 bits: the fp32 value in the low half and, in the
-  // high half, the number of the GEMM phase that wrote it (1, 2, ... within a launch).  A word is stored and
-  // loaded as one 64-bit access, so a reader that sees the phase number it expects also sees the value:
-  // no flag, no fence, and the reader polls the data itself.
-  // Two slots per block ([block][2][Rp][128]): slot 1 for the tile whose first K block it holds, slot 0 otherwise.
-  unsigned long long* pbuf;   //                               }
+  // Split-K partial sums, [blocks][2][Rp / 16][2 groups][3][128 features] words of 128 bits: the fp32 values of three
+  // rows and the number of the GEMM phase that wrote them (unique over the launches of a target: tag0 + 1, + 2, ...).  A
+  // word is stored and loaded as one 128-bit access, so a reader that sees the phase number it expects also sees the
+  // values: no flag, no fence, and the reader polls the data itself.  (Three values a word instead of one halve the
+  // exchange's bytes and take a third of its load instructions, which cost 30 ns each under the weight stream.)
+  // Two slots per block: slot 1 for the tile whose first K block it holds, slot 0 otherwise.
+  uint4* pbuf;
+  unsigned tag0;
   unsigned* gbar;             // device-wide barrier counter   } zeroed before every launch
   int* abort_g;               // device-wide abort word        }
   int n_tail_base;
@@ -178,6 +180,7 @@ __host__ __device__ __forceinline__ SiteInfo site_info(int site, const Dims& dm,
 // Block that owns unit u of a stream-K site.
 __device__ __forceinline__ int unit_owner(unsigned u, unsigned U, int G) {
   unsigned c = u * (unsigned)G / U;
+#pragma unroll 1
   while ((c + 1) * U / (unsigned)G <= u) ++c;
   return (int)c;
 }
@@ -228,6 +231,7 @@ __device__ __forceinline__ int site_units(const SiteSplit& s) {
   unsigned u = s.g_lo;
   Seg g;
   int n = 0;
+#pragma unroll 1
   while (seg_next(s, u, g)) n += g.b - g.a;
   return n;
 }
@@ -258,6 +262,7 @@ struct RingPos {
 template <typename FSite, typename FAtt>
 __device__ __forceinline__ void mega_walk(const MegaParams& p, FSite fsite, FAtt fatt) {
   const int n = mega_n_phases(p);
+#pragma unroll 1
   for (int ph = 0; ph < n; ++ph) {
     int site, l;
     mega_phase(p, ph, site, l);
@@ -276,13 +281,24 @@ __device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned* p) {
 __device__ __forceinline__ void red_relaxed_add(unsigned* p, unsigned v) {
   asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+__device__ __forceinline__ void st_partial(uint4* p, float a, float b, float c, unsigned tag) {
+  const unsigned long long lo = (unsigned long long)__float_as_uint(a) | (unsigned long long)__float_as_uint(b) << 32;
+  const unsigned long long hi = (unsigned long long)__float_as_uint(c) | (unsigned long long)tag << 32;
+  asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p), "l"(lo), "l"(hi) : "memory");
 }
-__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
+struct PartialWord {
+  unsigned long long lo, hi;
+  __device__ __forceinline__ unsigned tag() const { return (unsigned)(hi >> 32); }
+  __device__ __forceinline__ float val(int i) const { return __uint_as_float(i == 0 ? (unsigned)lo : (i == 1 ? (unsigned)(lo >> 32) : (unsigned)hi)); }
+};
+__device__ __forceinline__ PartialWord ld_partial(const uint4* p) {
+  PartialWord w;
+  asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}" : "=l"(w.lo), "=l"(w.hi) : "l"(p) : "memory");
+  return w;
+}
+// Offset of (block, slot, 16-row chunk, epilogue group, triple of rows, feature) in the partial buffer.
+__device__ __forceinline__ size_t partial_at(int block, int slot, int Rp, int chunk, int grp, int t, int f) {
+  return ((((size_t)(2 * block + slot) * (Rp >> 4) + chunk) * 2 + grp) * 3 + t) * kTileN + f;
 }
 
 // Bounded wait on a shared-memory barrier that also watches the device-wide abort word.
@@ -296,6 +312,7 @@ __device__ __forceinline__ bool mega_spin_ge(const unsigned* word, unsigned targ
                                              int* status, int where, int extra, uint32_t limit = kMegaSpin) {
   volatile int* af = &ctl->abort_flag;
   volatile int* ag = p.abort_g;
+#pragma unroll 1
   for (uint32_t i = 0; i < limit; ++i) {
     if (ld_relaxed_u32(word) >= target) return true;
     if (i > 16) {
@@ -309,6 +326,24 @@ __device__ __forceinline__ bool mega_spin_ge(const unsigned* word, unsigned targ
   *ag = 1;
   atomicCAS(status, DEV_OK, DEV_TIMEOUT);
   return false;
+}
+
+// One more poll of a partial-sum wait: false when the wait is over (aborted, or out of its limit).
+__device__ __forceinline__ bool mega_poll_again(uint32_t spin, MegaCtl* ctl, const MegaParams& p, int* status, int extra) {
+  volatile int* af = &ctl->abort_flag;
+  if (spin > 16) {
+    if (*af) return false;
+    if ((spin & 63) == 0 && *reinterpret_cast<volatile int*>(p.abort_g)) { *af = 1; return false; }
+    if (spin > 4096) __nanosleep(64);
+    if (spin >= kMegaSpin) {
+      *af = 1;
+      att_note_timeout(p.abort_g, 7, extra);
+      *reinterpret_cast<volatile int*>(p.abort_g) = 1;
+      atomicCAS(status, DEV_OK, DEV_TIMEOUT);
+      return false;
+    }
+  }
+  return true;
 }
 
 // Device-wide barrier for the 256 workers of every block.  Returns false once the step is aborting.
@@ -341,6 +376,7 @@ __device__ __forceinline__ bool mega_grid_sync(MegaCtl* ctl, const MegaParams& p
 __device__ __forceinline__ bool mega_wait_bars(int need, MegaCtl* ctl, const MegaParams& p, int* status, int where) {
   volatile int* bp = &ctl->bars_passed;
   volatile int* af = &ctl->abort_flag;
+#pragma unroll 1
   for (uint32_t i = 0; i < kMegaSpin; ++i) {
     if (*bp >= need) return true;
     if (*af) return false;
@@ -403,25 +439,30 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
   const unsigned U = ss.U;
   const int nt128 = dm.d / kTileN;
   const MegaLayerPtrs lp = p.lp[l];
-  // 1/rms of this phase's input rows (the planes hold x * gain; the scalar is applied here).  One warp
-  // per row, lanes over the column tiles, fixed shuffle tree: all loads of a row are in flight together.
+  // 1/rms of this phase's input rows (the planes hold x * gain; the scalar is applied here): one warp per row of its
+  // group, lanes over the column tiles, the loads of all its rows in flight together (72 rows, four at a time: 6 us
+  // before the QKV phase's first accumulator is looked at).
   if (site == SITE_QKV || site == SITE_GU || site == SITE_LM) {
+    constexpr int KR = NS == 8 ? kMegaMaxRows / 8 : 2;
     const int buf = (site == SITE_GU) ? 1 : 0;
-    for (int r0 = quarter; r0 < R; r0 += 16) {
-      float part[4];
+    float part[KR];
+    int row[KR];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int r = r0 + 4 * k;
-        part[k] = 0.f;
-        if (r < R && mega_row_group(r, R) == grp)
-          for (int t = lane; t < nt128; t += 32) part[k] += __ldcg(p.sumsq + ((size_t)buf * nt128 + t) * kMegaMaxRows + r);
-      }
+    for (int k = 0; k < KR; ++k) {
+      const int i = quarter + 4 * k, c16 = (i >> 3) * 16, n16 = min(16, R - c16), h16 = (n16 + 1) >> 1;   // i-th row slot of the group
+      row[k] = c16 < R && (i & 7) < (grp ? n16 - h16 : h16) ? c16 + (grp ? h16 : 0) + (i & 7) : -1;
+      part[k] = 0.f;
+      if (row[k] >= 0 && lane < nt128) part[k] = __ldcg(p.sumsq + ((size_t)buf * nt128 + lane) * kMegaMaxRows + row[k]);
+    }
+#pragma unroll 1
+    for (int t = lane + 32; t < nt128; t += 32)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int r = r0 + 4 * k;
-        const float s = warp_sum(part[k]);
-        if (lane == 0 && r < R && mega_row_group(r, R) == grp) ctl->inv[r] = 1.0f / sqrtf(s / (float)dm.d + dm.eps);
-      }
+      for (int k = 0; k < KR; ++k)
+        if (row[k] >= 0) part[k] += __ldcg(p.sumsq + ((size_t)buf * nt128 + t) * kMegaMaxRows + row[k]);
+#pragma unroll
+    for (int k = 0; k < KR; ++k) {
+      const float s = warp_sum(part[k]);
+      if (lane == 0 && row[k] >= 0) ctl->inv[row[k]] = 1.0f / sqrtf(s / (float)dm.d + dm.eps);
     }
     bar_sync(bar_id, 128);
   }
@@ -429,7 +470,7 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
   if (topk) {
     // The LM head stores no logits, so the rank of a drafted token is counted tile by tile against its own
     // logit, which therefore has to exist first: one dot product per row (this group's rows, a warp each).
-    const int gamma = rows - 1;
+#pragma unroll 1
     for (int r = quarter; r < R; r += 4) {
       if (mega_row_group(r, R) != grp) continue;
       const int tok = ctl->tgt_tok[r];
@@ -437,7 +478,6 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
       if (tok >= 0) z = planes_dot(reinterpret_cast<const bf16*>(w.A), R, dm.d, r, p.lm_head + (size_t)min(tok, dm.V - 1) * dm.d, lane) * ctl->inv[r];
       if (lane == 0) ctl->zd[r] = z;
     }
-    (void)gamma;
     bar_sync(bar_id, 128);
   }
   const int qd = dm.Hq * dm.hd, kd = dm.Hkv * dm.hd, tq = qd / kTileN, tk = kd / kTileN;
@@ -445,48 +485,213 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
   float* dbg_logits = (site == SITE_LM) ? args->dbg_logits : nullptr;
   const float qscale = 1.4426950408889634f / sqrtf((float)HD);
   const int fl = et;   // feature inside the tile == TMEM lane
+  const unsigned tag = p.tag0 + (unsigned)gseq;
+  // With fewer units than blocks a block holds at most one unit and most hold none: sharers are then found unit by unit.
+  const bool sparse = U < (unsigned)G;
 
-  int n_rs = 0, rs_tile0 = 0, rs_first0 = 0, rs_last0 = 0, rs_tile1 = 0, rs_first1 = 0, rs_last1 = 0;
-  float rs_gn0 = 1.f, rs_gn1 = 1.f;
+  // Per-feature constants of a tile's epilogue.  con: the QKV bias, or the gain of the norm that reads the result; it
+  // is loaded before the tile's accumulator is waited for (loaded later, its latency holds up the loads behind it).
+  struct Feature { int kind, head, dim; float con; };
+  auto feature = [&](int tile, float con) -> Feature {
+    Feature x{0, 0, 0, con};
+    if (site == SITE_QKV) {
+      x.kind = tile < tq ? 0 : (tile < tq + tk ? 1 : 2);
+      const int fs = (tile - (x.kind == 0 ? 0 : (x.kind == 1 ? tq : tq + tk))) * kTileN + fl;
+      x.head = fs / HD;
+      x.dim = fs % HD;
+    }
+    return x;
+  };
+  auto feature_con = [&](int tile) -> float {
+    if (site == SITE_QKV) {
+      const bf16* bp = tile < tq ? lp.bq : (tile < tq + tk ? lp.bk : lp.bv);
+      const int t0 = tile < tq ? 0 : (tile < tq + tk ? tq : tq + tk);
+      return bp ? __bfloat162float(bp[(tile - t0) * kTileN + fl]) : 0.f;
+    }
+    if (site == SITE_O) return __bfloat162float(lp.gain_ffn[tile * kTileN + fl]);
+    if (site == SITE_DOWN) return __bfloat162float(lp.gain_next[tile * kTileN + fl]);
+    return 0.f;
+  };
+  // What finishing `N` rows from row0 (cnt of them exist) reads besides the sums: residual rows or rotary table rows.
+  // Unpredicated (rows past the last repeat it), so that all loads are in flight together.
+  auto aux_loads = [&](auto& aux, const Feature& x, int tile, int row0, int cnt) {
+    constexpr int N = sizeof(aux) / sizeof(float2);
+    if (site == SITE_O || site == SITE_DOWN) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) aux[i].x = __ldcg(w.X + (size_t)max(min(row0 + i, row0 + cnt - 1), 0) * dm.d + tile * kTileN + fl);
+    } else if (site == SITE_QKV && x.kind < 2) {
+      const int ii = x.dim & (HD / 2 - 1);
+#pragma unroll
+      for (int i = 0; i < N; ++i) aux[i] = __ldcg(w.rope + (size_t)max(min(row0 + i, row0 + cnt - 1), 0) * (HD / 2) + ii);
+    }
+  };
+  // The epilogue proper: v holds the complete sums of N rows from row0 (cnt of them exist) of this thread's feature.
+  auto finish = [&](auto& v, auto& aux, const Feature& x, int tile, int row0, int cnt) {
+    constexpr int N = sizeof(v) / sizeof(float);
+    constexpr int RN = N <= 4 ? 4 : 8;   // N rounded up to what the warp reductions take
+    if (site == SITE_QKV) {
+      const int half = HD / 2;
+#pragma unroll
+      for (int i = 0; i < N; ++i) v[i] = v[i] * (i < cnt ? ctl->inv[row0 + i] : 0.f) + x.con;
+      if (x.kind < 2) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) ctl->u.exch[grp][fl][i] = v[i];
+        bar_sync(bar_id, 128);
+        const bool first = x.dim < half;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          const float xp = ctl->u.exch[grp][fl ^ half][i];
+          v[i] = first ? v[i] * aux[i].x - xp * aux[i].y : v[i] * aux[i].x + xp * aux[i].y;
+        }
+        bar_sync(bar_id, 128);
+      }
+      if (et == 0) MEGA_EV2(0, sidx, 6);
+      // query row (b, kvh, g, j) sits at ((b*Hq + head)*rows + j)*HD; a cache row at
+      // ((((layer*n_pages + page)*2 + K|V)*Hkv + head)*page_size + slot)*HD: the per-row parts are tabulated
+      if (x.kind == 0) {
+        __half* qb = w.Qb + (size_t)x.head * rows * HD + x.dim;
+        __half* ql = w.Qlo + (size_t)x.head * rows * HD + x.dim;
+        const bool two_term = l < p.att_precise_layers;   // block-uniform
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+          if (i < cnt) {
+            const float qv = v[i] * qscale;
+            const __half hq = __float2half_rn(qv);
+            qb[ctl->row_qoff[row0 + i]] = hq;
+            if (two_term) ql[ctl->row_qoff[row0 + i]] = __float2half_rn(qv - __half2float(hq));
+          }
+      } else {
+        bf16* kvb = reinterpret_cast<bf16*>(kv.pool) +
+                    ((size_t)l * kv.n_pages * 2 * dm.Hkv + (size_t)(x.kind - 1) * dm.Hkv + x.head) * kv.page_size * HD + x.dim;
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+          if (i < cnt && ctl->row_kvoff[row0 + i] >= 0) kvb[ctl->row_kvoff[row0 + i]] = __float2bfloat16_rn(v[i]);
+        __half* kn = w.KVn + (size_t)(x.head * 2 + x.kind - 1) * rows * HD + x.dim;
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+          if (i < cnt) kn[ctl->row_nkvoff[row0 + i]] = __float2half_rn(v[i]);
+      }
+    } else if (site == SITE_O || site == SITE_DOWN) {
+      const int f = tile * kTileN + fl;
+      const int buf = (site == SITE_O) ? 1 : 0;
+      float sq[RN];
+#pragma unroll
+      for (int i = 0; i < RN; ++i) sq[i] = 0.f;
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        if (i < cnt) {
+          const float y = aux[i].x + v[i];
+          w.X[(size_t)(row0 + i) * dm.d + f] = y;
+          store_act<bf16>(w.A, R, dm.d, row0 + i, f, y * x.con);
+          sq[i] = y * y;
+        }
+      if (et == 0) MEGA_EV2(0, sidx, 2);
+      const float tot = warp_sum_n<RN>(sq, lane);
+      if (lane % (32 / RN) == 0) ctl->red[grp][quarter][lane / (32 / RN)] = tot;
+      bar_sync(bar_id, 128);
+      if (et < cnt)
+        p.sumsq[((size_t)buf * nt128 + tile) * kMegaMaxRows + row0 + et] =
+            ctl->red[grp][0][et] + ctl->red[grp][1][et] + ctl->red[grp][2][et] + ctl->red[grp][3][et];
+      bar_sync(bar_id, 128);
+      if (et == 0) MEGA_EV2(0, sidx, 3);
+    } else if (site == SITE_GU) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) v[i] *= (i < cnt ? ctl->inv[row0 + i] : 0.f);
+      // gate threads finish the first half of the rows, up threads the others: each hands over its other values
+      constexpr int H = (N + 1) / 2;
+      const bool is_gate = fl < 64;
+#pragma unroll
+      for (int i = 0; i < H; ++i) ctl->u.exch[grp][fl][i] = is_gate ? v[min(H + i, N - 1)] : v[i];
+      bar_sync(bar_id, 128);
+      const int f = tile * 64 + (fl & 63), h0 = is_gate ? 0 : H;
+#pragma unroll
+      for (int i = 0; i < H; ++i) {
+        const float other = ctl->u.exch[grp][fl ^ 64][i];
+        const float g = is_gate ? v[i] : other, up = is_gate ? other : v[min(H + i, N - 1)];
+        if (h0 + i < cnt) store_act<bf16>(w.H, R, dm.F, row0 + h0 + i, f, g / (1.0f + expf(-g)) * up);
+      }
+      bar_sync(bar_id, 128);
+    } else {   // LM head
+      const int n = tile * kTileN + fl;
+      const int own = lane / (32 / RN);   // the row whose totals this lane ends up with
+      float z[RN];
+      int before = 0;
+#pragma unroll
+      for (int i = 0; i < RN; ++i) z[i] = -INFINITY;
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        const int r = min(row0 + i, R - 1);
+        const float raw = v[i] * ctl->inv[r];
+        const bool live = i < cnt && n < dm.V;
+        if (live) {
+          if (w.logits) w.logits[(size_t)r * dm.V + n] = raw;
+          if (dbg_logits) dbg_logits[(size_t)r * dm.V + n] = raw;
+          z[i] = raw * invT;
+          if (n == ctl->tgt_tok[r]) w.tgt_logit[r] = z[i];
+        }
+        if (topk) {
+          const int tg = ctl->tgt_tok[r];
+          const float zd = ctl->zd[r];
+          const int cnt_before = __popc(__ballot_sync(0xffffffffu, live && tg >= 0 && n != tg && (raw > zd || (raw == zd && n < tg))));
+          if (i == own) before = cnt_before;
+        }
+      }
+      float m;
+      int arg;
+      warp_max_n<RN>(z, n, lane, m, arg);
+#pragma unroll
+      for (int i = 0; i < RN; ++i) {
+        const float mi = __shfl_sync(0xffffffffu, m, i * (32 / RN));
+        z[i] = z[i] == -INFINITY ? 0.f : expf(z[i] - mi);
+      }
+      const float e = warp_sum_n<RN>(z, lane);
+      if (lane % (32 / RN) == 0) {
+        RowStat st; st.m = m; st.s = e; st.arg = arg; st.pad = before;
+        ctl->wstat[grp][quarter][own] = st;
+      }
+      bar_sync(bar_id, 128);
+      if (et < cnt) {
+        RowStat a = ctl->wstat[grp][0][et];
+        a = stat_merge(a, ctl->wstat[grp][1][et]);
+        a = stat_merge(a, ctl->wstat[grp][2][et]);
+        a = stat_merge(a, ctl->wstat[grp][3][et]);
+        w.stats[(size_t)tile * R + row0 + et] = a;
+      }
+      bar_sync(bar_id, 128);
+    }
+  };
+
+  // How a tile that several blocks share is finished.
+  //   by rows   every sharing block publishes all its rows and finishes R / n of them after the loop over its segments;
+  //   by owner  the block with the first K block gathers the others' words and finishes the tile at once.
+  // O and down are finished by rows (their epilogue is the longest), and everything is beyond 12 rows (NS 8), where
+  // one block finishing 16-row chunk after chunk while its partners idle at the barrier cost 10..15 us a phase at
+  // 48 and 72 rows.  At few rows the owner is faster for QKV and gate/up: finishing by rows is one more round trip for
+  // every block.
+  constexpr bool kAllRows = NS == 8;
+  constexpr int TR = (NS + 2) / 3;             // words per thread and chunk
+  constexpr int CB = 2;                        // owner: contributors whose words are in flight together
+  int n_rs = 0, rs_tile0 = 0, rs_first0 = 0, rs_n0 = 1, rs_j0 = 0, rs_tile1 = 0, rs_first1 = 0, rs_n1 = 1, rs_j1 = 0;
+  float rs_con0 = 0.f, rs_con1 = 0.f;
   unsigned u = ss.g_lo;
   Seg sg;
+#pragma unroll 1
   while (seg_next(ss, u, sg)) {
     const int tile = sg.tile, kb0 = sg.kb0;
-    const bool mine = sg.b > sg.a;   // this block computed a share of the segment
     const int acc = seg & 1, use = seg >> 1;
     const uint32_t taddr = ctl->tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 2 * Rp);
-
-    // per-tile constants of the fused epilogues; their global loads are issued before any wait
-    int kind = 0, head = 0, dim = 0;
-    float bias = 0.f, gn = 1.f;
-    if (site == SITE_QKV) {
-      int fs;
-      if (tile < tq) { kind = 0; fs = tile * kTileN + fl; }
-      else if (tile < tq + tk) { kind = 1; fs = (tile - tq) * kTileN + fl; }
-      else { kind = 2; fs = (tile - tq - tk) * kTileN + fl; }
-      head = fs / HD;
-      dim = fs % HD;
-      const bf16* bp = kind == 0 ? lp.bq : (kind == 1 ? lp.bk : lp.bv);
-      if (bp) bias = __bfloat162float(bp[fs]);
-    } else if (site == SITE_O) {
-      gn = __bfloat162float(lp.gain_ffn[tile * kTileN + fl]);
-    } else if (site == SITE_DOWN) {
-      gn = __bfloat162float(lp.gain_next[tile * kTileN + fl]);
-    }
-
     const bool complete = (kb0 == 0) && (sg.len == ss.KB);
-    // The O and down projections split a shared tile's epilogue by ROWS: the n blocks that hold K ranges of
-    // the tile each finish R / n of its rows (all 128 features of them) and publish their sums of the other
-    // rows, instead of one block finishing the whole tile while the others idle at the barrier.  (Needs every
-    // block to hold units, so that the sharing blocks are consecutive.)
-    const bool rowsplit = (site == SITE_O || site == SITE_DOWN) && !complete && U >= (unsigned)G;
+    const bool rowsplit = !complete && (kAllRows || ((site == SITE_O || site == SITE_DOWN) && !sparse));
     const bool owner = (kb0 == 0) && !rowsplit;
-    int c_first = c, c_last = c;   // first and last of the blocks that share this tile
-    if ((owner && !complete) || rowsplit) c_last = unit_owner((unsigned)(tile + 1) * (unsigned)ss.KB - 1u, U, G);
-    if (rowsplit) c_first = unit_owner((unsigned)tile * (unsigned)ss.KB, U, G);
+    int c_first = c, c_last = c;   // first and last of the blocks that share this tile (every block holds units)
+    if (!complete && !sparse) {
+      if (owner || rowsplit) c_last = unit_owner((unsigned)(tile + 1) * (unsigned)ss.KB - 1u, U, G);
+      if (rowsplit) c_first = unit_owner((unsigned)tile * (unsigned)ss.KB, U, G);
+    }
+    const float con = owner || rowsplit ? feature_con(tile) : 0.f;
+    const Feature x = feature(tile, con);
     if (et == 0) {
-      int ok = 1;
-      if (mine) ok = mega_wait(smem_u32(&ctl->tmem_full[acc]), use & 1, ctl, p, w.status, 6, gseq) ? 1 : 0;
+      const int ok = mega_wait(smem_u32(&ctl->tmem_full[acc]), use & 1, ctl, p, w.status, 6, gseq) ? 1 : 0;
       ctl->bcast[2 * grp + (seg & 1)] = ok;
     }
     bar_sync(bar_id, 128);
@@ -494,337 +699,139 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
     tc_fence_after();
     if (et == 0) MEGA_EV(sidx, 4);
 
+#pragma unroll 1
     for (int c16 = 0; c16 < Rp; c16 += 16) {
       // this group's rows of the 16-row chunk: the first or the second half of the rows that exist
       const int n16 = max(min(16, R - c16), 0), h16 = (n16 + 1) >> 1;
-      const int c0 = c16 + (grp ? h16 : 0), nr = grp ? n16 - h16 : h16, rend = c0 + nr;
-      float v[NS], xs[NS];
-      float2 cs[NS];
-      // every global load of this chunk is issued before anything waits on one of them
-      if (owner && (site == SITE_O || site == SITE_DOWN)) {   // residual rows
-        const int f = tile * kTileN + fl;
-#pragma unroll
-        for (int i = 0; i < NS; ++i) xs[i] = __ldcg(w.X + (size_t)max(min(c0 + i, rend - 1), 0) * dm.d + f);   // unpredicated: rows past R repeat the last row
-      }
-      if (owner && site == SITE_QKV && kind < 2) {            // rotary table rows
-        const int ii = dim & (HD / 2 - 1);
-#pragma unroll
-        for (int i = 0; i < NS; ++i)
-          cs[i] = __ldcg(w.rope + (size_t)max(min(c0 + i, rend - 1), 0) * (HD / 2) + ii);
-      }
-      if (mine) {
+      const int c0 = c16 + (grp ? h16 : 0), nr = grp ? n16 - h16 : h16, ntr = (nr + 2) / 3;
+      float v[NS];
+      float2 aux[NS];
+      if (owner) aux_loads(aux, x, tile, c0, nr);
+      {
         float hi8[8], lo8[8];
         tc_ld8(taddr + c0, hi8);
         tc_ld8(taddr + Rp + c0, lo8);
 #pragma unroll
         for (int i = 0; i < NS; ++i) v[i] = hi8[i] + lo8[i];
-      } else {
-#pragma unroll
-        for (int i = 0; i < NS; ++i) v[i] = 0.f;
       }
-      const unsigned long long tag = (unsigned long long)(unsigned)gseq << 32;
       if (et == 0 && owner) MEGA_EV2(0, sidx, 0);
-      if (rowsplit) {   // publish every row; the rows are finished after the loop over the segments
-        unsigned long long* dst = p.pbuf + ((size_t)(2 * c + (c == c_first ? 1 : 0)) * Rp + c0) * kTileN + fl;
+      if (!owner) {   // publish the partial sums, each word with this phase's number
+        uint4* dst = p.pbuf + partial_at(c, rowsplit && kb0 == 0 ? 1 : 0, Rp, c16 >> 4, grp, 0, fl);
 #pragma unroll
-        for (int i = 0; i < NS; ++i)
-          if (i < nr) st_relaxed_u64(dst + (size_t)i * kTileN, tag | __float_as_uint(v[i]));
+        for (int t = 0; t < TR; ++t)
+          if (t < ntr)
+            st_partial(dst + t * kTileN, v[3 * t], 3 * t + 1 < NS ? v[min(3 * t + 1, NS - 1)] : 0.f, 3 * t + 2 < NS ? v[min(3 * t + 2, NS - 1)] : 0.f, tag);
         continue;
       }
-      if (!owner) {   // publish the partial sums, each with this phase's number
-        unsigned long long* dst = p.pbuf + ((size_t)(2 * c) * Rp + c0) * kTileN + fl;
-#pragma unroll
-        for (int i = 0; i < NS; ++i)
-          if (i < nr) st_relaxed_u64(dst + (size_t)i * kTileN, tag | __float_as_uint(v[i]));
-        continue;
-      }
-      // The other blocks' shares of this tile: two blocks' words in flight at a time, all of them reloaded
-      // until every one carries this phase's number, then added in group order (so the sum does not depend
-      // on arrival order).  Often they were published long ago: a group's share of somebody else's tile is
-      // the first thing it computes.  A wait that runs out raises the abort word and goes on with whatever
-      // it read (the block leaves together at its next block-wide check).
-      for (int cb = c + 1; cb <= c_last; cb += 2) {
-        unsigned long long pw[2][NS];
-        const unsigned long long* src[2];
-        bool live[2];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const int c2 = cb + k;
-          live[k] = c2 <= c_last && has_units(c2, U, G);   // groups without units add nothing
-          src[k] = p.pbuf + ((size_t)(2 * (live[k] ? c2 : c)) * Rp + c0) * kTileN + fl;
-        }
-        volatile int* af = &ctl->abort_flag;
-        for (uint32_t spin = 0;; ++spin) {
-          bool ok = true;
-          // every load is issued before any result is looked at: rows past R read row 0 again (in
-          // bounds, ignored below) instead of being predicated off, which would put a select after each load
-#pragma unroll
-          for (int k = 0; k < 2; ++k)
-#pragma unroll
-            for (int i = 0; i < NS; ++i) pw[k][i] = ld_relaxed_u64(src[k] + (size_t)(i < nr ? i : 0) * kTileN);
-#pragma unroll
-          for (int k = 0; k < 2; ++k)
-#pragma unroll
-            for (int i = 0; i < NS; ++i) ok = ok && (!live[k] || i >= nr || (pw[k][i] >> 32) == (tag >> 32));
-          if (ok) break;
-          if (spin > 16) {
-            if (*af) break;
-            if ((spin & 63) == 0 && *reinterpret_cast<volatile int*>(p.abort_g)) { *af = 1; break; }
-            if (spin > 4096) __nanosleep(64);
-            if (spin >= kMegaSpin) {
-              *af = 1;
-              att_note_timeout(p.abort_g, 7, gseq);
-              *reinterpret_cast<volatile int*>(p.abort_g) = 1;
-              atomicCAS(w.status, DEV_OK, DEV_TIMEOUT);
-              break;
-            }
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-#pragma unroll
-          for (int i = 0; i < NS; ++i) v[i] += (live[k] && i < nr) ? __uint_as_float((unsigned)pw[k][i]) : 0.f;
-      }
-      if (et == 0) MEGA_EV(sidx, 5);
-      if (et == 0) MEGA_EV2(0, sidx, 1);
-      if (site == SITE_QKV) {
-        const int half = HD / 2;
-#pragma unroll
-        for (int i = 0; i < NS; ++i) {
-          const int r = c0 + i;
-          v[i] = v[i] * (r < rend ? ctl->inv[r] : 0.f) + bias;
-        }
-        if (kind < 2) {
-#pragma unroll
-          for (int i = 0; i < NS; ++i) ctl->u.exch[grp][fl][i] = v[i];
-          bar_sync(bar_id, 128);
-          const bool first = dim < half;
-#pragma unroll
-          for (int i = 0; i < NS; ++i) {
-            const float xp = ctl->u.exch[grp][fl ^ half][i];
-            v[i] = first ? v[i] * cs[i].x - xp * cs[i].y : v[i] * cs[i].x + xp * cs[i].y;
-          }
-          bar_sync(bar_id, 128);
-        }
-        if (et == 0) MEGA_EV2(0, sidx, 6);
-        // query row (b, kvh, g, j) sits at ((b*Hq + head)*rows + j)*HD; a cache row at
-        // ((((layer*n_pages + page)*2 + K|V)*Hkv + head)*page_size + slot)*HD: the per-row parts are tabulated
-        if (kind == 0) {
-          __half* qb = w.Qb + (size_t)head * rows * HD + dim;
-          __half* ql = w.Qlo + (size_t)head * rows * HD + dim;
-          const bool two_term = l < p.att_precise_layers;   // block-uniform
-#pragma unroll
-          for (int i = 0; i < NS; ++i)
-            if (i < nr) {
-              const float qv = v[i] * qscale;
-              const __half hq = __float2half_rn(qv);
-              qb[ctl->row_qoff[c0 + i]] = hq;
-              if (two_term) ql[ctl->row_qoff[c0 + i]] = __float2half_rn(qv - __half2float(hq));
-            }
-        } else {
-          bf16* kvb = reinterpret_cast<bf16*>(kv.pool) +
-                      ((size_t)l * kv.n_pages * 2 * dm.Hkv + (size_t)(kind - 1) * dm.Hkv + head) * kv.page_size * HD + dim;
-#pragma unroll
-          for (int i = 0; i < NS; ++i)
-            if (i < nr && ctl->row_kvoff[c0 + i] >= 0) kvb[ctl->row_kvoff[c0 + i]] = __float2bfloat16_rn(v[i]);
-          __half* kn = w.KVn + (size_t)(head * 2 + kind - 1) * rows * HD + dim;
-#pragma unroll
-          for (int i = 0; i < NS; ++i)
-            if (i < nr) kn[ctl->row_nkvoff[c0 + i]] = __float2half_rn(v[i]);
-        }
-      } else if (site == SITE_O || site == SITE_DOWN) {
-        const int f = tile * kTileN + fl;
-        const int buf = (site == SITE_O) ? 1 : 0;
-        float ss[NS];
-#pragma unroll
-        for (int i = 0; i < NS; ++i) {
-          const int r = c0 + i;
-          ss[i] = 0.f;
-          if (r < rend) {
-            const float x = xs[i] + v[i];
-            w.X[(size_t)r * dm.d + f] = x;
-            store_act<bf16>(w.A, R, dm.d, r, f, x * gn);
-            ss[i] = x * x;
-          }
-        }
-        if (et == 0) MEGA_EV2(0, sidx, 2);
-#pragma unroll
-        for (int i = 0; i < NS; ++i)
-          if (i < nr) ss[i] = warp_sum(ss[i]);   // block-uniform
-        if (lane == 0) {
-#pragma unroll
-          for (int i = 0; i < NS; ++i) ctl->red[grp][quarter][i] = ss[i];
-        }
-        bar_sync(bar_id, 128);
-        if (et < nr)
-          p.sumsq[((size_t)buf * nt128 + tile) * kMegaMaxRows + c0 + et] =
-              ctl->red[grp][0][et] + ctl->red[grp][1][et] + ctl->red[grp][2][et] + ctl->red[grp][3][et];
-        bar_sync(bar_id, 128);
-        if (et == 0) MEGA_EV2(0, sidx, 3);
-      } else if (site == SITE_GU) {
-#pragma unroll
-        for (int i = 0; i < NS; ++i) {
-          const int r = c0 + i;
-          v[i] *= (r < rend ? ctl->inv[r] : 0.f);
-        }
-        if (fl >= 64) {
-#pragma unroll
-          for (int i = 0; i < NS; ++i) ctl->u.exch[grp][fl - 64][i] = v[i];
-        }
-        bar_sync(bar_id, 128);
-        if (fl < 64) {
-          const int f = tile * 64 + fl;
-#pragma unroll
-          for (int i = 0; i < NS; ++i) {
-            const int r = c0 + i;
-            if (r < rend) {
-              const float g = v[i], up = ctl->u.exch[grp][fl][i];
-              store_act<bf16>(w.H, R, dm.F, r, f, g / (1.0f + expf(-g)) * up);
-            }
-          }
-        }
-        bar_sync(bar_id, 128);
-      } else {   // LM head
-        const int n = tile * kTileN + fl;
-#pragma unroll
-        for (int i = 0; i < NS; ++i) {
-          const int r = c0 + i;
-          float z = -INFINITY;
-          if (r < rend && n < dm.V) {
-            const float raw = v[i] * ctl->inv[r];
-            if (w.logits) w.logits[(size_t)r * dm.V + n] = raw;
-            if (dbg_logits) dbg_logits[(size_t)r * dm.V + n] = raw;
-            z = raw * invT;
-            if (n == ctl->tgt_tok[r]) w.tgt_logit[r] = z;
-          }
-          float m = z;
-          int arg = n;
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            const float om = __shfl_xor_sync(0xffffffffu, m, o);
-            const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
-            if (om > m || (om == m && oa < arg)) { m = om; arg = oa; }
-          }
-          float e = (z == -INFINITY) ? 0.f : expf(z - m);
-          e = warp_sum(e);
-          int before = 0;
-          if (topk) {
-            const int rr = min(r, R - 1), tg = ctl->tgt_tok[rr];
-            const float raw = v[i] * ctl->inv[rr], zd = ctl->zd[rr];
-            const bool bf = r < rend && n < dm.V && tg >= 0 && n != tg && (raw > zd || (raw == zd && n < tg));
-            before = __popc(__ballot_sync(0xffffffffu, bf));
-          }
-          if (lane == 0) {
-            RowStat st; st.m = m; st.s = e; st.arg = arg; st.pad = before;
-            ctl->wstat[grp][quarter][i] = st;
-          }
-        }
-        bar_sync(bar_id, 128);
-        if (et < nr) {
-          RowStat a = ctl->wstat[grp][0][et];
-          a = stat_merge(a, ctl->wstat[grp][1][et]);
-          a = stat_merge(a, ctl->wstat[grp][2][et]);
-          a = stat_merge(a, ctl->wstat[grp][3][et]);
-          w.stats[(size_t)tile * R + c0 + et] = a;
-        }
-        bar_sync(bar_id, 128);
-      }
-    }
-    if (et == 0) MEGA_EV2(0, sidx, 7);
-    if (mine) {
-      tc_fence_before();
-      mbar_arrive(smem_u32(&ctl->tmem_empty[acc]));
-      ++seg;
-    }
-    if (rowsplit) {   // at most two per phase: the block's first and last segment
-      if (n_rs == 0) { rs_tile0 = tile; rs_first0 = c_first; rs_last0 = c_last; rs_gn0 = gn; }
-      else { rs_tile1 = tile; rs_first1 = c_first; rs_last1 = c_last; rs_gn1 = gn; }
-      ++n_rs;
-    }
-  }
-  // Row-split tiles (O and down projections): this block's rows of each shared tile.  Every sharing block
-  // has published all its rows by now or will without waiting for anybody (publishing comes first in every
-  // block), so the waits below cannot form a chain.  A row's sums are added in block order.
+      if constexpr (!kAllRows) {
+        // The other blocks' shares of this tile: two blocks' words in flight at a time, all of them reloaded until every
+        // one carries this phase's number, then added in block order (so the sum does not depend on arrival
+        // order).  Often they were published long ago: a block's share of somebody else's tile is the first thing it
+        // computes.  A wait that runs out raises the abort word and goes on with whatever it read (the block leaves
+        // together at its next block-wide check).
+        const int n_con = complete ? 0 : (sparse ? ss.KB - 1 : c_last - c);
 #pragma unroll 1
-  for (int q = 0; q < n_rs; ++q) {
-    const int tile = q ? rs_tile1 : rs_tile0, c_first = q ? rs_first1 : rs_first0, c_last = q ? rs_last1 : rs_last0;
-    const float gn = q ? rs_gn1 : rs_gn0;
-    const int n = c_last - c_first + 1, j = c - c_first;
-    const int f = tile * kTileN + fl;
-    const int buf = (site == SITE_O) ? 1 : 0;
-    const unsigned long long tag = (unsigned long long)(unsigned)gseq << 32;
-    volatile int* af = &ctl->abort_flag;
-#pragma unroll 1
-    for (int c16 = 0; c16 < Rp; c16 += 16) {
-      const int n16 = max(min(16, R - c16), 0), h16 = (n16 + 1) >> 1;
-      const int c0 = c16 + (grp ? h16 : 0), nr = grp ? n16 - h16 : h16;
-      // Rows are dealt with weight 1 to the first and the last sharing block and weight 2 to the others:
-      // the first block of one tile is as a rule the last block of the tile before, and finishes rows of both.
-      const int wsum = 2 * n - 2, w_lo = j == 0 ? 0 : 2 * j - 1, w_hi = j == n - 1 ? wsum : 2 * j + 1;
-      const int a = max(w_lo * R / wsum - c0, 0), b = min(w_hi * R / wsum - c0, nr);   // this block's rows of the chunk: [a, b)
-#pragma unroll 1
-      for (int i = a; i < b; i += 2) {   // two rows at a time: their loads share one round trip
-        const int i1 = min(i + 1, b - 1);   // == i when the second row is absent: it repeats the first
-        const int r0 = c0 + i, r1 = c0 + i1;
-        const float x0 = __ldcg(w.X + (size_t)r0 * dm.d + f), x1 = __ldcg(w.X + (size_t)r1 * dm.d + f);
-        float s0 = 0.f, s1 = 0.f;
-#pragma unroll 1
-        for (int k0 = 0; k0 < n; k0 += 6) {   // the sharing blocks (this one included), six at a time
-          unsigned long long pw[2][6];
-          const unsigned long long* src[6];
+        for (int i0 = 0; i0 < n_con; i0 += CB) {
+          PartialWord pw[CB][TR];
+          const uint4* src[CB];
 #pragma unroll
-          for (int k = 0; k < 6; ++k) {
-            const int c2 = c_first + min(k0 + k, n - 1);   // past the last one: it is read again and ignored
-            src[k] = p.pbuf + ((size_t)(2 * c2 + (c2 == c_first ? 1 : 0)) * Rp + c0) * kTileN + fl;
+          for (int k = 0; k < CB; ++k) {
+            const int i = min(i0 + k, n_con - 1);   // past the last one: it is read again and ignored
+            const int c2 = sparse ? unit_owner((unsigned)tile * (unsigned)ss.KB + 1u + (unsigned)i, U, G) : c + 1 + i;
+            src[k] = p.pbuf + partial_at(c2, 0, Rp, c16 >> 4, grp, 0, fl);
           }
+#pragma unroll 1
           for (uint32_t spin = 0;; ++spin) {
             bool ok = true;
 #pragma unroll
-            for (int k = 0; k < 6; ++k) {
-              pw[0][k] = ld_relaxed_u64(src[k] + (size_t)i * kTileN);
-              pw[1][k] = ld_relaxed_u64(src[k] + (size_t)i1 * kTileN);
-            }
+            for (int k = 0; k < CB; ++k)
 #pragma unroll
-            for (int k = 0; k < 6; ++k) ok = ok && (pw[0][k] >> 32) == (tag >> 32) && (pw[1][k] >> 32) == (tag >> 32);
-            if (ok) break;
-            if (spin > 16) {
-              if (*af) break;
-              if ((spin & 63) == 0 && *reinterpret_cast<volatile int*>(p.abort_g)) { *af = 1; break; }
-              if (spin > 4096) __nanosleep(64);
-              if (spin >= kMegaSpin) {
-                *af = 1;
-                att_note_timeout(p.abort_g, 7, gseq);
-                *reinterpret_cast<volatile int*>(p.abort_g) = 1;
-                atomicCAS(w.status, DEV_OK, DEV_TIMEOUT);
-                break;
-              }
-            }
+              for (int t = 0; t < TR; ++t) pw[k][t] = ld_partial(src[k] + t * kTileN);   // all issued before any is looked at
+#pragma unroll
+            for (int k = 0; k < CB; ++k)
+#pragma unroll
+              for (int t = 0; t < TR; ++t) ok = ok && (t >= ntr || pw[k][t].tag() == tag);
+            if (ok || !mega_poll_again(spin, ctl, p, w.status, gseq)) break;
           }
 #pragma unroll
-          for (int k = 0; k < 6; ++k) {
-            const bool use = k0 + k < n;
-            s0 += use ? __uint_as_float((unsigned)pw[0][k]) : 0.f;
-            s1 += use ? __uint_as_float((unsigned)pw[1][k]) : 0.f;
-          }
-        }
-        const float y0 = x0 + s0, y1 = x1 + s1;
-        w.X[(size_t)r0 * dm.d + f] = y0;
-        store_act<bf16>(w.A, R, dm.d, r0, f, y0 * gn);
-        if (i1 != i) {
-          w.X[(size_t)r1 * dm.d + f] = y1;
-          store_act<bf16>(w.A, R, dm.d, r1, f, y1 * gn);
-        }
-        const float q0 = warp_sum(y0 * y0), q1 = warp_sum(y1 * y1);
-        if (lane == 0) {
-          ctl->red[grp][quarter][i] = q0;
-          ctl->red[grp][quarter][i1] = q1;
+          for (int k = 0; k < CB; ++k)
+#pragma unroll
+            for (int i = 0; i < NS; ++i) v[i] += (i0 + k < n_con && i < nr) ? pw[k][i / 3].val(i % 3) : 0.f;
         }
       }
-      bar_sync(bar_id, 128);
-      if (et >= a && et < b)
-        p.sumsq[((size_t)buf * nt128 + tile) * kMegaMaxRows + c0 + et] =
-            ctl->red[grp][0][et] + ctl->red[grp][1][et] + ctl->red[grp][2][et] + ctl->red[grp][3][et];
-      bar_sync(bar_id, 128);
+      if (et == 0) MEGA_EV(sidx, 5);
+      if (et == 0) MEGA_EV2(0, sidx, 1);
+      finish(v, aux, x, tile, c0, nr);
+    }
+    if (et == 0) MEGA_EV2(0, sidx, 7);
+    tc_fence_before();
+    mbar_arrive(smem_u32(&ctl->tmem_empty[acc]));
+    ++seg;
+    if (rowsplit) {   // at most two per phase: the block's first and last segment
+      const int n = sparse ? ss.KB : c_last - c_first + 1, j = sparse ? kb0 : c - c_first;
+      if (n_rs == 0) { rs_tile0 = tile; rs_first0 = c_first; rs_n0 = n; rs_j0 = j; rs_con0 = con; }
+      else { rs_tile1 = tile; rs_first1 = c_first; rs_n1 = n; rs_j1 = j; rs_con1 = con; }
+      ++n_rs;
+    }
+  }
+  // Tiles finished by rows: this block's rows of each.  Every sharing block has published all its rows by now or will
+  // without waiting for anybody (publishing comes first in every block), so the waits below cannot form a chain.  A row's
+  // sums are added in block order.
+#pragma unroll 1
+  for (int q = 0; q < n_rs; ++q) {
+    const int tile = q ? rs_tile1 : rs_tile0, c_first = q ? rs_first1 : rs_first0, n = q ? rs_n1 : rs_n0;
+    const int j = grp ? n - 1 - (q ? rs_j1 : rs_j0) : (q ? rs_j1 : rs_j0);   // the groups deal in opposite directions
+    const Feature x = feature(tile, q ? rs_con1 : rs_con0);
+    // Words (triples of rows) of this group: three in every full 16-row chunk, those of its rows in the last.  They are
+    // dealt with weight 1 to the first and the last sharing block and weight 2 to the others: the first block of one
+    // tile is as a rule the last block of the tile before, and finishes rows of both.
+    const int c16l = Rp - 16, n16l = R - c16l, nrl = grp ? n16l >> 1 : (n16l + 1) >> 1;
+    const int T = 3 * (c16l >> 4) + (nrl + 2) / 3;
+    const int wsum = max(2 * n - 2, 1), w_lo = j == 0 ? 0 : 2 * j - 1, w_hi = j == n - 1 ? wsum : 2 * j + 1;
+    const int tb = w_hi * T / wsum;
+    constexpr int TF = kAllRows ? 2 : 1;        // words finished together
+    constexpr int CR = kAllRows ? 4 : 6;        // sharing blocks whose words are in flight together
+    int t0 = w_lo * T / wsum;
+#pragma unroll 1
+    while (t0 < tb) {
+      const int chunk = t0 / 3, tri = t0 % 3, t1 = min(min(t0 + TF, tb), 3 * (chunk + 1));
+      const int n16 = min(16, R - 16 * chunk), h16 = (n16 + 1) >> 1, nr = grp ? n16 - h16 : h16;
+      const int row0 = 16 * chunk + (grp ? h16 : 0) + 3 * tri, cnt = min(3 * (t1 - t0), nr - 3 * tri);
+      float v[3 * TF];
+      float2 aux[3 * TF];
+      aux_loads(aux, x, tile, row0, cnt);
+#pragma unroll
+      for (int i = 0; i < 3 * TF; ++i) v[i] = 0.f;
+#pragma unroll 1
+      for (int k0 = 0; k0 < n; k0 += CR) {   // the sharing blocks, this one included
+        PartialWord pw[CR][TF];
+        const uint4* src[CR];
+#pragma unroll
+        for (int k = 0; k < CR; ++k) {
+          const int i = min(k0 + k, n - 1);   // past the last one: it is read again and ignored
+          const int c2 = sparse ? unit_owner((unsigned)tile * (unsigned)ss.KB + (unsigned)i, U, G) : c_first + i;
+          src[k] = p.pbuf + partial_at(c2, i == 0 ? 1 : 0, Rp, chunk, grp, tri, fl);
+        }
+#pragma unroll 1
+        for (uint32_t spin = 0;; ++spin) {
+          bool ok = true;
+#pragma unroll
+          for (int k = 0; k < CR; ++k)
+#pragma unroll
+            for (int t = 0; t < TF; ++t) pw[k][t] = ld_partial(src[k] + min(t, t1 - t0 - 1) * kTileN);
+#pragma unroll
+          for (int k = 0; k < CR; ++k)
+#pragma unroll
+            for (int t = 0; t < TF; ++t) ok = ok && pw[k][t].tag() == tag;
+          if (ok || !mega_poll_again(spin, ctl, p, w.status, gseq)) break;
+        }
+#pragma unroll
+        for (int k = 0; k < CR; ++k)
+#pragma unroll
+          for (int i = 0; i < 3 * TF; ++i) v[i] += k0 + k < n ? pw[k][i / 3].val(i % 3) : 0.f;
+      }
+      finish(v, aux, x, tile, row0, cnt);
+      t0 = t1;
     }
   }
   if (et == 0) MEGA_EV(sidx, 6);
@@ -835,6 +842,7 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
 __device__ __forceinline__ void mega_embed(MegaCtl* ctl, const MegaParams& p, const StepArgs* __restrict__ args,
                                            const KvView& kv, const Work& w, const Dims& dm, int wt) {
   const int ww = wt >> 5, lane = wt & 31, R = p.R, nt = dm.d / kTileN, gamma = p.rows - 1;
+#pragma unroll 1
   for (int item = blockIdx.x * 8 + ww; item < R * nt; item += gridDim.x * 8) {
     const int r = item / nt, tile = item % nt, b = ctl->row_b[r], j = ctl->row_j[r];
     const int seq = args->seq_ids[b];
@@ -856,6 +864,7 @@ __device__ __forceinline__ void mega_embed(MegaCtl* ctl, const MegaParams& p, co
     if (lane == 0) p.sumsq[(size_t)tile * kMegaMaxRows + r] = ss;
   }
   const int half = dm.hd / 2;
+#pragma unroll 1
   for (int idx = blockIdx.x * kMegaWorkers + wt; idx < R * half; idx += gridDim.x * kMegaWorkers) {
     const int r = idx / half, i = idx % half;
     const int pos = ctl->plan.L[ctl->row_b[r]] + ctl->row_j[r];
@@ -873,11 +882,13 @@ __device__ __forceinline__ void mega_finalize(MegaCtl* ctl, const MegaParams& p,
   const int seq = args->seq_ids[b];
   const int n_vtiles = (dm.V + kTileN - 1) / kTileN, nt128 = dm.d / kTileN;
   const bf16* gainF = p.lp[p.l1 - 1].gain_next;
+#pragma unroll 1
   for (int j = 0; j < rows; ++j) {
     const int r = b * rows + j;
     RowStat a; a.m = -INFINITY; a.s = 0.f; a.arg = 0; a.pad = 0;
     const int per = (n_vtiles + kMegaWorkers - 1) / kMegaWorkers;
     const int t0 = wt * per, t1 = min(t0 + per, n_vtiles);
+#pragma unroll 1
     for (int t = t0; t < t1; ++t) {
       RowStat x;
       const float4 raw = __ldcg(reinterpret_cast<const float4*>(w.stats + (size_t)t * R + r));
@@ -886,6 +897,7 @@ __device__ __forceinline__ void mega_finalize(MegaCtl* ctl, const MegaParams& p,
     }
     ctl->u.sred[wt] = a;
     bar_sync(1, kMegaWorkers);
+#pragma unroll 1
     for (int stride = 1; stride < kMegaWorkers; stride <<= 1) {
       if ((wt % (2 * stride)) == 0 && wt + stride < kMegaWorkers)
         ctl->u.sred[wt] = stat_merge(ctl->u.sred[wt], ctl->u.sred[wt + stride]);
@@ -897,20 +909,24 @@ __device__ __forceinline__ void mega_finalize(MegaCtl* ctl, const MegaParams& p,
   // 1/rms of the final norm for this sequence's rows
   if (wt < rows) {
     float s = 0.f;
+#pragma unroll 1
     for (int t = 0; t < nt128; ++t) s += __ldcg(p.sumsq + (size_t)t * kMegaMaxRows + b * rows + wt);
     ctl->inv[b * rows + wt] = 1.0f / sqrtf(s / (float)dm.d + dm.eps);
   }
   bar_sync(1, kMegaWorkers);
   if (args->dbg_hidden) {
+#pragma unroll 1
     for (int idx = wt; idx < rows * dm.d; idx += kMegaWorkers) {
       const int r = b * rows + idx / dm.d, i = idx % dm.d;
       args->dbg_hidden[(size_t)r * dm.d + i] = __ldcg(w.X + (size_t)r * dm.d + i) * __bfloat162float(gainF[i]) * ctl->inv[r];
     }
   }
+#pragma unroll 1
   for (int j = 1 + warp; j <= gamma; j += nwarp) {
     const int r = b * rows + j;
     float a = 0.f;
     if (args->has_judge)
+#pragma unroll 1
       for (int i = lane; i < dm.d; i += 32)
         a = fmaf(__ldcg(w.X + (size_t)r * dm.d + i) * __bfloat162float(gainF[i]) * ctl->inv[r], w.judge_w[i], a);
     a = warp_sum(a);
@@ -987,6 +1003,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
     ctl->abort_flag = 0;
     ctl->bars_passed = 0;
     int acc = 0;
+#pragma unroll 1
     for (int b = 0; b < B; ++b) {
       const int L = kv.kv_len[args->seq_ids[b]];
       ctl->plan.L[b] = L;
@@ -1028,6 +1045,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
   int n_att = (int)(t_hi - t_lo);
   if constexpr (A5) {
     int n_real = 0;
+#pragma unroll 1
     for (long long t = t_lo; t < t_hi;) {
       const AttTile x = att_locate(pl, B, g.KPS, (int)t);
       const int nv = (int)min((long long)(x.nt_b - x.ti), t_hi - t);
@@ -1068,6 +1086,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         const int tq = dm.Hq * dm.hd / kTileN, tk = dm.Hkv * dm.hd / kTileN;
         unsigned u = ss.g_lo;
         Seg sg;
+#pragma unroll 1
         while (seg_next(ss, u, sg)) {
           // the tensor map(s) and row of this segment's tile; only the K coordinate changes per unit
           const CUtensorMap* tm0;
@@ -1081,6 +1100,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
           else if (site == SITE_GU) { tm0 = &mp.wg[li]; tm1 = &mp.wu[li]; row = sg.tile * 64; }
           else if (site == SITE_DOWN) tm0 = &mp.wd[li];
           else tm0 = &mp.lm;
+#pragma unroll 1
           for (int kb = sg.a; kb < sg.b; ++kb) {
             if (!wait_slot()) { alive = false; return; }
             if (leader) {
@@ -1104,6 +1124,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
           rp.r = ap.r;
           return;
         }
+#pragma unroll 1
         for (long long t = t_lo; t < t_hi; ++t) {
           if (!wait_slot()) { alive = false; return; }
           const uint32_t bar = smem_u32(&ctl->full[rp.s]);
@@ -1137,6 +1158,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         if (u < ss.g_hi && !mega_wait_bars(nb, ctl, p, w.status, 10)) { alive = false; return; }
         nb += (site == SITE_QKV) ? 3 : 1;
         Seg sg;
+#pragma unroll 1
         while (seg_next(ss, u, sg)) {
           const int len = sg.b - sg.a;
           if (len == 0) continue;   // no share of this segment: no accumulator is used
@@ -1147,6 +1169,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
           }
           tc_fence_after();
           const uint32_t dcol = tmem_base + (uint32_t)(acc * 2 * Rp);
+#pragma unroll 1
           for (int i = 0; i < len; ++i) {
             if (!mega_wait(smem_u32(&ctl->full[rp.s]), (uint32_t)rp.r & 1u, ctl, p, w.status, 5, rp.r)) { alive = false; return; }
             tc_fence_after();
@@ -1203,7 +1226,9 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
           const CUtensorMap* tm = (site == SITE_O) ? &mp.a_q : (site == SITE_DOWN ? &mp.a_f : &mp.a_d);
           unsigned u = ss.g_lo;
           Seg sg;
+#pragma unroll 1
           while (seg_next(ss, u, sg)) {
+#pragma unroll 1
             for (int kb = sg.a; kb < sg.b; ++kb, ++n_unit) {
               if ((n_unit & 1) == mine) {
                 if (rp.r > 0 && !mega_wait(smem_u32(&ctl->empty[rp.s]), (uint32_t)(rp.r - 1) & 1u, ctl, p, w.status, 2, rp.r)) {
@@ -1259,6 +1284,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
       alive = mega_grid_sync<kTr>(ctl, p, w.status, nbar, wt);
     };
     const int n_ph = mega_n_phases(p);
+#pragma unroll 1
     for (int ph = 0; ph < n_ph; ++ph) {
       int site, l;
       mega_phase(p, ph, site, l);
@@ -1273,7 +1299,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
                                      ? p.trace + 2 * kMegaTraceBarriers + 8 * kMegaTraceSites + (size_t)(l - p.l0) * 4 * 8
                                      : nullptr;
         AttRing rg{ctl->full, ctl->empty, ctl->cons_cnt, ring, p.stage_bytes, NS, &ctl->abort_flag, p.abort_g, w.status, ev};
-        AttArgs aa{w.Qb, l < p.att_precise_layers ? w.Qlo : nullptr, w.KVn, AttPartials{w.tc_m, w.tc_l, w.tc_o}, p.n_tail_base, l};
+        AttArgs aa{w.Qb, l < p.att_precise_layers ? w.Qlo : nullptr, w.KVn, AttPartials{w.tc_m, w.tc_l, w.tc_o}, p.n_tail_base, l, B};
         if constexpr (A5) {
           if ((ww & 3) < 2) {
             // softmax warps: lane quarter ww & 3, key / dim half ww >> 2
@@ -1284,12 +1310,13 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
             // all blocks from the last block down
             AttWarp<HD, 2> st;
             const int k = (ww & 1) + 2 * (ww >> 2);
+#pragma unroll 1
             for (int q = (G - 1 - c) * 4 + k; q < B * dm.Hkv * g.MT; q += G * 4)
               att_tail_task<HD, 2>(st, g, aa, q / g.MT, (q % g.MT) * 16, lane);
           }
         } else {
           int it2 = it;
-          att_consume_dispatch<HD>(rg, it2, pl, g, args, kv, aa, dm.Hkv, c, G, ww, lane);
+          att_consume_dispatch<HD>(rg, it2, pl, g, aa, dm.Hkv, c, G, ww, lane);
         }
       }
       it += n_att;
@@ -1297,6 +1324,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
       if (alive) {
         const AttPartials P{w.tc_m, w.tc_l, w.tc_o};
         const int items = B * dm.Hkv * g.nq * AttCombineSplit<HD>::value;
+#pragma unroll 1
         for (int item = ww * G + c; item < items; item += G * 8)   // spread over blocks first
           att_combine_item<bf16, HD, A5 ? 8 : 0>(P, pl, g, G, p.n_tail_base, dm.Hkv, item, w.ATT, R, dm.Hq, lane,
                                      (kTr && p.trace && c == 0 && ww == 0 && (l - p.l0) * 4 < kMegaTraceSites)

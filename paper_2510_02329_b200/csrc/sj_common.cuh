@@ -196,4 +196,54 @@ __device__ __forceinline__ RowStat stat_merge(const RowStat& a, const RowStat& b
   return r;
 }
 
+// The same for sets in any vocabulary order: on equal maxima the lower index is kept.
+__device__ __forceinline__ RowStat stat_merge_any(const RowStat& a, const RowStat& b) {
+  return (b.m == a.m && b.arg < a.arg) ? stat_merge(b, a) : stat_merge(a, b);
+}
+
+// Merged statistics of the block rows [r0, r0 + rows) over all vocabulary tiles, by the eight warps of a block: a warp
+// takes half of a row's tiles, 16 of them per lane in flight (a thread walking through its tiles one load at a time took
+// 4 us a row, 60 us of a 9-row step in all).  part: [rows][2], shared memory; the caller synchronises and merges the halves.
+__device__ __forceinline__ void merge_row_stats(const RowStat* stats, int n_vtiles, int R, int r0, int rows, int warp, int lane,
+                                                RowStat (*part)[2]) {
+  const int half = (n_vtiles + 1) / 2;
+#pragma unroll 1
+  for (int item = warp; item < 2 * rows; item += 8) {
+    const int j = item >> 1, t0 = (item & 1) * half, t1 = min(t0 + half, n_vtiles);
+    RowStat a; a.m = -INFINITY; a.s = 0.f; a.arg = 0x7fffffff; a.pad = 0;
+#pragma unroll 1
+    for (int tb = t0; tb < t1; tb += 512) {
+      float4 raw[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        raw[k] = __ldcg(reinterpret_cast<const float4*>(stats + (size_t)min(tb + 32 * k + lane, t1 - 1) * R + r0 + j));
+      float m = -INFINITY, sum = 0.f;
+      int arg = 0x7fffffff;
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        if (tb + 32 * k + lane >= t1) { raw[k].x = -INFINITY; raw[k].w = 0.f; }
+        const int ak = __float_as_int(raw[k].z);
+        if (raw[k].x > m || (raw[k].x == m && ak < arg)) { m = raw[k].x; arg = ak; }
+      }
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        sum += raw[k].x == -INFINITY ? 0.f : raw[k].y * expf(raw[k].x - m);
+        a.pad += __float_as_int(raw[k].w);
+      }
+      RowStat b; b.m = m; b.s = sum; b.arg = arg; b.pad = 0;
+      a = stat_merge_any(a, b);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      RowStat b;
+      b.m = __shfl_xor_sync(0xffffffffu, a.m, o);
+      b.s = __shfl_xor_sync(0xffffffffu, a.s, o);
+      b.arg = __shfl_xor_sync(0xffffffffu, a.arg, o);
+      b.pad = __shfl_xor_sync(0xffffffffu, a.pad, o);
+      a = stat_merge_any(a, b);
+    }
+    if (lane == 0) part[j][item & 1] = a;
+  }
+}
+
 }  // namespace sj

@@ -571,41 +571,35 @@ static __global__ void k_lm_stats_from_logits(const StepArgs* __restrict__ args,
 static __global__ void k_finalize(const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, int n_vtiles, int R) {
   pdl_wait();
   pdl_launch();
-  __shared__ RowStat sred[256];
+  __shared__ RowStat part[kMaxGamma + 1][2];
   __shared__ RowStat rs[kMaxGamma + 1];
   __shared__ float score[kMaxGamma + 1];
   const int b = blockIdx.x, gamma = args->gamma, rows = gamma + 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = blockDim.x >> 5;
   const int seq = args->seq_ids[b];
-  // merged statistics of every row: thread t folds tiles t, t+T, ... in order, then a fixed tree
-  for (int j = 0; j < rows; ++j) {
-    const int r = b * rows + j;
-    RowStat a; a.m = -INFINITY; a.s = 0.f; a.arg = 0; a.pad = 0;
-    // contiguous ranges keep vocabulary order inside and across threads
-    int per = (n_vtiles + blockDim.x - 1) / blockDim.x;
-    int t0 = tid * per, t1 = min(t0 + per, n_vtiles);
-    for (int t = t0; t < t1; ++t) a = stat_merge(a, w.stats[(size_t)t * R + r]);
-    sred[tid] = a;
-    __syncthreads();
-    for (int stride = 1; stride < (int)blockDim.x; stride <<= 1) {
-      if ((tid % (2 * stride)) == 0 && tid + stride < (int)blockDim.x) sred[tid] = stat_merge(sred[tid], sred[tid + stride]);
-      __syncthreads();
-    }
-    if (tid == 0) { rs[j] = sred[0]; w.rowstat[r] = sred[0]; }
-    __syncthreads();
-  }
+  merge_row_stats(w.stats, n_vtiles, R, b * rows, rows, warp, lane, part);
   // judge scores: Verifier(h_j) = sigmoid(w.h_j + b), j = 1..gamma, one warp per row
   for (int j = 1 + warp; j <= gamma; j += nwarp) {
     const float* h = w.Hf + (size_t)(b * rows + j) * dm.d;
     float a = 0.f;
-    if (args->has_judge)
-      for (int i = lane; i < dm.d; i += 32) a = fmaf(h[i], w.judge_w[i], a);
+    if (args->has_judge) {
+#pragma unroll 8
+      for (int i = 4 * lane; i < dm.d; i += 128) {   // d is a multiple of 8
+        const float4 hv = *reinterpret_cast<const float4*>(h + i), jv = *reinterpret_cast<const float4*>(w.judge_w + i);
+        a = fmaf(hv.x, jv.x, fmaf(hv.y, jv.y, fmaf(hv.z, jv.z, fmaf(hv.w, jv.w, a))));
+      }
+    }
     a = warp_sum(a);
     if (lane == 0) {
       float s = args->has_judge ? 1.0f / (1.0f + expf(-(a + args->judge_bias))) : 0.f;
       score[j] = s;
       args->judge_scores[b * gamma + j - 1] = s;
     }
+  }
+  __syncthreads();
+  if (tid < rows) {
+    rs[tid] = stat_merge_any(part[tid][0], part[tid][1]);
+    w.rowstat[b * rows + tid] = rs[tid];
   }
   __syncthreads();
   if (warp == 0) {

@@ -154,7 +154,7 @@ struct MegaCtl {
   union {
     float exch[2][128][9];      // [group][feature][row of the chunk]
     float a5_mx[2][2][64];      // tcgen05 attention: [tile parity][key half][query row] maxima / sums of a row's two threads
-    RowStat sred[kMegaWorkers];
+    RowStat part[kMaxGamma + 1][2];
   } u;
 };
 
@@ -882,38 +882,21 @@ __device__ __forceinline__ void mega_finalize(MegaCtl* ctl, const MegaParams& p,
   const int seq = args->seq_ids[b];
   const int n_vtiles = (dm.V + kTileN - 1) / kTileN, nt128 = dm.d / kTileN;
   const bf16* gainF = p.lp[p.l1 - 1].gain_next;
-#pragma unroll 1
-  for (int j = 0; j < rows; ++j) {
-    const int r = b * rows + j;
-    RowStat a; a.m = -INFINITY; a.s = 0.f; a.arg = 0; a.pad = 0;
-    const int per = (n_vtiles + kMegaWorkers - 1) / kMegaWorkers;
-    const int t0 = wt * per, t1 = min(t0 + per, n_vtiles);
-#pragma unroll 1
-    for (int t = t0; t < t1; ++t) {
-      RowStat x;
-      const float4 raw = __ldcg(reinterpret_cast<const float4*>(w.stats + (size_t)t * R + r));
-      x.m = raw.x; x.s = raw.y; x.arg = __float_as_int(raw.z); x.pad = __float_as_int(raw.w);
-      a = stat_merge(a, x);
-    }
-    ctl->u.sred[wt] = a;
-    bar_sync(1, kMegaWorkers);
-#pragma unroll 1
-    for (int stride = 1; stride < kMegaWorkers; stride <<= 1) {
-      if ((wt % (2 * stride)) == 0 && wt + stride < kMegaWorkers)
-        ctl->u.sred[wt] = stat_merge(ctl->u.sred[wt], ctl->u.sred[wt + stride]);
-      bar_sync(1, kMegaWorkers);
-    }
-    if (wt == 0) { ctl->rs[j] = ctl->u.sred[0]; w.rowstat[r] = ctl->u.sred[0]; }
-    bar_sync(1, kMegaWorkers);
-  }
+  merge_row_stats(w.stats, n_vtiles, R, b * rows, rows, warp, lane, ctl->u.part);
   // 1/rms of the final norm for this sequence's rows
-  if (wt < rows) {
-    float s = 0.f;
 #pragma unroll 1
-    for (int t = 0; t < nt128; ++t) s += __ldcg(p.sumsq + (size_t)t * kMegaMaxRows + b * rows + wt);
-    ctl->inv[b * rows + wt] = 1.0f / sqrtf(s / (float)dm.d + dm.eps);
+  for (int j = warp; j < rows; j += nwarp) {
+    float s = 0.f;
+#pragma unroll 4
+    for (int t = lane; t < nt128; t += 32) s += __ldcg(p.sumsq + (size_t)t * kMegaMaxRows + b * rows + j);
+    s = warp_sum(s);
+    if (lane == 0) ctl->inv[b * rows + j] = 1.0f / sqrtf(s / (float)dm.d + dm.eps);
   }
   bar_sync(1, kMegaWorkers);
+  if (wt < rows) {
+    ctl->rs[wt] = stat_merge_any(ctl->u.part[wt][0], ctl->u.part[wt][1]);
+    w.rowstat[b * rows + wt] = ctl->rs[wt];
+  }
   if (args->dbg_hidden) {
 #pragma unroll 1
     for (int idx = wt; idx < rows * dm.d; idx += kMegaWorkers) {
@@ -925,10 +908,16 @@ __device__ __forceinline__ void mega_finalize(MegaCtl* ctl, const MegaParams& p,
   for (int j = 1 + warp; j <= gamma; j += nwarp) {
     const int r = b * rows + j;
     float a = 0.f;
-    if (args->has_judge)
-#pragma unroll 1
-      for (int i = lane; i < dm.d; i += 32)
-        a = fmaf(__ldcg(w.X + (size_t)r * dm.d + i) * __bfloat162float(gainF[i]) * ctl->inv[r], w.judge_w[i], a);
+    if (args->has_judge) {
+#pragma unroll 4
+      for (int i = 4 * lane; i < dm.d; i += 128) {   // d is a multiple of 128 here
+        const float4 xv = __ldcg(reinterpret_cast<const float4*>(w.X + (size_t)r * dm.d + i));
+        const float4 jv = *reinterpret_cast<const float4*>(w.judge_w + i);
+        const float g0 = __bfloat162float(gainF[i]), g1 = __bfloat162float(gainF[i + 1]), g2 = __bfloat162float(gainF[i + 2]), g3 = __bfloat162float(gainF[i + 3]);
+        const float inv = ctl->inv[r];
+        a = fmaf(xv.x * g0 * inv, jv.x, fmaf(xv.y * g1 * inv, jv.y, fmaf(xv.z * g2 * inv, jv.z, fmaf(xv.w * g3 * inv, jv.w, a))));
+      }
+    }
     a = warp_sum(a);
     if (lane == 0) {
       const float s = args->has_judge ? 1.0f / (1.0f + expf(-(a + args->judge_bias))) : 0.f;

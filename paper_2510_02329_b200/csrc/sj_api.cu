@@ -1034,10 +1034,20 @@ static sj_status enqueue_resample(sj_target* t, sj_kv* kv, int B, const Work& W,
   return SJ_OK;
 }
 
+// Rows per pass: enough for all rows where the registers allow it (4 features x 12 rows of accumulators).  Warps that
+// share a group of features: enough that every SM has two blocks, while a warp keeps at least two steps of K.
+template <typename T>
+static cudaError_t launch_gemm_simt(cudaStream_t s, bool pdl, int sms, const T* A, const GemmSegs& g, float* Y, int R, int N, int K, int planes) {
+  int ks = 1;
+  while (ks < 8 && (long)N * ks < 2L * sms * 32 && K >= 2 * 32 * Vec<T>::n * 2 * ks) ks *= 2;
+  const dim3 grid((N * ks + 31) / 32), block(256);   // 8 / ks groups of 4 features
+  if (R <= 4) return launch(k_gemm_simt<T, 4, 4>, grid, block, 0, s, pdl, A, g, Y, R, N, K, planes, ks);
+  if (R <= 8 || (R > 12 && R <= 16)) return launch(k_gemm_simt<T, 8, 4>, grid, block, 0, s, pdl, A, g, Y, R, N, K, planes, ks);
+  return launch(k_gemm_simt<T, 12, 4>, grid, block, 0, s, pdl, A, g, Y, R, N, K, planes, ks);
+}
 template <typename T>
 static cudaError_t launch_simt(sj_target* t, const void* A, const GemmSegs& segs, float* Y, int R, int N, int K, bool pdl) {
-  return launch(k_gemm_simt<T, 8>, dim3((N + 7) / 8), dim3(256), 0, t->stream, pdl, (const T*)A, segs, Y, R, N, K,
-                t->bf ? 2 : 1);
+  return launch_gemm_simt<T>(t->stream, pdl, t->sm_count, (const T*)A, segs, Y, R, N, K, t->bf ? 2 : 1);
 }
 
 // Launch `expr`; in timing mode bracket it with events filed under `name`.
@@ -1798,10 +1808,13 @@ extern "C" sj_status sj_gemm_skinny(int dtype, int impl, int R, int N, int K, co
   cudaStream_t s = (cudaStream_t)cuda_stream;
   if (impl == 0) {
     GemmSegs g{{w, nullptr, nullptr}, {N, 0, 0}, 1};
+    int dev0 = 0, sms = 0;
+    CU_TRY(cudaGetDevice(&dev0));
+    CU_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev0));
     if (dtype == SJ_DTYPE_BF16)
-      CU_TRY(launch(k_gemm_simt<bf16, 8>, dim3((N + 7) / 8), dim3(256), 0, s, false, (const bf16*)a, g, y, R, N, K, 1));
+      CU_TRY(launch_gemm_simt<bf16>(s, false, sms, (const bf16*)a, g, y, R, N, K, 1));
     else if (dtype == SJ_DTYPE_F32)
-      CU_TRY(launch(k_gemm_simt<float, 8>, dim3((N + 7) / 8), dim3(256), 0, s, false, (const float*)a, g, y, R, N, K, 1));
+      CU_TRY(launch_gemm_simt<float>(s, false, sms, (const float*)a, g, y, R, N, K, 1));
     else
       return fail(SJ_ERR_INVALID_ARG, "unknown dtype");
     return SJ_OK;

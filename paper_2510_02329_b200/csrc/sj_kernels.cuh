@@ -255,8 +255,14 @@ __global__ void k_swiglu(Work w, Dims dm, SplitPlan sp, size_t slot_stride) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// CUDA-core skinny GEMM: one warp per output feature, RT rows at a time.  Used for fp32 models
+// CUDA-core skinny GEMM: a warp computes NF output features for RT rows, lanes over K.  Used for fp32 models
 // and as a cross-check of the tensor-core kernel.
+//
+// What bounds it is the load path: every weight is used once per row, and its activations come from L1 / L2.  With one
+// feature per warp a 16-byte weight load came with RT activation loads and the rows beyond RT = 8 read the weights again
+// (1B-shaped fp32 model, 10 rows: 730 GB/s of weights, the GEMMs 2.8 ms of a 3.3 ms step).  NF = 4 features share each
+// activation load, RT is picked to cover the rows in one pass where it can, and where N leaves SMs without a block, `ks`
+// of a block's eight warps share a group of features and split K (their sums meet in shared memory, in warp order).
 // ---------------------------------------------------------------------------------------------
 struct GemmSegs {
   const void* w[3];  // up to three weight matrices stacked along the output dimension
@@ -280,47 +286,75 @@ __device__ __forceinline__ void unpack(const uint4& v, float* f) {
 }
 
 // `planes` = 2: the input is a hi/lo pair of bf16 planes (see Work); the two are added before use.
-template <typename T, int RT>
-__global__ void k_gemm_simt(const T* __restrict__ A, GemmSegs segs, float* __restrict__ Y, int R, int N, int K,
-                            int planes) {
+template <typename T, int RT, int NF>
+__global__ void __launch_bounds__(256)
+k_gemm_simt(const T* __restrict__ A, GemmSegs segs, float* __restrict__ Y, int R, int N, int K, int planes, int ks) {
   pdl_wait();
   pdl_launch();
   constexpr int VN = Vec<T>::n;
   typedef typename Vec<T>::type V;
-  const int lane = threadIdx.x & 31;
-  const int n = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (n >= N) return;
-  int nn = n, s = 0;
-  while (s < segs.nseg - 1 && nn >= segs.rows[s]) { nn -= segs.rows[s]; ++s; }
-  const T* wrow = reinterpret_cast<const T*>(segs.w[s]) + (size_t)nn * K;
-  for (int r0 = 0; r0 < R; r0 += RT) {
-    float acc[RT];
+  static_assert(NF * RT % 16 == 0, "sums are reduced sixteen at a time");
+  __shared__ float part[8][NF * RT];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, kp = warp % ks;
+  const int n0 = (blockIdx.x * (8 / ks) + warp / ks) * NF;   // past N in the last block's last warps: nothing is stored
+  const T* wrow[NF];
 #pragma unroll
-    for (int i = 0; i < RT; ++i) acc[i] = 0.f;
-    for (int k = lane * VN; k < K; k += 32 * VN) {
-      float wf[VN];
-      unpack(*reinterpret_cast<const V*>(wrow + k), wf);
+  for (int f = 0; f < NF; ++f) {
+    int nn = min(n0 + f, N - 1), s = 0;   // features past the last repeat it and are not stored
+    while (s < segs.nseg - 1 && nn >= segs.rows[s]) { nn -= segs.rows[s]; ++s; }
+    wrow[f] = reinterpret_cast<const T*>(segs.w[s]) + (size_t)nn * K;
+  }
+#pragma unroll 1
+  for (int r0 = 0; r0 < R; r0 += RT) {
+    const T* arow[RT];   // rows past the last repeat it
+#pragma unroll
+    for (int i = 0; i < RT; ++i) arow[i] = A + (size_t)min(r0 + i, R - 1) * K;
+    float acc[NF][RT];
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+      for (int i = 0; i < RT; ++i) acc[f][i] = 0.f;
+    V wn[NF];   // the next step's weights, requested a step ahead
+#pragma unroll
+    for (int f = 0; f < NF; ++f) wn[f] = *reinterpret_cast<const V*>(wrow[f] + min((lane + 32 * kp) * VN, K - VN));
+#pragma unroll 1
+    for (int k = (lane + 32 * kp) * VN; k < K; k += 32 * VN * ks) {
+      float wf[NF][VN];
+#pragma unroll
+      for (int f = 0; f < NF; ++f) unpack(wn[f], wf[f]);
+      const int kn = min(k + 32 * VN * ks, K - VN);
+#pragma unroll
+      for (int f = 0; f < NF; ++f) wn[f] = *reinterpret_cast<const V*>(wrow[f] + kn);
 #pragma unroll
       for (int i = 0; i < RT; ++i) {
-        if (r0 + i < R) {
-          float af[VN];
-          unpack(*reinterpret_cast<const V*>(A + (size_t)(r0 + i) * K + k), af);
-          if (planes == 2) {
-            float lo[VN];
-            unpack(*reinterpret_cast<const V*>(A + ((size_t)pad16(R) + r0 + i) * K + k), lo);
+        float af[VN];
+        unpack(*reinterpret_cast<const V*>(arow[i] + k), af);
+        if (planes == 2) {
+          float lo[VN];
+          unpack(*reinterpret_cast<const V*>(arow[i] + (size_t)pad16(R) * K + k), lo);
 #pragma unroll
-            for (int e = 0; e < VN; ++e) af[e] += lo[e];
-          }
-#pragma unroll
-          for (int e = 0; e < VN; ++e) acc[i] = fmaf(af[e], wf[e], acc[i]);
+          for (int e = 0; e < VN; ++e) af[e] += lo[e];
         }
+#pragma unroll
+        for (int f = 0; f < NF; ++f)
+#pragma unroll
+          for (int e = 0; e < VN; ++e) acc[f][i] = fmaf(af[e], wf[f][e], acc[f][i]);
       }
     }
 #pragma unroll
-    for (int i = 0; i < RT; ++i) {
-      float v = warp_sum(acc[i]);
-      if (lane == 0 && r0 + i < R) Y[(size_t)(r0 + i) * N + n] = v;
+    for (int g = 0; g < NF * RT / 16; ++g) {
+      const float t = warp_sum_n<16>(&acc[0][0] + 16 * g, lane);
+      if ((lane & 1) == 0) part[warp][16 * g + (lane >> 1)] = t;
     }
+    __syncthreads();
+    if (kp == 0)
+      for (int e = lane; e < NF * RT; e += 32) {
+        const int f = e / RT, i = e % RT;
+        float v = 0.f;
+        for (int u = 0; u < ks; ++u) v += part[warp + u][e];
+        if (r0 + i < R && n0 + f < N) Y[(size_t)(r0 + i) * N + n0 + f] = v;
+      }
+    __syncthreads();
   }
 }
 
@@ -380,17 +414,35 @@ __global__ void k_attn_simt(const StepArgs* __restrict__ args, KvView kv, Work w
     for (int i = 0; i < 48; ++i) acc[i] = 0.f;
     for (int k0 = k_begin; k0 < k_end; k0 += kAttKT) {
       __syncthreads();
-      for (int i = tid; i < kAttKT * hd; i += kAttThreads) {
-        int kk = i / hd, dd = i % hd, key = k0 + kk;
-        float kvv = 0.f, vvv = 0.f;
-        if (key < k_end) {
-          int page = kv.block_table[(size_t)seq * kv.max_pages_per_seq + key / kv.page_size];
-          int slot = key % kv.page_size;
-          kvv = to_f(kv_row<T>(kv, layer, page, 0, kvh, slot)[dd]);
-          vvv = to_f(kv_row<T>(kv, layer, page, 1, kvh, slot)[dd]);
+      {   // 16-byte loads, all of a thread's requested before any is stored (two to four: hd 64 or 128, fp32 or bf16)
+        constexpr int VN = Vec<T>::n, MAXV = kAttKT * 128 / VN / kAttThreads;
+        typedef typename Vec<T>::type V;
+        V kv4[MAXV], vv4[MAXV];
+#pragma unroll
+        for (int u = 0; u < MAXV; ++u) {
+          const int i = (tid + u * kAttThreads) * VN, kk = i / hd, dd = i % hd, key = min(k0 + kk, k_end - 1);
+          if (kk < kAttKT) {
+            const int page = kv.block_table[(size_t)seq * kv.max_pages_per_seq + key / kv.page_size];
+            const T* kr = kv_row<T>(kv, layer, page, 0, kvh, key % kv.page_size) + dd;
+            kv4[u] = *reinterpret_cast<const V*>(kr);
+            vv4[u] = *reinterpret_cast<const V*>(kr + (size_t)kv.n_kv_heads * kv.page_size * kv.head_dim);
+          }
         }
-        ks[kk * (hd + 1) + dd] = kvv;
-        vs[kk * hd + dd] = vvv;
+#pragma unroll
+        for (int u = 0; u < MAXV; ++u) {
+          const int i = (tid + u * kAttThreads) * VN, kk = i / hd, dd = i % hd;
+          if (kk < kAttKT) {
+            float kf[VN], vf[VN];
+            unpack(kv4[u], kf);
+            unpack(vv4[u], vf);
+            const bool live = k0 + kk < k_end;
+#pragma unroll
+            for (int e = 0; e < VN; ++e) {
+              ks[kk * (hd + 1) + dd + e] = live ? kf[e] : 0.f;
+              vs[kk * hd + dd + e] = live ? vf[e] : 0.f;
+            }
+          }
+        }
       }
       __syncthreads();
       // scores: one (q, key) pair per thread-iteration; a warp covers the 32 keys of one q

@@ -530,7 +530,8 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
   }
 #undef ALLOC
   if (t->bf && c.head_dim == 128) {
-    cudaError_t e = cudaFuncSetAttribute(k_attn_t5, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kT5SmemBytes + sizeof(T5Ctl) + 1024));
+    cudaError_t e = cudaFuncSetAttribute(k_attn_t5<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_attn_t5<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) { fail(SJ_ERR_CUDA, "smem opt-in: %s", cudaGetErrorString(e)); return bail(SJ_ERR_CUDA); }
   }
   if (t->bf) {
@@ -1139,8 +1140,9 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
       // one warp per (sequence, KV head, query row, half of the head dimension): every task's loads are in flight at once
       const int items = B * dm.Hkv * nq, cgrid = std::max(1, std::min(32 * t->sm_count, (items * (dm.hd >= 128 ? 2 : 1) + 7) / 8));
       if (dm.hd == 128 && t->opt_attn == 2 && nq <= 128) {   // one 128-lane accumulator holds a KV head's query rows
-        const size_t t5_smem = kT5SmemBytes + sizeof(T5Ctl) + 1024;
-        TIMED("attn", launch(k_attn_t5, dim3(t->sm_count), dim3(kT5Threads), t5_smem, s, pdl, kv->tm_pool, args, kv->view, W, dm, aa));
+        const T5Geom tg = t5_geom(nq);
+        TIMED("attn", launch(a5_split(nq) <= 32 ? k_attn_t5<4> : k_attn_t5<8>, dim3(t->sm_count), dim3(kT5Threads), tg.smem, s, pdl, kv->tm_pool, args,
+                             kv->view, W, dm, aa, tg.stages));
         TIMED("attn_combine", launch(k_attn_combine_tc<128, 8>, dim3(cgrid), dim3(256), 0, s, pdl, args, W, dm, parts, t->sm_count, aa.n_tail_base, kT5Keys, kT5Pad));
       } else if (dm.hd == 128) {
         TIMED("attn", launch(k_attn_tc<128>, dim3(t->sm_count), dim3(kAttTcThreads), tc_smem, s, pdl, kv->tm_pool, args, kv->view, W, dm, aa));

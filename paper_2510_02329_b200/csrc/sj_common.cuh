@@ -155,6 +155,21 @@ __device__ __forceinline__ void warp_max_n(const float* v, int id, int lane, flo
   arg = b[0];
 }
 
+// Maximum of each of 8 values over the warp: a lane returns that of value lane / 4.
+__device__ __forceinline__ float warp_max8(const float* v, int lane) {
+  float a[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) a[i] = v[i];
+#pragma unroll
+  for (int h = 4; h >= 1; h >>= 1) {
+    const bool up = lane & (4 * h);
+#pragma unroll
+    for (int i = 0; i < h; ++i) a[i] = fmaxf(up ? a[i + h] : a[i], __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + h], 4 * h));
+  }
+  a[0] = fmaxf(a[0], __shfl_xor_sync(0xffffffffu, a[0], 2));
+  return fmaxf(a[0], __shfl_xor_sync(0xffffffffu, a[0], 1));
+}
+
 // Block-wide sum with a fixed reduction tree (deterministic).  `red` holds >= 32 floats.
 __device__ __forceinline__ float block_sum(float v, float* red) {
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;

@@ -28,9 +28,9 @@
 //   LM head -> softmax statistics per (vocabulary tile, row), logit of the drafted token
 // Attention: its cache tiles travel through the same ring.  Two implementations, chosen per launch: fp16 mma.sync in
 // the worker warps (sj_attn_tc.cuh), or -- head dimension 128, at most 64 query rows per KV head and sequence --
-// tcgen05 (the routines at the end of sj_attn_t5.cuh; ring stages of at least 32 KiB): warps 1 and 2 issue the MMAs of
-// the even and the odd 128-key tiles, four worker warps run the softmax on tensor memory, the other four the causal tails; the queries sit in an area of their own
-// after the ring, the accumulators alias the GEMM phases' tensor-memory columns.
+// tcgen05 (the routines of sj_attn_t5.cuh; ring stages of at least 32 KiB): warp 1 issues the MMAs, the workers run the
+// softmax on tensor memory; the queries sit in an area of their own after the ring, a tile's probabilities in a ring
+// stage, the accumulators alias the GEMM phases' tensor-memory columns.
 //
 // Every wait is bounded; the first one to run out raises a device-wide abort word that all other waits
 // poll, so that a logic error ends the kernel with SJ_ERR_TIMEOUT instead of hanging the GPU.
@@ -137,7 +137,7 @@ struct MegaCtl {
   int abort_flag;
   int bars_passed;
   A5Bars a5;                   // tcgen05 attention: score / probability / output hand-offs
-  uint64_t a5_pair[2];         // ... and the barrier of each lane quarter's two softmax warps
+  A5Smem a5s;                  // ... and the softmax state
   int bcast[6];   // [2 * group + accumulator]: the group's wait on that accumulator succeeded; [4], [5] spare
   float inv[kMegaMaxRows];
   float zd[kMegaMaxRows];      // top-k test: raw logit of each row's drafted token, computed before the LM head
@@ -153,14 +153,9 @@ struct MegaCtl {
   int att_pages[kAttPageCache];   // page ids of this block's first ring tiles (the same in every layer)
   union {
     float exch[2][128][9];      // [group][feature][row of the chunk]
-    float a5_mx[2][2][64];      // tcgen05 attention: [tile parity][key half][query row] maxima / sums of a row's two threads
     RowStat part[kMaxGamma + 1][2];
   } u;
 };
-
-// The tcgen05 attention's M = 128 descriptors read up to 16 KiB past the last half of the query area, which this
-// block follows: those bytes must be the kernel's own.
-static_assert(sizeof(MegaCtl) >= 16384, "the control block no longer covers the query area's over-read");
 
 struct SiteInfo {
   int n_tiles, KB;
@@ -983,12 +978,8 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&ctl->tmem_full[i]), 1);
       mbar_init(smem_u32(&ctl->tmem_empty[i]), kMegaWorkers);
-      mbar_init(smem_u32(&ctl->a5.s_full[i]), 1);
-      mbar_init(smem_u32(&ctl->a5.p_full[i]), 128);
-      mbar_init(smem_u32(&ctl->a5.o_done[i]), 1);
-      mbar_init(smem_u32(&ctl->a5_pair[i]), 64);
     }
-    mbar_init(smem_u32(&ctl->a5.q_ready), 128);
+    a5_bars_init(&ctl->a5);
     ctl->abort_flag = 0;
     ctl->bars_passed = 0;
     int acc = 0;
@@ -1030,7 +1021,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
 
   const AttPlan& pl = ctl->plan;
   const long long t_lo = (long long)c * pl.T / G, t_hi = (long long)(c + 1) * pl.T / G;
-  // ring stages of one attention phase: one per tile, or (tcgen05) a key stage and a value stage per real tile
+  // ring stages of one attention phase: one per tile, or (tcgen05) a key stage, a value stage and one for the probabilities per real tile
   int n_att = (int)(t_hi - t_lo);
   if constexpr (A5) {
     int n_real = 0;
@@ -1041,7 +1032,12 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
       n_real += max(0, min(nv, x.nt_real - x.ti));
       t += nv;
     }
-    n_att = 2 * n_real;
+    n_att = A5Entry<true>::n * n_real;
+  }
+  if constexpr (A5) {   // padding query rows stay zero for the whole kernel
+#pragma unroll 1
+    for (int i = threadIdx.x; i < p.q_area_bytes / 16; i += blockDim.x) reinterpret_cast<uint4*>(q_area)[i] = make_uint4(0, 0, 0, 0);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read them
   }
   const A5Ring a5r{ctl->full, ctl->empty, ring, p.stage_bytes, NS, &ctl->abort_flag, p.abort_g, w.status};
   att_fill_pages(ctl->att_pages, pl, kv, args, B, g.KPS, t_lo, t_hi, threadIdx.x, blockDim.x);
@@ -1108,7 +1104,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         if (!alive) return;
         if constexpr (A5) {
           A5Pos ap{rp.s, rp.r};
-          alive = a5_produce(a5r, ap, &mp.pool, kv, args, pl, B, l, t_lo, t_hi, ctl->att_pages, lane);
+          alive = a5_produce<true>(a5r, ap, &mp.pool, kv, args, pl, B, l, t_lo, t_hi, ctl->att_pages, lane);
           rp.s = ap.s;
           rp.r = ap.r;
           return;
@@ -1181,7 +1177,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         if constexpr (A5) {
           if (!alive) return;
           A5Pos ap{rp.s, rp.r};
-          alive = a5_issue(a5r, ap, &ctl->a5, tmem_base, smem_u32(q_area), g.nq, 0, pl, B, t_lo, t_hi, a5_tiles, a5_segs);
+          alive = a5_issue<true>(a5r, ap, &ctl->a5, tmem_base, smem_u32(q_area), 0u, g.nq, pl, B, t_lo, t_hi, a5_tiles, a5_segs);
           rp.s = ap.s;
           rp.r = ap.r;
         } else {
@@ -1236,21 +1232,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         ++sidx;
         nb += (site == SITE_QKV) ? 3 : 1;
       };
-      int a5_tiles = 0, a5_segs = 0;
-      auto fatt = [&](int l) {
-        if constexpr (A5) {
-          // warp 2 issues the attention MMAs of the odd tiles (warp 1 those of the even ones)
-          if (mine == 0) {
-            if (!alive) return;
-            A5Pos ap{rp.s, rp.r};
-            alive = a5_issue(a5r, ap, &ctl->a5, ctl->tmem_base, smem_u32(q_area), g.nq, 1, pl, B, t_lo, t_hi, a5_tiles, a5_segs);
-            rp.s = ap.s;
-            rp.r = ap.r;
-            return;
-          }
-        }
-        rp.advance(n_att);
-      };
+      auto fatt = [&](int l) { rp.advance(n_att); };
       mega_walk(p, fsite, fatt);
     }
   }
@@ -1259,7 +1241,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
     // ------------------------------ workers ------------------------------
     const int wt = threadIdx.x - 128, ww = wt >> 5;
     int nbar = 0, gseq = 0, seg = 0, it = 0;
-    int a5_tiles = 0, a5_pairs = 0;
+    int a5_tiles = 0;
     bool alive = true;
     if (p.do_embed) {
       mega_embed(ctl, p, args, kv, w, dm, wt);
@@ -1290,19 +1272,14 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         AttRing rg{ctl->full, ctl->empty, ctl->cons_cnt, ring, p.stage_bytes, NS, &ctl->abort_flag, p.abort_g, w.status, ev};
         AttArgs aa{w.Qb, l < p.att_precise_layers ? w.Qlo : nullptr, w.KVn, AttPartials{w.tc_m, w.tc_l, w.tc_o}, p.n_tail_base, l, B};
         if constexpr (A5) {
-          if ((ww & 3) < 2) {
-            // softmax warps: lane quarter ww & 3, key / dim half ww >> 2
-            alive = a5_softmax(a5r, &ctl->a5, ctl->tmem_base, q_area, &ctl->u.a5_mx[0][0][0], &ctl->a5_pair[ww & 3], a5_pairs, aa, pl, B,
-                               dm.Hkv, g.nq, t_lo, t_hi, a5_tiles, c, ww & 3, ww >> 2, lane, ev);
-          } else {
-            // the other four warps: the causal tails (one m-tile of one (sequence, KV head) per task), dealt over
-            // all blocks from the last block down
-            AttWarp<HD, 2> st;
-            const int k = (ww & 1) + 2 * (ww >> 2);
+          // all eight warps: lane quarter ww & 3, query group ww >> 2; then the causal tails, dealt over all blocks' warps
+          // from the last block down
+          A5Pos ap{it % NS, it / NS};
+          alive = a5_softmax<true, 4>(a5r, ap, &ctl->a5, &ctl->a5s, ctl->tmem_base, q_area, nullptr, aa, pl, B, dm.Hkv, g.nq, t_lo, t_hi, a5_tiles, c,
+                                      ww & 3, ww >> 2, 2 + (ww >> 2), lane, ev);
+          AttWarp<HD, 2> st;
 #pragma unroll 1
-            for (int q = (G - 1 - c) * 4 + k; q < B * dm.Hkv * g.MT; q += G * 4)
-              att_tail_task<HD, 2>(st, g, aa, q / g.MT, (q % g.MT) * 16, lane);
-          }
+          for (int q = (G - 1 - c) * 8 + ww; q < B * dm.Hkv * g.MT; q += G * 8) att_tail_task<HD, 2>(st, g, aa, q / g.MT, (q % g.MT) * 16, lane);
         } else {
           int it2 = it;
           att_consume_dispatch<HD>(rg, it2, pl, g, aa, dm.Hkv, c, G, ww, lane);

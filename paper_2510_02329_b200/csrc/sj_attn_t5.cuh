@@ -33,7 +33,7 @@ namespace sj {
 
 constexpr int kT5Keys = 128;               // keys per tile
 constexpr int kT5Pad = 4;                  // empty tiles the plan counts per (sequence, KV head): what a segment costs a block beyond its tiles
-constexpr int kT5Threads = 320;            // warp 0 TMA, warp 1 MMA, warps 2..9 softmax and, after their tiles, the causal tails
+constexpr int kT5Threads = 352;            // warp 0 key tiles, warp 10 value tiles, warp 1 MMA, warps 2..9 softmax and, after their tiles, the causal tails
 constexpr int kT5MaxRows = 128;
 constexpr int kA5Keys = kT5Keys;           // the same in the persistent kernel
 constexpr int kA5MaxRows = 64;
@@ -149,6 +149,7 @@ struct alignas(16) A5Smem {   // softmax state in shared memory, read four float
   float m[kT5MaxRows];          // stabiliser per query
   float f[kT5MaxRows];          // the factor of its last move
   float red[4][kT5MaxRows];     // per lane quarter
+  int claimed;                  // value stages the first producer warp has claimed
 };
 __device__ __forceinline__ void a5_bars_init(A5Bars* b) {
   for (int i = 0; i < 2; ++i) {
@@ -206,14 +207,18 @@ __device__ __forceinline__ void a5_run_at(const AttPlan& pl, int B, long long t,
   n = max(0, min(nv, x.nt_real - x.ti));
 }
 
-// All 32 lanes of one warp (same control flow): the TMA loads of the block's tiles [t_lo, t_hi) of one layer.  A key or
-// value tile is sixteen boxes of 2 KiB (16 keys x 64 dims: a page's slots, one swizzle span wide), one per lane (half =
-// lane / 8, page = lane % 8), so it costs one instruction.  Lane 0 announces the bytes.  pages: the block's page ids, eight
-// per tile (clamped to the sequence's last page), for its first kAttPageCache / 8 tiles.
+// The TMA loads of the block's tiles [t_lo, t_hi) of one layer, by two warps (all 32 lanes of each in the same control
+// flow).  A key or value tile is sixteen boxes of 2 KiB (16 keys x 64 dims: a page's slots, one swizzle span wide), one
+// per lane (half = lane / 8, page = lane % 8); sixteen lanes get theirs out in 1250 clocks, so one warp for both would
+// take longer than HBM needs for the bytes.  The first warp claims every stage in ring order and loads the key tiles; it
+// hands a value stage over by a count in shared memory (`claimed`: value stages claimed so far, over all layers).  The
+// second warp may not wait on the stages' barriers itself: key stages are freed ahead of value stages, and a warp that is
+// lapped waits for a parity that has passed.  pages: the block's page ids, eight per tile (clamped to the sequence's last
+// page), for its first kAttPageCache / 8 tiles.  vals: value tiles of earlier layers (advanced).
 template <bool PRING>
 __device__ __forceinline__ bool a5_produce(const A5Ring& rg, A5Pos& pos, const CUtensorMap* tmKV, const KvView& kv,
                                            const StepArgs* __restrict__ args, const AttPlan& pl, int B, int layer,
-                                           long long t_lo, long long t_hi, const int* pages, int lane) {
+                                           long long t_lo, long long t_hi, const int* pages, int lane, int which, volatile int* claimed, int& vals) {
   const int half = (lane >> 3) & 1, p = lane & 7;
 #pragma unroll 1
   for (long long t = t_lo; t < t_hi; ++t) {
@@ -224,27 +229,44 @@ __device__ __forceinline__ bool a5_produce(const A5Ring& rg, A5Pos& pos, const C
     if (pi > last_page) pi = last_page;   // keys there are masked; reload a valid page
     const int page = (tb + 1) * 8 <= kAttPageCache ? pages[tb * 8 + p]
                                                    : __ldg(kv.block_table + (size_t)seq * kv.max_pages_per_seq + pi);
+    const long long row = ((((long long)layer * kv.n_pages + page) * 2 + which) * kv.n_kv_heads + x.h) * 16;
+    ++vals;
+    if (which == 1) {
+      for (uint32_t i = 0; *claimed < vals; ++i) {
+        if (i > 64) {
+          if (*rg.abort_flag) return false;
+          __nanosleep(20);
+        }
+        if (i >= kAttSpin) { *rg.abort_flag = 1; atomicCAS(rg.status, DEV_OK, DEV_TIMEOUT); return false; }
+      }
+      __syncwarp();
+    }
 #pragma unroll 1
-    for (int which = 0; which < A5Entry<PRING>::n; ++which) {
-      if (pos.r > 0 && !a5_wait(rg, &rg.empty[pos.s], (uint32_t)(pos.r - 1) & 1u, 1, pos.r)) return false;
+    for (int e = 0; e < A5Entry<PRING>::n; ++e) {
       const uint32_t bar = att_smem_u32(&rg.full[pos.s]);
-      if (lane == 0) {
-        if (which < 2) att_mbar_expect_tx(bar, kA5Part);
-        else att_mbar_arrive(bar);
-        att_mbar_arrive(bar);   // the stage's second arrival
+      if (which == 0) {
+        if (pos.r > 0 && !a5_wait(rg, &rg.empty[pos.s], (uint32_t)(pos.r - 1) & 1u, 1, pos.r)) return false;
+        if (lane == 0) {
+          if (e < 2) att_mbar_expect_tx(bar, kA5Part);
+          else att_mbar_arrive(bar);
+          att_mbar_arrive(bar);   // the stage's second arrival
+          if (e == 1) {
+            __threadfence_block();
+            *claimed = vals;
+          }
+        }
       }
-      if (which < 2 && lane < 16) {
-        const long long row = ((((long long)layer * kv.n_pages + page) * 2 + which) * kv.n_kv_heads + x.h) * 16;
+      if (e == which && lane < 16)
         att_tma_2d(att_smem_u32(rg.base + (size_t)pos.s * rg.stage_stride) + (uint32_t)(half * 16384 + p * 2048), tmKV, bar, half * 64, (int)row);
-      }
       pos.next(rg.stages);
     }
   }
   return true;
 }
 
-// One elected thread: the MMAs of the block's tiles.  Order: scores(0), then scores(i + 1), output(i), so that a tile's
-// scores are ready while the softmax of the one before runs.  gt: tiles of earlier layers (the barriers' phases run on
+// One elected thread: the MMAs of the block's tiles.  Order: scores(0) .. scores(n_s - 1), then output(i), scores(i + n_s),
+// so that a tile's scores are ready while the softmax of the one before runs, and an output never waits behind scores
+// whose keys have not arrived (with output(i) after scores(i + 1) a tile took 4000 clocks).  gt: tiles of earlier layers (the barriers' phases run on
 // across layers), segs: segments of earlier layers; both advanced.  p_area: address of the probabilities without PRING.
 template <bool PRING>
 __device__ __forceinline__ bool a5_issue(const A5Ring& rg, A5Pos& pos, A5Bars* ab, uint32_t tmem, uint32_t q_area, uint32_t p_area, int nq,
@@ -264,13 +286,25 @@ __device__ __forceinline__ bool a5_issue(const A5Ring& rg, A5Pos& pos, A5Bars* a
     if (n == 0) continue;   // only empty tiles of this (sequence, KV head): no segment
     if (!a5_wait(rg, &ab->q_ready, (uint32_t)segs & 1u, 2, segs)) return false;
     tc_fence_after();
-    A5Entry<PRING> prev = {};
+    A5Entry<PRING> pend[2];   // entries of the tiles whose scores have been issued and outputs have not: pend[i & 1]
 #pragma unroll 1
-    for (int i = 0; i <= n; ++i) {
-      A5Entry<PRING> e = prev;
-      if (i < n) {
-        e = a5_entry<PRING>(rg, pos);
-        const int g = gt + i, b = n_s == 2 ? g & 1 : 0, use = n_s == 2 ? g >> 1 : g;
+    for (int i = -n_s; i < n; ++i) {
+      if (i >= 0) {   // output of tile i
+        const int g = gt + i;
+        const A5Entry<PRING> e = n_s == 2 && (i & 1) ? pend[1] : pend[0];
+        if (!a5_wait(rg, &ab->p_full, (uint32_t)g & 1u, 5, g) || !a5_wait(rg, &rg.full[e.s[1]], e.par[1], 6, g)) return false;
+        tc_fence_after();
+        const uint64_t dv = smem_desc_mn_sw128(e.a[1], 16384u), dp = smem_desc_mn_sw128(PRING ? e.a[A5Entry<PRING>::n - 1] : p_area, 16384u);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)   // 16 keys each
+          tc_mma_bf16(d_o, dv + (uint64_t)(k * (2048 >> 4)), dp + (uint64_t)(k * (2048 >> 4)), id_o, (i > 0 || k > 0) ? 1u : 0u);
+        tc_commit(att_smem_u32(&ab->o_done));
+        tc_commit(att_smem_u32(&rg.empty[e.s[1]]));
+        if (PRING) tc_commit(att_smem_u32(&rg.empty[e.s[A5Entry<PRING>::n - 1]]));
+      }
+      if (i + n_s < n) {   // scores of tile i + n_s
+        const A5Entry<PRING> e = a5_entry<PRING>(rg, pos);
+        const int g = gt + i + n_s, b = n_s == 2 ? g & 1 : 0, use = n_s == 2 ? g >> 1 : g;
         if (use > 0 && !a5_wait(rg, &ab->s_free[b], (uint32_t)(use - 1) & 1u, 3, g)) return false;
         if (!a5_wait(rg, &rg.full[e.s[0]], e.par[0], 3, g)) return false;
         tc_fence_after();
@@ -280,22 +314,11 @@ __device__ __forceinline__ bool a5_issue(const A5Ring& rg, A5Pos& pos, A5Bars* a
         for (int k = 0; k < 8; ++k)
           tc_mma_bf16(d_s, dk + (uint64_t)(k >> 2) * k_half + (uint64_t)(2 * (k & 3)), dq + (uint64_t)(k >> 2) * q_half + (uint64_t)(2 * (k & 3)), id_s,
                       k > 0 ? 1u : 0u);
-        tc_commit(att_smem_u32(&rg.empty[e.s[0]]));
         tc_commit(att_smem_u32(&ab->s_full[b]));
+        tc_commit(att_smem_u32(&rg.empty[e.s[0]]));
+        if (n_s == 2 && ((i + n_s) & 1)) pend[1] = e;
+        else pend[0] = e;
       }
-      if (i > 0) {
-        const int g = gt + i - 1;
-        if (!a5_wait(rg, &ab->p_full, (uint32_t)g & 1u, 5, g) || !a5_wait(rg, &rg.full[prev.s[1]], prev.par[1], 6, g)) return false;
-        tc_fence_after();
-        const uint64_t dv = smem_desc_mn_sw128(prev.a[1], 16384u), dp = smem_desc_mn_sw128(PRING ? prev.a[A5Entry<PRING>::n - 1] : p_area, 16384u);
-#pragma unroll
-        for (int k = 0; k < 8; ++k)   // 16 keys each
-          tc_mma_bf16(d_o, dv + (uint64_t)(k * (2048 >> 4)), dp + (uint64_t)(k * (2048 >> 4)), id_o, (i > 1 || k > 0) ? 1u : 0u);
-        tc_commit(att_smem_u32(&rg.empty[prev.s[1]]));
-        if (PRING) tc_commit(att_smem_u32(&rg.empty[prev.s[A5Entry<PRING>::n - 1]]));
-        tc_commit(att_smem_u32(&ab->o_done));
-      }
-      prev = e;
     }
     gt += n;
     ++segs;
@@ -610,6 +633,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
       att_mbar_init(att_smem_u32(&ctl->empty[i]), 1);
     }
     a5_bars_init(&ctl->bars);
+    ctl->sh.claimed = 0;
     ctl->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -634,8 +658,8 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   const A5Ring rg{ctl->full, ctl->empty, sm, (int)kA5Part, stages, &ctl->abort_flag, nullptr, w.status};
   A5Pos pos{0, 0};
   int gt = 0, segs = 0;
-  if (warp == 0) {
-    a5_produce<false>(rg, pos, &tmKV, kv, args, pl, B, a.layer, t_lo, t_hi, ctl->pages, lane);
+  if (warp == 0 || warp == 10) {
+    a5_produce<false>(rg, pos, &tmKV, kv, args, pl, B, a.layer, t_lo, t_hi, ctl->pages, lane, warp == 0 ? 0 : 1, &ctl->sh.claimed, gt);
   } else if (warp == 1) {
     if (elect_one()) a5_issue<false>(rg, pos, &ctl->bars, tmem, att_smem_u32(q_area), att_smem_u32(p_area), nq, pl, B, t_lo, t_hi, gt, segs);
   } else {

@@ -980,6 +980,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
       mbar_init(smem_u32(&ctl->tmem_empty[i]), kMegaWorkers);
     }
     a5_bars_init(&ctl->a5);
+    ctl->a5s.claimed = 0;
     ctl->abort_flag = 0;
     ctl->bars_passed = 0;
     int acc = 0;
@@ -1052,9 +1053,9 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kMegaRegsLight));
   if (warp == 0) {
     // ------------------------------ weight / cache-tile producer ------------------------------
-    // One lane; all 32 with the tcgen05 attention, whose cache tiles are 32 small copies each (one per lane, one
-    // instruction per tile).  All lanes run the same control flow and wait on the same barriers; lane 0 alone announces
-    // bytes and issues the weight copies (the elected lane).
+    // One lane; all 32 with the tcgen05 attention, whose key tiles are sixteen small copies each (one per lane; the value
+    // tiles are warp 3's).  All lanes run the same control flow and wait on the same barriers; the elected lane alone
+    // issues the weight copies.
     const bool leader = elect_one();
     if (A5 || leader) {
       const uint64_t pol_w = l2_policy_evict_first();
@@ -1100,11 +1101,12 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         if (leader) MEGA_EV(sidx, 7);
         ++sidx;
       };
+      int a5_vals = 0;
       auto fatt = [&](int l) {
         if (!alive) return;
         if constexpr (A5) {
           A5Pos ap{rp.s, rp.r};
-          alive = a5_produce<true>(a5r, ap, &mp.pool, kv, args, pl, B, l, t_lo, t_hi, ctl->att_pages, lane);
+          alive = a5_produce<true>(a5r, ap, &mp.pool, kv, args, pl, B, l, t_lo, t_hi, ctl->att_pages, lane, 0, &ctl->a5s.claimed, a5_vals);
           rp.s = ap.s;
           rp.r = ap.r;
           return;
@@ -1190,8 +1192,10 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
     // ------------------------------ activation producers (warps 2 and 3) ------------------------------
     // Two threads, alternate units: right after a device-wide barrier the ring already holds the phase's first
     // weight tiles, and the MMAs can start only as fast as their activation slices are requested (a wait, an
-    // expect and a TMA per slice cost one thread about a quarter of a microsecond).
-    if (elect_one()) {
+    // expect and a TMA per slice cost one thread about a quarter of a microsecond).  With the tcgen05 attention warp 3 also
+    // loads the value tiles, all its lanes in the same flow.
+    const bool leader = elect_one();
+    if (leader || (A5 && warp == 3)) {
       const int mine = warp - 2;
       int n_unit = 0;
       const uint64_t pol_a = l2_policy_evict_last();
@@ -1220,9 +1224,11 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
                   alive = false;
                   return;
                 }
-                const uint32_t bar = smem_u32(&ctl->full[rp.s]);
-                mbar_expect_tx(bar, a_tx);
-                tma_load_2d(stage_addr(rp.s) + kWTileBytes, tm, bar, kb * kBK, 0, pol_a);
+                if (leader) {
+                  const uint32_t bar = smem_u32(&ctl->full[rp.s]);
+                  mbar_expect_tx(bar, a_tx);
+                  tma_load_2d(stage_addr(rp.s) + kWTileBytes, tm, bar, kb * kBK, 0, pol_a);
+                }
               }
               rp.next();
             }
@@ -1232,7 +1238,20 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         ++sidx;
         nb += (site == SITE_QKV) ? 3 : 1;
       };
-      auto fatt = [&](int l) { rp.advance(n_att); };
+      int a5_vals = 0;
+      auto fatt = [&](int l) {
+        if constexpr (A5) {
+          if (warp == 3) {
+            if (!alive) return;
+            A5Pos ap{rp.s, rp.r};
+            alive = a5_produce<true>(a5r, ap, &mp.pool, kv, args, pl, B, l, t_lo, t_hi, ctl->att_pages, lane, 1, &ctl->a5s.claimed, a5_vals);
+            rp.s = ap.s;
+            rp.r = ap.r;
+            return;
+          }
+        }
+        rp.advance(n_att);
+      };
       mega_walk(p, fsite, fatt);
     }
   }

@@ -16,13 +16,12 @@ LIB = os.path.join(HERE, "libsjverify.so")
 
 def units():
     """(name, source, macros) of every object file: the library, and the persistent kernel's instantiations
-    (minutes of compile time in one translation unit) by head dimension, attention phase and timeline code."""
+    (minutes of compile time in one translation unit) by head dimension and timeline code."""
     out = [("sj_api", SRC, [])]
-    for hd, t5 in ((64, 0), (128, 0), (128, 1)):
+    for hd in (64, 128):
         for trace in (0, 1):
-            name = f"mega_kernel_{hd}" + ("_t5" if t5 else "") + ("_trace" if trace else "")
-            out.append((name, INST, [f"-DSJ_INST_NAME={name}", f"-DSJ_INST_HD={hd}", f"-DSJ_INST_T5={t5}",
-                                     f"-DSJ_INST_TRACE={trace}"]))
+            name = f"mega_kernel_{hd}" + ("_trace" if trace else "")
+            out.append((name, INST, [f"-DSJ_INST_NAME={name}", f"-DSJ_INST_HD={hd}", f"-DSJ_INST_TRACE={trace}"]))
     return out
 
 

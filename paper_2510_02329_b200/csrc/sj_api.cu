@@ -188,10 +188,11 @@ struct LayerW {
 };
 
 struct StepKey {
+  const sj_kv* kv;   // a captured step holds its cache's pointers; destroying the cache drops the graphs
   int B, gamma, mode, chunk_len, gemm_impl, attn_impl, pdl, scratch;
   bool operator<(const StepKey& o) const {
-    return std::tie(B, gamma, mode, chunk_len, gemm_impl, attn_impl, pdl, scratch) <
-           std::tie(o.B, o.gamma, o.mode, o.chunk_len, o.gemm_impl, o.attn_impl, o.pdl, o.scratch);
+    return std::tie(kv, B, gamma, mode, chunk_len, gemm_impl, attn_impl, pdl, scratch) <
+           std::tie(o.kv, o.B, o.gamma, o.mode, o.chunk_len, o.gemm_impl, o.attn_impl, o.pdl, o.scratch);
   }
 };
 
@@ -306,10 +307,9 @@ static bool tc_shapes_ok(const sj_model_config& c) {
 }
 
 // The persistent kernel for a head dimension (64 or 128), a number of row slots (4, 6 or 8), with or without
-// the timeline code, with the mma.sync or (head dimension 128 only) the tcgen05 attention phase.
-static MegaKernel mega_kernel(int hd, int ns, bool trace, bool a5) {
+// the timeline code.
+static MegaKernel mega_kernel(int hd, int ns, bool trace) {
   if (hd != 128) return trace ? mega_kernel_64_trace(ns) : mega_kernel_64(ns);
-  if (a5) return trace ? mega_kernel_128_t5_trace(ns) : mega_kernel_128_t5(ns);
   return trace ? mega_kernel_128_trace(ns) : mega_kernel_128(ns);
 }
 
@@ -511,9 +511,8 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
     if (e == cudaSuccess) e = cudaMemset(t->d_sumsq, 0, sizeof(float) * 2 * (c.d_model / kTileN) * kMegaMaxRows);
     if (e == cudaSuccess) e = cudaMemset(t->d_sync, 0, sizeof(unsigned) * (64 + mega_partial_words(t, pad16(Rm))));
     for (int ns = 4; ns <= 8 && e == cudaSuccess; ns += 2)
-      for (int v = 0; v < 4 && e == cudaSuccess; ++v)
-        e = cudaFuncSetAttribute(mega_kernel(c.head_dim, ns, (v & 1) != 0, (v & 2) != 0 && c.head_dim == 128),
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+      for (int v = 0; v < 2 && e == cudaSuccess; ++v)
+        e = cudaFuncSetAttribute(mega_kernel(c.head_dim, ns, v != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) { fail(SJ_ERR_CUDA, "whole-step kernel set-up: %s", cudaGetErrorString(e)); return bail(SJ_ERR_CUDA); }
     for (int l0 = 0; l0 < c.n_layers; l0 += kMegaMaxLayers) {
       t->mega_maps.emplace_back();
@@ -1013,8 +1012,9 @@ static sj_status launch_pair(sj_target* t, sj_kv* kv, int site, int n_tiles, int
   return SJ_OK;
 }
 
-// Steps of more rows than the persistent kernel takes run their projections on pairs of SMs.
-constexpr int kPairMinRows = kMegaMaxRows + 1;
+// The per-stage path runs the projections of wider steps on pairs of SMs (below, the pairs' tiles of 256 features leave most
+// of them without work).
+constexpr int kPairMinRows = 33;
 static bool pair_usable(const sj_target* t, const sj_kv* kv, int R) {
   return t->opt_gemm == 1 && t->opt_attn >= 1 && t->bf && kv->has_tm_pool && R >= kPairMinRows;
 }
@@ -1246,14 +1246,18 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
 #undef TIMED_BEGIN
 #undef TIMED_END
 
-// The whole step as one cooperative launch per chunk of kMegaMaxLayers layers.
-static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma) {
+// The whole step as one cooperative launch per chunk of kMegaMaxLayers layers, up to kMegaMaxRows rows.  From kPairMinRows
+// rows on and with caches of several 128-key tiles per SM the attention decides: the persistent kernel's mma.sync phase
+// takes about three times as long a key as the tcgen05 kernel (8B-shaped, 16 layers, 4 x 9 rows: 4 x 4000 keys 3062 us
+// against 2681 per stage, 4 x 300 keys 2429 against 2518).
+static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma, long total_keys) {
   const int rows = gamma + 1, R = B * rows, group = t->dm.Hq / t->dm.Hkv;
+  if (R >= kPairMinRows && t->dm.hd == 128 && t->opt_attn == 2 && total_keys * t->dm.Hkv / kT5Keys / t->sm_count >= t->opt_a5_min_tiles) return false;
   return t->opt_step == 1 && t->opt_gemm == 1 && t->mega_shapes && kv->has_tm_pool && R <= kMegaMaxRows &&
          group * rows <= 16 * 6 && t->stream != nullptr;
 }
 
-static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode, bool use_scratch, long total_keys) {
+static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode, bool use_scratch) {
   const Dims& dm = t->dm;
   const int rows = gamma + 1, R = B * rows, Rp = pad16(R), qd = dm.Hq * dm.hd;
   cudaStream_t s = t->stream;
@@ -1268,23 +1272,14 @@ static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode
   memset(&p, 0, sizeof(p));
   p.B = B; p.rows = rows; p.R = R; p.Rp = Rp;
   p.stage_bytes = kWTileBytes + round_up(2 * Rp * 128, 1024);
-  // tcgen05 attention phase: head dimension 128, a KV head's query rows within two TMEM lane quarters, ring stages
-  // that hold a 32 KiB key or value tile (49 block rows or more), and caches long enough that the phase is bound by
-  // throughput (at a few tiles per block it is a chain of latencies, and the mma.sync phase, which needs no hand-over
-  // between warps, is as fast)
-  const int nq = (dm.Hq / dm.Hkv) * rows;
-  const long tiles_per_block = total_keys * dm.Hkv / kA5Keys / t->sm_count;
-  const bool a5 = dm.hd == 128 && nq <= kA5MaxRows && t->opt_attn == 2 && p.stage_bytes >= (int)kA5Part &&
-                  tiles_per_block >= t->opt_a5_min_tiles;
-  p.q_area_bytes = a5 ? a5_q_area_bytes(nq) : 0;
   const int ctl_bytes = ((int)sizeof(MegaCtl) + 127) & ~127;
-  const int budget = 227 * 1024 - 1024 - ctl_bytes - p.q_area_bytes;
+  const int budget = 227 * 1024 - 1024 - ctl_bytes;
   p.stages = std::min(8, std::min(kMegaMaxStages, budget / p.stage_bytes));   // deeper rings did not measure faster; the rest stays L1
   if (p.stages < 3) return fail(SJ_ERR_SHAPE, "too many rows for the whole-step kernel");
   if (t->opt_ring) p.stages = std::min(p.stages, t->opt_ring);
   uint32_t tc = 32;
   while (tc < (uint32_t)(4 * Rp)) tc <<= 1;
-  p.tmem_cols = a5 ? std::max(tc, (uint32_t)kA5TmemCols) : tc;
+  p.tmem_cols = tc;
   p.lp = t->d_layer_ptrs;
   p.embed = (const bf16*)t->embed;
   p.lm_head = (const bf16*)t->lm_head;
@@ -1298,7 +1293,7 @@ static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode
   p.trace = t->opt_trace ? t->d_trace : nullptr;
   p.trace_block = t->opt_trace ? (unsigned)std::min(t->opt_trace - 1, t->sm_count - 1) : 0u;
   const int grid = t->sm_count;
-  const size_t smem = (size_t)p.stages * p.stage_bytes + p.q_area_bytes + ctl_bytes + 1024;
+  const size_t smem = (size_t)p.stages * p.stage_bytes + ctl_bytes + 1024;
   const bool timing = t->opt_timing != 0;
   const int NL = dm.n_layers;
   for (size_t ci = 0; ci < t->mega_maps.size(); ++ci) {
@@ -1336,7 +1331,7 @@ static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode
     const StepArgs* args = t->d_args;
     // row slots per epilogue thread: a group gets at most (min(R, 16) + 1) / 2 rows of a 16-row chunk
     const int ns = R <= 8 ? 4 : (R <= 12 ? 6 : 8);
-    CU_TRY(cudaLaunchKernelEx(&cfg, mega_kernel(dm.hd, ns, t->opt_trace != 0, a5), mm, p, args, kv->view, W, dm));
+    CU_TRY(cudaLaunchKernelEx(&cfg, mega_kernel(dm.hd, ns, t->opt_trace != 0), mm, p, args, kv->view, W, dm));
     if (timing) {
       CU_TRY(cudaEventRecord(eb, s));
       t->timed.push_back({"verify_step", ea, eb});
@@ -1464,13 +1459,14 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
   const int chunk_len = pick_chunk_len(t, total_keys);
   for (int i = 0; i < B; ++i) chunk_need_base += (size_t)(kv->len_hi[a->seq_ids[i]] + rows + chunk_len - 1) / chunk_len;
 
-  const bool use_mega = mega_usable(t, kv, B, gamma);
+  const bool use_mega = mega_usable(t, kv, B, gamma, total_keys);
   // [R, V] logits exist only for the CUDA-core LM head (fp32 models, cross-checks); the tensor-core paths keep
   // softmax statistics per vocabulary tile and, in sampling mode, the logits of one row per sequence ([B, V])
   const bool use_scratch = t->opt_gemm == 0 && !use_mega;
   const size_t logit_rows_needed = use_scratch ? (size_t)R : (a->mode == SJ_MODE_SAMPLING ? (size_t)B : 0);
   // grow lazily-sized buffers (outside any capture)
-  if (chunk_need_base > t->att_chunks_cap || rows > t->att_rows_cap) {
+  const bool simt_attn = t->opt_attn == 0 || !t->bf || !kv->has_tm_pool;
+  if (simt_attn && (chunk_need_base > t->att_chunks_cap || rows > t->att_rows_cap)) {
     CU_TRY(cudaStreamSynchronize(t->stream));
     clear_graphs(t);
     size_t cap = std::max(chunk_need_base * 2, (size_t)64);
@@ -1489,7 +1485,7 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
     t->att_chunks_cap = cap;
     t->att_rows_cap = rcap;
   }
-  if ((t->opt_attn >= 1 || use_mega) && t->bf && kv->has_tm_pool)
+  if ((!simt_attn || use_mega) && kv->has_tm_pool)
     if ((st = ensure_attn_partials(t, B, rows)) != SJ_OK) return st;
   if (logit_rows_needed > t->logits_rows) {
     CU_TRY(cudaStreamSynchronize(t->stream));
@@ -1523,9 +1519,10 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
   memcpy(h.seq_ids, a->seq_ids, sizeof(int) * B);
   CU_TRY(cudaMemcpyAsync(t->d_args, &h, sizeof(h), cudaMemcpyHostToDevice, t->stream));
 
-  StepKey key{B, gamma, a->mode, chunk_len, t->opt_gemm, t->opt_attn, t->opt_pdl, use_scratch ? 1 : 0};
+  // chunk_len shapes only the CUDA-core attention's grid: a growing cache captures no new step elsewhere
+  StepKey key{kv, B, gamma, a->mode, simt_attn ? chunk_len : 0, t->opt_gemm, t->opt_attn, t->opt_pdl, use_scratch ? 1 : 0};
   if (use_mega) {
-    if ((st = launch_mega(t, kv, B, gamma, a->mode, use_scratch, total_keys)) != SJ_OK) return st;
+    if ((st = launch_mega(t, kv, B, gamma, a->mode, use_scratch)) != SJ_OK) return st;
   } else if (t->opt_graph) {
     auto it = t->graphs.find(key);
     if (it == t->graphs.end()) {
@@ -1658,10 +1655,10 @@ extern "C" sj_status sj_semantic_score(sj_target* t, sj_kv* kv, int seq, int y_i
 // bf16 pages, so another partition would give slightly other results) over the same sequence -- entry b attends to the stored cache plus the b * c rows before it
 // (its projection has stored them in the pages by the time the attention kernel runs) and to its own rows, which is
 // exactly what B verification steps of c rows one after another would do, at one read of the weights (8B-shaped model,
-// 1000 tokens and a step: 190 ms in blocks of 24 rows, PF_MS ms in two of 504).  Only the last token's row meets the
+// 1000 tokens and a step: 190 ms in blocks of 24 rows, 34 ms in two of 504).  Only the last token's row meets the
 // LM head, and a block that is not the last one ends with its key / value rows.
 constexpr int kPrefillRows = SJ_MAX_ROWS;   // rows of a wide block
-constexpr int kPrefillWideMin = 33;    // shorter prompts: one or two narrow blocks through the whole-step kernel
+constexpr int kPrefillWideMin = kPairMinRows;   // shorter prompts: one or two narrow blocks through the whole-step kernel
 
 static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* tokens, int n_tokens, int c, int* d_next, bool* done) {
   const Dims& dm = t->dm;
@@ -1672,7 +1669,6 @@ static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* token
     const size_t mark = t->owned.size();
     memset(&t->pf_work, 0, sizeof(Work));
     st = alloc_rows(t, t->pf_work, kPrefillRows);
-    if (st == SJ_OK) st = alloc_partials(t, t->pf_work, kPairMinRows - 1);   // wider blocks need none
     if (st != SJ_OK) {   // no memory for it: the narrow blocks need none
       while (t->owned.size() > mark) { counted_free(t->owned.back()); t->owned.pop_back(); }
       t->pf_rows = -1;

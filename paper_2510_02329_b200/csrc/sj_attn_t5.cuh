@@ -15,12 +15,12 @@
 //                 as well.  O^T has the dims in the lanes: the segment's partial is stored coalesced.
 // 16 MMAs of N = 2 NQ per tile.  With the query rows as M = 128 (the kernel before this one) 36 rows of a group of four
 // heads and gamma 8 left 72 % of the accumulator lanes and softmax lanes idle and the softmax took 2060 clocks a tile,
-// where HBM delivers one in 2600 to every SM; it is now MEASURED.
+// where HBM delivers one in 2600 to every SM; a layer of 32 sequences of 512 to 8192 keys and 8 KV
+// heads (570 MB, 86 us at the copy rate) took 153 us, with this one 127 us (B200).
 //
 // A segment (the block's run of tiles of one (sequence, KV head)) ends with the unnormalised partial (m, l, o) per query
 // row, in the format of sj_attn_tc.cuh, whose combine pass merges them; the block's own gamma+1 rows (the causal tail)
-// are handled with that file's mma.sync routine.  The routines below are shared by the stand-alone kernel k_attn_t5 and
-// the attention phase of the persistent step kernel, whose ring also carries the weights.
+// are handled with that file's mma.sync routine, by a warp of their own beside the tiles.
 //
 // Every wait is bounded; one that runs out raises the abort flag, after which all others return at once: the flow goes
 // on to its end with whatever it reads (named barriers are met by every warp), and the status word tells the host.
@@ -32,40 +32,13 @@
 namespace sj {
 
 constexpr int kT5Keys = 128;               // keys per tile
-constexpr int kT5Pad = 4;                  // empty tiles the plan counts per (sequence, KV head): what a segment costs a block beyond its tiles
-constexpr int kT5Threads = 352;            // warp 0 key tiles, warp 10 value tiles, warp 1 MMA, warps 2..9 softmax and, after their tiles, the causal tails
+constexpr int kT5Pad = 2;                  // empty tiles the plan counts per (sequence, KV head): what a segment costs a block beyond its tiles
+constexpr int kT5Threads = 384;            // warp 0 key tiles, warp 10 value tiles, warp 1 MMA, warps 2..9 softmax, warp 11 the causal tails
 constexpr int kT5MaxRows = 128;
-constexpr int kA5Keys = kT5Keys;           // the same in the persistent kernel
-constexpr int kA5MaxRows = 64;
-constexpr int kA5Pad = 3;
-constexpr uint32_t kA5Part = 32768;        // bytes of a key tile or a value tile: the least a ring stage must hold
+constexpr uint32_t kT5Part = 32768;        // bytes of a key tile or a value tile: a ring stage
 constexpr int kA5TmemCols = 512;
 constexpr float kA5Raise = 16.f;           // log2: how far a score may exceed the stabiliser
 
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,"
-      "%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-        "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tc_ld32_nowait(uint32_t taddr, float* v) {   // results valid after tc_wait_ld()
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,"
-      "%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]), "=f"(v[9]),
-        "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15]), "=f"(v[16]), "=f"(v[17]), "=f"(v[18]),
-        "=f"(v[19]), "=f"(v[20]), "=f"(v[21]), "=f"(v[22]), "=f"(v[23]), "=f"(v[24]), "=f"(v[25]), "=f"(v[26]), "=f"(v[27]),
-        "=f"(v[28]), "=f"(v[29]), "=f"(v[30]), "=f"(v[31])
-      : "r"(taddr));
-}
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t* r) {
   asm volatile(
@@ -73,13 +46,6 @@ __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t* r) {
       "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
       "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
       : "memory");
-}
-__device__ __forceinline__ void tc_st32f(uint32_t taddr, const float* v) {
-  uint32_t r[32];
-#pragma unroll
-  for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(v[i]);
-  tc_st16(taddr, r);
-  tc_st16(taddr + 16, r + 16);
 }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
@@ -162,12 +128,11 @@ __device__ __forceinline__ void a5_bars_init(A5Bars* b) {
 }
 static_assert(alignof(A5Smem) == 16 && sizeof(float) * kT5MaxRows % 16 == 0, "float4 reads of the softmax state");
 struct A5Ring {
-  uint64_t* full;    // [stages], each completes on two arrivals (the expecting one and a second)
+  uint64_t* full;    // [stages], one arrival
   uint64_t* empty;   // [stages], one arrival
   uint8_t* base;
-  int stage_stride, stages;
+  int stages;
   volatile int* abort_flag;
-  volatile int* abort_g;
   int* status;
 };
 struct A5Pos {
@@ -176,33 +141,29 @@ struct A5Pos {
     if (++s == NS) { s = 0; ++r; }
   }
 };
-// A tile's ring entries: the key tile, the value tile and, with PRING, a stage without a load that holds its
-// probabilities (a ring that is sized for other traffic has no room for an area of their own).
-template <bool PRING>
+// A tile's ring entries: the key tile (0) and the value tile (1).
 struct A5Entry {
-  static constexpr int n = PRING ? 3 : 2;
-  int s[n];
-  uint32_t par[n], a[n];   // stage, parity of this use, address
+  int s[2];
+  uint32_t par[2], a[2];   // stage, parity of this use, address
 };
-template <bool PRING>
-__device__ __forceinline__ A5Entry<PRING> a5_entry(const A5Ring& rg, A5Pos& pos) {   // the tile at pos; pos moves past it
-  A5Entry<PRING> e;
+__device__ __forceinline__ A5Entry a5_entry(const A5Ring& rg, A5Pos& pos) {   // the tile at pos; pos moves past it
+  A5Entry e;
 #pragma unroll
-  for (int i = 0; i < A5Entry<PRING>::n; ++i) {
+  for (int i = 0; i < 2; ++i) {
     e.s[i] = pos.s;
     e.par[i] = (uint32_t)pos.r & 1u;
-    e.a[i] = att_smem_u32(rg.base + (size_t)pos.s * rg.stage_stride);
+    e.a[i] = att_smem_u32(rg.base + (size_t)pos.s * kT5Part);
     pos.next(rg.stages);
   }
   return e;
 }
 __device__ __forceinline__ bool a5_wait(const A5Ring& rg, uint64_t* bar, uint32_t parity, int where, int extra) {
-  return att_mbar_wait(att_smem_u32(bar), parity, rg.abort_flag, rg.status, rg.abort_g, where, extra);
+  return att_mbar_wait(att_smem_u32(bar), parity, rg.abort_flag, rg.status, nullptr, where, extra);
 }
 // The block's run of real tiles at tile t: (sequence, KV head, first tile), its length n, and nv, the same with the
 // plan's empty tiles; n == 0 when only empty tiles of that (sequence, KV head) fell to this block.
 __device__ __forceinline__ void a5_run_at(const AttPlan& pl, int B, long long t, long long t_hi, AttTile& x, int& n, int& nv) {
-  x = att_locate(pl, B, kA5Keys, (int)t);
+  x = att_locate(pl, B, kT5Keys, (int)t);
   nv = (int)min((long long)(x.nt_b - x.ti), t_hi - t);
   n = max(0, min(nv, x.nt_real - x.ti));
 }
@@ -211,18 +172,18 @@ __device__ __forceinline__ void a5_run_at(const AttPlan& pl, int B, long long t,
 // flow).  A key or value tile is sixteen boxes of 2 KiB (16 keys x 64 dims: a page's slots, one swizzle span wide), one
 // per lane (half = lane / 8, page = lane % 8); sixteen lanes get theirs out in 1250 clocks, so one warp for both would
 // take longer than HBM needs for the bytes.  The first warp claims every stage in ring order and loads the key tiles; it
-// hands a value stage over by a count in shared memory (`claimed`: value stages claimed so far, over all layers).  The
+// hands a value stage over by a count in shared memory (`claimed`: value stages claimed so far).  The
 // second warp may not wait on the stages' barriers itself: key stages are freed ahead of value stages, and a warp that is
 // lapped waits for a parity that has passed.  pages: the block's page ids, eight per tile (clamped to the sequence's last
-// page), for its first kAttPageCache / 8 tiles.  vals: value tiles of earlier layers (advanced).
-template <bool PRING>
+// page), for its first kAttPageCache / 8 tiles.
 __device__ __forceinline__ bool a5_produce(const A5Ring& rg, A5Pos& pos, const CUtensorMap* tmKV, const KvView& kv,
                                            const StepArgs* __restrict__ args, const AttPlan& pl, int B, int layer,
-                                           long long t_lo, long long t_hi, const int* pages, int lane, int which, volatile int* claimed, int& vals) {
+                                           long long t_lo, long long t_hi, const int* pages, int lane, int which, volatile int* claimed) {
+  int vals = 0;
   const int half = (lane >> 3) & 1, p = lane & 7;
 #pragma unroll 1
   for (long long t = t_lo; t < t_hi; ++t) {
-    const AttTile x = att_locate(pl, B, kA5Keys, (int)t);
+    const AttTile x = att_locate(pl, B, kT5Keys, (int)t);
     if (x.ti >= x.nt_real) continue;   // one of the plan's empty tiles: no ring entry
     const int seq = args->seq_ids[x.b], last_page = (x.L - 1) / 16, tb = (int)(t - t_lo);
     int pi = x.ti * 8 + p;
@@ -242,14 +203,12 @@ __device__ __forceinline__ bool a5_produce(const A5Ring& rg, A5Pos& pos, const C
       __syncwarp();
     }
 #pragma unroll 1
-    for (int e = 0; e < A5Entry<PRING>::n; ++e) {
+    for (int e = 0; e < 2; ++e) {
       const uint32_t bar = att_smem_u32(&rg.full[pos.s]);
       if (which == 0) {
         if (pos.r > 0 && !a5_wait(rg, &rg.empty[pos.s], (uint32_t)(pos.r - 1) & 1u, 1, pos.r)) return false;
         if (lane == 0) {
-          if (e < 2) att_mbar_expect_tx(bar, kA5Part);
-          else att_mbar_arrive(bar);
-          att_mbar_arrive(bar);   // the stage's second arrival
+          att_mbar_expect_tx(bar, kT5Part);
           if (e == 1) {
             __threadfence_block();
             *claimed = vals;
@@ -257,7 +216,7 @@ __device__ __forceinline__ bool a5_produce(const A5Ring& rg, A5Pos& pos, const C
         }
       }
       if (e == which && lane < 16)
-        att_tma_2d(att_smem_u32(rg.base + (size_t)pos.s * rg.stage_stride) + (uint32_t)(half * 16384 + p * 2048), tmKV, bar, half * 64, (int)row);
+        att_tma_2d(att_smem_u32(rg.base + (size_t)pos.s * kT5Part) + (uint32_t)(half * 16384 + p * 2048), tmKV, bar, half * 64, (int)row);
       pos.next(rg.stages);
     }
   }
@@ -266,9 +225,7 @@ __device__ __forceinline__ bool a5_produce(const A5Ring& rg, A5Pos& pos, const C
 
 // One elected thread: the MMAs of the block's tiles.  Order: scores(0) .. scores(n_s - 1), then output(i), scores(i + n_s),
 // so that a tile's scores are ready while the softmax of the one before runs, and an output never waits behind scores
-// whose keys have not arrived (with output(i) after scores(i + 1) a tile took 4000 clocks).  gt: tiles of earlier layers (the barriers' phases run on
-// across layers), segs: segments of earlier layers; both advanced.  p_area: address of the probabilities without PRING.
-template <bool PRING>
+// whose keys have not arrived (with output(i) after scores(i + 1) a tile took 4000 clocks).  gt, segs: tiles and segments so far (advanced).  p_area: address of the probabilities.
 __device__ __forceinline__ bool a5_issue(const A5Ring& rg, A5Pos& pos, A5Bars* ab, uint32_t tmem, uint32_t q_area, uint32_t p_area, int nq,
                                          const AttPlan& pl, int B, long long t_lo, long long t_hi, int& gt, int& segs) {
   const int NQ2 = 2 * a5_nq(nq), n_s = a5_s_bufs(nq);
@@ -286,24 +243,23 @@ __device__ __forceinline__ bool a5_issue(const A5Ring& rg, A5Pos& pos, A5Bars* a
     if (n == 0) continue;   // only empty tiles of this (sequence, KV head): no segment
     if (!a5_wait(rg, &ab->q_ready, (uint32_t)segs & 1u, 2, segs)) return false;
     tc_fence_after();
-    A5Entry<PRING> pend[2];   // entries of the tiles whose scores have been issued and outputs have not: pend[i & 1]
+    A5Entry pend[2];   // entries of the tiles whose scores have been issued and outputs have not: pend[i & 1]
 #pragma unroll 1
     for (int i = -n_s; i < n; ++i) {
       if (i >= 0) {   // output of tile i
         const int g = gt + i;
-        const A5Entry<PRING> e = n_s == 2 && (i & 1) ? pend[1] : pend[0];
+        const A5Entry e = n_s == 2 && (i & 1) ? pend[1] : pend[0];
         if (!a5_wait(rg, &ab->p_full, (uint32_t)g & 1u, 5, g) || !a5_wait(rg, &rg.full[e.s[1]], e.par[1], 6, g)) return false;
         tc_fence_after();
-        const uint64_t dv = smem_desc_mn_sw128(e.a[1], 16384u), dp = smem_desc_mn_sw128(PRING ? e.a[A5Entry<PRING>::n - 1] : p_area, 16384u);
+        const uint64_t dv = smem_desc_mn_sw128(e.a[1], 16384u), dp = smem_desc_mn_sw128(p_area, 16384u);
 #pragma unroll
         for (int k = 0; k < 8; ++k)   // 16 keys each
           tc_mma_bf16(d_o, dv + (uint64_t)(k * (2048 >> 4)), dp + (uint64_t)(k * (2048 >> 4)), id_o, (i > 0 || k > 0) ? 1u : 0u);
         tc_commit(att_smem_u32(&ab->o_done));
         tc_commit(att_smem_u32(&rg.empty[e.s[1]]));
-        if (PRING) tc_commit(att_smem_u32(&rg.empty[e.s[A5Entry<PRING>::n - 1]]));
       }
       if (i + n_s < n) {   // scores of tile i + n_s
-        const A5Entry<PRING> e = a5_entry<PRING>(rg, pos);
+        const A5Entry e = a5_entry(rg, pos);
         const int g = gt + i + n_s, b = n_s == 2 ? g & 1 : 0, use = n_s == 2 ? g >> 1 : g;
         if (use > 0 && !a5_wait(rg, &ab->s_free[b], (uint32_t)(use - 1) & 1u, 3, g)) return false;
         if (!a5_wait(rg, &rg.full[e.s[0]], e.par[0], 3, g)) return false;
@@ -332,19 +288,15 @@ __device__ __forceinline__ uint32_t a5_q_off(int row, int dim, int NQ2) {
 }
 
 // The softmax side: eight warps in two groups of 128 threads, thread = key = TMEM lane; group `grp` handles the queries
-// [0, a5_split) or the rest and meets at named barrier `bar_id`.  MAXC: most 8-query chunks of a group.  pos: the block's
-// first ring entry (advanced).  The partial slot of the block's segment is slot0 + b * Hkv + h (sub-partial 0).
-// ev: optional timeline of the block's last segment (global-timer ns), stamped by the first softmax thread:
-// [0] queries delivered, [1] last tile's probabilities delivered, [2] partial stored, [3] first scores seen.
-template <bool PRING, int MAXC>
-__device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Pos& pos, A5Bars* ab, A5Smem* sh, uint32_t tmem, uint8_t* q_area, uint8_t* p_area,
+// [0, a5_split) or the rest and meets at named barrier `bar_id`.  MAXC: most 8-query chunks of a group.  The partial slot of the block's segment is slot0 + b * Hkv + h (sub-partial 0).
+template <int MAXC>
+__device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Bars* ab, A5Smem* sh, uint32_t tmem, uint8_t* q_area, uint8_t* p_area,
                                            const AttArgs& a, const AttPlan& pl, int B, int Hkv, int nq, long long t_lo, long long t_hi, int& gt,
-                                           int slot0, int quarter, int grp, int bar_id, int lane, unsigned long long* ev = nullptr) {
+                                           int slot0, int quarter, int grp, int bar_id, int lane) {
   constexpr int HD = 128;
   const int NQ = a5_nq(nq), NQ2 = 2 * NQ, n_s = a5_s_bufs(nq), split = a5_split(nq);
   const int q0 = grp ? split : 0, nch = (grp ? NQ - split : split) / 8;
   const int key = 32 * quarter + lane;
-  const bool stamp = ev && grp == 0 && key == 0;
   const uint32_t lane_addr = tmem + ((uint32_t)(32 * quarter) << 16);
   const uint32_t o_addr = lane_addr + (uint32_t)(n_s * NQ2);
   // queries of a (sequence, KV head): fp16 (plus what its rounding dropped, in the two-term layers) -> two bf16 terms
@@ -409,7 +361,6 @@ __device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Pos& pos, A5Bars*
     }
     if (first_seg) deliver_q(x);   // later segments' queries were delivered while the segment before them ended
     first_seg = false;
-    if (stamp) ev[0] = att_timer_ns();
     float l[MAXC][8];
 #pragma unroll
     for (int c = 0; c < MAXC; ++c)
@@ -418,10 +369,8 @@ __device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Pos& pos, A5Bars*
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
       const int g = gt + i, b = n_s == 2 ? g & 1 : 0, use = n_s == 2 ? g >> 1 : g;
-      const A5Entry<PRING> en = a5_entry<PRING>(rg, pos);
       a5_wait(rg, &ab->s_full[b], (uint32_t)use & 1u, 7, g);
       __syncwarp();
-      if (stamp && i == 0) ev[3] = att_timer_ns();
       tc_fence_after();
       const uint32_t s_addr = lane_addr + (uint32_t)(b * NQ2 + q0);
       float s[MAXC][8];
@@ -443,7 +392,7 @@ __device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Pos& pos, A5Bars*
       }
       tc_fence_before();
       att_mbar_arrive(att_smem_u32(&ab->s_free[b]));
-      if (key >= x.L - (x.ti + i) * kA5Keys) {   // only in a sequence's last tile
+      if (key >= x.L - (x.ti + i) * kT5Keys) {   // only in a sequence's last tile
 #pragma unroll
         for (int c = 0; c < MAXC; ++c)
 #pragma unroll
@@ -503,11 +452,6 @@ __device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Pos& pos, A5Bars*
         }
       }
       // the tile's place for the probabilities is free once the output MMAs that read the one before have completed
-      uint8_t* pb = p_area;
-      if (PRING) {
-        a5_wait(rg, &rg.full[en.s[A5Entry<PRING>::n - 1]], en.par[A5Entry<PRING>::n - 1], 9, g);
-        pb = rg.base + (size_t)en.s[A5Entry<PRING>::n - 1] * rg.stage_stride;
-      }
       if (i > 0) a5_wait(rg, &ab->o_done, (uint32_t)(g - 1) & 1u, 9, g);   // (every phase is waited for: a parity wait may not skip one)
       __syncwarp();
       // probabilities as two bf16 terms: hi = p truncated to bf16, lo = the rest rounded to bf16 (16 significant bits)
@@ -528,14 +472,13 @@ __device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Pos& pos, A5Bars*
             lo[e >> 1] = *reinterpret_cast<const uint32_t*>(&bl);
           }
           const int nh = q0 + 8 * c, nl = NQ + nh;   // columns; [64-column atom][key][128 B], 128-byte swizzle
-          *reinterpret_cast<uint4*>(pb + (nh >> 6) * 16384 + key * 128 + ((((nh & 63) >> 3) ^ (key & 7)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-          *reinterpret_cast<uint4*>(pb + (nl >> 6) * 16384 + key * 128 + ((((nl & 63) >> 3) ^ (key & 7)) << 4)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+          *reinterpret_cast<uint4*>(p_area + (nh >> 6) * 16384 + key * 128 + ((((nh & 63) >> 3) ^ (key & 7)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+          *reinterpret_cast<uint4*>(p_area + (nl >> 6) * 16384 + key * 128 + ((((nl & 63) >> 3) ^ (key & 7)) << 4)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read these generic-proxy stores
       tc_fence_before();
       att_mbar_arrive(att_smem_u32(&ab->p_full));
     }
-    if (stamp) ev[1] = att_timer_ns();
     // The next segment's queries, before this one is wound up: every score MMA of this segment has completed (this
     // thread saw the scores of its last tile), so the query area is free once every thread is here, and the issuer starts
     // on the next segment's scores while the partial below is read out (its first output MMAs wait for probabilities that
@@ -583,16 +526,15 @@ __device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Pos& pos, A5Bars*
       tc_fence_before();
     }
     bar_sync128(bar_id);   // the sums have been read before the next segment's first tile reuses their place
-    if (stamp) ev[2] = att_timer_ns();
     gt += n;
     t += nv;
   }
   return *rg.abort_flag == 0;
 }
 
-// =============================================================================================
-// the stand-alone kernel: one block per SM
-// =============================================================================================
+// ---------------------------------------------------------------------------------------------
+// the kernel: one block per SM
+// ---------------------------------------------------------------------------------------------
 constexpr int kT5MaxStages = 6;
 struct T5Ctl {
   uint64_t full[kT5MaxStages], empty[kT5MaxStages];
@@ -607,9 +549,9 @@ struct T5Geom { int stages; size_t smem; };
 __host__ __forceinline__ T5Geom t5_geom(int nq) {
   const size_t fixed = (size_t)a5_q_area_bytes(nq) + a5_p_bytes(nq) + sizeof(T5Ctl) + 1024;
   T5Geom g;
-  g.stages = (int)((227 * 1024 - fixed) / kA5Part);
+  g.stages = (int)((227 * 1024 - fixed) / kT5Part);
   if (g.stages > kT5MaxStages) g.stages = kT5MaxStages;
-  g.smem = fixed + (size_t)g.stages * kA5Part;
+  g.smem = fixed + (size_t)g.stages * kT5Part;
   return g;
 }
 
@@ -624,12 +566,12 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   pdl_launch();
   const int B = args->B, rows = args->gamma + 1, Hkv = dm.Hkv, group = dm.Hq / dm.Hkv, nq = group * rows;
   const int G = gridDim.x, c = blockIdx.x;
-  uint8_t* p_area = sm + (size_t)stages * kA5Part;
+  uint8_t* p_area = sm + (size_t)stages * kT5Part;
   uint8_t* q_area = p_area + a5_p_bytes(nq);
   T5Ctl* ctl = reinterpret_cast<T5Ctl*>(q_area + a5_q_area_bytes(nq));
   if (threadIdx.x == 0) {
     for (int i = 0; i < stages; ++i) {
-      att_mbar_init(att_smem_u32(&ctl->full[i]), 2);
+      att_mbar_init(att_smem_u32(&ctl->full[i]), 1);
       att_mbar_init(att_smem_u32(&ctl->empty[i]), 1);
     }
     a5_bars_init(&ctl->bars);
@@ -655,26 +597,23 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   att_fill_pages(ctl->pages, pl, kv, args, B, kT5Keys, t_lo, t_hi, threadIdx.x, blockDim.x);
   __syncthreads();
   const uint32_t tmem = ctl->tmem_base;
-  const A5Ring rg{ctl->full, ctl->empty, sm, (int)kA5Part, stages, &ctl->abort_flag, nullptr, w.status};
+  const A5Ring rg{ctl->full, ctl->empty, sm, stages, &ctl->abort_flag, w.status};
   A5Pos pos{0, 0};
   int gt = 0, segs = 0;
   if (warp == 0 || warp == 10) {
-    a5_produce<false>(rg, pos, &tmKV, kv, args, pl, B, a.layer, t_lo, t_hi, ctl->pages, lane, warp == 0 ? 0 : 1, &ctl->sh.claimed, gt);
+    a5_produce(rg, pos, &tmKV, kv, args, pl, B, a.layer, t_lo, t_hi, ctl->pages, lane, warp == 0 ? 0 : 1, &ctl->sh.claimed);
   } else if (warp == 1) {
-    if (elect_one()) a5_issue<false>(rg, pos, &ctl->bars, tmem, att_smem_u32(q_area), att_smem_u32(p_area), nq, pl, B, t_lo, t_hi, gt, segs);
-  } else {
+    if (elect_one()) a5_issue(rg, pos, &ctl->bars, tmem, att_smem_u32(q_area), att_smem_u32(p_area), nq, pl, B, t_lo, t_hi, gt, segs);
+  } else if (warp < 10) {
     const int grp = (warp - 2) >> 2;
-    const bool alive = a5_softmax<false, MAXC>(rg, pos, &ctl->bars, &ctl->sh, tmem, q_area, p_area, a, pl, B, Hkv, nq, t_lo, t_hi, gt, c, warp & 3, grp,
-                                               2 + grp, lane);
+    a5_softmax<MAXC>(rg, &ctl->bars, &ctl->sh, tmem, q_area, p_area, a, pl, B, Hkv, nq, t_lo, t_hi, gt, c, warp & 3, grp, 2 + grp, lane);
+  } else {
     // the causal tails (the step's own rows as keys; mma.sync): one m-tile of one (sequence, KV head) per task, dealt
-    // over all blocks' softmax warps from the last block down
-    if (alive) {
-      const AttGeom g = att_geom(HD, group, rows);
-      AttWarp<HD, 2> st;
+    // over all blocks from the last block down, beside the tiles
+    const AttGeom g = att_geom(HD, group, rows);
+    AttWarp<HD, 2> st;
 #pragma unroll 1
-      for (int task = (G - 1 - c) * 8 + (warp - 2); task < B * Hkv * g.MT; task += G * 8)
-        att_tail_task<HD, 2>(st, g, a, task / g.MT, (task % g.MT) * 16, lane);
-    }
+    for (int task = G - 1 - c; task < B * Hkv * g.MT; task += G) att_tail_task<HD, 2>(st, g, a, task / g.MT, (task % g.MT) * 16, lane);
   }
   tc_fence_before();
   __syncthreads();

@@ -26,11 +26,13 @@
 //   gate/up (tiles interleave 64 gate and 64 up features) -> silu(g) * u -> down-projection input planes
 //   down  -> as O
 //   LM head -> softmax statistics per (vocabulary tile, row), logit of the drafted token
-// Attention: its cache tiles travel through the same ring.  Two implementations, chosen per launch: fp16 mma.sync in
-// the worker warps (sj_attn_tc.cuh), or -- head dimension 128, at most 64 query rows per KV head and sequence --
-// tcgen05 (the routines of sj_attn_t5.cuh; ring stages of at least 32 KiB): warp 1 issues the MMAs, the workers run the
-// softmax on tensor memory; the queries sit in an area of their own after the ring, a tile's probabilities in a ring
-// stage, the accumulators alias the GEMM phases' tensor-memory columns.
+// Attention: its cache tiles travel through the same ring and are consumed by fp16 mma.sync in the worker warps
+// (sj_attn_tc.cuh).
+//
+// Up to kMegaMaxRows = 48 block rows.  Beyond that the step is no longer bound by the chain of its phases, and one kernel
+// per stage with the paired projections and the tcgen05 attention is faster (B200, us a step, persistent against per
+// stage: 32B-shaped 16 layers, 72 rows, 8 x 8192 keys 6735 / 5744; 8B-shaped 16 layers, 54 rows, 6 x 4000 keys 3643 / 2860;
+// 1B-shaped, 72 rows 2057 / 1713, 48 rows 1605 / 1608, 9 rows 1107 / 1823).
 //
 // Every wait is bounded; the first one to run out raises a device-wide abort word that all other waits
 // poll, so that a logic error ends the kernel with SJ_ERR_TIMEOUT instead of hanging the GPU.
@@ -38,14 +40,13 @@
 
 #include "sj_attn_tc.cuh"
 #include "sj_gemm_tc.cuh"
-#include "sj_attn_t5.cuh"
 
 namespace sj {
 
 constexpr int kMegaThreads = 384;
 constexpr int kMegaWorkers = 256;
 constexpr int kMegaMaxLayers = 32;   // per launch (tensor maps travel as kernel parameters)
-constexpr int kMegaMaxRows = 80;
+constexpr int kMegaMaxRows = 48;
 constexpr int kMegaMaxStages = 12;
 constexpr uint32_t kMegaSpin = 1u << 22;
 constexpr int kMegaRegsLight = 80;    // registers per thread of warps 0..3 after reallocation
@@ -96,7 +97,6 @@ struct MegaParams {
   int* abort_g;               // device-wide abort word        }
   int n_tail_base;
   int att_precise_layers;     // layers [0, n) run the attention with two-term (hi + lo fp16) queries and probabilities
-  int q_area_bytes;           // tcgen05 attention: bytes of the query area between the ring and the control block
   // optional timeline (global-timer nanoseconds), block `trace_block`:
   //   [2k], [2k+1]                      arrival at / release from device-wide barrier k (k >= 1)
   //   [2*kMegaTraceBarriers + 8*s + e]  event e of GEMM phase s: 0 activation producer released, 1 its last
@@ -136,8 +136,6 @@ struct MegaCtl {
   uint32_t tmem_base;
   int abort_flag;
   int bars_passed;
-  A5Bars a5;                   // tcgen05 attention: score / probability / output hand-offs
-  A5Smem a5s;                  // ... and the softmax state
   int bcast[6];   // [2 * group + accumulator]: the group's wait on that accumulator succeeded; [4], [5] spare
   float inv[kMegaMaxRows];
   float zd[kMegaMaxRows];      // top-k test: raw logit of each row's drafted token, computed before the LM head
@@ -179,11 +177,6 @@ __device__ __forceinline__ int unit_owner(unsigned u, unsigned U, int G) {
   while ((c + 1) * U / (unsigned)G <= u) ++c;
   return (int)c;
 }
-// Whether block c owns at least one unit when U units are dealt to G blocks.
-__device__ __forceinline__ bool has_units(int c, unsigned U, int G) {
-  return (unsigned)(c + 1) * U / (unsigned)G > (unsigned)c * U / (unsigned)G;
-}
-
 // How a site's units are dealt.  A "group" is CS consecutive blocks that share segments (CS = 1 everywhere
 // at present: a B200 holds only 33 clusters of four of these blocks, and streaming with 132 of its 148 SMs
 // cost more than an exchange through distributed shared memory saved).  Groups take [g*U/n, (g+1)*U/n);
@@ -382,27 +375,6 @@ __device__ __forceinline__ bool mega_wait_bars(int need, MegaCtl* ctl, const Meg
   *p.abort_g = 1;
   atomicCAS(status, DEV_OK, DEV_TIMEOUT);
   return false;
-}
-
-// TMA loads of one weight unit into a ring stage.
-__device__ __forceinline__ void mega_issue_w(const MegaMaps& mp, int site, int li, const Dims& dm, int tile, int kb,
-                                             uint32_t dst, uint32_t bar, uint64_t pol) {
-  switch (site) {
-    case SITE_QKV: {
-      const int tq = dm.Hq * dm.hd / kTileN, tk = dm.Hkv * dm.hd / kTileN;
-      if (tile < tq) tma_load_2d(dst, &mp.wq[li], bar, kb * kBK, tile * kTileN, pol);
-      else if (tile < tq + tk) tma_load_2d(dst, &mp.wk[li], bar, kb * kBK, (tile - tq) * kTileN, pol);
-      else tma_load_2d(dst, &mp.wv[li], bar, kb * kBK, (tile - tq - tk) * kTileN, pol);
-      break;
-    }
-    case SITE_O: tma_load_2d(dst, &mp.wo[li], bar, kb * kBK, tile * kTileN, pol); break;
-    case SITE_GU:
-      tma_load_2d(dst, &mp.wg[li], bar, kb * kBK, tile * 64, pol);
-      tma_load_2d(dst + 8192u, &mp.wu[li], bar, kb * kBK, tile * 64, pol);
-      break;
-    case SITE_DOWN: tma_load_2d(dst, &mp.wd[li], bar, kb * kBK, tile * kTileN, pol); break;
-    default: tma_load_2d(dst, &mp.lm, bar, kb * kBK, tile * kTileN, pol); break;
-  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -956,18 +928,16 @@ __device__ __forceinline__ void mega_finalize(MegaCtl* ctl, const MegaParams& p,
 // ---------------------------------------------------------------------------------------------
 // the kernel
 // ---------------------------------------------------------------------------------------------
-template <int HD, int SLOTS, bool kTr, bool A5>
+template <int HD, int SLOTS, bool kTr>
 __global__ void __launch_bounds__(kMegaThreads, 1)
 k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const StepArgs* __restrict__ args, const KvView kv,
               const Work w, const Dims dm) {
   extern __shared__ uint8_t mega_smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(mega_smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint8_t* q_area = ring + (size_t)p.stages * p.stage_bytes;
-  MegaCtl* ctl = reinterpret_cast<MegaCtl*>(q_area + p.q_area_bytes);
+  MegaCtl* ctl = reinterpret_cast<MegaCtl*>(ring + (size_t)p.stages * p.stage_bytes);
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int c = blockIdx.x, G = gridDim.x, NS = p.stages, B = p.B, R = p.R, Rp = p.Rp, rows = p.rows;
-  AttGeom g = att_geom(HD, dm.Hq / dm.Hkv, rows);
-  if constexpr (A5) { g.KPS = kA5Keys; g.KS = 1; g.KW = kA5Keys; }   // one sub-partial per block segment
+  const AttGeom g = att_geom(HD, dm.Hq / dm.Hkv, rows);
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < NS; ++i) {
@@ -979,8 +949,6 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
       mbar_init(smem_u32(&ctl->tmem_full[i]), 1);
       mbar_init(smem_u32(&ctl->tmem_empty[i]), kMegaWorkers);
     }
-    a5_bars_init(&ctl->a5);
-    ctl->a5s.claimed = 0;
     ctl->abort_flag = 0;
     ctl->bars_passed = 0;
     int acc = 0;
@@ -989,11 +957,11 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
       const int L = kv.kv_len[args->seq_ids[b]];
       ctl->plan.L[b] = L;
       ctl->plan.pre[b] = acc;
-      acc += L > 0 ? dm.Hkv * ((L + g.KPS - 1) / g.KPS + (A5 ? kA5Pad : 0)) : 0;
+      acc += L > 0 ? dm.Hkv * ((L + g.KPS - 1) / g.KPS) : 0;
     }
     ctl->plan.pre[B] = acc;
     ctl->plan.T = acc;
-    ctl->plan.pad = A5 ? kA5Pad : 0;
+    ctl->plan.pad = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -1022,25 +990,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
 
   const AttPlan& pl = ctl->plan;
   const long long t_lo = (long long)c * pl.T / G, t_hi = (long long)(c + 1) * pl.T / G;
-  // ring stages of one attention phase: one per tile, or (tcgen05) a key stage, a value stage and one for the probabilities per real tile
-  int n_att = (int)(t_hi - t_lo);
-  if constexpr (A5) {
-    int n_real = 0;
-#pragma unroll 1
-    for (long long t = t_lo; t < t_hi;) {
-      const AttTile x = att_locate(pl, B, g.KPS, (int)t);
-      const int nv = (int)min((long long)(x.nt_b - x.ti), t_hi - t);
-      n_real += max(0, min(nv, x.nt_real - x.ti));
-      t += nv;
-    }
-    n_att = A5Entry<true>::n * n_real;
-  }
-  if constexpr (A5) {   // padding query rows stay zero for the whole kernel
-#pragma unroll 1
-    for (int i = threadIdx.x; i < p.q_area_bytes / 16; i += blockDim.x) reinterpret_cast<uint4*>(q_area)[i] = make_uint4(0, 0, 0, 0);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read them
-  }
-  const A5Ring a5r{ctl->full, ctl->empty, ring, p.stage_bytes, NS, &ctl->abort_flag, p.abort_g, w.status};
+  const int n_att = (int)(t_hi - t_lo);   // ring stages of one attention phase
   att_fill_pages(ctl->att_pages, pl, kv, args, B, g.KPS, t_lo, t_hi, threadIdx.x, blockDim.x);
   __syncthreads();
   auto stage_addr = [&](int s) -> uint32_t { return smem_u32(ring + (size_t)s * p.stage_bytes); };
@@ -1053,11 +1003,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
   asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kMegaRegsLight));
   if (warp == 0) {
     // ------------------------------ weight / cache-tile producer ------------------------------
-    // One lane; all 32 with the tcgen05 attention, whose key tiles are sixteen small copies each (one per lane; the value
-    // tiles are warp 3's).  All lanes run the same control flow and wait on the same barriers; the elected lane alone
-    // issues the weight copies.
-    const bool leader = elect_one();
-    if (A5 || leader) {
+    if (elect_one()) {
       const uint64_t pol_w = l2_policy_evict_first();
       RingPos rp{0, 0, NS};
       int sidx = 0;
@@ -1089,28 +1035,18 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
 #pragma unroll 1
           for (int kb = sg.a; kb < sg.b; ++kb) {
             if (!wait_slot()) { alive = false; return; }
-            if (leader) {
-              const uint32_t bar = smem_u32(&ctl->full[rp.s]), dst = stage_addr(rp.s);
-              mbar_expect_tx(bar, kWTileBytes);
-              tma_load_2d(dst, tm0, bar, kb * kBK, row, pol_w);
-              if (site == SITE_GU) tma_load_2d(dst + 8192u, tm1, bar, kb * kBK, row, pol_w);
-            }
+            const uint32_t bar = smem_u32(&ctl->full[rp.s]), dst = stage_addr(rp.s);
+            mbar_expect_tx(bar, kWTileBytes);
+            tma_load_2d(dst, tm0, bar, kb * kBK, row, pol_w);
+            if (site == SITE_GU) tma_load_2d(dst + 8192u, tm1, bar, kb * kBK, row, pol_w);
             rp.next();
           }
         }
-        if (leader) MEGA_EV(sidx, 7);
+        MEGA_EV(sidx, 7);
         ++sidx;
       };
-      int a5_vals = 0;
       auto fatt = [&](int l) {
         if (!alive) return;
-        if constexpr (A5) {
-          A5Pos ap{rp.s, rp.r};
-          alive = a5_produce<true>(a5r, ap, &mp.pool, kv, args, pl, B, l, t_lo, t_hi, ctl->att_pages, lane, 0, &ctl->a5s.claimed, a5_vals);
-          rp.s = ap.s;
-          rp.r = ap.r;
-          return;
-        }
 #pragma unroll 1
         for (long long t = t_lo; t < t_hi; ++t) {
           if (!wait_slot()) { alive = false; return; }
@@ -1174,28 +1110,15 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         MEGA_EV(sidx, 3);
         ++sidx;
       };
-      int a5_tiles = 0, a5_segs = 0;
-      auto fatt = [&](int l) {
-        if constexpr (A5) {
-          if (!alive) return;
-          A5Pos ap{rp.s, rp.r};
-          alive = a5_issue<true>(a5r, ap, &ctl->a5, tmem_base, smem_u32(q_area), 0u, g.nq, pl, B, t_lo, t_hi, a5_tiles, a5_segs);
-          rp.s = ap.s;
-          rp.r = ap.r;
-        } else {
-          rp.advance(n_att);
-        }
-      };
+      auto fatt = [&](int l) { rp.advance(n_att); };
       mega_walk(p, fsite, fatt);
     }
   } else {
     // ------------------------------ activation producers (warps 2 and 3) ------------------------------
     // Two threads, alternate units: right after a device-wide barrier the ring already holds the phase's first
     // weight tiles, and the MMAs can start only as fast as their activation slices are requested (a wait, an
-    // expect and a TMA per slice cost one thread about a quarter of a microsecond).  With the tcgen05 attention warp 3 also
-    // loads the value tiles, all its lanes in the same flow.
-    const bool leader = elect_one();
-    if (leader || (A5 && warp == 3)) {
+    // expect and a TMA per slice cost one thread about a quarter of a microsecond).
+    if (elect_one()) {
       const int mine = warp - 2;
       int n_unit = 0;
       const uint64_t pol_a = l2_policy_evict_last();
@@ -1224,11 +1147,9 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
                   alive = false;
                   return;
                 }
-                if (leader) {
-                  const uint32_t bar = smem_u32(&ctl->full[rp.s]);
-                  mbar_expect_tx(bar, a_tx);
-                  tma_load_2d(stage_addr(rp.s) + kWTileBytes, tm, bar, kb * kBK, 0, pol_a);
-                }
+                const uint32_t bar = smem_u32(&ctl->full[rp.s]);
+                mbar_expect_tx(bar, a_tx);
+                tma_load_2d(stage_addr(rp.s) + kWTileBytes, tm, bar, kb * kBK, 0, pol_a);
               }
               rp.next();
             }
@@ -1238,20 +1159,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         ++sidx;
         nb += (site == SITE_QKV) ? 3 : 1;
       };
-      int a5_vals = 0;
-      auto fatt = [&](int l) {
-        if constexpr (A5) {
-          if (warp == 3) {
-            if (!alive) return;
-            A5Pos ap{rp.s, rp.r};
-            alive = a5_produce<true>(a5r, ap, &mp.pool, kv, args, pl, B, l, t_lo, t_hi, ctl->att_pages, lane, 1, &ctl->a5s.claimed, a5_vals);
-            rp.s = ap.s;
-            rp.r = ap.r;
-            return;
-          }
-        }
-        rp.advance(n_att);
-      };
+      auto fatt = [&](int l) { rp.advance(n_att); };
       mega_walk(p, fsite, fatt);
     }
   }
@@ -1260,7 +1168,6 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
     // ------------------------------ workers ------------------------------
     const int wt = threadIdx.x - 128, ww = wt >> 5;
     int nbar = 0, gseq = 0, seg = 0, it = 0;
-    int a5_tiles = 0;
     bool alive = true;
     if (p.do_embed) {
       mega_embed(ctl, p, args, kv, w, dm, wt);
@@ -1290,16 +1197,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
                                      : nullptr;
         AttRing rg{ctl->full, ctl->empty, ctl->cons_cnt, ring, p.stage_bytes, NS, &ctl->abort_flag, p.abort_g, w.status, ev};
         AttArgs aa{w.Qb, l < p.att_precise_layers ? w.Qlo : nullptr, w.KVn, AttPartials{w.tc_m, w.tc_l, w.tc_o}, p.n_tail_base, l, B};
-        if constexpr (A5) {
-          // all eight warps: lane quarter ww & 3, query group ww >> 2; then the causal tails, dealt over all blocks' warps
-          // from the last block down
-          A5Pos ap{it % NS, it / NS};
-          alive = a5_softmax<true, 4>(a5r, ap, &ctl->a5, &ctl->a5s, ctl->tmem_base, q_area, nullptr, aa, pl, B, dm.Hkv, g.nq, t_lo, t_hi, a5_tiles, c,
-                                      ww & 3, ww >> 2, 2 + (ww >> 2), lane, ev);
-          AttWarp<HD, 2> st;
-#pragma unroll 1
-          for (int q = (G - 1 - c) * 8 + ww; q < B * dm.Hkv * g.MT; q += G * 8) att_tail_task<HD, 2>(st, g, aa, q / g.MT, (q % g.MT) * 16, lane);
-        } else {
+        {
           int it2 = it;
           att_consume_dispatch<HD>(rg, it2, pl, g, aa, dm.Hkv, c, G, ww, lane);
         }
@@ -1311,7 +1209,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         const int items = B * dm.Hkv * g.nq * AttCombineSplit<HD>::value;
 #pragma unroll 1
         for (int item = ww * G + c; item < items; item += G * 8)   // spread over blocks first
-          att_combine_item<bf16, HD, A5 ? 8 : 0>(P, pl, g, G, p.n_tail_base, dm.Hkv, item, w.ATT, R, dm.Hq, lane,
+          att_combine_item<bf16, HD, 0>(P, pl, g, G, p.n_tail_base, dm.Hkv, item, w.ATT, R, dm.Hq, lane,
                                      (kTr && p.trace && c == 0 && ww == 0 && (l - p.l0) * 4 < kMegaTraceSites)
                                          ? p.trace + 2 * kMegaTraceBarriers + 8 * kMegaTraceSites + (size_t)(l - p.l0) * 4 * 8 + 4
                                          : nullptr);
@@ -1330,13 +1228,11 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
 }
 
 typedef void (*MegaKernel)(const MegaMaps, const MegaParams, const StepArgs*, const KvView, const Work, const Dims);
-// The kernel's instantiations by head dimension, attention phase and timeline code, each in a translation unit of
+// The kernel's instantiations by head dimension and timeline code, each in a translation unit of
 // its own (sj_mega_inst.cu) so that they compile side by side; ns: row slots (4, 6 or 8).
 MegaKernel mega_kernel_64(int ns);
 MegaKernel mega_kernel_64_trace(int ns);
 MegaKernel mega_kernel_128(int ns);
 MegaKernel mega_kernel_128_trace(int ns);
-MegaKernel mega_kernel_128_t5(int ns);
-MegaKernel mega_kernel_128_t5_trace(int ns);
 
 }  // namespace sj

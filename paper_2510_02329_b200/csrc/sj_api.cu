@@ -228,6 +228,7 @@ struct sj_target {
   int att_rows_cap = 0;
   size_t tc_part_cap = 0;   // floats in tc_m / tc_l
   size_t logits_rows = 0;
+  int pair_clusters[kPairMaxSplit + 1] = {};
   std::map<StepKey, cudaGraphExec_t> graphs;
   std::map<std::pair<const void*, int>, CUtensorMap> act_maps;   // per activation matrix and row count
   std::map<std::tuple<const void*, int, int>, CUtensorMap> pair_maps;   // the same per box height, for the paired projections
@@ -487,6 +488,23 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
     for (int site = PAIR_QKV; site <= PAIR_LM && e == cudaSuccess; ++site)
       e = cudaFuncSetAttribute(pair_kernel(site, c.head_dim), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) { fail(SJ_ERR_CUDA, "smem opt-in: %s", cudaGetErrorString(e)); return bail(SJ_ERR_CUDA); }
+    // clusters of S pairs, one CTA per SM, that are resident at once (all of a site's kernels take most of an SM)
+    t->pair_clusters[1] = t->sm_count / 2;
+    for (int S = 2; tc && S <= kPairMaxSplit; ++S) {
+      cudaLaunchConfig_t cfg;
+      memset(&cfg, 0, sizeof(cfg));
+      cfg.gridDim = dim3(2 * S);
+      cfg.blockDim = dim3(kPairThreads);
+      cfg.dynamicSmemBytes = 200 * 1024;
+      cudaLaunchAttribute at;
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = 2 * S; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, pair_kernel(PAIR_RES, c.head_dim), &cfg) != cudaSuccess) { n = 0; cudaGetLastError(); }
+      t->pair_clusters[S] = n;
+    }
   }
   if ((st = alloc_partials(t, W, R)) != SJ_OK) return bail(st);
   {
@@ -525,7 +543,7 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
       }
       mm.lm = t->m_lm;
     }
-    t->opt_step = 1;
+    t->opt_step = 2;
   }
 #undef ALLOC
   if (t->bf && c.head_dim == 128) {
@@ -585,8 +603,8 @@ extern "C" sj_status sj_set_option(sj_target* t, const char* name, int value) {
     if (value == 2 && t->dm.hd != 128) return fail(SJ_ERR_UNSUPPORTED, "the tcgen05 attention needs head_dim 128");
     t->opt_attn = value;
   } else if (n == "step_impl") {
-    if (value != 0 && value != 1) return fail(SJ_ERR_INVALID_ARG, "step_impl must be 0 or 1");
-    if (value == 1 && !t->mega_shapes) return fail(SJ_ERR_UNSUPPORTED, "the whole-step kernel needs bf16, 128-multiples and cooperative launch");
+    if (value < 0 || value > 2) return fail(SJ_ERR_INVALID_ARG, "step_impl must be 0, 1 or 2");
+    if (value >= 1 && !t->mega_shapes) return fail(SJ_ERR_UNSUPPORTED, "the whole-step kernel needs bf16, 128-multiples and cooperative launch");
     t->opt_step = value;
   } else if (n == "ring_stages") {
     if (value != 0 && (value < 3 || value > kMegaMaxStages)) return fail(SJ_ERR_INVALID_ARG, "ring_stages must be 0 (auto) or 3..%d", kMegaMaxStages);
@@ -934,23 +952,35 @@ static cudaError_t launch_tc(sj_target* t, const TcSite& s, const CUtensorMap* m
                 *(w2 ? w2 : w0), p, (const StepArgs*)t->d_args, W, t->dm.V);
 }
 
-// Paired projections (sj_gemm_pair.cuh): geometry of a site of n_tiles 128-feature tiles for R rows.
-struct PairGeom { int rb, n_rb, stages, stage_bytes; uint32_t tmem_cols; size_t smem; };
-static PairGeom pair_geom(int R, int n_tiles, int n_pairs, int site) {
+// Paired projections (sj_gemm_pair.cuh): geometry of a site of n_tiles 128-feature tiles and KB K blocks for R rows.
+// clusters[S]: clusters of S pairs that fit on the device.
+struct PairGeom { int rb, n_rb, n_split, n_groups, xch_js, stages, stage_bytes; uint32_t tmem_cols; size_t smem; };
+static PairGeom pair_geom(int R, int n_tiles, int KB, const int* clusters, int site) {
   PairGeom g;
   memset(&g, 0, sizeof(g));
-  // rows per block: fewest rounds of items times the clocks a K step takes (shared-memory port, tensor pipe)
-  long best = 0;
-  for (int n_rb = (R + 127) / 128; n_rb <= (R + 15) / 16; ++n_rb) {
-    const int rb = round_up((R + n_rb - 1) / n_rb, 16), n = (R + rb - 1) / rb;
-    const long rounds = ((n_tiles + 1) / 2 * n + n_pairs - 1) / n_pairs, cost = rounds * std::max(256 + 2 * rb, 4 * rb);
-    if (!best || cost < best) { best = cost; g.rb = rb; g.n_rb = n; }
+  // Rows per block and pairs per item: the fewest clocks, rounds of items times the K steps of one at a step's clocks
+  // (shared-memory port, tensor pipe) and its epilogue -- the exchange of a split item costs about as much again -- but
+  // no less than the weights take from HBM.
+  const int tiles2 = (n_tiles + 1) / 2;
+  const double hbm = 32768.0 * tiles2 * KB / kPairHbmBytesPerClk;
+  double best = 0;
+  for (int S = 1; S <= kPairMaxSplit; ++S) {
+    if (clusters[S] <= 0 || (S > 1 && KB < 8 * S)) continue;
+    for (int n_rb = (R + 127) / 128; n_rb <= (R + 15) / 16; ++n_rb) {
+      const int rb = round_up((R + n_rb - 1) / n_rb, 16), n = (R + rb - 1) / rb;
+      const int rounds = (tiles2 * n + clusters[S] - 1) / clusters[S], steps = (KB + S - 1) / S;
+      const double cost = std::max((double)rounds * (steps * std::max(256 + 2 * rb, 4 * rb) + (S > 1 ? kPairXchClk : 0)), hbm + (S > 1 ? kPairXchClk : 0));
+      if (best == 0 || cost < best) { best = cost; g.rb = rb; g.n_rb = n; g.n_split = S; }
+    }
   }
+  g.n_groups = std::min(clusters[g.n_split], tiles2 * g.n_rb);
   g.tmem_cols = 32;
   while (g.tmem_cols < (uint32_t)(4 * g.rb)) g.tmem_cols <<= 1;
   g.stage_bytes = kWTileBytes + g.rb * 128;
-  const size_t ctl = site == PAIR_QKV ? sizeof(PairSmem<PAIR_QKV>) : site == PAIR_RES ? sizeof(PairSmem<PAIR_RES>)
-                     : site == PAIR_GU ? sizeof(PairSmem<PAIR_GU>) : sizeof(PairSmem<PAIR_LM>);
+  g.xch_js = ((g.rb + 31) / 32 + g.n_split - 1) / g.n_split;
+  const size_t ctl = (site == PAIR_QKV ? sizeof(PairSmem<PAIR_QKV>) : site == PAIR_RES ? sizeof(PairSmem<PAIR_RES>)
+                      : site == PAIR_GU ? sizeof(PairSmem<PAIR_GU>) : sizeof(PairSmem<PAIR_LM>)) +
+                     (size_t)(g.n_split - 1) * 2 * g.xch_js * 8192;
   g.stages = std::min<int>(kPairMaxStages, (int)((227 * 1024 - 1024 - ctl) / g.stage_bytes));
   g.smem = (size_t)g.stages * g.stage_bytes + ctl + 1024;
   return g;
@@ -981,28 +1011,27 @@ struct PairOut {   // what a site's epilogue needs beyond the step's workspace
 static sj_status launch_pair(sj_target* t, sj_kv* kv, int site, int n_tiles, int K, const void* act, const CUtensorMap* w0, const CUtensorMap* w1,
                              const CUtensorMap* w2, int R, bool pdl, const Work& W, const PairOut& o) {
   const Dims& dm = t->dm;
-  const int n_pairs = t->sm_count / 2;
-  const PairGeom g = pair_geom(R, n_tiles, n_pairs, site);
+  const PairGeom g = pair_geom(R, n_tiles, K / kBK, t->pair_clusters, site);
   const CUtensorMap* mA = nullptr;
   sj_status st = pair_map(t, act, R, g.rb, K, &mA);
   if (st != SJ_OK) return st;
   PairParams p;
   memset(&p, 0, sizeof(p));
   p.n_tiles = n_tiles; p.KB = K / kBK; p.R = R; p.rb = g.rb; p.n_rb = g.n_rb; p.plane_rows = pad16(R);
-  p.n_pairs = std::min(n_pairs, (n_tiles + 1) / 2 * g.n_rb);
+  p.n_groups = g.n_groups; p.n_split = g.n_split; p.xch_js = g.xch_js;
   p.stages = g.stages; p.stage_bytes = g.stage_bytes; p.tmem_cols = g.tmem_cols;
   p.tile_q = dm.Hq * dm.hd / kTileN; p.tile_k = p.tile_q + dm.Hkv * dm.hd / kTileN;
   p.ssq_in = o.ssq_in; p.ssq_out = o.ssq_out; p.gain = (const bf16*)o.gain; p.planes_out = o.planes_out; p.K_out = o.K_out; p.layer = o.layer;
   p.bq = (const bf16*)o.bq; p.bk = (const bf16*)o.bk; p.bv = (const bf16*)o.bv;
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3(2 * p.n_pairs);
+  cfg.gridDim = dim3(2 * g.n_split * g.n_groups);
   cfg.blockDim = dim3(kPairThreads);
   cfg.dynamicSmemBytes = g.smem;
   cfg.stream = t->stream;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[0].val.clusterDim.x = 2 * g.n_split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
@@ -1012,11 +1041,8 @@ static sj_status launch_pair(sj_target* t, sj_kv* kv, int site, int n_tiles, int
   return SJ_OK;
 }
 
-// The per-stage path runs the projections of wider steps on pairs of SMs (below, the pairs' tiles of 256 features leave most
-// of them without work).
-constexpr int kPairMinRows = 33;
-static bool pair_usable(const sj_target* t, const sj_kv* kv, int R) {
-  return t->opt_gemm == 1 && t->opt_attn >= 1 && t->bf && kv->has_tm_pool && R >= kPairMinRows;
+static bool pair_usable(const sj_target* t, const sj_kv* kv) {
+  return t->opt_gemm == 1 && t->opt_attn >= 1 && t->bf && kv->has_tm_pool;
 }
 
 // a14 in sampling mode with the tensor-core LM head: re-normalise the one row per sequence that the emitted
@@ -1102,7 +1128,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
     if ((st = activation_map(t, W.ATT, R, qd, &mA_q)) != SJ_OK) return st;
     if ((st = activation_map(t, W.H, R, dm.F, &mA_f)) != SJ_OK) return st;
   }
-  const bool pair = pair_usable(t, kv, R);
+  const bool pair = pair_usable(t, kv);
   const size_t ssq_n = (size_t)(dm.d / kTileN) * R;
   auto plan_of = [&](const TcSite& site) { return tc ? SplitPlan{site.d_tile_slots, site.n_tiles} : one; };
 
@@ -1220,7 +1246,7 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
   const int n_vtiles = (dm.V + kTileN - 1) / kTileN;
   if (tc) {
     TIMED("target_logits", launch(k_target_logits, dim3((R + 7) / 8), dim3(256), 0, s, pdl, args, W, dm, (const bf16*)t->lm_head, R));
-    if (pair_usable(t, kv, R))
+    if (pair_usable(t, kv))
       TIMED_ST("gemm_lm_head", launch_pair(t, kv, PAIR_LM, n_vtiles, dm.d, W.A, &t->m_lm, nullptr, nullptr, R, pdl, W, PairOut()));
     else
       TIMED("gemm_lm_head", launch_tc(t, t->s_lm, mA_d, &t->m_lm, nullptr, nullptr, R, pdl, true, W));   // W: no [R, V] logit store
@@ -1246,15 +1272,21 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
 #undef TIMED_BEGIN
 #undef TIMED_END
 
-// The whole step as one cooperative launch per chunk of kMegaMaxLayers layers, up to kMegaMaxRows rows.  From kPairMinRows
-// rows on and with caches of several 128-key tiles per SM the attention decides: the persistent kernel's mma.sync phase
-// takes about three times as long a key as the tcgen05 kernel (8B-shaped, 16 layers, 4 x 9 rows: 4 x 4000 keys 3062 us
-// against 2681 per stage, 4 x 300 keys 2429 against 2518).
+// The whole step as one cooperative launch per chunk of kMegaMaxLayers layers.  "step_impl" 1 takes it up to kMegaMaxRows
+// rows; the default (2) where it is the faster of the two (B200, us a step, persistent / per stage):
+//   rows: its barriers cost less than launches, the paired projections are the better GEMM.  16 layers, 8B-shaped: 9 rows
+//     1927 / 2099, 18 rows 2200 / 2143, 27 rows 2270 / 2135; 1B-shaped: 18 rows 1228 / 1270, 24 rows 1308 / 1302, 36 rows
+//     1487 / 1384; 32B-shaped: 9 rows 3275 / 3434, 18 rows 3671 / 3519, 72 rows 6735 / 4871;
+//   layers: it has a fixed cost of tens of us (its 300 KB of code come from memory once a step).  2 layers of small
+//     widths: 148 / 120.
+// Caches of several 128-key tiles per SM (and head dimension 128): its mma.sync attention takes about three times as long a
+// key as the tcgen05 kernel (8B-shaped, 9 rows: 8000 keys, 3.4 tiles, 2156 / 2159).
 static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma, long total_keys) {
   const int rows = gamma + 1, R = B * rows, group = t->dm.Hq / t->dm.Hkv;
-  if (R >= kPairMinRows && t->dm.hd == 128 && t->opt_attn == 2 && total_keys * t->dm.Hkv / kT5Keys / t->sm_count >= t->opt_a5_min_tiles) return false;
-  return t->opt_step == 1 && t->opt_gemm == 1 && t->mega_shapes && kv->has_tm_pool && R <= kMegaMaxRows &&
-         group * rows <= 16 * 6 && t->stream != nullptr;
+  if (t->opt_step == 0 || t->opt_gemm != 1 || !t->mega_shapes || !kv->has_tm_pool || R > kMegaMaxRows || group * rows > 16 * 6 || !t->stream)
+    return false;
+  if (t->dm.hd == 128 && t->opt_attn == 2 && total_keys * t->dm.Hkv / kT5Keys / t->sm_count >= t->opt_a5_min_tiles) return false;
+  return t->opt_step == 1 || t->opt_attn == 0 || (R <= kMegaAutoRows && t->dm.n_layers >= kMegaAutoLayers);
 }
 
 static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode, bool use_scratch) {
@@ -1658,7 +1690,6 @@ extern "C" sj_status sj_semantic_score(sj_target* t, sj_kv* kv, int seq, int y_i
 // 1000 tokens and a step: 190 ms in blocks of 24 rows, 34 ms in two of 504).  Only the last token's row meets the
 // LM head, and a block that is not the last one ends with its key / value rows.
 constexpr int kPrefillRows = SJ_MAX_ROWS;   // rows of a wide block
-constexpr int kPrefillWideMin = kPairMinRows;   // shorter prompts: one or two narrow blocks through the whole-step kernel
 
 static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* tokens, int n_tokens, int c, int* d_next, bool* done) {
   const Dims& dm = t->dm;
@@ -1747,7 +1778,7 @@ extern "C" sj_status sj_prefill(sj_target* t, sj_kv* kv, int seq, const int* tok
   o.judge_scores = reinterpret_cast<float*>(t->d_prefill + 3 * (SJ_MAX_GAMMA + 1));
   o.p_draft = reinterpret_cast<float*>(t->d_prefill + 5 * (SJ_MAX_GAMMA + 1));
   bool done = false;
-  if (n_tokens >= kPrefillWideMin && t->bf && t->opt_gemm == 1 && t->opt_attn >= 1 && kv->has_tm_pool) {
+  if (n_tokens > c_max && pair_usable(t, kv)) {   // else one narrow block
     sj_status st = prefill_wide(t, kv, seq, tokens, n_tokens, c_max, o.next_token, &done);
     if (st != SJ_OK) return st;
   }

@@ -1,4 +1,4 @@
-// Projections of wide steps (more block rows than the persistent kernel takes) on pairs of SMs, with fused epilogues.
+// Projections of the per-stage step on pairs of SMs, with fused epilogues.
 //
 //   D[256 features, rb rows] (fp32, tensor memory) = W_tile[256, K] (bf16) x A[rb, K]^T (two bf16 planes)
 // A pair of CTAs (tcgen05 cta_group::2) computes one 256-feature tile for a block of rb <= 128 rows over the whole of K:
@@ -18,8 +18,15 @@
 // run side by side) but no exchange of sums: a first version of this kernel that split K over the pairs was bound by
 // the pair that finished a tile for all of them.
 //
-// Items (tile, row block), row blocks fastest, are dealt round robin: pair g takes items g, g + n_pairs, ...  The host
-// picks rb by the model above (pair_geom): fewest rounds times clocks per round.
+// Where the items (tile, row block) leave pairs idle (down has 16 to 20 tiles of 256 features), a cluster of n_split <= 4
+// pairs shares an item's K.  Every pair sends its sums of the rows that another one finishes into that one's shared
+// memory and finishes its own: chunk j (32 rows) belongs to split j % n_split, so all of them work on the epilogue and
+// no sum crosses L2.  A cluster is scheduled as a whole, so its pairs can wait for one another.
+// Down at 72 rows (20 tiles, K 27648, 283 MB): 94.5 us with row blocks of 32 on 60 pairs, 60.4 as 80 rows on 40 pairs;
+// steps (B200): 32B-shaped 72 rows 5434 -> 4871 us, 8B-shaped 44 rows 5150 -> 4440, 1B-shaped 48 rows 1610 -> 1447.
+//
+// Items, row blocks fastest, are dealt round robin: cluster g takes items g, g + n_groups, ...  The host picks rb and
+// n_split by the model above (pair_geom).
 //
 // Epilogues (template SITE) -- the same arithmetic as the persistent kernel's: the planes hold x * gain and the row scalar
 // 1/rms, from per-tile sums of squares, is applied by the consumer.
@@ -39,6 +46,9 @@ constexpr int kPairWorkers = 256;
 constexpr int kPairMaxStages = 10;
 constexpr int kPairMaxRows = kMaxRows;
 constexpr int kPairSegKB = 16;          // K blocks of 64 per accumulation chain
+constexpr int kPairMaxSplit = 4;        // pairs that share an item's K (a cluster of 8)
+constexpr double kPairHbmBytesPerClk = 3600;   // HBM against the SM clock, for the host's choice of a geometry
+constexpr int kPairXchClk = 3000;       // an exchange between the splits
 constexpr uint32_t kPairSpin = 1u << 22;
 
 enum PairSite { PAIR_QKV = 0, PAIR_RES = 1, PAIR_GU = 2, PAIR_LM = 3 };
@@ -46,7 +56,9 @@ enum PairSite { PAIR_QKV = 0, PAIR_RES = 1, PAIR_GU = 2, PAIR_LM = 3 };
 struct PairParams {
   int n_tiles;            // 128-feature tiles (gate/up: 64 + 64); an odd last one is paired with zeros
   int KB;                 // K blocks of 64
-  int n_pairs;
+  int n_groups;           // clusters
+  int n_split;            // pairs of a cluster: they share an item's K blocks
+  int xch_js;             // 32-row chunks of a row block that one split finishes, at most
   int R, rb, n_rb;        // rows, rows per block (a multiple of 16, at most 128: an M = 256 MMA takes N = 32, 64 .. 256), row blocks
   int plane_rows;         // row of the lo plane in the activation matrix
   int stages, stage_bytes;
@@ -63,6 +75,7 @@ struct PairParams {
 
 struct PairCtl {
   uint64_t full[kPairMaxStages], empty[kPairMaxStages], tmem_full[2], tmem_empty[2];
+  uint64_t xch_full[2], xch_free[2];   // per epilogue group: the other splits' sums are here; the others have read mine
   uint32_t tmem_base;
   int abort_flag;
   float inv[kPairMaxRows];
@@ -104,9 +117,9 @@ __device__ __forceinline__ void pair_tma_2d(uint32_t dst, const CUtensorMap* tm,
       "l"(reinterpret_cast<uint64_t>(tm)), "r"(bar & kPeerMask), "r"(c0), "r"(c1), "l"(policy)
       : "memory");
 }
-__device__ __forceinline__ void pair_commit(uint32_t bar) {   // arrives on `bar` of both CTAs
+__device__ __forceinline__ void pair_commit(uint32_t bar, uint32_t mask) {   // arrives on `bar` of both CTAs of the pair (mask)
   asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((uint16_t)3)
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((uint16_t)mask)
       : "memory");
 }
 __device__ __forceinline__ void pair_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
@@ -117,10 +130,27 @@ __device__ __forceinline__ void pair_mma(uint32_t d_tmem, uint64_t a_desc, uint6
       "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-__device__ __forceinline__ void pair_arrive_rank0(uint32_t bar) {
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, int cta) {   // the same shared-memory address in CTA `cta` of the cluster
   uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(bar));
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(cta));
+  return remote;
+}
+__device__ __forceinline__ void cluster_arrive(uint32_t bar, int cta) {   // releases this warp's earlier writes to that CTA
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr(bar, cta)) : "memory");
+}
+__device__ __forceinline__ bool cluster_try_wait(uint32_t bar, uint32_t parity) {   // acquires what other CTAs of the cluster released
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ void cluster_st4(uint32_t remote, const float* v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(remote), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
 }
 __device__ __forceinline__ uint32_t instr_desc_pair(int n) {   // M = 256
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
@@ -133,10 +163,14 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const Dims dm) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  PairSmem<SITE>* sm = reinterpret_cast<PairSmem<SITE>*>(smem + (size_t)p.stages * p.stage_bytes);
+  // ring | the other splits' sums [n_split - 1][2 groups][xch_js][4][128 features] of 4 rows each | control
+  float4* xch = reinterpret_cast<float4*>(smem + (size_t)p.stages * p.stage_bytes);
+  PairSmem<SITE>* sm = reinterpret_cast<PairSmem<SITE>*>(xch + (size_t)(p.n_split - 1) * 2 * p.xch_js * 512);
   PairCtl* ctl = &sm->c;
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  const int rank = (int)cluster_rank(), g = blockIdx.x >> 1;
+  const int S = p.n_split, crank = (int)cluster_rank(), rank = crank & 1, split = crank >> 1, g = blockIdx.x / (2 * S);
+  const int kb_lo = p.KB * split / S, kb_hi = p.KB * (split + 1) / S;   // this pair's K blocks
+  const uint32_t pair_mask = 3u << (crank & ~1);
   volatile int* abort_flag = &ctl->abort_flag;
   const int n_items = (p.n_tiles + 1) / 2 * p.n_rb;
 
@@ -148,6 +182,8 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&ctl->tmem_full[i]), 1);
       mbar_init(smem_u32(&ctl->tmem_empty[i]), 16);   // the epilogue warps of both CTAs
+      mbar_init(smem_u32(&ctl->xch_full[i]), 4 * max(S - 1, 1));   // a group's warps of every other split
+      mbar_init(smem_u32(&ctl->xch_free[i]), 4 * max(S - 1, 1));
     }
     ctl->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -186,14 +222,14 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       };
       // the first ring-full of weights before the programmatic wait: they do not depend on the previous kernel
       int pre = 0;
-      for (int item = g; item < n_items && pre < p.stages; item += p.n_pairs)
-        for (int kb = 0; kb < p.KB && pre < p.stages; ++kb) w_load(pre++, item / p.n_rb, kb);
+      for (int item = g; item < n_items && pre < p.stages; item += p.n_groups)
+        for (int kb = kb_lo; kb < kb_hi && pre < p.stages; ++kb) w_load(pre++, item / p.n_rb, kb);
       pdl_wait();
       int s = 0, r = 0;
       bool alive = true;
-      for (int item = g; item < n_items && alive; item += p.n_pairs) {
+      for (int item = g; item < n_items && alive; item += p.n_groups) {
         const int tile2 = item / p.n_rb, row = rank * p.plane_rows + (item % p.n_rb) * p.rb;
-        for (int kb = 0; kb < p.KB; ++kb) {
+        for (int kb = kb_lo; kb < kb_hi; ++kb) {
           if (r > 0) {
             if (!mbar_wait(smem_u32(&ctl->empty[s]), (uint32_t)(r - 1) & 1u, abort_flag, w.status, kPairSpin)) { alive = false; break; }
             w_load(s, tile2, kb);
@@ -212,11 +248,11 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       const uint32_t idesc = instr_desc_pair(2 * p.rb);
       int s = 0, r = 0, n = 0;
       bool alive = true;
-      for (int item = g; item < n_items && alive; item += p.n_pairs) {
+      for (int item = g; item < n_items && alive; item += p.n_groups) {
         uint32_t dcol = 0;
         int acc = 0;
-        for (int kb = 0; kb < p.KB; ++kb) {
-          const bool first = kb % kPairSegKB == 0;
+        for (int kb = kb_lo; kb < kb_hi; ++kb) {
+          const bool first = (kb - kb_lo) % kPairSegKB == 0;
           if (first) {
             acc = n & 1;
             const int use = n >> 1;
@@ -230,9 +266,9 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           const uint64_t dw = smem_desc_sw128(wa), da = smem_desc_sw128(wa + kWTileBytes);
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k) pair_mma(dcol, dw + 2 * k, da + 2 * k, idesc, (!first || k > 0) ? 1u : 0u);
-          pair_commit(smem_u32(&ctl->empty[s]));
+          pair_commit(smem_u32(&ctl->empty[s]), pair_mask);
           if (++s == p.stages) { s = 0; ++r; }
-          if (kb % kPairSegKB == kPairSegKB - 1 || kb == p.KB - 1) pair_commit(smem_u32(&ctl->tmem_full[acc]));
+          if ((kb - kb_lo) % kPairSegKB == kPairSegKB - 1 || kb == kb_hi - 1) pair_commit(smem_u32(&ctl->tmem_full[acc]), pair_mask);
         }
       }
     }
@@ -273,9 +309,11 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       }
     }
     all_sync();
-    const int n_seg = (p.KB + kPairSegKB - 1) / kPairSegKB;
-    int n = 0;
-    for (int item = g; item < n_items; item += p.n_pairs) {
+    const int n_seg = (kb_hi - kb_lo + kPairSegKB - 1) / kPairSegKB;
+    int n = 0, n_x = 0;   // segments, exchanges so far
+    uint32_t mine = 0;    // the chunks j that this split finishes
+    for (int j = split; j < 4; j += S) mine |= 1u << j;
+    for (int item = g; item < n_items; item += p.n_groups) {
       const int tile = 2 * (item / p.n_rb) + rank, r_lo = item % p.n_rb * p.rb, r_hi = min(r_lo + p.rb, R);
       const bool real = tile < p.n_tiles;   // an odd last tile's partner has no features
       // the segments' sums: chunk j of this group in registers
@@ -306,7 +344,45 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) pair_arrive_rank0(smem_u32(&ctl->tmem_empty[acc]));
+        if (lane == 0) cluster_arrive(smem_u32(&ctl->tmem_empty[acc]), crank & ~1);
+      }
+      if (S > 1) {   // send the sums that others finish, add theirs to mine
+        auto xch_wait = [&](uint64_t* bar, uint32_t parity) {
+          if (fl == 0) mbar_wait(smem_u32(bar), parity, abort_flag, w.status, kPairSpin);
+          group_sync();
+          cluster_try_wait(smem_u32(bar), parity);   // every thread acquires the completed phase
+        };
+        if (n_x > 0) xch_wait(&ctl->xch_free[grp], (uint32_t)(n_x - 1) & 1u);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (!(mine >> j & 1u) && r_lo + 16 * grp + 32 * j < r_hi) {
+            const int f = j % S, slot = split < f ? split : split - 1;
+            const uint32_t dst = cluster_addr(smem_u32(xch + ((size_t)(slot * 2 + grp) * p.xch_js + j / S) * 512 + fl), 2 * f + rank);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) cluster_st4(dst + (uint32_t)q * 2048u, &sum[j][4 * q]);
+          }
+        __syncwarp();
+        if (lane == 0)
+          for (int f = 0; f < S; ++f)
+            if (f != split) cluster_arrive(smem_u32(&ctl->xch_full[grp]), 2 * f + rank);
+        xch_wait(&ctl->xch_full[grp], (uint32_t)n_x & 1u);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if ((mine >> j & 1u) && r_lo + 16 * grp + 32 * j < r_hi) {
+            for (int slot = 0; slot < S - 1; ++slot) {
+              const float4* src = xch + ((size_t)(slot * 2 + grp) * p.xch_js + j / S) * 512 + fl;
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const float4 x = src[q * 128];
+                sum[j][4 * q] += x.x; sum[j][4 * q + 1] += x.y; sum[j][4 * q + 2] += x.z; sum[j][4 * q + 3] += x.w;
+              }
+            }
+          }
+        __syncwarp();
+        if (lane == 0)
+          for (int f = 0; f < S; ++f)
+            if (f != split) cluster_arrive(smem_u32(&ctl->xch_free[grp]), 2 * f + rank);
+        ++n_x;
       }
 
       // per-feature constants
@@ -327,6 +403,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       for (int j = 0; j < 4; ++j) {
         const int c0 = r_lo + 16 * grp + 32 * j, nr = min(16, r_hi - c0);
         if (nr <= 0 || !real) break;   // uniform over the group
+        if (!(mine >> j & 1u)) continue;
         float (&v)[16] = sum[j];
         float xs[16];
         if constexpr (SITE == PAIR_RES) {   // residual rows, requested before the accumulator is waited for
@@ -462,7 +539,8 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         all_sync();
         if (real)
           for (int r = r_lo + wt; r < r_hi; r += kPairWorkers)
-            p.ssq_out[(size_t)tile * R + r] = (sm->x.sums[0][r] + sm->x.sums[1][r]) + (sm->x.sums[2][r] + sm->x.sums[3][r]);
+            if (mine >> ((r - r_lo) >> 5) & 1u)
+              p.ssq_out[(size_t)tile * R + r] = (sm->x.sums[0][r] + sm->x.sums[1][r]) + (sm->x.sums[2][r] + sm->x.sums[3][r]);
         all_sync();
       }
     }

@@ -29,10 +29,8 @@
 // Attention: its cache tiles travel through the same ring and are consumed by fp16 mma.sync in the worker warps
 // (sj_attn_tc.cuh).
 //
-// Up to kMegaMaxRows = 48 block rows.  Beyond that the step is no longer bound by the chain of its phases, and one kernel
-// per stage with the paired projections and the tcgen05 attention is faster (B200, us a step, persistent against per
-// stage: 32B-shaped 16 layers, 72 rows, 8 x 8192 keys 6735 / 5744; 8B-shaped 16 layers, 54 rows, 6 x 4000 keys 3643 / 2860;
-// 1B-shaped, 72 rows 2057 / 1713, 48 rows 1605 / 1608, 9 rows 1107 / 1823).
+// Up to kMegaMaxRows = 48 block rows; which steps it runs by default, and what it measured against one kernel per stage,
+// stands at mega_usable() in sj_api.cu.
 //
 // Every wait is bounded; the first one to run out raises a device-wide abort word that all other waits
 // poll, so that a logic error ends the kernel with SJ_ERR_TIMEOUT instead of hanging the GPU.
@@ -47,6 +45,7 @@ constexpr int kMegaThreads = 384;
 constexpr int kMegaWorkers = 256;
 constexpr int kMegaMaxLayers = 32;   // per launch (tensor maps travel as kernel parameters)
 constexpr int kMegaMaxRows = 48;
+constexpr int kMegaAutoRows = 24, kMegaAutoLayers = 5;   // by default: at most that many rows, at least that many layers
 constexpr int kMegaMaxStages = 12;
 constexpr uint32_t kMegaSpin = 1u << 22;
 constexpr int kMegaRegsLight = 80;    // registers per thread of warps 0..3 after reallocation

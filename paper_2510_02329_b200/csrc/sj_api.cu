@@ -338,7 +338,14 @@ static sj_status alloc_rows(sj_target* t, Work& W, int R) {
   act(&W.A, d);
   act(&W.ATT, qd);
   act(&W.H, c.d_ffn);
-  act(&W.Asel, d);   // at most one row per sequence is used
+  {   // one row (two planes of 16)
+    uint8_t* q = nullptr;
+    if (get(&q, 32 * d * esz)) {
+      W.Asel = q;
+      if (cudaMemset(q, 0, 32 * d * esz) != cudaSuccess) st = fail(SJ_ERR_CUDA, "workspace clear failed");
+    }
+  }
+  get(&W.rs_part, (size_t)std::min<int>(R, SJ_MAX_BATCH) * ((c.vocab + kResampleChunk - 1) / kResampleChunk));
   get(&W.Q, R * qd);
   if (t->bf) {
     get(&W.Qb, R * qd);
@@ -934,8 +941,7 @@ static sj_status activation_map(sj_target* t, const void* base, int R, int K, co
 }
 
 static cudaError_t launch_tc(sj_target* t, const TcSite& s, const CUtensorMap* mA, const CUtensorMap* w0,
-                             const CUtensorMap* w1, const CUtensorMap* w2, int R, bool pdl, bool planes, const Work& W,
-                             int lm_mode = -1) {
+                             const CUtensorMap* w1, const CUtensorMap* w2, int R, bool pdl, bool planes, const Work& W) {
   RowGeom g = feed_geom(R, planes);
   TcGemmParams p;
   memset(&p, 0, sizeof(p));
@@ -947,7 +953,7 @@ static cudaError_t launch_tc(sj_target* t, const TcSite& s, const CUtensorMap* m
   p.stages = g.stages; p.a_stage_bytes = g.a_stage_bytes; p.tmem_cols = g.tmem_cols;
   p.acc_bufs = g.acc_bufs; p.acc_stride = g.acc_stride;
   p.P = W.P; p.slot_stride = (size_t)R * s.N; p.tile_slots = s.d_tile_slots;
-  p.lm_mode = lm_mode >= 0 ? lm_mode : (s.lm ? 1 : 0); p.status = W.status;
+  p.lm_mode = s.lm ? 1 : 0; p.status = W.status;
   return launch(k_gemm_tc, dim3(s.G), dim3(kTcThreads), g.smem_bytes, t->stream, pdl, *mA, *w0, *(w1 ? w1 : w0),
                 *(w2 ? w2 : w0), p, (const StepArgs*)t->d_args, W, t->dm.V);
 }
@@ -1045,19 +1051,12 @@ static bool pair_usable(const sj_target* t, const sj_kv* kv) {
   return t->opt_gemm == 1 && t->opt_attn >= 1 && t->bf && kv->has_tm_pool;
 }
 
-// a14 in sampling mode with the tensor-core LM head: re-normalise the one row per sequence that the emitted
-// token is drawn from, run the LM head over those B rows into the [B, V] logit scratch, draw the token.
-template <typename T>
-static sj_status enqueue_resample(sj_target* t, sj_kv* kv, int B, const Work& W, bool pdl) {
+// a14 in sampling mode: draw the emitted token from the stored logits of one row per sequence.
+static sj_status enqueue_resample(sj_target* t, sj_kv* kv, int B, bool pdl_first, bool pdl) {
   const Dims& dm = t->dm;
-  cudaStream_t s = t->stream;
-  const CUtensorMap* mA = nullptr;
-  sj_status st = activation_map(t, W.Asel, B, dm.d, &mA);
-  if (st != SJ_OK) return st;
-  CU_TRY(launch(k_select_rows<T>, dim3(B), dim3(256), sizeof(float) * dm.d, s, pdl, (const StepArgs*)t->d_args, W, dm,
-                (const T*)t->final_norm, -1));
-  CU_TRY(launch_tc(t, t->s_lm, mA, &t->m_lm, nullptr, nullptr, B, pdl, true, W, 2));
-  CU_TRY(launch(k_resample, dim3(B), dim3(1024), 0, s, pdl, (const StepArgs*)t->d_args, kv->view, W, dm, 1));
+  const int n_chunks = (dm.V + kResampleChunk - 1) / kResampleChunk;
+  CU_TRY(launch(k_resample_sums, dim3(n_chunks, B), dim3(kResampleThreads), 0, t->stream, pdl_first, (const StepArgs*)t->d_args, t->work, dm));
+  CU_TRY(launch(k_resample_pick, dim3(B), dim3(kResampleThreads), 0, t->stream, pdl, (const StepArgs*)t->d_args, kv->view, t->work, dm, n_chunks));
   return SJ_OK;
 }
 
@@ -1228,7 +1227,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
 }
 
 template <typename T>
-static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mode, int chunk_len, bool use_scratch,
+static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mode, int chunk_len, bool use_logits,
                                size_t n_chunks_hi) {
   const Dims& dm = t->dm;
   const int R = B * (gamma + 1);
@@ -1236,7 +1235,7 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
   const bool pdl = t->opt_pdl != 0 && !timing, tc = t->opt_gemm == 1;
   const StepArgs* args = t->d_args;
   Work W = t->work;
-  if (!use_scratch) W.logits = nullptr;
+  if (!use_logits) W.logits = nullptr;
   cudaStream_t s = t->stream;
   const CUtensorMap* mA_d = nullptr;
   sj_status st = enqueue_layers<T>(t, kv, B, gamma, chunk_len, W, n_chunks_hi, false);
@@ -1256,14 +1255,7 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
     TIMED("lm_stats", launch(k_lm_stats_from_logits, dim3(n_vtiles, (R + 7) / 8), dim3(256), 0, s, pdl, args, W, dm, R));
   }
   TIMED("finalize", launch(k_finalize, dim3(B), dim3(256), 0, s, pdl, args, kv->view, W, dm, n_vtiles, R));
-  if (mode == SJ_MODE_SAMPLING) {
-    if (tc) {
-      sj_status st = enqueue_resample<T>(t, kv, B, t->work, pdl);   // t->work: with the [B, V] logit scratch
-      if (st != SJ_OK) return st;
-    } else {
-      TIMED("resample", launch(k_resample, dim3(B), dim3(1024), 0, s, pdl, args, kv->view, W, dm, 0));
-    }
-  }
+  if (mode == SJ_MODE_SAMPLING) TIMED_ST("resample", enqueue_resample(t, kv, B, pdl, pdl));
   return SJ_OK;
 }
 
@@ -1289,12 +1281,12 @@ static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma, l
   return t->opt_step == 1 || t->opt_attn == 0 || (R <= kMegaAutoRows && t->dm.n_layers >= kMegaAutoLayers);
 }
 
-static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode, bool use_scratch) {
+static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode, bool use_logits) {
   const Dims& dm = t->dm;
   const int rows = gamma + 1, R = B * rows, Rp = pad16(R), qd = dm.Hq * dm.hd;
   cudaStream_t s = t->stream;
   Work W = t->work;
-  if (!use_scratch) W.logits = nullptr;
+  if (!use_logits) W.logits = nullptr;
   const CUtensorMap *mA_d = nullptr, *mA_q = nullptr, *mA_f = nullptr;
   sj_status st;
   if ((st = activation_map(t, W.A, R, dm.d, &mA_d)) != SJ_OK) return st;
@@ -1369,7 +1361,7 @@ static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode
       t->timed.push_back({"verify_step", ea, eb});
     }
   }
-  if (mode == SJ_MODE_SAMPLING) return enqueue_resample<bf16>(t, kv, B, t->work, false);
+  if (mode == SJ_MODE_SAMPLING) return enqueue_resample(t, kv, B, false, t->opt_pdl != 0 && !timing);
   return SJ_OK;
 }
 
@@ -1492,10 +1484,10 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
   for (int i = 0; i < B; ++i) chunk_need_base += (size_t)(kv->len_hi[a->seq_ids[i]] + rows + chunk_len - 1) / chunk_len;
 
   const bool use_mega = mega_usable(t, kv, B, gamma, total_keys);
-  // [R, V] logits exist only for the CUDA-core LM head (fp32 models, cross-checks); the tensor-core paths keep
-  // softmax statistics per vocabulary tile and, in sampling mode, the logits of one row per sequence ([B, V])
-  const bool use_scratch = t->opt_gemm == 0 && !use_mega;
-  const size_t logit_rows_needed = use_scratch ? (size_t)R : (a->mode == SJ_MODE_SAMPLING ? (size_t)B : 0);
+  // [R, V] logits exist for the CUDA-core LM head (fp32 models, cross-checks) and in sampling mode; else the tensor-core
+  // paths keep softmax statistics per vocabulary tile
+  const bool use_logits = (t->opt_gemm == 0 && !use_mega) || a->mode == SJ_MODE_SAMPLING;
+  const size_t logit_rows_needed = use_logits ? (size_t)R : 0;
   // grow lazily-sized buffers (outside any capture)
   const bool simt_attn = t->opt_attn == 0 || !t->bf || !kv->has_tm_pool;
   if (simt_attn && (chunk_need_base > t->att_chunks_cap || rows > t->att_rows_cap)) {
@@ -1552,9 +1544,9 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
   CU_TRY(cudaMemcpyAsync(t->d_args, &h, sizeof(h), cudaMemcpyHostToDevice, t->stream));
 
   // chunk_len shapes only the CUDA-core attention's grid: a growing cache captures no new step elsewhere
-  StepKey key{kv, B, gamma, a->mode, simt_attn ? chunk_len : 0, t->opt_gemm, t->opt_attn, t->opt_pdl, use_scratch ? 1 : 0};
+  StepKey key{kv, B, gamma, a->mode, simt_attn ? chunk_len : 0, t->opt_gemm, t->opt_attn, t->opt_pdl, use_logits ? 1 : 0};
   if (use_mega) {
-    if ((st = launch_mega(t, kv, B, gamma, a->mode, use_scratch)) != SJ_OK) return st;
+    if ((st = launch_mega(t, kv, B, gamma, a->mode, use_logits)) != SJ_OK) return st;
   } else if (t->opt_graph) {
     auto it = t->graphs.find(key);
     if (it == t->graphs.end()) {
@@ -1564,8 +1556,8 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
       }
       cudaGraph_t graph = nullptr;
       CU_TRY(cudaStreamBeginCapture(t->stream, cudaStreamCaptureModeThreadLocal));
-      st = t->bf ? enqueue_step<bf16>(t, kv, B, gamma, a->mode, chunk_len, use_scratch, chunk_need_base)
-                 : enqueue_step<float>(t, kv, B, gamma, a->mode, chunk_len, use_scratch, chunk_need_base);
+      st = t->bf ? enqueue_step<bf16>(t, kv, B, gamma, a->mode, chunk_len, use_logits, chunk_need_base)
+                 : enqueue_step<float>(t, kv, B, gamma, a->mode, chunk_len, use_logits, chunk_need_base);
       cudaError_t e = cudaStreamEndCapture(t->stream, &graph);
       if (st != SJ_OK) {
         if (graph) cudaGraphDestroy(graph);
@@ -1581,8 +1573,8 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
     }
     CU_TRY(cudaGraphLaunch(it->second, t->stream));
   } else {
-    st = t->bf ? enqueue_step<bf16>(t, kv, B, gamma, a->mode, chunk_len, use_scratch, chunk_need_base)
-               : enqueue_step<float>(t, kv, B, gamma, a->mode, chunk_len, use_scratch, chunk_need_base);
+    st = t->bf ? enqueue_step<bf16>(t, kv, B, gamma, a->mode, chunk_len, use_logits, chunk_need_base)
+               : enqueue_step<float>(t, kv, B, gamma, a->mode, chunk_len, use_logits, chunk_need_base);
     if (st != SJ_OK) return st;
   }
   if (a->commit) {
@@ -1743,7 +1735,7 @@ static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* token
     if (last) {
       const CUtensorMap* mA = nullptr;
       if ((st = activation_map(t, W.Asel, 1, dm.d, &mA)) != SJ_OK) return st;
-      CU_TRY(launch(k_select_rows<bf16>, dim3(1), dim3(256), sizeof(float) * dm.d, s, t->opt_pdl != 0, (const StepArgs*)t->d_args, W, dm,
+      CU_TRY(launch(k_select_row<bf16>, dim3(1), dim3(256), sizeof(float) * dm.d, s, t->opt_pdl != 0, W, dm,
                     (const bf16*)t->final_norm, n - 1));
       CU_TRY(launch_tc(t, t->s_lm, mA, &t->m_lm, nullptr, nullptr, 1, t->opt_pdl != 0, true, W));
     }

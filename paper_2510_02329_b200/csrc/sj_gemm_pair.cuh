@@ -490,7 +490,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           const int n_id = tile * kTileN + fl;
           const float invT = args->inv_temperature;
           const bool topk = args->top_k >= 2;
-          float* dbg = args->dbg_logits;
+          float *dbg = args->dbg_logits, *keep = w.logits;   // asked for; sampling mode
           const int own = lane >> 1;   // the chunk's row whose totals this lane ends up with
           int before = 0;
 #pragma unroll
@@ -505,6 +505,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             }
             if (i < nr && n_id < dm.V) {
               if (dbg) dbg[(size_t)r * dm.V + n_id] = v[i];
+              if (keep) keep[(size_t)r * dm.V + n_id] = v[i];
               v[i] *= invT;
               if (n_id == sm->x.tok[r]) w.tgt_logit[r] = v[i];
             } else {

@@ -42,7 +42,8 @@ struct Work {
   RowStat* rowstat;  // [R]   merged statistics
   float* logits;     // fp32 logit scratch, or null: [R, V] for the CUDA-core LM head; [B, V] in sampling mode with
                      // the tensor-core LM head (only the one row per sequence that the emitted token is drawn from)
-  void* Asel;        // GEMM input planes of those B rows (final-norm hidden states), K = d
+void* Asel;        // GEMM input planes of one row (the last of a prefill), K = d
+  double2* rs_part;  // [B][chunks of the vocabulary] sums of p and max(0, p - q) of the row that is drawn from
   const double* inv_freq;  // [hd/2] rope_theta^(-2i/hd)
   const float* judge_w;    // [d]
   int* status;
@@ -686,71 +687,159 @@ static __global__ void k_finalize(const StepArgs* __restrict__ args, KvView kv, 
   }
 }
 
-// a14, sampling mode, first half: the row the emitted token is drawn from (row n_b of sequence b, known only
-// after the first-rejection scan; a given row when row >= 0: prefill) is normalised again into a compact set of GEMM input planes, one row per
-// sequence; a second LM-head pass over those B rows then yields the only logits the step ever stores.
+// One row of the residual stream (the last of a prefill) through the final norm into GEMM input planes of their own.
 template <typename T>
-__global__ void k_select_rows(const StepArgs* __restrict__ args, Work w, Dims dm, const T* __restrict__ gain, int row) {
+__global__ void k_select_row(Work w, Dims dm, const T* __restrict__ gain, int row) {
   extern __shared__ float xs[];
   __shared__ float red[32];
   pdl_wait();
   pdl_launch();
-  const int b = blockIdx.x, rows = args->gamma + 1;
-  const int r = row >= 0 ? row : b * rows + min(max(args->accepted_len[b], 0), rows - 1);
-  for (int i = threadIdx.x; i < dm.d; i += blockDim.x) xs[i] = w.X[(size_t)r * dm.d + i];
+  for (int i = threadIdx.x; i < dm.d; i += blockDim.x) xs[i] = w.X[(size_t)row * dm.d + i];
   __syncthreads();
-  norm_row_from_smem<T>(xs, dm.d, gain, dm.eps, w.Asel, gridDim.x, b, nullptr, nullptr, red);
+  norm_row_from_smem<T>(xs, dm.d, gain, dm.eps, w.Asel, 1, 0, nullptr, nullptr, red);
 }
 
 // a14, sampling mode: inverse CDF over the vocabulary of norm(max(0, p_n - q_{n+1})) (first
 // rejection) or of p_gamma (everything accepted), driven by uniforms[:, gamma].  fp64 prefix sums.
-// per_seq: the logit scratch holds one row per sequence (row b) instead of every block row.
-static __global__ void k_resample(const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, int per_seq) {
+//
+// The LM head's pass has stored the logits of all rows (4 bytes an entry against the 2 d bytes of weights that a second
+// pass over the chosen row would read).  One block of 1024 threads per sequence that walked the row in 1024 contiguous
+// pieces spent its time on a chain of uncoalesced loads and fp64 adds; now chunks of kResampleChunk entries are summed by a
+// block each, and one block per sequence finds the chunk and the entry.  The second pass and the old draw took 350 us of a
+// step of an 8B-shaped target (128256 entries), what is left of both 20 (B200).
+constexpr int kResampleThreads = 256, kResamplePer = 8, kResampleChunk = kResampleThreads * kResamplePer;
+
+struct ResampleRow {
+  const float* lg;   // the row's logits
+  const float* q;    // the draft's probabilities there; null: everything was accepted
+  float invT, m;
+  double inv_s;
+};
+__device__ __forceinline__ ResampleRow resample_row(const StepArgs* args, const Work& w, const Dims& dm, int b) {
+  const int gamma = args->gamma, n = args->accepted_len[b], r = b * (gamma + 1) + n;
+  const RowStat st = w.rowstat[r];
+  return ResampleRow{w.logits + (size_t)r * dm.V, n < gamma ? args->q_full + ((size_t)b * gamma + n) * dm.V : nullptr,
+                     args->inv_temperature, st.m, 1.0 / (double)st.s};
+}
+// This thread's kResamplePer entries of chunk c: p, and max(0, p - q) in `res`; 0 beyond the vocabulary.
+__device__ __forceinline__ void resample_load(const ResampleRow& x, int V, int c, double (&p)[kResamplePer], double (&res)[kResamplePer]) {
+  const int v0 = c * kResampleChunk + (int)threadIdx.x * kResamplePer;
+  float lg[kResamplePer], q[kResamplePer];
+#pragma unroll
+  for (int i = 0; i < kResamplePer; ++i) {
+    lg[i] = __ldcg(x.lg + min(v0 + i, V - 1));
+    q[i] = x.q ? x.q[min(v0 + i, V - 1)] : 0.f;
+  }
+#pragma unroll
+  for (int i = 0; i < kResamplePer; ++i) {
+    p[i] = v0 + i < V ? (double)expf(lg[i] * x.invT - x.m) * x.inv_s : 0.0;
+    res[i] = fmax(0.0, p[i] - (double)q[i]);
+  }
+}
+// Inclusive prefix sum over the block's threads, left in sm[1 ..]; sm[0] = 0.  sm: [kResampleThreads + 1 + 8].
+__device__ __forceinline__ void resample_scan(double v, double* sm) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const double up = __shfl_up_sync(0xffffffffu, v, d);
+    if (lane >= d) v += up;
+  }
+  double* wsum = sm + kResampleThreads + 1;
+  if (lane == 31) wsum[warp] = v;
+  __syncthreads();
+  double before = 0.0;
+  for (int k = 0; k < warp; ++k) before += wsum[k];
+  sm[threadIdx.x + 1] = before + v;
+  if (threadIdx.x == 0) sm[0] = 0.0;
+  __syncthreads();
+}
+
+// grid (chunks, B): the chunk's sums of p and of max(0, p - q)
+static __global__ void k_resample_sums(const StepArgs* __restrict__ args, Work w, Dims dm) {
   pdl_wait();
   pdl_launch();
-  __shared__ double part[1024];
-  __shared__ double total_s;
-  __shared__ int winner;
-  const int b = blockIdx.x, gamma = args->gamma, rows = gamma + 1, tid = threadIdx.x, T = blockDim.x;
-  const int n = args->accepted_len[b];
-  const int r = b * rows + n;
-  const RowStat st = w.rowstat[r];
-  const float invT = args->inv_temperature;
-  const float* lg = w.logits + (size_t)(per_seq ? b : r) * dm.V;
-  const float* q = (n < gamma) ? args->q_full + ((size_t)b * gamma + n) * dm.V : nullptr;
-  const int per = (dm.V + T - 1) / T, v0 = tid * per, v1 = min(v0 + per, dm.V);
-  const double inv_s = 1.0 / (double)st.s;
-  for (int pass = 0; pass < 2; ++pass) {
-    const bool residual = (q != nullptr) && pass == 0;
-    double acc = 0.0;
-    for (int v = v0; v < v1; ++v) {
-      double p = (double)expf(lg[v] * invT - st.m) * inv_s;
-      acc += residual ? fmax(0.0, p - (double)q[v]) : p;
-    }
-    part[tid] = acc;
+  __shared__ double sm[kResampleThreads + 9];
+  const int c = blockIdx.x, b = blockIdx.y;
+  double p[kResamplePer], res[kResamplePer], tp = 0.0, tr = 0.0;
+  resample_load(resample_row(args, w, dm, b), dm.V, c, p, res);
+#pragma unroll
+  for (int i = 0; i < kResamplePer; ++i) { tp += p[i]; tr += res[i]; }
+  double2 out;
+  resample_scan(tp, sm);
+  out.x = sm[kResampleThreads];
+  __syncthreads();
+  resample_scan(tr, sm);
+  out.y = sm[kResampleThreads];
+  if (threadIdx.x == 0) w.rs_part[(size_t)b * gridDim.x + c] = out;
+}
+
+// grid B: the chunk, then the entry, whose prefix sum first exceeds u times the total
+static __global__ void k_resample_pick(const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, int n_chunks) {
+  pdl_wait();
+  pdl_launch();
+  __shared__ double sm[kResampleThreads + 9];
+  __shared__ int pick, last;
+  const int b = blockIdx.x, tid = threadIdx.x, rows = args->gamma + 1;
+  const ResampleRow x = resample_row(args, w, dm, b);
+  const double2* part = w.rs_part + (size_t)b * n_chunks;
+  double total_p = 0.0, total_r = 0.0;
+  for (int c0 = 0; c0 < n_chunks; c0 += kResampleThreads) {
+    const double2 v = c0 + tid < n_chunks ? __ldcg(part + c0 + tid) : make_double2(0.0, 0.0);
+    resample_scan(v.x, sm);
+    total_p += sm[kResampleThreads];
     __syncthreads();
-    if (tid == 0) {
+    resample_scan(v.y, sm);
+    total_r += sm[kResampleThreads];
+    __syncthreads();
+  }
+  const bool residual = x.q != nullptr && total_r > 0.0;   // no residual mass: fall back to p
+  const double target = (double)args->uniforms[b * rows + args->gamma] * (residual ? total_r : total_p);
+  double carry = 0.0;
+  int chunk = -1;
+  for (int c0 = 0; c0 < n_chunks && chunk < 0; c0 += kResampleThreads) {
+    if (tid == 0) pick = kResampleThreads;
+    const double2 v = c0 + tid < n_chunks ? __ldcg(part + c0 + tid) : make_double2(0.0, 0.0);
+    resample_scan(residual ? v.y : v.x, sm);
+    if (carry + sm[tid + 1] > target) atomicMin(&pick, tid);
+    __syncthreads();
+    const int k = pick;
+    if (k < kResampleThreads) {
+      chunk = c0 + k;
+      carry += sm[k];
+    } else {
+      carry += sm[kResampleThreads];
+    }
+    __syncthreads();
+  }
+  if (tid == 0) { pick = kResampleThreads; last = -1; }
+  double p[kResamplePer], res[kResamplePer], own = 0.0;
+  if (chunk >= 0) {
+    resample_load(x, dm.V, chunk, p, res);
+#pragma unroll
+    for (int i = 0; i < kResamplePer; ++i) {
+      if (residual) p[i] = res[i];
+      own += p[i];
+    }
+  }
+  resample_scan(own, sm);
+  if (carry + sm[tid + 1] > target) atomicMin(&pick, tid);
+  if (own > 0.0) atomicMax(&last, tid);   // a sum that rounding left short of the target ends at the last entry with mass
+  __syncthreads();
+  const int who = chunk < 0 ? 0 : (pick < kResampleThreads ? pick : max(last, 0));
+  if (tid == who) {
+    int winner = dm.V - 1;
+    if (chunk >= 0) {
+      const int v0 = chunk * kResampleChunk + tid * kResamplePer;
       double run = 0.0;
-      for (int i = 0; i < T; ++i) { double t = part[i]; part[i] = run; run += t; }  // exclusive prefix
-      total_s = run;
-      winner = dm.V - 1;
+      bool found = false;
+#pragma unroll
+      for (int i = 0; i < kResamplePer; ++i) {
+        run += p[i];
+        if (!found && p[i] > 0.0) { winner = v0 + i; found = carry + (sm[tid] + run) > target; }
+      }
     }
-    __syncthreads();
-    const double total = total_s;
-    if (residual && !(total > 0.0)) { __syncthreads(); continue; }  // no residual mass: fall back to p
-    const double target = (double)args->uniforms[b * rows + gamma] * total;
-    double run = part[tid];
-    for (int v = v0; v < v1; ++v) {
-      double p = (double)expf(lg[v] * invT - st.m) * inv_s;
-      run += residual ? fmax(0.0, p - (double)q[v]) : p;
-      if (run > target) { atomicMin(&winner, v); break; }
-    }
-    __syncthreads();
-    if (tid == 0) {
-      args->next_token[b] = winner;
-      if (args->commit) kv.pending[args->seq_ids[b]] = winner;
-    }
-    break;
+    args->next_token[b] = winner;
+    if (args->commit) kv.pending[args->seq_ids[b]] = winner;
   }
 }
 

@@ -189,10 +189,10 @@ struct LayerW {
 
 struct StepKey {
   const sj_kv* kv;   // a captured step holds its cache's pointers; destroying the cache drops the graphs
-  int B, gamma, mode, chunk_len, gemm_impl, attn_impl, pdl, scratch;
+  int B, gamma, mode, chunk_len, gemm_impl, attn_impl, pdl, top_k;
   bool operator<(const StepKey& o) const {
-    return std::tie(kv, B, gamma, mode, chunk_len, gemm_impl, attn_impl, pdl, scratch) <
-           std::tie(o.kv, o.B, o.gamma, o.mode, o.chunk_len, o.gemm_impl, o.attn_impl, o.pdl, o.scratch);
+    return std::tie(kv, B, gamma, mode, chunk_len, gemm_impl, attn_impl, pdl, top_k) <
+           std::tie(o.kv, o.B, o.gamma, o.mode, o.chunk_len, o.gemm_impl, o.attn_impl, o.pdl, o.top_k);
   }
 };
 
@@ -227,7 +227,6 @@ struct sj_target {
   size_t att_chunks_cap = 0;
   int att_rows_cap = 0;
   size_t tc_part_cap = 0;   // floats in tc_m / tc_l
-  size_t logits_rows = 0;
   int pair_clusters[kPairMaxSplit + 1] = {};
   std::map<StepKey, cudaGraphExec_t> graphs;
   std::map<std::pair<const void*, int>, CUtensorMap> act_maps;   // per activation matrix and row count
@@ -373,7 +372,11 @@ static sj_status alloc_partials(sj_target* t, Work& W, int R) {
     n = 0;
     for (TcSite* s : {&t->s_qkv, &t->s_o, &t->s_gu, &t->s_down}) n = std::max(n, (size_t)s->max_slots * R * s->N);
   }
-  return dev_alloc(t, &W.P, n);
+  // the logits' place as well: they are written when the last projection's sums have been read
+  n = std::max(n, (size_t)R * c.vocab);
+  const sj_status st = dev_alloc(t, &W.P, n);
+  W.logits = W.P;
+  return st;
 }
 
 typedef void (*PairKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const PairParams, const StepArgs*,
@@ -1162,19 +1165,20 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
       AttArgs aa{W.Qb, l < t->opt_att_precise ? W.Qlo : nullptr, W.KVn, AttPartials{W.tc_m, W.tc_l, W.tc_o}, t->sm_count + B * dm.Hkv, l, B};
       const size_t tc_smem = kAttStages * kAttStageBytes + sizeof(AttSmemCtl) + 1024;
       const AttPartials parts{W.tc_m, W.tc_l, W.tc_o};
-      // one warp per (sequence, KV head, query row, half of the head dimension): every task's loads are in flight at once
-      const int items = B * dm.Hkv * nq, cgrid = std::max(1, std::min(32 * t->sm_count, (items * (dm.hd >= 128 ? 2 : 1) + 7) / 8));
+      // as many blocks per (sequence, KV head) as its rows keep busy, about four to an SM altogether
+      const int per = kCombineRows * kCombineThreads / 32;
+      const dim3 cgrid(B * dm.Hkv, std::max(1, std::min((nq + per - 1) / per, 4 * t->sm_count / (B * dm.Hkv))));
       if (dm.hd == 128 && t->opt_attn == 2 && nq <= 128) {   // one 128-lane accumulator holds a KV head's query rows
         const T5Geom tg = t5_geom(nq);
         TIMED("attn", launch(a5_split(nq) <= 32 ? k_attn_t5<4> : k_attn_t5<8>, dim3(t->sm_count), dim3(kT5Threads), tg.smem, s, pdl, kv->tm_pool, args,
                              kv->view, W, dm, aa, tg.stages));
-        TIMED("attn_combine", launch(k_attn_combine_tc<128, 8>, dim3(cgrid), dim3(256), 0, s, pdl, args, W, dm, parts, t->sm_count, aa.n_tail_base, kT5Keys, kT5Pad));
+        TIMED("attn_combine", launch(k_attn_combine_tc<128>, cgrid, dim3(kCombineThreads), 0, s, pdl, args, W, dm, parts, t->sm_count, aa.n_tail_base, kT5Keys, kT5Pad));
       } else if (dm.hd == 128) {
         TIMED("attn", launch(k_attn_tc<128>, dim3(t->sm_count), dim3(kAttTcThreads), tc_smem, s, pdl, kv->tm_pool, args, kv->view, W, dm, aa));
-        TIMED("attn_combine", launch(k_attn_combine_tc<128, 0>, dim3(cgrid), dim3(256), 0, s, pdl, args, W, dm, parts, t->sm_count, aa.n_tail_base, 0, 0));
+        TIMED("attn_combine", launch(k_attn_combine_tc<128>, cgrid, dim3(kCombineThreads), 0, s, pdl, args, W, dm, parts, t->sm_count, aa.n_tail_base, 0, 0));
       } else {
         TIMED("attn", launch(k_attn_tc<64>, dim3(t->sm_count), dim3(kAttTcThreads), tc_smem, s, pdl, kv->tm_pool, args, kv->view, W, dm, aa));
-        TIMED("attn_combine", launch(k_attn_combine_tc<64, 0>, dim3(cgrid), dim3(256), 0, s, pdl, args, W, dm, parts, t->sm_count, aa.n_tail_base, 0, 0));
+        TIMED("attn_combine", launch(k_attn_combine_tc<64>, cgrid, dim3(kCombineThreads), 0, s, pdl, args, W, dm, parts, t->sm_count, aa.n_tail_base, 0, 0));
       }
     } else {
       TIMED("attn", launch(k_attn_simt<T>, dim3(att_grid), dim3(kAttThreads), att_smem, s, pdl, args, kv->view, W, dm, l, chunk_len));
@@ -1227,7 +1231,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
 }
 
 template <typename T>
-static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mode, int chunk_len, bool use_logits,
+static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mode, int top_k, int chunk_len, bool use_logits,
                                size_t n_chunks_hi) {
   const Dims& dm = t->dm;
   const int R = B * (gamma + 1);
@@ -1244,7 +1248,7 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
   // LM head + statistics
   const int n_vtiles = (dm.V + kTileN - 1) / kTileN;
   if (tc) {
-    TIMED("target_logits", launch(k_target_logits, dim3((R + 7) / 8), dim3(256), 0, s, pdl, args, W, dm, (const bf16*)t->lm_head, R));
+    if (top_k >= 2) TIMED("target_logits", launch(k_target_logits, dim3((R + 7) / 8), dim3(256), 0, s, pdl, args, W, dm, (const bf16*)t->lm_head, R));
     if (pair_usable(t, kv))
       TIMED_ST("gemm_lm_head", launch_pair(t, kv, PAIR_LM, n_vtiles, dm.d, W.A, &t->m_lm, nullptr, nullptr, R, pdl, W, PairOut()));
     else
@@ -1487,7 +1491,6 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
   // [R, V] logits exist for the CUDA-core LM head (fp32 models, cross-checks) and in sampling mode; else the tensor-core
   // paths keep softmax statistics per vocabulary tile
   const bool use_logits = (t->opt_gemm == 0 && !use_mega) || a->mode == SJ_MODE_SAMPLING;
-  const size_t logit_rows_needed = use_logits ? (size_t)R : 0;
   // grow lazily-sized buffers (outside any capture)
   const bool simt_attn = t->opt_attn == 0 || !t->bf || !kv->has_tm_pool;
   if (simt_attn && (chunk_need_base > t->att_chunks_cap || rows > t->att_rows_cap)) {
@@ -1511,17 +1514,6 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
   }
   if ((!simt_attn || use_mega) && kv->has_tm_pool)
     if ((st = ensure_attn_partials(t, B, rows)) != SJ_OK) return st;
-  if (logit_rows_needed > t->logits_rows) {
-    CU_TRY(cudaStreamSynchronize(t->stream));
-    clear_graphs(t);
-    if (t->work.logits) {
-      counted_free(t->work.logits);
-      t->owned.erase(std::remove(t->owned.begin(), t->owned.end(), (void*)t->work.logits), t->owned.end());
-      t->work.logits = nullptr;
-    }
-    if ((st = dev_alloc(t, &t->work.logits, logit_rows_needed * t->dm.V)) != SJ_OK) return st;
-    t->logits_rows = logit_rows_needed;
-  }
 
   // per-call arguments: one small copy (the driver stages pageable memory before returning)
   StepArgs h;
@@ -1544,7 +1536,7 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
   CU_TRY(cudaMemcpyAsync(t->d_args, &h, sizeof(h), cudaMemcpyHostToDevice, t->stream));
 
   // chunk_len shapes only the CUDA-core attention's grid: a growing cache captures no new step elsewhere
-  StepKey key{kv, B, gamma, a->mode, simt_attn ? chunk_len : 0, t->opt_gemm, t->opt_attn, t->opt_pdl, use_logits ? 1 : 0};
+  StepKey key{kv, B, gamma, a->mode, simt_attn ? chunk_len : 0, t->opt_gemm, t->opt_attn, t->opt_pdl, h.top_k};
   if (use_mega) {
     if ((st = launch_mega(t, kv, B, gamma, a->mode, use_logits)) != SJ_OK) return st;
   } else if (t->opt_graph) {
@@ -1556,8 +1548,8 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
       }
       cudaGraph_t graph = nullptr;
       CU_TRY(cudaStreamBeginCapture(t->stream, cudaStreamCaptureModeThreadLocal));
-      st = t->bf ? enqueue_step<bf16>(t, kv, B, gamma, a->mode, chunk_len, use_logits, chunk_need_base)
-                 : enqueue_step<float>(t, kv, B, gamma, a->mode, chunk_len, use_logits, chunk_need_base);
+      st = t->bf ? enqueue_step<bf16>(t, kv, B, gamma, a->mode, h.top_k, chunk_len, use_logits, chunk_need_base)
+                 : enqueue_step<float>(t, kv, B, gamma, a->mode, h.top_k, chunk_len, use_logits, chunk_need_base);
       cudaError_t e = cudaStreamEndCapture(t->stream, &graph);
       if (st != SJ_OK) {
         if (graph) cudaGraphDestroy(graph);
@@ -1573,8 +1565,8 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
     }
     CU_TRY(cudaGraphLaunch(it->second, t->stream));
   } else {
-    st = t->bf ? enqueue_step<bf16>(t, kv, B, gamma, a->mode, chunk_len, use_logits, chunk_need_base)
-               : enqueue_step<float>(t, kv, B, gamma, a->mode, chunk_len, use_logits, chunk_need_base);
+    st = t->bf ? enqueue_step<bf16>(t, kv, B, gamma, a->mode, h.top_k, chunk_len, use_logits, chunk_need_base)
+               : enqueue_step<float>(t, kv, B, gamma, a->mode, h.top_k, chunk_len, use_logits, chunk_need_base);
     if (st != SJ_OK) return st;
   }
   if (a->commit) {

@@ -562,7 +562,6 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   extern __shared__ uint8_t t5_smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(t5_smem_raw) + 1023) & ~(uintptr_t)1023);
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  pdl_wait();
   pdl_launch();
   const int B = args->B, rows = args->gamma + 1, Hkv = dm.Hkv, group = dm.Hq / dm.Hkv, nq = group * rows;
   const int G = gridDim.x, c = blockIdx.x;
@@ -597,6 +596,9 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   att_fill_pages(ctl->pages, pl, kv, args, B, kT5Keys, t_lo, t_hi, threadIdx.x, blockDim.x);
   __syncthreads();
   const uint32_t tmem = ctl->tmem_base;
+  // All of the above reads what kernels before the previous one have written.  So do the loads of the cache's tiles, but
+  // in a prefill, whose entries attend to rows that the previous kernel stores.
+  if (!((warp == 0 || warp == 10) && args->pos_step == 0)) pdl_wait();
   const A5Ring rg{ctl->full, ctl->empty, sm, stages, &ctl->abort_flag, w.status};
   A5Pos pos{0, 0};
   int gt = 0, segs = 0;

@@ -691,7 +691,6 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(att_smem_raw) + 1023) & ~(uintptr_t)1023);
   AttSmemCtl* ctl = reinterpret_cast<AttSmemCtl*>(ring + kAttStages * kAttStageBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_wait();
   pdl_launch();
   const int B = args->B, rows = args->gamma + 1, Hkv = dm.Hkv;
   const AttGeom g = att_geom(HD, dm.Hq / dm.Hkv, rows);
@@ -714,6 +713,9 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
     att_fill_pages(ctl->pages, pl, kv, args, B, g.KPS, t_lo, t_hi, threadIdx.x, blockDim.x);
   }
   __syncthreads();
+  // All of the above reads what kernels before the previous one have written.  So do the loads of the cache's tiles, but in
+  // a prefill, whose entries attend to rows that the previous kernel stores.
+  if (!(warp == 0 && args->pos_step == 0)) pdl_wait();
   if (warp == 0) {
     if (lane == 0) {
       const long long t_lo = (long long)c * pl.T / G, t_hi = (long long)(c + 1) * pl.T / G;
@@ -761,10 +763,7 @@ template <> struct AttVec<2> {
 // dims a lane holds per sub-partial are one 8-byte load and all sub-partials of a config-3 item (39) are in
 // flight at once; with one warp per item they need two dependent batches.
 template <int HD> struct AttCombineSplit { static constexpr int value = HD >= 128 ? 2 : 1; };
-// OBN: output rows one lane keeps in flight (0: 40 or 24, sized for the 30..40 sub-partials of short tiles; 8 where long
-// tiles leave an item a handful of sub-partials: the clamped repeats of the last row would be most of the pass's L2
-// traffic)
-template <typename T, int HD, int OBN = 0>
+template <typename T, int HD>
 __device__ __forceinline__ void att_combine_item(const AttPartials& P, const AttPlan& pl, const AttGeom& g, int G_att,
                                                  int n_tail_base, int Hkv, int item_part, void* ATT, int R, int Hq, int lane,
                                                  unsigned long long* ev = nullptr) {
@@ -795,7 +794,7 @@ __device__ __forceinline__ void att_combine_item(const AttPartials& P, const Att
     return (long long)(cc + 1) * pl.T / G_att > (long long)cc * pl.T / G_att;
   };
   constexpr int DPL = HD / 32 / SPLIT;   // dims per lane
-  constexpr int OB = OBN > 0 ? OBN : (DPL <= 2 ? 40 : 24);   // output rows whose loads one lane keeps in flight
+  constexpr int OB = DPL <= 2 ? 40 : 24;   // output rows whose loads one lane keeps in flight
   constexpr int RS = HD / DPL;             // row stride of the outputs in units of V
   typedef typename AttVec<DPL>::type V;
   const V* Po = reinterpret_cast<const V*>(P.o) + part * 32 + lane;   // row r of the outputs starts at Po + r * RS
@@ -861,24 +860,128 @@ __device__ __forceinline__ void att_combine_item(const AttPartials& P, const Att
   for (int i = 0; i < DPL; ++i) store_act<T>(ATT, R, Hq * HD, r, head * HD + (part * 32 + lane) * DPL + i, acc[i] * inv);
 }
 
+// The merge as a kernel of its own (the persistent kernel's phase is att_combine_item): a block takes query rows of ONE
+// (sequence, KV head), so the blocks of the attention pass that hold its partials are worked out once, before the wait for
+// that pass; a warp merges two rows side by side, a lane 4 (2) dims of each, with four partials of both in flight.  Bound
+// by the latency of two dependent rounds of L2 loads: one warp per half row that looked its blocks up by itself took
+// 25 us for 9216 rows of two to three partials, this kernel 17 (B200, launch included; a trivial kernel measures 6).
 // keys_per_tile > 0: the partials come from a pass that cut the cache into tiles of that many keys (plus tile_pad empty
 // ones per (sequence, KV head)) with one sub-partial per block segment (the tcgen05 attention); 0: this file's own
 // geometry.
-template <int HD, int OBN>
-__global__ void k_attn_combine_tc(const StepArgs* __restrict__ args, Work w, Dims dm, AttPartials P, int G_att,
-                                  int n_tail_base, int keys_per_tile, int tile_pad) {
+constexpr int kCombineThreads = 256, kCombineRows = 2;   // rows a warp merges at a time
+template <int HD>
+static __global__ void __launch_bounds__(kCombineThreads)
+k_attn_combine_tc(const StepArgs* __restrict__ args, Work w, Dims dm, AttPartials P, int G_att, int n_tail_base, int keys_per_tile, int tile_pad) {
+  constexpr int DPL = HD / 32, NR = kCombineRows, OB = 4;
+  typedef typename AttVec<DPL>::type V;
   __shared__ AttPlan pl;
-  pdl_wait();
   pdl_launch();
-  const int B = args->B, rows = args->gamma + 1;
-  AttGeom g = att_geom(HD, dm.Hq / dm.Hkv, rows);
-  if (keys_per_tile > 0) { g.KPS = keys_per_tile; g.KS = 1; g.KW = keys_per_tile; }
+  const int B = args->B, rows = args->gamma + 1, group = dm.Hq / dm.Hkv, nq = group * rows;
+  AttGeom g = att_geom(HD, group, rows);
+  if (keys_per_tile > 0) { g.KPS = keys_per_tile; g.KS = 1; }
+  // the row positions are the work of a kernel before the one that this one waits for
   if (threadIdx.x < 32) att_plan_fill(&pl, w.row_pos, B, rows, dm.Hkv, g.KPS, threadIdx.x, keys_per_tile > 0 ? tile_pad : 0);
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-  const int items = B * dm.Hkv * g.nq * AttCombineSplit<HD>::value;
-  for (int item = warp * gridDim.x + blockIdx.x; item < items; item += gridDim.x * wpb)   // spread over blocks first
-    att_combine_item<bf16, HD, OBN>(P, pl, g, G_att, n_tail_base, dm.Hkv, item, w.ATT, B * rows, dm.Hq, lane);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int bh = blockIdx.x, b = bh / dm.Hkv, h = bh % dm.Hkv, L = pl.L[b];
+  const int nt_b = L > 0 ? (L + g.KPS - 1) / g.KPS + pl.pad : 0;
+  int c_first = 0, n_cta = 0;
+  if (nt_b > 0) {
+    const long long t0 = (long long)pl.pre[b] + (long long)h * nt_b;
+    c_first = att_owner(t0, pl.T, G_att);
+    n_cta = att_owner(t0 + nt_b - 1, pl.T, G_att) - c_first + 1;
+  }
+  const int n_sub = n_cta * g.KS + 1;   // the last one is the tail
+  const int ks_shift = g.KS == 4 ? 2 : (g.KS == 2 ? 1 : 0), ks_mask = g.KS - 1;
+  auto sub_row = [&](int k) -> size_t {   // row 0 of sub-partial k (ring: block c_first + k / KS, key share k % KS)
+    const size_t slot = k >= n_sub - 1 ? (size_t)n_tail_base + bh : (size_t)c_first + (k >> ks_shift) + bh;
+    return (slot * kAttMaxSub + (k >= n_sub - 1 ? 0 : k & ks_mask)) * nq;
+  };
+  const bool all_live = pl.T >= G_att;   // every block of the attention pass owns at least one tile
+  auto sub_live = [&](int k) -> bool {
+    if (all_live || k == n_sub - 1) return true;
+    const int cc = c_first + (k >> ks_shift);
+    return (long long)(cc + 1) * pl.T / G_att > (long long)cc * pl.T / G_att;
+  };
+  pdl_wait();
+  const V* Po = reinterpret_cast<const V*>(P.o) + lane;   // row r of the outputs starts at Po + 32 r
+#pragma unroll 1
+  for (int q0 = (blockIdx.y * (kCombineThreads / 32) + warp) * NR; q0 < nq; q0 += gridDim.y * (kCombineThreads / 32) * NR) {
+    int q[NR];
+    float M[NR], lsum[NR], acc[NR][DPL];
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      q[i] = min(q0 + i, nq - 1);
+      M[i] = -INFINITY;
+      lsum[i] = 0.f;
+#pragma unroll
+      for (int e = 0; e < DPL; ++e) acc[i][e] = 0.f;
+    }
+#pragma unroll 1
+    for (int k0 = 0; k0 < n_sub; k0 += 32) {
+      const int kn = min(32, n_sub - k0), k = k0 + lane;
+      const bool live = k < n_sub && sub_live(k);
+      const size_t row = sub_row(min(k, n_sub - 1));
+      float mk[NR], lk[NR], wk[NR];
+      V ob[NR][OB];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        mk[i] = live ? __ldcg(P.m + row + q[i]) : -INFINITY;
+        lk[i] = live ? __ldcg(P.l + row + q[i]) : 0.f;
+      }
+      auto load = [&](int kb) {
+#pragma unroll
+        for (int u = 0; u < OB; ++u) {
+          const size_t r = sub_row(k0 + min(kb + u, kn - 1));
+#pragma unroll
+          for (int i = 0; i < NR; ++i) ob[i][u] = __ldcg(Po + (r + q[i]) * 32);
+        }
+      };
+      load(0);
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        const float Mnew = fmaxf(M[i], warp_max(mk[i]));
+        const float rescale = M[i] == -INFINITY ? 0.f : exp2f(M[i] - Mnew);
+        wk[i] = mk[i] == -INFINITY ? 0.f : exp2f(mk[i] - Mnew);
+        lsum[i] = lsum[i] * rescale + warp_sum(lk[i] * wk[i]);
+        M[i] = Mnew;
+#pragma unroll
+        for (int e = 0; e < DPL; ++e) acc[i][e] *= rescale;
+      }
+#pragma unroll 1
+      for (int kb = 0; kb < kn; kb += OB) {
+        if (kb > 0) load(kb);
+#pragma unroll
+        for (int u = 0; u < OB; ++u)
+#pragma unroll
+          for (int i = 0; i < NR; ++i) {
+            const float wgt = __shfl_sync(0xffffffffu, wk[i], (kb + u) & 31);
+            AttVec<DPL>::fma(acc[i], ob[i][u], kb + u < kn ? wgt : 0.f);
+          }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      if (q0 + i >= nq) break;
+      const int r = b * rows + q[i] % rows, head = h * group + q[i] / rows, R = B * rows;
+      const float inv = 1.0f / lsum[i];
+      bf16* dst = reinterpret_cast<bf16*>(w.ATT) + (size_t)r * dm.Hq * HD + head * HD + lane * DPL;
+      __align__(8) bf16 hi[DPL], lo[DPL];
+#pragma unroll
+      for (int e = 0; e < DPL; ++e) {
+        const float y = acc[i][e] * inv;
+        hi[e] = __float2bfloat16_rn(y);
+        lo[e] = __float2bfloat16_rn(y - __bfloat162float(hi[e]));
+      }
+      if constexpr (DPL == 4) {
+        *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(hi);
+        *reinterpret_cast<uint2*>(dst + (size_t)pad16(R) * dm.Hq * HD) = *reinterpret_cast<const uint2*>(lo);
+      } else {
+        *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(hi);
+        *reinterpret_cast<uint32_t*>(dst + (size_t)pad16(R) * dm.Hq * HD) = *reinterpret_cast<const uint32_t*>(lo);
+      }
+    }
+  }
 }
 
 }  // namespace sj

@@ -1208,7 +1208,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
         const int items = B * dm.Hkv * g.nq * AttCombineSplit<HD>::value;
 #pragma unroll 1
         for (int item = ww * G + c; item < items; item += G * 8)   // spread over blocks first
-          att_combine_item<bf16, HD, 0>(P, pl, g, G, p.n_tail_base, dm.Hkv, item, w.ATT, R, dm.Hq, lane,
+          att_combine_item<bf16, HD>(P, pl, g, G, p.n_tail_base, dm.Hkv, item, w.ATT, R, dm.Hq, lane,
                                      (kTr && p.trace && c == 0 && ww == 0 && (l - p.l0) * 4 < kMegaTraceSites)
                                          ? p.trace + 2 * kMegaTraceBarriers + 8 * kMegaTraceSites + (size_t)(l - p.l0) * 4 * 8 + 4
                                          : nullptr);

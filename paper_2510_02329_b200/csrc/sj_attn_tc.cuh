@@ -107,6 +107,12 @@ __device__ __forceinline__ int att_owner(long long t, long long T, int G) {
   return c;
 }
 
+// First ring tile of block c.
+__device__ __forceinline__ long long att_first_tile(int c, long long T, int G) {
+  if (T < (1 << 22) && G < 512) return (unsigned)c * (unsigned)T / (unsigned)G;
+  return (long long)c * T / G;
+}
+
 // Partial storage: slot s, sub-partial ks, query row q.
 struct AttPartials {
   float* m;   // [slots][kAttMaxSub][nq]
@@ -791,7 +797,7 @@ __device__ __forceinline__ void att_combine_item(const AttPartials& P, const Att
   auto sub_live = [&](int k) -> bool {
     if (all_live || k == n_sub - 1) return true;
     const int cc = c_first + (k >> ks_shift);
-    return (long long)(cc + 1) * pl.T / G_att > (long long)cc * pl.T / G_att;
+    return att_first_tile(cc + 1, pl.T, G_att) > att_first_tile(cc, pl.T, G_att);
   };
   constexpr int DPL = HD / 32 / SPLIT;   // dims per lane
   constexpr int OB = DPL <= 2 ? 40 : 24;   // output rows whose loads one lane keeps in flight
@@ -901,7 +907,7 @@ k_attn_combine_tc(const StepArgs* __restrict__ args, Work w, Dims dm, AttPartial
   auto sub_live = [&](int k) -> bool {
     if (all_live || k == n_sub - 1) return true;
     const int cc = c_first + (k >> ks_shift);
-    return (long long)(cc + 1) * pl.T / G_att > (long long)cc * pl.T / G_att;
+    return att_first_tile(cc + 1, pl.T, G_att) > att_first_tile(cc, pl.T, G_att);
   };
   pdl_wait();
   const V* Po = reinterpret_cast<const V*>(P.o) + lane;   // row r of the outputs starts at Po + 32 r

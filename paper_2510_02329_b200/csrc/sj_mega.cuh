@@ -756,7 +756,9 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
     const int wsum = max(2 * n - 2, 1), w_lo = j == 0 ? 0 : 2 * j - 1, w_hi = j == n - 1 ? wsum : 2 * j + 1;
     const int tb = w_hi * T / wsum;
     constexpr int TF = kAllRows ? 2 : 1;        // words finished together
-    constexpr int CR = kAllRows ? 4 : 6;        // sharing blocks whose words are in flight together
+    // sharing blocks whose words are in flight together: at few rows all of them as a rule (O of a 1B-shaped model: ten
+    // blocks; six at a time are a second round trip to L2 in the phase's last microseconds)
+    constexpr int CR = kAllRows ? 4 : 12;
     int t0 = w_lo * T / wsum;
 #pragma unroll 1
     while (t0 < tb) {
@@ -771,12 +773,16 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
 #pragma unroll 1
       for (int k0 = 0; k0 < n; k0 += CR) {   // the sharing blocks, this one included
         PartialWord pw[CR][TF];
-        const uint4* src[CR];
+        const uint4* src[kAllRows ? CR : 1];
+        const uint4* first = p.pbuf + partial_at(c_first, 0, Rp, chunk, grp, tri, fl);   // slot 0; a block's slots lie `slot` apart
+        const int slot = (Rp >> 4) * 6 * kTileN;
+        if constexpr (kAllRows) {
 #pragma unroll
-        for (int k = 0; k < CR; ++k) {
-          const int i = min(k0 + k, n - 1);   // past the last one: it is read again and ignored
-          const int c2 = sparse ? unit_owner((unsigned)tile * (unsigned)ss.KB + (unsigned)i, U, G) : c_first + i;
-          src[k] = p.pbuf + partial_at(c2, i == 0 ? 1 : 0, Rp, chunk, grp, tri, fl);
+          for (int k = 0; k < CR; ++k) {
+            const int i = min(k0 + k, n - 1);   // past the last one: it is read again and ignored
+            const int c2 = sparse ? unit_owner((unsigned)tile * (unsigned)ss.KB + (unsigned)i, U, G) : c_first + i;
+            src[k] = first + (2 * (c2 - c_first) + (i == 0 ? 1 : 0)) * slot;
+          }
         }
 #pragma unroll 1
         for (uint32_t spin = 0;; ++spin) {
@@ -784,7 +790,10 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
 #pragma unroll
           for (int k = 0; k < CR; ++k)
 #pragma unroll
-            for (int t = 0; t < TF; ++t) pw[k][t] = ld_partial(src[k] + min(t, t1 - t0 - 1) * kTileN);
+            for (int t = 0; t < TF; ++t) {
+              const int i = min(k0 + k, n - 1);
+              pw[k][t] = ld_partial((kAllRows ? src[kAllRows ? k : 0] : first + (i == 0 ? slot : 2 * i * slot)) + min(t, t1 - t0 - 1) * kTileN);
+            }
 #pragma unroll
           for (int k = 0; k < CR; ++k)
 #pragma unroll

@@ -32,6 +32,10 @@ class SpeculativeDecoder:
         self.pending: List[int] = [0] * self.B        # next token to feed (not yet in the caches)
         self.cycles = 0
         self.accepted_total = 0
+        # device buffers of a cycle: the draft's decode steps write `_step`, their tokens collect in `_drafts`
+        self._step, self._dummy = binding.VerifyBuffers(self.B, 1), torch.zeros((self.B, 1), dtype=torch.int32, device="cuda")
+        self._drafts = torch.zeros((self.B, self.gamma), dtype=torch.int32, device="cuda")
+        self._block = binding.VerifyBuffers(self.B, self.gamma)
 
     # ---- set-up -------------------------------------------------------------------------------
     def prefill(self, prompts: Sequence[Sequence[int]]) -> None:
@@ -61,12 +65,16 @@ class SpeculativeDecoder:
         B, gamma = self.B, self.gamma
         self.draft_kv.set_pending(self.seq_ids, self.pending)
         self.target_kv.set_pending(self.seq_ids, self.pending)
-        drafts = torch.zeros((B, gamma), dtype=torch.int32, device="cuda")
-        for j in range(gamma):                                        # the draft's gamma sequential passes
-            nxt = self._decode(self.draft, self.draft_kv, self.seq_ids)
-            self.draft.stream.synchronize()
-            drafts[:, j] = nxt
-        out = binding.VerifyBuffers(B, gamma)
+        # The draft's gamma sequential passes, queued on its stream without waiting for any: a pass finds its token in the
+        # cache's pending slot.  (Waiting for each pass and filling new buffers left the GPU idle between passes.)
+        drafts, out = self._drafts, self._block
+        self.draft.stream.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(self.draft.stream):
+            for j in range(gamma):
+                binding.verify(self.draft, self.draft_kv, self.seq_ids, self._dummy, self._step, mode=binding.MODE_GREEDY,
+                               use_align=False, use_judge=False, commit=True)
+                drafts[:, j].copy_(self._step.next_token)
+        self.target.stream.wait_stream(self.draft.stream)
         binding.verify(self.target, self.target_kv, self.seq_ids, drafts, out, mode=binding.MODE_GREEDY,
                        use_align=True, use_judge=use_judge, theta=theta, top_k=top_k, commit=True)
         self.target.sync()

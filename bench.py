@@ -497,10 +497,10 @@ def main():
                              "achieved": per_launch_bytes / per_launch_s / 1e9,
                              "avg_launch_us": per_launch_s * 1e6, "algorithmic_bytes_per_launch": per_launch_bytes})
         else:
-            # k_gemm_tc: all projections + LM head; algorithmic bytes = every streamed weight byte once
+            # k_gemm_pair: all projections + LM head; algorithmic bytes = every streamed weight byte once
             per_launch_bytes = w_bytes / (g_n / n_inst)
             per_launch_s = (g_ms / g_n) / 1e3
-            roofline.update({"kernel": "k_gemm_tc", "launches_per_step": g_n // n_inst,
+            roofline.update({"kernel": "k_gemm_pair", "launches_per_step": g_n // n_inst,
                              "achieved": per_launch_bytes / per_launch_s / 1e9,
                              "avg_launch_us": per_launch_s * 1e6, "algorithmic_bytes_per_launch": per_launch_bytes})
         roofline["frac"] = roofline["achieved"] / peak
@@ -526,7 +526,7 @@ def main():
         "algorithmic_bytes_per_step": w_bytes + kv_bytes,
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "ms_per_step": ms_e2e},
-        "gpu_launches": (mega_launches + 1 + (1 if mode == binding.MODE_SAMPLING else 0) if mega_launches
+        "gpu_launches": (mega_launches + 1 + (2 if mode == binding.MODE_SAMPLING else 0) if mega_launches
                          else dw.launches_per_step(mode)) * args.steps,
         "clocks": clocks, "roofline": roofline, "cpu_baseline": cpu_baseline,
         "kernel_breakdown": {} if args.no_breakdown else breakdown,

@@ -22,6 +22,8 @@
 // pairs shares an item's K.  Every pair sends its sums of the rows that another one finishes into that one's shared
 // memory and finishes its own: chunk j (32 rows) belongs to split j % n_split, so all of them work on the epilogue and
 // no sum crosses L2.  A cluster is scheduled as a whole, so its pairs can wait for one another.
+// The sums go as st.async: their arrival is the signal.  (A release after plain stores is one more trip: 1B-shaped 48 rows
+// 954 -> 934 us a step, 8B-shaped 44 rows 4459 -> 4377, with the residual rows requested beside the MMAs.)
 // Down at 72 rows (20 tiles, K 27648, 283 MB): 94.5 us with row blocks of 32 on 60 pairs, 60.4 as 80 rows on 40 pairs;
 // steps (B200): 32B-shaped 72 rows 5434 -> 4871 us, 8B-shaped 44 rows 5150 -> 4440, 1B-shaped 48 rows 1610 -> 1447.
 //
@@ -149,8 +151,11 @@ __device__ __forceinline__ bool cluster_try_wait(uint32_t bar, uint32_t parity) 
       : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ void cluster_st4(uint32_t remote, const float* v) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(remote), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+// Four values to another CTA of the cluster; their arrival counts 16 bytes on that CTA's barrier (an address there).
+__device__ __forceinline__ void cluster_st4_async(uint32_t remote, const float* v, uint32_t remote_bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(remote), "f"(v[0]), "f"(v[1]),
+               "f"(v[2]), "f"(v[3]), "r"(remote_bar)
+               : "memory");
 }
 __device__ __forceinline__ uint32_t instr_desc_pair(int n) {   // M = 256
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
@@ -182,8 +187,8 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&ctl->tmem_full[i]), 1);
       mbar_init(smem_u32(&ctl->tmem_empty[i]), 16);   // the epilogue warps of both CTAs
-      mbar_init(smem_u32(&ctl->xch_full[i]), 4 * max(S - 1, 1));   // a group's warps of every other split
-      mbar_init(smem_u32(&ctl->xch_free[i]), 4 * max(S - 1, 1));
+      mbar_init(smem_u32(&ctl->xch_full[i]), 1);   // and the bytes of the other splits' sums
+      mbar_init(smem_u32(&ctl->xch_free[i]), 4 * max(S - 1, 1));   // a group's warps of every other split
     }
     ctl->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -316,6 +321,13 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     for (int item = g; item < n_items; item += p.n_groups) {
       const int tile = 2 * (item / p.n_rb) + rank, r_lo = item % p.n_rb * p.rb, r_hi = min(r_lo + p.rb, R);
       const bool real = tile < p.n_tiles;   // an odd last tile's partner has no features
+      // residual rows of the first chunk that this split finishes, requested beside the MMAs
+      float x_first[16];
+      if constexpr (SITE == PAIR_RES) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          x_first[i] = __ldcg(w.X + (size_t)min(r_lo + 16 * grp + 32 * split + i, R - 1) * dm.d + min(tile, p.n_tiles - 1) * kTileN + fl);
+      }
       // the segments' sums: chunk j of this group in registers
       float sum[4][16];
 #pragma unroll
@@ -352,19 +364,22 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           group_sync();
           cluster_try_wait(smem_u32(bar), parity);   // every thread acquires the completed phase
         };
+        if (fl == 0) {
+          uint32_t bytes = 0;
+          for (int j = split; j < 4; j += S)
+            if (r_lo + 16 * grp + 32 * j < r_hi) bytes += (uint32_t)(S - 1) * 8192u;
+          mbar_expect_tx(smem_u32(&ctl->xch_full[grp]), bytes);
+        }
         if (n_x > 0) xch_wait(&ctl->xch_free[grp], (uint32_t)(n_x - 1) & 1u);
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           if (!(mine >> j & 1u) && r_lo + 16 * grp + 32 * j < r_hi) {
             const int f = j % S, slot = split < f ? split : split - 1;
             const uint32_t dst = cluster_addr(smem_u32(xch + ((size_t)(slot * 2 + grp) * p.xch_js + j / S) * 512 + fl), 2 * f + rank);
+            const uint32_t bar = cluster_addr(smem_u32(&ctl->xch_full[grp]), 2 * f + rank);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) cluster_st4(dst + (uint32_t)q * 2048u, &sum[j][4 * q]);
+            for (int q = 0; q < 4; ++q) cluster_st4_async(dst + (uint32_t)q * 2048u, &sum[j][4 * q], bar);
           }
-        __syncwarp();
-        if (lane == 0)
-          for (int f = 0; f < S; ++f)
-            if (f != split) cluster_arrive(smem_u32(&ctl->xch_full[grp]), 2 * f + rank);
         xch_wait(&ctl->xch_full[grp], (uint32_t)n_x & 1u);
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -406,7 +421,11 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         if (!(mine >> j & 1u)) continue;
         float (&v)[16] = sum[j];
         float xs[16];
-        if constexpr (SITE == PAIR_RES) {   // residual rows, requested before the accumulator is waited for
+        if constexpr (SITE == PAIR_RES) {
+          if (j == split) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) xs[i] = x_first[i];
+          } else
 #pragma unroll
           for (int i = 0; i < 16; ++i) xs[i] = __ldcg(w.X + (size_t)min(c0 + i, R - 1) * dm.d + tile * kTileN + fl);
         }

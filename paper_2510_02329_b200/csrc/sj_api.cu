@@ -1270,11 +1270,12 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
 
 // The whole step as one cooperative launch per chunk of kMegaMaxLayers layers.  "step_impl" 1 takes it up to kMegaMaxRows
 // rows; the default (2) where it is the faster of the two (B200, us a step, persistent / per stage):
-//   rows: its barriers cost less than launches, the paired projections are the better GEMM.  16 layers, 8B-shaped: 9 rows
-//     1927 / 2099, 18 rows 2200 / 2143, 27 rows 2270 / 2135; 1B-shaped: 18 rows 1228 / 1270, 24 rows 1308 / 1302, 36 rows
-//     1487 / 1384; 32B-shaped: 9 rows 3275 / 3434, 18 rows 3671 / 3519, 72 rows 6735 / 4871;
-//   layers: it has a fixed cost of tens of us (its 300 KB of code come from memory once a step).  2 layers of small
-//     widths: 148 / 120.
+//   rows: its barriers cost less than launches, the paired projections are the better GEMM, and at head dimension 128 the
+//     tcgen05 kernel the better attention.  16 layers, 8B-shaped: 9 rows 1928 / 2088, 17 rows 2198 / 2275, 18 rows
+//     2250 / 2113, 24 rows 2359 / 2136; 32B-shaped: 9 rows 3271 / 3412, 17 rows 3661 / 3648, 18 rows 3690 / 3476; 1B-shaped
+//     (head dimension 64): 9 rows 1039 / 1246, 18 rows 1222 / 1250, 24 rows 1270 / 1267, 36 rows 1487 / 1384;
+//   widths: where gate/up has fewer units than there are blocks, the phases stream nothing that could hide the barriers
+//     or the 0.3 MB of code.  2 layers: d 256, ffn 1024 147 / 121, 1B-shaped 240 / 257, 8B-shaped 405 / 430.
 // Caches of several 128-key tiles per SM (and head dimension 128): its mma.sync attention takes about three times as long a
 // key as the tcgen05 kernel (8B-shaped, 9 rows: 8000 keys, 3.4 tiles, 2156 / 2159).
 static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma, long total_keys) {
@@ -1282,7 +1283,8 @@ static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma, l
   if (t->opt_step == 0 || t->opt_gemm != 1 || !t->mega_shapes || !kv->has_tm_pool || R > kMegaMaxRows || group * rows > 16 * 6 || !t->stream)
     return false;
   if (t->dm.hd == 128 && t->opt_attn == 2 && total_keys * t->dm.Hkv / kT5Keys / t->sm_count >= t->opt_a5_min_tiles) return false;
-  return t->opt_step == 1 || t->opt_attn == 0 || (R <= kMegaAutoRows && t->dm.n_layers >= kMegaAutoLayers);
+  return t->opt_step == 1 || t->opt_attn == 0 ||
+         (R <= (t->dm.hd == 128 ? kMegaAutoRows128 : kMegaAutoRows64) && (t->dm.F / 64) * (t->dm.d / kBK) >= t->sm_count);
 }
 
 static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode, bool use_logits) {

@@ -205,11 +205,13 @@ typedef struct {
  * Errors before launch: INVALID_ARG, SHAPE (B*(gamma+1) > max_rows), OOM (page pool), STATE. */
 sj_status sj_verify(sj_target *t, sj_kv *kv, const sj_verify_args *args, const sj_verify_out *out);
 
-/* Chunked prefill through the verification step's own kernels: Eq. 2 applied to tokens that are known
- * rather than drafted.  Appends the n_tokens tokens `tokens` (host) to sequence `seq` in blocks of up to
+/* Prefill through the verification step's own kernels: Eq. 2 applied to tokens that are known rather than
+ * drafted.  Appends the n_tokens tokens `tokens` (host) to sequence `seq` in blocks of up to
  * min(32, 96 / (Hq/Hkv), max_rows) tokens: each block runs as a verification step whose first row is the
  * block's first token and whose "drafts" are the following ones, every position accepted and committed
- * (accept_all), so the cache receives exactly the K/V rows a verification step would read.  On return (the
+ * (accept_all), so the cache receives exactly the K/V rows a verification step would read.  bf16 models with
+ * tensor-core options take up to SJ_MAX_ROWS tokens' blocks through the layers at once (a workspace for them is
+ * allocated by the first such call; without memory for it the blocks run one by one).  On return (the
  * work is queued on the target's stream) the sequence is n_tokens longer and its pending token is the target's
  * greedy token after the last appended one; with next_token != NULL (host) that token is also copied out,
  * which waits for the stream.  The sequence's previous pending token is dropped: the first appended token

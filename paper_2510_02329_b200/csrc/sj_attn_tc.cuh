@@ -92,9 +92,14 @@ __host__ __device__ __forceinline__ AttGeom att_geom(int hd, int group, int rows
   return g;
 }
 
-// Which block owns ring tile t when T tiles are dealt to G blocks as [c*T/G, (c+1)*T/G).
+// T ring tiles are dealt to G blocks as [c*T/G, (c+1)*T/G); fewer tiles than blocks go one each to the first T of them, so
+// that the blocks from a tile's owner to a later one's all hold tiles.  (Spread over all G, as they were, every block in
+// between counted as a sub-partial of the merge: 80 of them at 128 keys and 4 heads, a toy step 64 us against 54.)
+// Which block owns tile t; first tile of block c.  32-bit arithmetic where it suffices (64-bit division is slow): t*G and
+// (c+1)*T stay below 2^31.
 __device__ __forceinline__ int att_owner(long long t, long long T, int G) {
-  if (T < (1 << 22) && G < 512) {   // 32-bit arithmetic (64-bit division is slow): t*G and (c+1)*T stay below 2^31
+  if (T <= G) return (int)t;
+  if (T < (1 << 22) && G < 512) {
     const unsigned tt = (unsigned)t, TT = (unsigned)T, GG = (unsigned)G;
     unsigned c = tt * GG / TT;
 #pragma unroll 1
@@ -106,9 +111,8 @@ __device__ __forceinline__ int att_owner(long long t, long long T, int G) {
   while ((long long)(c + 1) * T / G <= t) ++c;
   return c;
 }
-
-// First ring tile of block c.
 __device__ __forceinline__ long long att_first_tile(int c, long long T, int G) {
+  if (T <= G) return min((long long)c, T);
   if (T < (1 << 22) && G < 512) return (unsigned)c * (unsigned)T / (unsigned)G;
   return (long long)c * T / G;
 }
@@ -591,7 +595,7 @@ __device__ __forceinline__ bool att_consume(const AttRing& rg, int& it, const At
   AttWarp<HD, NT> st;
   const int mi = cw / g.KS, ks = cw % g.KS, row0 = mi * 16;
   const long long T = pl.T;
-  const long long t_lo = (long long)c * T / G, t_hi = (long long)(c + 1) * T / G;
+  const long long t_lo = att_first_tile(c, T, G), t_hi = att_first_tile(c + 1, T, G);
   long long t = t_lo;
 #pragma unroll 1
   while (t < t_hi) {
@@ -661,7 +665,7 @@ __device__ __forceinline__ bool att_consume_dispatch(const AttRing& rg, int& it,
 }
 
 // ---------------------------------------------------------------------------------------------
-// stand-alone kernel (used by the multi-kernel step): warp 0 streams the ring, warps 1..8 consume
+// the kernel of the per-stage step: warp 0 streams the ring, warps 1..8 consume
 // ---------------------------------------------------------------------------------------------
 constexpr int kAttStages = 8;
 constexpr int kAttTcThreads = 32 * (1 + kAttMaxWarps);
@@ -715,7 +719,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   const int G = gridDim.x, c = blockIdx.x;
   volatile int* abort_flag = &ctl->abort_flag;
   {
-    const long long t_lo = (long long)c * pl.T / G, t_hi = (long long)(c + 1) * pl.T / G;
+    const long long t_lo = att_first_tile(c, pl.T, G), t_hi = att_first_tile(c + 1, pl.T, G);
     att_fill_pages(ctl->pages, pl, kv, args, B, g.KPS, t_lo, t_hi, threadIdx.x, blockDim.x);
   }
   __syncthreads();
@@ -724,7 +728,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   if (!(warp == 0 && args->pos_step == 0)) pdl_wait();
   if (warp == 0) {
     if (lane == 0) {
-      const long long t_lo = (long long)c * pl.T / G, t_hi = (long long)(c + 1) * pl.T / G;
+      const long long t_lo = att_first_tile(c, pl.T, G), t_hi = att_first_tile(c + 1, pl.T, G);
       const int npg = g.KPS / 16;
       int it = 0;
 #pragma unroll 1
@@ -793,12 +797,6 @@ __device__ __forceinline__ void att_combine_item(const AttPartials& P, const Att
   auto sub_index = [&](int k) -> int {
     return k >= n_sub - 1 ? tail_idx : base + (k >> ks_shift) * step_c + (k & ks_mask) * g.nq;
   };
-  const bool all_live = pl.T >= G_att;   // every block of the attention pass owns at least one tile
-  auto sub_live = [&](int k) -> bool {
-    if (all_live || k == n_sub - 1) return true;
-    const int cc = c_first + (k >> ks_shift);
-    return att_first_tile(cc + 1, pl.T, G_att) > att_first_tile(cc, pl.T, G_att);
-  };
   constexpr int DPL = HD / 32 / SPLIT;   // dims per lane
   constexpr int OB = DPL <= 2 ? 40 : 24;   // output rows whose loads one lane keeps in flight
   constexpr int RS = HD / DPL;             // row stride of the outputs in units of V
@@ -815,7 +813,7 @@ __device__ __forceinline__ void att_combine_item(const AttPartials& P, const Att
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
       const int k = k0 + u * 32 + lane;
-      const bool live = k < n_sub && sub_live(k);
+      const bool live = k < n_sub;
       mk[u] = live ? __ldcg(P.m + sub_index(k)) : -INFINITY;
       lk[u] = live ? __ldcg(P.l + sub_index(k)) : 0.f;
     }
@@ -903,12 +901,6 @@ k_attn_combine_tc(const StepArgs* __restrict__ args, Work w, Dims dm, AttPartial
     const size_t slot = k >= n_sub - 1 ? (size_t)n_tail_base + bh : (size_t)c_first + (k >> ks_shift) + bh;
     return (slot * kAttMaxSub + (k >= n_sub - 1 ? 0 : k & ks_mask)) * nq;
   };
-  const bool all_live = pl.T >= G_att;   // every block of the attention pass owns at least one tile
-  auto sub_live = [&](int k) -> bool {
-    if (all_live || k == n_sub - 1) return true;
-    const int cc = c_first + (k >> ks_shift);
-    return att_first_tile(cc + 1, pl.T, G_att) > att_first_tile(cc, pl.T, G_att);
-  };
   pdl_wait();
   const V* Po = reinterpret_cast<const V*>(P.o) + lane;   // row r of the outputs starts at Po + 32 r
 #pragma unroll 1
@@ -926,7 +918,7 @@ k_attn_combine_tc(const StepArgs* __restrict__ args, Work w, Dims dm, AttPartial
 #pragma unroll 1
     for (int k0 = 0; k0 < n_sub; k0 += 32) {
       const int kn = min(32, n_sub - k0), k = k0 + lane;
-      const bool live = k < n_sub && sub_live(k);
+      const bool live = k < n_sub;
       const size_t row = sub_row(min(k, n_sub - 1));
       float mk[NR], lk[NR], wk[NR];
       V ob[NR][OB];

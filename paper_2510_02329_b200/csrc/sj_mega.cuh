@@ -997,7 +997,7 @@ k_verify_mega(const __grid_constant__ MegaMaps mp, const MegaParams p, const Ste
   __syncthreads();
 
   const AttPlan& pl = ctl->plan;
-  const long long t_lo = (long long)c * pl.T / G, t_hi = (long long)(c + 1) * pl.T / G;
+  const long long t_lo = att_first_tile(c, pl.T, G), t_hi = att_first_tile(c + 1, pl.T, G);
   const int n_att = (int)(t_hi - t_lo);   // ring stages of one attention phase
   att_fill_pages(ctl->att_pages, pl, kv, args, B, g.KPS, t_lo, t_hi, threadIdx.x, blockDim.x);
   __syncthreads();

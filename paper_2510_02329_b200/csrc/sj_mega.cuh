@@ -275,7 +275,14 @@ __device__ __forceinline__ void st_partial(uint4* p, float a, float b, float c, 
 }
 struct PartialWord {
   unsigned long long lo, hi;
-  __device__ __forceinline__ unsigned tag() const { return (unsigned)(hi >> 32); }
+  // Whether this is the word of `tag` that carries NV values (1 to 3; the others were written as zero).  Looks at every bit
+  // of the word: where only the first value and the tag were used (the fourth row of a group, steps of 7 and 8 rows), the
+  // load behaved as two narrower ones and a value of the phase before came with the new tag.  8B-shaped, 2 layers, 7 rows:
+  // six steps of six off by 2e-3 to 0.4 of the hidden state, none with this.
+  template <int NV>
+  __device__ __forceinline__ bool is(unsigned tag) const {
+    return (unsigned)(hi >> 32) == tag && (NV >= 3 || (unsigned)hi == 0u) && (NV >= 2 || (unsigned)(lo >> 32) == 0u);
+  }
   __device__ __forceinline__ float val(int i) const { return __uint_as_float(i == 0 ? (unsigned)lo : (i == 1 ? (unsigned)(lo >> 32) : (unsigned)hi)); }
 };
 __device__ __forceinline__ PartialWord ld_partial(const uint4* p) {
@@ -716,7 +723,7 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
 #pragma unroll
             for (int k = 0; k < CB; ++k)
 #pragma unroll
-              for (int t = 0; t < TR; ++t) ok = ok && (t >= ntr || pw[k][t].tag() == tag);
+              for (int t = 0; t < TR; ++t) ok = ok && (t >= ntr || (3 * t + 3 <= NS ? pw[k][t].template is<3>(tag) : pw[k][t].template is<NS % 3>(tag)));
             if (ok || !mega_poll_again(spin, ctl, p, w.status, gseq)) break;
           }
 #pragma unroll
@@ -797,7 +804,7 @@ __device__ __forceinline__ void mega_epilogue(int site, int l, int gseq, int& se
 #pragma unroll
           for (int k = 0; k < CR; ++k)
 #pragma unroll
-            for (int t = 0; t < TF; ++t) ok = ok && pw[k][t].tag() == tag;
+            for (int t = 0; t < TF; ++t) ok = ok && pw[k][t].template is<3>(tag);
           if (ok || !mega_poll_again(spin, ctl, p, w.status, gseq)) break;
         }
 #pragma unroll

@@ -1014,7 +1014,7 @@ struct PairOut {   // what a site's epilogue needs beyond the step's workspace
   float* ssq_out = nullptr;
   const void* gain = nullptr;
   void* planes_out = nullptr;
-  int K_out = 0, layer = 0;
+  int K_out = 0, layer = 0, seg_kb = kPairSegKB;
   const void *bq = nullptr, *bk = nullptr, *bv = nullptr;
 };
 static sj_status launch_pair(sj_target* t, sj_kv* kv, int site, int n_tiles, int K, const void* act, const CUtensorMap* w0, const CUtensorMap* w1,
@@ -1027,7 +1027,7 @@ static sj_status launch_pair(sj_target* t, sj_kv* kv, int site, int n_tiles, int
   PairParams p;
   memset(&p, 0, sizeof(p));
   p.n_tiles = n_tiles; p.KB = K / kBK; p.R = R; p.rb = g.rb; p.n_rb = g.n_rb; p.plane_rows = pad16(R);
-  p.n_groups = g.n_groups; p.n_split = g.n_split; p.xch_js = g.xch_js;
+  p.n_groups = g.n_groups; p.n_split = g.n_split; p.xch_js = g.xch_js; p.seg_kb = o.seg_kb;
   p.stages = g.stages; p.stage_bytes = g.stage_bytes; p.tmem_cols = g.tmem_cols;
   p.tile_q = dm.Hq * dm.hd / kTileN; p.tile_k = p.tile_q + dm.Hkv * dm.hd / kTileN;
   p.ssq_in = o.ssq_in; p.ssq_out = o.ssq_out; p.gain = (const bf16*)o.gain; p.planes_out = o.planes_out; p.K_out = o.K_out; p.layer = o.layer;
@@ -1108,11 +1108,11 @@ static cudaError_t launch_simt(sj_target* t, const void* A, const GemmSegs& segs
   } while (0)
 
 // The decoder layers of a step (set-up and embedding included): from the step's arguments to the GEMM input planes of
-// the final norm.  kv_only: the block's key / value rows are all that is wanted (prefill blocks before the last), so the
-// last layer ends after its projection.
+// the final norm.  prefill: a wide block of known tokens; kv_only: its key / value rows are all that is wanted (blocks
+// before the last), so the last layer ends after its projection.
 template <typename T>
 static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int chunk_len, Work W, size_t n_chunks_hi,
-                                bool kv_only) {
+                                bool prefill, bool kv_only) {
   const Dims& dm = t->dm;
   const int R = B * (gamma + 1), qd = dm.Hq * dm.hd, kd = dm.Hkv * dm.hd;
   const bool timing = t->opt_timing != 0 && !t->opt_graph;
@@ -1131,12 +1131,17 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
     if ((st = activation_map(t, W.H, R, dm.F, &mA_f)) != SJ_OK) return st;
   }
   const bool pair = pair_usable(t, kv);
+  // A prefill's sums of few K blocks (1B-shaped widths: 32) in chains half as long.  The persistent kernel, which runs the
+  // narrow blocks, deals such a projection in shares of about five blocks; with chains of 16 the step on a prefilled cache
+  // of 400 tokens was off by 1.97e-4 of the hidden state where its was 1.43e-4, with 8 by 1.63e-4 (4 layers).  Wider models have
+  // longer shares there (8B-shaped 2.58e-4 against 2.71e-4), and a step on a given cache shows no difference (1.105e-4, 1.109e-4).
+  auto seg_kb = [&](int K) { return prefill && K / kBK <= kPairShortKB ? kPairSegKB / 2 : kPairSegKB; };
   const size_t ssq_n = (size_t)(dm.d / kTileN) * R;
   auto plan_of = [&](const TcSite& site) { return tc ? SplitPlan{site.d_tile_slots, site.n_tiles} : one; };
 
   TIMED("plan", launch(k_plan, dim3(1), dim3(256), 0, s, false, args, kv->view, W, chunk_len));
   TIMED("embed_norm", launch(k_embed_norm<T>, dim3(R), dim3(256), row_smem, s, pdl, args, kv->view, W, dm, (const T*)t->embed,
-                (const T*)t->layers[0].na));
+                (const T*)t->layers[0].na, pair ? W.ssq : (float*)nullptr));
   const int nq = (dm.Hq / dm.Hkv) * (gamma + 1);
   const size_t att_smem = sizeof(float) * ((size_t)nq * dm.hd + kAttKT * (dm.hd + 1) + kAttKT * dm.hd + (size_t)nq * kAttKT + 3 * nq);
   const int att_grid = std::max(1, std::min<int>(t->sm_count * 2, (int)n_chunks_hi * dm.Hkv));
@@ -1145,9 +1150,10 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
     // QKV projection, bias, rotary embedding, cache append
     if (pair) {
       PairOut o;
-      o.ssq_in = l > 0 ? W.ssq : nullptr;
+      o.ssq_in = W.ssq;
       o.layer = l;
       o.bq = L.bq; o.bk = L.bk; o.bv = L.bv;
+      o.seg_kb = seg_kb(dm.d);
       TIMED_ST("gemm_qkv", launch_pair(t, kv, PAIR_QKV, t->s_qkv.n_tiles, dm.d, W.A, &L.m_q, &L.m_k, &L.m_v, R, pdl, W, o));
     } else {
       if (tc) {
@@ -1186,11 +1192,11 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
     }
     if (pair) {   // O, gate/up and down with their epilogues
       PairOut o, gu, dn;
-      o.ssq_out = W.ssq + ssq_n; o.gain = L.nf; o.planes_out = W.A;
+      o.ssq_out = W.ssq + ssq_n; o.gain = L.nf; o.planes_out = W.A; o.seg_kb = seg_kb(qd);
       TIMED_ST("gemm_o", launch_pair(t, kv, PAIR_RES, dm.d / kTileN, qd, W.ATT, &L.m_o, nullptr, nullptr, R, pdl, W, o));
-      gu.ssq_in = W.ssq + ssq_n; gu.planes_out = W.H; gu.K_out = dm.F;
+      gu.ssq_in = W.ssq + ssq_n; gu.planes_out = W.H; gu.K_out = dm.F; gu.seg_kb = seg_kb(dm.d);
       TIMED_ST("gemm_gateup", launch_pair(t, kv, PAIR_GU, dm.F / 64, dm.d, W.A, &L.m_g64, &L.m_u64, nullptr, R, pdl, W, gu));
-      dn.ssq_out = W.ssq; dn.planes_out = W.A;
+      dn.ssq_out = W.ssq; dn.planes_out = W.A; dn.seg_kb = seg_kb(dm.F);
       dn.gain = l + 1 < dm.n_layers ? t->layers[l + 1].na : t->final_norm;
       TIMED_ST("gemm_down", launch_pair(t, kv, PAIR_RES, dm.d / kTileN, dm.F, W.H, &L.m_d, nullptr, nullptr, R, pdl, W, dn));
       if (l == dm.n_layers - 1)
@@ -1242,7 +1248,7 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
   if (!use_logits) W.logits = nullptr;
   cudaStream_t s = t->stream;
   const CUtensorMap* mA_d = nullptr;
-  sj_status st = enqueue_layers<T>(t, kv, B, gamma, chunk_len, W, n_chunks_hi, false);
+  sj_status st = enqueue_layers<T>(t, kv, B, gamma, chunk_len, W, n_chunks_hi, false, false);
   if (st != SJ_OK) return st;
   if (tc && (st = activation_map(t, W.A, R, dm.d, &mA_d)) != SJ_OK) return st;
   // LM head + statistics
@@ -1724,7 +1730,7 @@ static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* token
     h.B = B; h.gamma = c - 1; h.mode = SJ_MODE_GREEDY; h.inv_temperature = 1.f; h.top_k = 1; h.accept_all = 1;
     for (int b = 0; b < B; ++b) h.seq_ids[b] = seq;
     CU_TRY(cudaMemcpyAsync(t->d_args, &h, sizeof(h), cudaMemcpyHostToDevice, s));
-    if ((st = enqueue_layers<bf16>(t, kv, B, c - 1, 4096, W, 0, !last)) != SJ_OK) return st;
+    if ((st = enqueue_layers<bf16>(t, kv, B, c - 1, 4096, W, 0, true, !last)) != SJ_OK) return st;
     const int n_vtiles = (dm.V + kTileN - 1) / kTileN;
     if (last) {
       const CUtensorMap* mA = nullptr;

@@ -7,7 +7,7 @@
 // both.  The epilogue adds the two halves.
 //
 // The tensor core's accumulation truncates (measured against fp64: a chain of 896 MMAs comes out 1.4e-5 too small, one
-// of 64 about 1e-6), so K is summed in segments of kPairSegKB K blocks whose results the epilogue warps add in fp32
+// of 64 about 1e-6), so K is summed in segments of up to kPairSegKB K blocks whose results the epilogue warps add in fp32
 // registers.  Segments alternate between two accumulators: the adding, and an item's epilogue, run beside the next
 // segment's MMAs.
 //
@@ -47,7 +47,7 @@ constexpr int kPairThreads = 384;      // warp 0 TMA, warp 1 MMA (rank 0), warp 
 constexpr int kPairWorkers = 256;
 constexpr int kPairMaxStages = 10;
 constexpr int kPairMaxRows = kMaxRows;
-constexpr int kPairSegKB = 16;          // K blocks of 64 per accumulation chain
+constexpr int kPairSegKB = 16, kPairShortKB = 32;   // K blocks of 64 per accumulation chain; half of them in a prefill's sums of up to kPairShortKB
 constexpr int kPairMaxSplit = 4;        // pairs that share an item's K (a cluster of 8)
 constexpr double kPairHbmBytesPerClk = 3600;   // HBM against the SM clock, for the host's choice of a geometry
 constexpr int kPairXchClk = 3000;       // an exchange between the splits
@@ -60,13 +60,14 @@ struct PairParams {
   int KB;                 // K blocks of 64
   int n_groups;           // clusters
   int n_split;            // pairs of a cluster: they share an item's K blocks
+  int seg_kb;             // K blocks per accumulation chain
   int xch_js;             // 32-row chunks of a row block that one split finishes, at most
   int R, rb, n_rb;        // rows, rows per block (a multiple of 16, at most 128: an M = 256 MMA takes N = 32, 64 .. 256), row blocks
   int plane_rows;         // row of the lo plane in the activation matrix
   int stages, stage_bytes;
   uint32_t tmem_cols;     // two accumulators of 2 rb columns
   int tile_q, tile_k;     // QKV: tiles of Wq, tiles of Wq and Wk together
-  const float* ssq_in;    // [d / 128][R] sums of squares of this GEMM's input rows (null: the planes are normalised)
+  const float* ssq_in;    // [d / 128][R] sums of squares of this GEMM's input rows (null: LM head, whose planes are normalised)
   float* ssq_out;         // [d / 128][R] PAIR_RES
   const bf16* gain;       // PAIR_RES: gain of the norm that reads the result next
   void* planes_out;       // PAIR_RES: W.A; PAIR_GU: W.H
@@ -255,9 +256,9 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       bool alive = true;
       for (int item = g; item < n_items && alive; item += p.n_groups) {
         uint32_t dcol = 0;
-        int acc = 0;
+        int acc = 0, at = 0;   // block of the chain
         for (int kb = kb_lo; kb < kb_hi; ++kb) {
-          const bool first = (kb - kb_lo) % kPairSegKB == 0;
+          const bool first = at == 0;
           if (first) {
             acc = n & 1;
             const int use = n >> 1;
@@ -273,7 +274,10 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           for (int k = 0; k < kBK / 16; ++k) pair_mma(dcol, dw + 2 * k, da + 2 * k, idesc, (!first || k > 0) ? 1u : 0u);
           pair_commit(smem_u32(&ctl->empty[s]), pair_mask);
           if (++s == p.stages) { s = 0; ++r; }
-          if ((kb - kb_lo) % kPairSegKB == kPairSegKB - 1 || kb == kb_hi - 1) pair_commit(smem_u32(&ctl->tmem_full[acc]), pair_mask);
+          if (++at == p.seg_kb || kb == kb_hi - 1) {
+            pair_commit(smem_u32(&ctl->tmem_full[acc]), pair_mask);
+            at = 0;
+          }
         }
       }
     }
@@ -314,7 +318,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       }
     }
     all_sync();
-    const int n_seg = (kb_hi - kb_lo + kPairSegKB - 1) / kPairSegKB;
+    const int n_seg = (kb_hi - kb_lo + p.seg_kb - 1) / p.seg_kb;
     int n = 0, n_x = 0;   // segments, exchanges so far
     uint32_t mine = 0;    // the chunks j that this split finishes
     for (int j = split; j < 4; j += S) mine |= 1u << j;

@@ -109,10 +109,14 @@ __device__ __forceinline__ void norm_row_from_smem(const float* xs, int d, const
   }
 }
 
-// a1 + first a2: embedding gather, RMSNorm, and this step's rotary table.
+// a1 + first a2: embedding gather, RMSNorm, and this step's rotary table.  With `ssq` ([d / 128][R]; the paired projections,
+// whose d is a multiple of 128) the planes hold embedding x gain and the reader applies the row scalar, as in the other
+// layers and in the persistent kernel: a product of two bf16 numbers fits the two planes, so the first layer's keys and
+// values carry no activation rounding.  Normalised rows lose 2^-17 in the planes, which turned the bf16 rounding of 2.5e-3 of
+// the first layer's cached numbers (6.5e-4 without it, 8e-4 by the persistent kernel), and of more in every layer after.
 template <typename T>
 __global__ void k_embed_norm(const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, const T* __restrict__ embed,
-                             const T* __restrict__ gain) {
+                             const T* __restrict__ gain, float* __restrict__ ssq) {
   extern __shared__ float xs[];
   __shared__ float red[32];
   pdl_wait();
@@ -137,6 +141,22 @@ __global__ void k_embed_norm(const StepArgs* __restrict__ args, KvView kv, Work 
     w.rope[(size_t)r * (dm.hd / 2) + i] = make_float2((float)c, (float)s);
   }
   __syncthreads();
+  if (ssq) {   // uniform
+    const int lane = threadIdx.x & 31;
+    for (int t = threadIdx.x >> 5; t < dm.d / 128; t += blockDim.x >> 5) {
+      float ss = 0.f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int f = t * 128 + 32 * i + lane;
+        const float x = xs[f];
+        store_act<T>(w.A, gridDim.x, dm.d, r, f, x * to_f(gain[f]));
+        ss += x * x;
+      }
+      ss = warp_sum(ss);
+      if (lane == 0) ssq[(size_t)t * gridDim.x + r] = ss;
+    }
+    return;
+  }
   norm_row_from_smem<T>(xs, dm.d, gain, dm.eps, w.A, gridDim.x, r, nullptr, nullptr, red);
 }
 

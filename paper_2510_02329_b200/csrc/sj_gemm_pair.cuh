@@ -51,6 +51,12 @@ constexpr int kPairSegKB = 16, kPairShortKB = 32;   // K blocks of 64 per accumu
 constexpr int kPairMaxSplit = 4;        // pairs that share an item's K (a cluster of 8)
 constexpr double kPairHbmBytesPerClk = 3600;   // HBM against the SM clock, for the host's choice of a geometry
 constexpr int kPairXchClk = 3000;       // an exchange between the splits
+// "My sums have been read" barriers per epilogue group, taken in turn by successive exchanges.  A split that receives
+// nothing in an exchange (all of the row block's chunks belong to others) does not wait for its partners there and may
+// finish it before a partner has looked at the phase of the exchange before; on one barrier that phase would be overtaken,
+// and a wait that knows only its parity would see it as not yet complete.  To finish the second exchange after, a split
+// needs its partners' arrivals of the first, which they give after their look: two barriers are never overtaken.
+constexpr int kPairFreeBars = 2;
 constexpr uint32_t kPairSpin = 1u << 22;
 
 enum PairSite { PAIR_QKV = 0, PAIR_RES = 1, PAIR_GU = 2, PAIR_LM = 3 };
@@ -78,7 +84,8 @@ struct PairParams {
 
 struct PairCtl {
   uint64_t full[kPairMaxStages], empty[kPairMaxStages], tmem_full[2], tmem_empty[2];
-  uint64_t xch_full[2], xch_free[2];   // per epilogue group: the other splits' sums are here; the others have read mine
+  uint64_t xch_full[2];                  // per epilogue group: the other splits' sums are here
+  uint64_t xch_free[2][kPairFreeBars];   // the others have read mine
   uint32_t tmem_base;
   int abort_flag;
   float inv[kPairMaxRows];
@@ -189,7 +196,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       mbar_init(smem_u32(&ctl->tmem_full[i]), 1);
       mbar_init(smem_u32(&ctl->tmem_empty[i]), 16);   // the epilogue warps of both CTAs
       mbar_init(smem_u32(&ctl->xch_full[i]), 1);   // and the bytes of the other splits' sums
-      mbar_init(smem_u32(&ctl->xch_free[i]), 4 * max(S - 1, 1));   // a group's warps of every other split
+      for (int k = 0; k < kPairFreeBars; ++k) mbar_init(smem_u32(&ctl->xch_free[i][k]), 4 * max(S - 1, 1));   // a group's warps of every other split
     }
     ctl->abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -374,7 +381,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             if (r_lo + 16 * grp + 32 * j < r_hi) bytes += (uint32_t)(S - 1) * 8192u;
           mbar_expect_tx(smem_u32(&ctl->xch_full[grp]), bytes);
         }
-        if (n_x > 0) xch_wait(&ctl->xch_free[grp], (uint32_t)(n_x - 1) & 1u);
+        if (n_x > 0) xch_wait(&ctl->xch_free[grp][(n_x - 1) % kPairFreeBars], (uint32_t)((n_x - 1) / kPairFreeBars) & 1u);
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           if (!(mine >> j & 1u) && r_lo + 16 * grp + 32 * j < r_hi) {
@@ -400,7 +407,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         __syncwarp();
         if (lane == 0)
           for (int f = 0; f < S; ++f)
-            if (f != split) cluster_arrive(smem_u32(&ctl->xch_free[grp]), 2 * f + rank);
+            if (f != split) cluster_arrive(smem_u32(&ctl->xch_free[grp][n_x % kPairFreeBars]), 2 * f + rank);
         ++n_x;
       }
 

@@ -31,6 +31,28 @@ def test_split_projections(shape, n, gamma):
         case.close()
 
 
+def test_exchanges_that_one_split_receives_in():
+    """Down has 67 tiles and 286 K blocks: with 48 rows its clusters of three pairs take two items each (B200), and the second
+    epilogue group's only chunk belongs to the first split, so the others finish an exchange without waiting."""
+    shape = synth.ModelShape("wide-down", 1, 67 * 128, 2, 1, 128, 143 * 128, 512)
+    case = harness.Case(shape, torch.bfloat16, [3 + 61 * b for b in range(8)], 5, seed=19, cache="fill", gen_device="cuda").gpu_setup(max_rows=48)
+    try:
+        v, f = case.run_oracle(orc.GREEDY)
+        want = np.stack([x.hidden for x in f])
+        off = lambda g: np.linalg.norm(g["hidden"] - want)
+        case.target.set_option("step_impl", 1)
+        persistent = case.run_gpu(orc.GREEDY)      # no exchange; off by as much, up to 3.2e-3: the fp16 copies of the block's own rows
+        case.target.set_option("step_impl", 0)
+        runs = [case.run_gpu(orc.GREEDY) for _ in range(20)]
+        rep = harness.compare(case, v, f, runs[0], orc.GREEDY)
+        assert rep.exact + rep.margin == 8
+        assert off(runs[0]) <= 1.1 * off(persistent)
+        for again in runs[1:]:
+            np.testing.assert_array_equal(again["hidden"], runs[0]["hidden"])
+    finally:
+        case.close()
+
+
 def test_captured_steps_belong_to_their_cache():
     """Two caches of one target, the same call on both in turn: a captured step holds its cache's pointers."""
     from paper_2510_02329_b200 import binding

@@ -32,10 +32,7 @@ class SpeculativeDecoder:
         self.pending: List[int] = [0] * self.B        # next token to feed (not yet in the caches)
         self.cycles = 0
         self.accepted_total = 0
-        # device buffers of a cycle: the draft's decode steps write `_step`, their tokens collect in `_drafts`
-        self._step, self._dummy = binding.VerifyBuffers(self.B, 1), torch.zeros((self.B, 1), dtype=torch.int32, device="cuda")
-        self._drafts = torch.zeros((self.B, self.gamma), dtype=torch.int32, device="cuda")
-        self._block = binding.VerifyBuffers(self.B, self.gamma)
+        self._made_for = None                         # (B, gamma) of the cycle's device buffers
 
     # ---- set-up -------------------------------------------------------------------------------
     def prefill(self, prompts: Sequence[Sequence[int]]) -> None:
@@ -58,11 +55,22 @@ class SpeculativeDecoder:
         binding.verify(target, kv, seqs, dummy, out, mode=binding.MODE_GREEDY, use_align=False, use_judge=False, commit=True)
         return out.next_token
 
+    def _buffers(self) -> None:
+        """Device buffers of a cycle, kept while B and gamma stay: the draft's passes write `_step`, their tokens collect in
+        `_drafts`, the verification writes `_block`."""
+        if self._made_for == (self.B, self.gamma):
+            return
+        self._step, self._dummy = binding.VerifyBuffers(self.B, 1), torch.zeros((self.B, 1), dtype=torch.int32, device="cuda")
+        self._drafts = torch.zeros((self.B, self.gamma), dtype=torch.int32, device="cuda")
+        self._block = binding.VerifyBuffers(self.B, self.gamma)
+        self._made_for = (self.B, self.gamma)
+
     # ---- one cycle ----------------------------------------------------------------------------------
     def cycle(self, use_judge: bool = True, theta: float = -1.0, top_k: int = 0) -> List[List[int]]:
         """Draft gamma tokens, verify, commit.  Returns, per sequence, the tokens this cycle appended to the
         output: the accepted drafts followed by the token the target emitted."""
         B, gamma = self.B, self.gamma
+        self._buffers()
         self.draft_kv.set_pending(self.seq_ids, self.pending)
         self.target_kv.set_pending(self.seq_ids, self.pending)
         # The draft's gamma sequential passes, queued on its stream without waiting for any: a pass finds its token in the

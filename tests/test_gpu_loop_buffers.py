@@ -1,0 +1,37 @@
+"""The host loop's device buffers: they follow the attributes that a cycle reads, and nobody gets their memory while a queued pass
+still writes it."""
+import pytest
+import torch
+
+from paper_2510_02329_b200 import loop, synth
+from test_gpu_extensions import _target_and_cache
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture
+def pair():
+    """A target, the same model as its own draft, and a third copy to decode alone; fp32, so every draft is accepted."""
+    made = [_target_and_cache(synth.TINY, torch.float32, 0, 2)[1:] for _ in range(3)]
+    yield made
+    torch.cuda.synchronize()
+    for target, kv in made:
+        kv.close()
+        target.close()
+
+
+def test_cycles_follow_gamma_and_the_sequences(pair):
+    (draft, draft_kv), (target, target_kv), (solo, solo_kv) = pair
+    prompts = [[int(t) for t in synth.token_ids(synth.TINY.vocab, n, seed=60 + n, stream=3)] for n in (9, 5)]
+    dec = loop.SpeculativeDecoder(draft, draft_kv, target, target_kv, [0, 1], 4)
+    dec.prefill(prompts)
+    got = [[], []]
+    for gamma in (4, 7, 2, 5):
+        dec.gamma = gamma
+        for o, p in zip(got, dec.cycle(use_judge=False)):
+            assert len(p) == gamma + 1
+            o.extend(p)
+    dec.seq_ids, dec.B, dec.lens, dec.pending = [1], 1, dec.lens[1:], dec.pending[1:]
+    got[1].extend(dec.cycle(use_judge=False)[0])
+    for s in (0, 1):
+        assert got[s] == loop.greedy_decode(solo, solo_kv, s, prompts[s], len(got[s]))

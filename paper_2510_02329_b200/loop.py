@@ -20,6 +20,14 @@ import torch
 from . import binding
 
 
+def _used_on(stream: torch.cuda.Stream, *buffers) -> None:
+    """The buffers (tensors, VerifyBuffers) are used by work queued on `stream`: nobody gets their memory before it has run."""
+    for b in buffers:
+        for t in [b] if isinstance(b, torch.Tensor) else vars(b).values():
+            if t is not None:
+                t.record_stream(stream)
+
+
 class SpeculativeDecoder:
     """A draft (target, cache) pair and a verifying (target, cache) pair over the same sequence slots."""
 
@@ -52,6 +60,7 @@ class SpeculativeDecoder:
         n = len(seqs)
         out = binding.VerifyBuffers(n, 1)
         dummy = torch.zeros((n, 1), dtype=torch.int32, device="cuda")
+        _used_on(target.stream, dummy, out)
         binding.verify(target, kv, seqs, dummy, out, mode=binding.MODE_GREEDY, use_align=False, use_judge=False, commit=True)
         return out.next_token
 
@@ -63,6 +72,8 @@ class SpeculativeDecoder:
         self._step, self._dummy = binding.VerifyBuffers(self.B, 1), torch.zeros((self.B, 1), dtype=torch.int32, device="cuda")
         self._drafts = torch.zeros((self.B, self.gamma), dtype=torch.int32, device="cuda")
         self._block = binding.VerifyBuffers(self.B, self.gamma)
+        for stream in (self.draft.stream, self.target.stream):
+            _used_on(stream, self._dummy, self._drafts, self._step, self._block)
         self._made_for = (self.B, self.gamma)
 
     # ---- one cycle ----------------------------------------------------------------------------------

@@ -35,3 +35,25 @@ def test_cycles_follow_gamma_and_the_sequences(pair):
     got[1].extend(dec.cycle(use_judge=False)[0])
     for s in (0, 1):
         assert got[s] == loop.greedy_decode(solo, solo_kv, s, prompts[s], len(got[s]))
+
+
+def test_a_queued_pass_keeps_its_buffers(pair):
+    """A cycle that accepts everything ends with a draft pass that nobody waits for: while it is held back, no new tensor of the
+    same size gets the memory that it will write."""
+    (draft, draft_kv), (target, target_kv), _ = pair
+    dec = loop.SpeculativeDecoder(draft, draft_kv, target, target_kv, [0, 1], 3)
+    dec.prefill([[int(t) for t in synth.token_ids(synth.TINY.vocab, n, seed=60 + n, stream=3)] for n in (9, 5)])
+    dec.cycle(use_judge=False)
+    plain = loop.SpeculativeDecoder._decode
+
+    def held_back(target, kv, seqs):
+        with torch.cuda.stream(target.stream):
+            torch.cuda._sleep(200_000_000)            # about a tenth of a second on the draft's stream
+        return plain(target, kv, seqs)
+
+    dec._decode = held_back
+    dec.cycle(use_judge=False)
+    got = [torch.full((2,), -7, dtype=torch.int32, device="cuda") for _ in range(64)]
+    got += [torch.full((2, 1), -7.0, device="cuda") for _ in range(64)]
+    torch.cuda.synchronize()
+    assert all(bool((t == -7).all()) for t in got)

@@ -97,6 +97,7 @@ class SpeculativeDecoder:
         binding.verify(self.target, self.target_kv, self.seq_ids, drafts, out, mode=binding.MODE_GREEDY,
                        use_align=True, use_judge=use_judge, theta=theta, top_k=top_k, commit=True)
         self.target.sync()
+        self.draft.sync()      # its passes have ended too: the target's stream waited for them; this asks how
         n_acc = out.accepted_len.cpu().numpy()
         emitted = out.next_token.cpu().numpy()
         d_host = drafts.cpu().numpy()

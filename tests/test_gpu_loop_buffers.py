@@ -57,3 +57,18 @@ def test_a_queued_pass_keeps_its_buffers(pair):
     got += [torch.full((2, 1), -7.0, device="cuda") for _ in range(64)]
     torch.cuda.synchronize()
     assert all(bool((t == -7).all()) for t in got)
+
+
+def test_a_draft_pass_that_timed_out_is_reported():
+    from paper_2510_02329_b200 import binding
+    shape = synth.ModelShape("gqa-small", 3, 256, 4, 2, 64, 512, 1024, rope_theta=5e5)
+    (_, target, target_kv), (_, draft, draft_kv) = (_target_and_cache(shape, torch.bfloat16, 0, 1) for _ in range(2))
+    try:
+        dec = loop.SpeculativeDecoder(draft, draft_kv, target, target_kv, [0], 3)
+        dec.prefill([[int(t) for t in synth.token_ids(shape.vocab, 9, seed=60, stream=3)]])
+        draft.expire_wait(0)
+        with pytest.raises(binding.SjError) as e:
+            dec.cycle()
+        assert e.value.status == 7
+    finally:
+        target_kv.close(); draft_kv.close(); target.close(); draft.close()

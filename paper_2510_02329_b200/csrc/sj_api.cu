@@ -227,6 +227,7 @@ struct sj_target {
   size_t att_chunks_cap = 0;
   int att_rows_cap = 0;
   size_t tc_part_cap = 0;   // floats in tc_m / tc_l
+  size_t p_cap = 0, logits_cap = 0;   // floats in work.P, work.logits
   int pair_clusters[kPairMaxSplit + 1] = {};
   std::map<StepKey, cudaGraphExec_t> graphs;
   std::map<std::pair<const void*, int>, CUtensorMap> act_maps;   // per activation matrix and row count
@@ -372,10 +373,32 @@ static sj_status alloc_partials(sj_target* t, Work& W, int R) {
     n = 0;
     for (TcSite* s : {&t->s_qkv, &t->s_o, &t->s_gu, &t->s_down}) n = std::max(n, (size_t)s->max_slots * R * s->N);
   }
-  // the logits' place as well: they are written when the last projection's sums have been read
-  n = std::max(n, (size_t)R * c.vocab);
   const sj_status st = dev_alloc(t, &W.P, n);
-  W.logits = W.P;
+  if (st == SJ_OK) t->p_cap = n;
+  return st;
+}
+
+// Room for the [R, V] logits that sampling and the CUDA-core LM head keep, taken by the first step that needs it (outside any
+// capture): targets that only decode greedily never do.  The partial sums' buffer where it is large enough: the logits are
+// written when the last projection's sums have been read.
+static sj_status ensure_logits(sj_target* t, size_t R) {
+  const size_t need = R * t->dm.V;
+  if (need <= t->logits_cap) return SJ_OK;
+  CU_TRY(cudaStreamSynchronize(t->stream));
+  clear_graphs(t);
+  if (t->work.logits && t->work.logits != t->work.P) {
+    counted_free(t->work.logits);
+    t->owned.erase(std::remove(t->owned.begin(), t->owned.end(), (void*)t->work.logits), t->owned.end());
+  }
+  t->work.logits = nullptr;
+  t->logits_cap = 0;
+  if (need <= t->p_cap) {
+    t->work.logits = t->work.P;
+    t->logits_cap = t->p_cap;
+    return SJ_OK;
+  }
+  const sj_status st = dev_alloc(t, &t->work.logits, need);
+  if (st == SJ_OK) t->logits_cap = need;
   return st;
 }
 
@@ -1258,7 +1281,7 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
     if (pair_usable(t, kv))
       TIMED_ST("gemm_lm_head", launch_pair(t, kv, PAIR_LM, n_vtiles, dm.d, W.A, &t->m_lm, nullptr, nullptr, R, pdl, W, PairOut()));
     else
-      TIMED("gemm_lm_head", launch_tc(t, t->s_lm, mA_d, &t->m_lm, nullptr, nullptr, R, pdl, true, W));   // W: no [R, V] logit store
+      TIMED("gemm_lm_head", launch_tc(t, t->s_lm, mA_d, &t->m_lm, nullptr, nullptr, R, pdl, true, W));   // stores logits where W has them
   } else {
     GemmSegs g{{t->lm_head, nullptr, nullptr}, {dm.V, 0, 0}, 1};
     TIMED("gemm_cudacore", launch_simt<T>(t, W.A, g, W.logits, R, dm.V, dm.d, pdl));
@@ -1522,6 +1545,7 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
   }
   if ((!simt_attn || use_mega) && kv->has_tm_pool)
     if ((st = ensure_attn_partials(t, B, rows)) != SJ_OK) return st;
+  if (use_logits && (st = ensure_logits(t, R)) != SJ_OK) return st;
 
   // per-call arguments: one small copy (the driver stages pageable memory before returning)
   StepArgs h;

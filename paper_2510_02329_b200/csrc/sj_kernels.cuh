@@ -40,9 +40,9 @@ struct Work {
   float* tgt_logit;  // [R]   logit of the drafted token d_{j+1} in row j
   float* tgt_pre;    // [R]   the same logit (raw), computed BEFORE the LM head when the top-k test needs it to count ranks
   RowStat* rowstat;  // [R]   merged statistics
-  float* logits;     // fp32 logit scratch, or null: [R, V] for the CUDA-core LM head; [B, V] in sampling mode with
-                     // the tensor-core LM head (only the one row per sequence that the emitted token is drawn from)
-void* Asel;        // GEMM input planes of one row (the last of a prefill), K = d
+  float* logits;     // [R, V] fp32, or null: stored for the CUDA-core LM head and in sampling mode (the row that a token is
+                     // drawn from is known only after the head); may be P
+  void* Asel;        // GEMM input planes of one row (the last of a prefill), K = d
   double2* rs_part;  // [B][chunks of the vocabulary] sums of p and max(0, p - q) of the row that is drawn from
   const double* inv_freq;  // [hd/2] rope_theta^(-2i/hd)
   const float* judge_w;    // [d]

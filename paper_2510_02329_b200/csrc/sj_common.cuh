@@ -218,7 +218,8 @@ __device__ __forceinline__ RowStat stat_merge_any(const RowStat& a, const RowSta
 
 // Merged statistics of the block rows [r0, r0 + rows) over all vocabulary tiles, by the eight warps of a block: a warp
 // takes half of a row's tiles, 16 of them per lane in flight (a thread walking through its tiles one load at a time took
-// 4 us a row, 60 us of a 9-row step in all).  part: [rows][2], shared memory; the caller synchronises and merges the halves.
+// 4 us a row, 60 us of a 9-row step in all).  part: [rows][2], shared memory; the caller synchronises and merges the halves
+// with merge_row_halves().
 __device__ __forceinline__ void merge_row_stats(const RowStat* stats, int n_vtiles, int R, int r0, int rows, int warp, int lane,
                                                 RowStat (*part)[2]) {
   const int half = (n_vtiles + 1) / 2;
@@ -236,7 +237,7 @@ __device__ __forceinline__ void merge_row_stats(const RowStat* stats, int n_vtil
       int arg = 0x7fffffff;
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
-        if (tb + 32 * k + lane >= t1) { raw[k].x = -INFINITY; raw[k].w = 0.f; }
+        if (tb + 32 * k + lane >= t1) { raw[k].x = -INFINITY; raw[k].z = __int_as_float(0x7fffffff); raw[k].w = 0.f; }
         const int ak = __float_as_int(raw[k].z);
         if (raw[k].x > m || (raw[k].x == m && ak < arg)) { m = raw[k].x; arg = ak; }
       }
@@ -259,6 +260,12 @@ __device__ __forceinline__ void merge_row_stats(const RowStat* stats, int n_vtil
     }
     if (lane == 0) part[j][item & 1] = a;
   }
+}
+
+__device__ __forceinline__ RowStat merge_row_halves(const RowStat (&part)[2]) {
+  RowStat a = stat_merge_any(part[0], part[1]);
+  if (a.arg == 0x7fffffff) a.arg = 0;   // no logit is larger than -infinity (all are NaN): a token of the vocabulary all the same
+  return a;
 }
 
 }  // namespace sj

@@ -671,7 +671,7 @@ static __global__ void k_finalize(const StepArgs* __restrict__ args, KvView kv, 
   }
   __syncthreads();
   if (tid < rows) {
-    rs[tid] = stat_merge_any(part[tid][0], part[tid][1]);
+    rs[tid] = merge_row_halves(part[tid]);
     w.rowstat[b * rows + tid] = rs[tid];
   }
   __syncthreads();

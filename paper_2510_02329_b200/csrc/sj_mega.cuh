@@ -876,7 +876,7 @@ __device__ __forceinline__ void mega_finalize(MegaCtl* ctl, const MegaParams& p,
   }
   bar_sync(1, kMegaWorkers);
   if (wt < rows) {
-    ctl->rs[wt] = stat_merge_any(ctl->u.part[wt][0], ctl->u.part[wt][1]);
+    ctl->rs[wt] = merge_row_halves(ctl->u.part[wt]);
     w.rowstat[b * rows + wt] = ctl->rs[wt];
   }
   if (args->dbg_hidden) {

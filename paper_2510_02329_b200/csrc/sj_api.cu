@@ -188,7 +188,7 @@ struct LayerW {
 };
 
 struct StepKey {
-  const sj_kv* kv;   // a captured step holds its cache's pointers; destroying the cache drops the graphs
+  const sj_kv* kv;   // a captured step holds its cache's pointers; destroying the cache drops its graphs
   int B, gamma, mode, chunk_len, gemm_impl, attn_impl, pdl, top_k;
   bool operator<(const StepKey& o) const {
     return std::tie(kv, B, gamma, mode, chunk_len, gemm_impl, attn_impl, pdl, top_k) <
@@ -791,7 +791,11 @@ extern "C" sj_status sj_kv_create(sj_target* t, int max_seqs, long max_pages, in
 extern "C" sj_status sj_kv_destroy(sj_kv* kv) {
   if (!kv) return SJ_OK;
   cudaStreamSynchronize(kv->t->stream);
-  clear_graphs(kv->t);  // captured steps hold this cache's pointers
+  for (auto it = kv->t->graphs.begin(); it != kv->t->graphs.end();) {   // captured steps hold this cache's pointers
+    if (it->first.kv != kv) { ++it; continue; }
+    cudaGraphExecDestroy(it->second);
+    it = kv->t->graphs.erase(it);
+  }
   counted_free(kv->view.pool);
   counted_free(kv->d_block_table);
   delete kv;

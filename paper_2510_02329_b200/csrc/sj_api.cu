@@ -196,6 +196,14 @@ struct StepKey {
   }
 };
 
+struct StepGraph {
+  cudaGraphExec_t exec;
+  unsigned long used;   // sj_target::graph_clock at its last use
+};
+// Captured steps that a target keeps; beyond them the one that was not used for the longest time goes.  Two batch sizes' worth of
+// SJ_MAX_BATCH; a captured step of 32 layers holds about half a megabyte, mostly on the device (B200: 64 of them 21 MB).
+constexpr size_t kMaxStepGraphs = 512;
+
 struct sj_target {
   sj_model_config cfg;
   Dims dm;
@@ -229,7 +237,8 @@ struct sj_target {
   size_t tc_part_cap = 0;   // floats in tc_m / tc_l
   size_t p_cap = 0, logits_cap = 0;   // floats in work.P, work.logits
   int pair_clusters[kPairMaxSplit + 1] = {};
-  std::map<StepKey, cudaGraphExec_t> graphs;
+  std::map<StepKey, StepGraph> graphs;
+  unsigned long graph_clock = 0;
   std::map<std::pair<const void*, int>, CUtensorMap> act_maps;   // per activation matrix and row count
   std::map<std::tuple<const void*, int, int>, CUtensorMap> pair_maps;   // the same per box height, for the paired projections
   // prefill in wide blocks (allocated by the first call that can use it): a workspace of kPrefillRows rows, the tokens
@@ -256,7 +265,7 @@ struct sj_kv {
 };
 
 static void clear_graphs(sj_target* t) {
-  for (auto& kvp : t->graphs) cudaGraphExecDestroy(kvp.second);
+  for (auto& kvp : t->graphs) cudaGraphExecDestroy(kvp.second.exec);
   t->graphs.clear();
 }
 
@@ -793,7 +802,7 @@ extern "C" sj_status sj_kv_destroy(sj_kv* kv) {
   cudaStreamSynchronize(kv->t->stream);
   for (auto it = kv->t->graphs.begin(); it != kv->t->graphs.end();) {   // captured steps hold this cache's pointers
     if (it->first.kv != kv) { ++it; continue; }
-    cudaGraphExecDestroy(it->second);
+    cudaGraphExecDestroy(it->second.exec);
     it = kv->t->graphs.erase(it);
   }
   counted_free(kv->view.pool);
@@ -1597,9 +1606,16 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
       e = cudaGraphInstantiate(&exec, graph, 0);
       cudaGraphDestroy(graph);
       CU_TRY(e);
-      it = t->graphs.emplace(key, exec).first;
+      if (t->graphs.size() >= kMaxStepGraphs) {
+        auto oldest = std::min_element(t->graphs.begin(), t->graphs.end(), [](auto& x, auto& y) { return x.second.used < y.second.used; });
+        CU_TRY(cudaStreamSynchronize(t->stream));
+        cudaGraphExecDestroy(oldest->second.exec);
+        t->graphs.erase(oldest);
+      }
+      it = t->graphs.emplace(key, StepGraph{exec, 0}).first;
     }
-    CU_TRY(cudaGraphLaunch(it->second, t->stream));
+    it->second.used = ++t->graph_clock;
+    CU_TRY(cudaGraphLaunch(it->second.exec, t->stream));
   } else {
     st = t->bf ? enqueue_step<bf16>(t, kv, B, gamma, a->mode, h.top_k, chunk_len, use_logits, chunk_need_base)
                : enqueue_step<float>(t, kv, B, gamma, a->mode, h.top_k, chunk_len, use_logits, chunk_need_base);

@@ -102,11 +102,13 @@ sj_status sj_load_judge_head(sj_target *t, const float *w_host, float bias, floa
  *   "attn_impl"  0 = CUDA-core kernel,  1 = tensor-core (mma.sync, fp16 operands) kernel (bf16 models),
  *                2 = tcgen05 kernel (bf16 models, head_dim 128, at most 128 query rows per KV head and sequence, else
  *                it runs as 1); default: 2 at head_dim 128, else 1, for bf16 models; 0 for fp32 models.
+ *                Of steps that run as one kernel per stage: the persistent kernel has an mma.sync attention of its own, and
+ *                with 0 the default "step_impl" takes it for every step that it can run.
  *   "attn_tcgen05_min_tiles"  n >= 0 (default 4; 0 = always): with "attn_impl" 2, a step whose caches hold at least this
  *                many 128-key tiles per SM runs as one kernel per stage, with the tcgen05 attention, whatever "step_impl"
  *   "step_impl"  1 = the whole step as one persistent cooperative kernel (bf16, tcgen05 GEMMs, at most 48
- *                block rows), 0 = one kernel per stage, 2 = whichever is the faster for the step's rows and the model's
- *                widths (default when the shape allows)
+ *                block rows), 0 = one kernel per stage, 2 = whichever is the faster for the step's rows and sequences and
+ *                the model's widths (default when the shape allows)
  *   "attn_two_term_layers"  n >= 0 (default 1): in layers [0, n) the tensor-core attention carries queries and
  *                probabilities as a sum of two fp16 terms (twice the MMAs).  Where the residual stream is still
  *                small (the first layer: an embedding row), the attention output is most of what the next

@@ -1312,12 +1312,20 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
 
 // The whole step as one cooperative launch per chunk of kMegaMaxLayers layers.  "step_impl" 1 takes it up to kMegaMaxRows
 // rows; the default (2) where it is the faster of the two (B200, us a step, persistent / per stage):
-//   rows: its barriers cost less than launches, the paired projections are the better GEMM, and at head dimension 128 the
-//     tcgen05 kernel the better attention.  16 layers, 8B-shaped: 9 rows 1928 / 2088, 17 rows 2198 / 2275, 18 rows
-//     2250 / 2113, 24 rows 2359 / 2136; 32B-shaped: 9 rows 3271 / 3412, 17 rows 3661 / 3648, 18 rows 3690 / 3476; 1B-shaped
-//     (head dimension 64): 9 rows 1039 / 1246, 18 rows 1222 / 1250, 24 rows 1270 / 1267, 36 rows 1487 / 1384;
-//   widths: where gate/up has fewer units than there are blocks, the phases stream nothing that could hide the barriers
-//     or the 0.3 MB of code.  2 layers: d 256, ffn 1024 147 / 121, 1B-shaped 240 / 257, 8B-shaped 405 / 430.
+//   widths: a phase has to stream for longer than its barrier takes: ten 16 KiB units of gate/up for every block, 3.6 us at the
+//     copy rate.  One sequence, 9 rows, 24 layers: d 512, ffn 2048 (1.7 units) 1419 / 1054; d 1024, ffn 4096 (6.9) 1232 / 1161; d 1536,
+//     ffn 6144 (15.6) 1197 / 1257; 1B-shaped (27.7, 16 layers) 1012 / 1274.
+//   rows: its barriers cost less than launches, the paired projections are the better GEMM, and the per-stage attention kernels
+//     spread several sequences better.  8B-shaped, 16 layers, 1024 / 4000 keys a sequence: one sequence, 12 rows 1895 / 2000 and
+//     2029 / 2114, 16 rows 2049 / 2005 and 2189 / 2116, 17 rows 2102 / 2191 and 2322 / 2318, 24 rows 2233 / 2233 and 2475 / 2390; two
+//     sequences, 12 rows 1903 / 2024 and 2083 / 2065, 16 rows 1997 / 2033 and 2233 / 2075, 18 rows 2094 / 2103 and 2364 / 2154; four, 12 rows
+//     1956 / 1993, 16 rows 2056 / 2007; eight, 16 rows 2166 / 2016.  32B-shaped, 12 layers: one sequence, 9 rows 2470 / 2543, 16 rows
+//     2654 / 2680, 17 rows 2773 / 2754; two, 12 rows 2542 / 2608, 16 rows 2649 / 2608; four, 12 rows 2588 / 2592, 16 rows 2664 / 2594.
+//     (Between 12 and 24 rows of one sequence the two are within 4 % of each other, either way: the line is the last row count
+//     at which neither key count is slower.)
+//     1B-shaped (head dimension 64; no per-stage tcgen05 attention): one sequence, 20 rows 1196 / 1224, 24 rows 1232 / 1222; two, 24 rows
+//     1254 / 1260; four, 16 rows 1158 / 1214, 24 rows 1287 / 1287, 36 rows 1470 / 1296; six, 18 rows 1234 / 1220; eight, 16 rows
+//     1201 / 1187, 24 rows 1289 / 1239.
 // Caches of several 128-key tiles per SM (and head dimension 128): its mma.sync attention takes about three times as long a
 // key as the tcgen05 kernel (8B-shaped, 9 rows: 8000 keys, 3.4 tiles, 2156 / 2159).
 static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma, long total_keys) {
@@ -1325,8 +1333,8 @@ static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma, l
   if (t->opt_step == 0 || t->opt_gemm != 1 || !t->mega_shapes || !kv->has_tm_pool || R > kMegaMaxRows || group * rows > 16 * 6 || !t->stream)
     return false;
   if (t->dm.hd == 128 && t->opt_attn == 2 && total_keys * t->dm.Hkv / kT5Keys / t->sm_count >= t->opt_a5_min_tiles) return false;
-  return t->opt_step == 1 || t->opt_attn == 0 ||
-         (R <= (t->dm.hd == 128 ? kMegaAutoRows128 : kMegaAutoRows64) && (t->dm.F / 64) * (t->dm.d / kBK) >= t->sm_count);
+  const int most = t->dm.hd == 128 ? (B == 1 ? 17 : 12) : (B <= 4 ? 24 : 12);
+  return t->opt_step == 1 || t->opt_attn == 0 || (R <= most && (long)(t->dm.F / 64) * (t->dm.d / kBK) >= 10L * t->sm_count);
 }
 
 static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode, bool use_logits) {

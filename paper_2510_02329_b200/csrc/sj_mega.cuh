@@ -45,7 +45,6 @@ constexpr int kMegaThreads = 384;
 constexpr int kMegaWorkers = 256;
 constexpr int kMegaMaxLayers = 32;   // per launch (tensor maps travel as kernel parameters)
 constexpr int kMegaMaxRows = 48;
-constexpr int kMegaAutoRows128 = 17, kMegaAutoRows64 = 24;   // rows that run here by default, by head dimension
 constexpr int kMegaMaxStages = 12;
 constexpr uint32_t kMegaSpin = 1u << 22;
 constexpr int kMegaRegsLight = 80;    // registers per thread of warps 0..3 after reallocation

@@ -393,11 +393,13 @@ static sj_status alloc_partials(sj_target* t, Work& W, int R) {
 static sj_status ensure_logits(sj_target* t, size_t R) {
   const size_t need = R * t->dm.V;
   if (need <= t->logits_cap) return SJ_OK;
-  CU_TRY(cudaStreamSynchronize(t->stream));
-  clear_graphs(t);
-  if (t->work.logits && t->work.logits != t->work.P) {
-    counted_free(t->work.logits);
-    t->owned.erase(std::remove(t->owned.begin(), t->owned.end(), (void*)t->work.logits), t->owned.end());
+  if (t->work.logits) {   // captured steps hold it
+    CU_TRY(cudaStreamSynchronize(t->stream));
+    clear_graphs(t);
+    if (t->work.logits != t->work.P) {
+      counted_free(t->work.logits);
+      t->owned.erase(std::remove(t->owned.begin(), t->owned.end(), (void*)t->work.logits), t->owned.end());
+    }
   }
   t->work.logits = nullptr;
   t->logits_cap = 0;

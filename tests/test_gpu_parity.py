@@ -379,26 +379,25 @@ def test_tcgen05_attention(name, shape, kv_lens, gamma):
         case.close()
 
 
-# at least 49 block rows each: the persistent kernel's ring stages then hold a 32 KiB key or value tile
-A5_CASES = [
+# tile edges (64 and 128 keys), an empty cache, one and two query chunks per group, 41 to 72 rows
+T5_EDGE_CASES = [
     ("llama-8b-cut2-b6", synth.LLAMA_8B.cut(2), [4096, 210, 1, 129, 128, 777], 8),       # config 3 widths; 36 query rows
     ("llama-8b-cut1-edges", synth.LLAMA_8B.cut(1), [1, 63, 64, 65, 0, 127, 128, 129, 255, 256, 257, 300], 4),  # tile edges; an empty cache
     ("llama-8b-cut2-g10", synth.LLAMA_8B.cut(2), [3000, 500, 40, 1000, 2000], 10),      # 44 query rows
-    ("qwen-32b-cut1-b8", synth.QWEN_32B.cut(1), [40, 1300, 515, 2048, 1, 900, 128, 3000], 8),  # group 5 (45 query rows), qkv bias, 36 KiB stages
+    ("qwen-32b-cut1-b8", synth.QWEN_32B.cut(1), [40, 1300, 515, 2048, 1, 900, 128, 3000], 8),  # group 5 (45 query rows), qkv bias
 ]
 
 
-@pytest.mark.parametrize("name,shape,kv_lens,gamma", A5_CASES, ids=[c[0] for c in A5_CASES])
-def test_tcgen05_attention_in_persistent_kernel(name, shape, kv_lens, gamma):
-    """The persistent kernel's tcgen05 attention phase (128-key tiles through the shared ring, two issuing threads),
-    forced on whatever the cache lengths, against the oracle and against the mma.sync phase on the same inputs."""
+@pytest.mark.parametrize("name,shape,kv_lens,gamma", T5_EDGE_CASES, ids=[c[0] for c in T5_EDGE_CASES])
+def test_tcgen05_attention_at_tile_edges(name, shape, kv_lens, gamma):
+    """k_attn_t5 against the oracle and against the mma.sync kernel on the same inputs, one kernel per stage each."""
     case = harness.Case(shape, torch.bfloat16, kv_lens, gamma, seed=8, cache="fill",
                         gen_device="cuda").gpu_setup(max_rows=len(kv_lens) * (gamma + 1))
     try:
         for mode, T in [(orc.GREEDY, 1.0), (orc.SAMPLING, 1.0)]:
-            rep, g = _run(case, mode, T, options={"gemm_impl": 1, "step_impl": 1, "attn_impl": 2, "attn_tcgen05_min_tiles": 0})
+            rep, g = _run(case, mode, T, options={"gemm_impl": 1, "step_impl": 0, "attn_impl": 2})
             assert rep.exact + rep.margin == len(kv_lens)
-            rep1, g1 = _run(case, mode, T, options={"gemm_impl": 1, "step_impl": 1, "attn_impl": 1})
+            rep1, g1 = _run(case, mode, T, options={"gemm_impl": 1, "step_impl": 0, "attn_impl": 1})
             d = np.abs(g["hidden"] - g1["hidden"]).max()
             assert 0 < d < 5e-3 or max(kv_lens) == 0   # close, and not the same code path
             print(name, "mode", mode, rep, "vs mma.sync", d)
@@ -406,17 +405,52 @@ def test_tcgen05_attention_in_persistent_kernel(name, shape, kv_lens, gamma):
         case.close()
 
 
-def test_more_than_256_rows_keep_both_activation_planes():
-    """29 sequences x 9 rows = 261 rows: the two bf16 activation planes no longer fit side by side in tensor
-    memory and the lo plane is accumulated into the hi plane's columns."""
+# 13 to 48 rows at head dimension 128: the persistent kernel with every tile finished by rows
+PERSISTENT_CASES = [
+    ("llama-8b-cut2-13", synth.LLAMA_8B.cut(2), [777], 12),                                  # 13 rows: a second word of one row and none
+    ("llama-8b-cut2-g16", synth.LLAMA_8B.cut(2), [210], 16),                                 # 17 rows: a chunk of one row
+    ("llama-8b-cut1-edges", synth.LLAMA_8B.cut(1), [1, 63, 64, 65, 0, 129], 4),              # 30 rows; tile edges; an empty cache
+    ("qwen-32b-cut1-b3", synth.QWEN_32B.cut(1), [40, 515, 128], 8),                          # 27 rows, group 5, qkv bias
+    ("qwen-32b-cut1-48", synth.QWEN_32B.cut(1), [40, 300, 1, 128], 11),                      # 48 rows: the most there are
+]
+
+
+@pytest.mark.parametrize("name,shape,kv_lens,gamma", PERSISTENT_CASES, ids=[c[0] for c in PERSISTENT_CASES])
+def test_persistent_kernel_at_13_to_48_rows(name, shape, kv_lens, gamma):
+    """Against the oracle and against one kernel per stage on the same inputs, on the path that it names."""
+    case = harness.Case(shape, torch.bfloat16, kv_lens, gamma, seed=8, cache="fill",
+                        gen_device="cuda").gpu_setup(max_rows=len(kv_lens) * (gamma + 1))
+    try:
+        for name_, value in (("graph", 0), ("timing", 1)):
+            case.target.set_option(name_, value)
+        for mode, T in [(orc.GREEDY, 1.0), (orc.SAMPLING, 1.0)]:
+            case.target.set_option("timing", 1)      # clears the records
+            rep, g = _run(case, mode, T, options={"gemm_impl": 1, "step_impl": 1, "attn_impl": 2})
+            assert rep.exact + rep.margin == len(kv_lens)
+            assert case.target.kernel_time("verify_step")[1] == 1 and case.target.kernel_time("gemm")[1] == 0
+            rep1, g1 = _run(case, mode, T, options={"gemm_impl": 1, "step_impl": 0, "attn_impl": 2})
+            assert case.target.kernel_time("verify_step")[1] == 1 and case.target.kernel_time("gemm")[1] > 0
+            d = np.abs(g["hidden"] - g1["hidden"]).max()
+            assert 0 < d < 5e-3                      # close, and not the same code path
+            print(name, "mode", mode, rep, "vs per stage", d)
+    finally:
+        case.close()
+
+
+@pytest.mark.parametrize("options", [{}, {"gemm_impl": 1, "attn_impl": 0, "step_impl": 0}], ids=["paired", "one-SM-tiles"])
+def test_more_than_256_rows_keep_both_activation_planes(options):
+    """29 sequences x 9 rows = 261 rows.  The paired projections cut them into row blocks; with tiles of one SM (the GEMM of steps with
+    the CUDA-core attention) the two bf16 activation planes no longer fit side by side in tensor memory and the lo plane is
+    accumulated into the hi plane's columns."""
     kv_lens = [5 + 7 * b for b in range(29)]
     case = harness.Case(GQA, torch.bfloat16, kv_lens, 8, seed=6).gpu_setup(max_rows=29 * 9)
     try:
         for mode, T in [(orc.GREEDY, 1.0), (orc.SAMPLING, 0.5)]:
-            rep, g = _run(case, mode, T)
+            rep, g = _run(case, mode, T, options=options)
             assert rep.exact + rep.margin == len(kv_lens)
-            # the hidden states are as accurate as with few rows (plain bf16 activations are ~30x worse)
-            assert rep.max_hidden_err < 2e-3, rep
+            # the hidden states are as accurate as with few rows (plain bf16 activations are ~30x worse); the CUDA-core attention
+            # reads the block's own rows from the pages, rounded to bf16 (2^-9) and not to fp16: 3.0e-3 seen
+            assert rep.max_hidden_err < (6e-3 if options else 2e-3), rep
     finally:
         case.close()
 

@@ -464,7 +464,7 @@ def main():
                 dw.step(mode)
             dw.target.sync()
             tot = 0.0
-            for name in ("plan", "embed_norm", "gemm_qkv", "gemm_o", "gemm_gateup", "gemm_down", "gemm_lm_head",
+            for name in ("embed_norm", "gemm_qkv", "gemm_o", "gemm_gateup", "gemm_down", "gemm_lm_head",
                          "qkv_rope", "attn_combine", "reduce_norm", "swiglu", "finalize", "resample"):
                 ms, n = dw.target.kernel_time(name)
                 if n:
@@ -526,7 +526,7 @@ def main():
         "algorithmic_bytes_per_step": w_bytes + kv_bytes,
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "ms_per_step": ms_e2e},
-        "gpu_launches": (mega_launches + 1 + (2 if mode == binding.MODE_SAMPLING else 0) if mega_launches
+        "gpu_launches": (mega_launches + 3 + (2 if mode == binding.MODE_SAMPLING else 0) if mega_launches
                          else dw.launches_per_step(mode)) * args.steps,
         "clocks": clocks, "roofline": roofline, "cpu_baseline": cpu_baseline,
         "kernel_breakdown": {} if args.no_breakdown else breakdown,

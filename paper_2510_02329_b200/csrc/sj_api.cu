@@ -259,7 +259,6 @@ struct sj_kv {
   std::vector<int> len_hi;              // upper bound of the live length known to the host
   std::vector<char> exact;              // len_hi is the exact length
   int* d_block_table = nullptr;
-  int* d_tmp = nullptr;                 // [2 * SJ_MAX_BATCH] staging for rollback / set_len
   CUtensorMap tm_pool;                  // bf16 pool as a [rows, head_dim] matrix, box = 16 slots x 64 dims
   bool has_tm_pool = false;
 };
@@ -756,7 +755,7 @@ extern "C" sj_status sj_kv_create(sj_target* t, int max_seqs, long max_pages, in
   cudaError_t e = counted_malloc(&pool, bytes);
   int* meta = nullptr;
   const int mpps = (int)std::min<long>(max_pages, 1 << 20);
-  if (e == cudaSuccess) e = counted_malloc((void**)&meta, sizeof(int) * ((size_t)max_seqs * (mpps + 2) + 2 * SJ_MAX_BATCH));
+  if (e == cudaSuccess) e = counted_malloc((void**)&meta, sizeof(int) * (size_t)max_seqs * (mpps + 2));
   if (e != cudaSuccess) {
     cudaGetLastError();
     if (pool) counted_free(pool);
@@ -764,7 +763,7 @@ extern "C" sj_status sj_kv_create(sj_target* t, int max_seqs, long max_pages, in
     return fail(e == cudaErrorMemoryAllocation ? SJ_ERR_OOM : SJ_ERR_CUDA, "KV pool of %zu bytes: %s", bytes,
                 cudaGetErrorString(e));
   }
-  cudaMemset(meta, 0, sizeof(int) * ((size_t)max_seqs * (mpps + 2) + 2 * SJ_MAX_BATCH));
+  cudaMemset(meta, 0, sizeof(int) * (size_t)max_seqs * (mpps + 2));
   // Slots past a sequence's length are read (and masked) by the tensor-core attention: keep them finite.
   e = cudaMemset(pool, 0, bytes);
   if (e == cudaSuccess && t->bf) {
@@ -784,7 +783,6 @@ extern "C" sj_status sj_kv_create(sj_target* t, int max_seqs, long max_pages, in
   kv->view.block_table = meta;
   kv->view.kv_len = meta + (size_t)max_seqs * mpps;
   kv->view.pending = kv->view.kv_len + max_seqs;
-  kv->d_tmp = kv->view.pending + max_seqs;
   kv->view.n_pages = max_pages;
   kv->view.max_pages_per_seq = mpps;
   kv->view.page_size = page_size;
@@ -814,8 +812,9 @@ extern "C" sj_status sj_kv_destroy(sj_kv* kv) {
   return SJ_OK;
 }
 
-// Make sure `seq` owns pages for `tokens` tokens; uploads the new block-table entries.
-static sj_status reserve(sj_kv* kv, int seq, long tokens, std::vector<std::pair<int, int>>* undo) {
+// Make sure `seq` owns pages for `tokens` tokens; new block-table entries go into `edits` (the caller launches them) as long
+// as they fit there, else they are uploaded.
+static sj_status reserve(sj_kv* kv, int seq, long tokens, std::vector<std::pair<int, int>>* undo, KvEdits* edits) {
   const int ps = kv->view.page_size;
   const long need = (tokens + ps - 1) / ps;
   std::vector<int>& pg = kv->pages[seq];
@@ -829,9 +828,38 @@ static sj_status reserve(sj_kv* kv, int seq, long tokens, std::vector<std::pair<
     kv->free_pages.pop_back();
   }
   if (undo) undo->push_back({seq, (int)had});
+  if (edits && edits->n + (int)(pg.size() - had) <= kMaxEdits) {
+    for (size_t i = had; i < pg.size(); ++i) edits->e[edits->n++] = {seq, (int)i, pg[i]};
+    return SJ_OK;
+  }
   CU_TRY(cudaMemcpyAsync(kv->d_block_table + (size_t)seq * kv->view.max_pages_per_seq + had, pg.data() + had,
                          sizeof(int) * (pg.size() - had), cudaMemcpyHostToDevice, kv->t->stream));
   return SJ_OK;
+}
+// Pages reserved for a step that is not launched after all go back to the pool.
+struct ReservedPages {
+  sj_kv* kv;
+  std::vector<std::pair<int, int>> undo;   // (sequence, pages it had), in the order of the reservations
+  ~ReservedPages() {
+    for (auto u = undo.rbegin(); u != undo.rend(); ++u) {
+      std::vector<int>& pg = kv->pages[u->first];
+      while ((int)pg.size() > u->second) { kv->free_pages.push_back(pg.back()); pg.pop_back(); }
+    }
+  }
+};
+
+// The launch that starts a step: arguments and page numbers to the device (k_begin).  W: workspace to plan a per-stage
+// step in, or null.
+static sj_status begin_step(sj_target* t, sj_kv* kv, const StepArgs& h, const KvEdits& edits, const Work* W, int chunk_len, unsigned* sync) {
+  CU_TRY(launch(k_begin, dim3(1), dim3(256), 0, t->stream, false, h, edits, t->d_args, kv->view, W ? *W : Work{}, chunk_len, W ? 1 : 0, sync));
+  return SJ_OK;
+}
+// One kind of bookkeeping entry of B sequences.
+static KvEdits edits_of(const int* seq_ids, const int* values, int B, int at) {
+  KvEdits x;
+  x.n = B;
+  for (int i = 0; i < B; ++i) x.e[i] = {seq_ids[i], at, values[i]};
+  return x;
 }
 
 static void release_beyond(sj_kv* kv, int seq, long tokens) {
@@ -856,7 +884,7 @@ extern "C" sj_status sj_kv_fill(sj_kv* kv, int seq, int layer, int start, int n_
   if (!kv || !k || !v) return fail(SJ_ERR_INVALID_ARG, "null argument");
   if (seq < 0 || seq >= kv->max_seqs || layer < 0 || layer >= kv->t->dm.n_layers || start < 0 || n_tokens <= 0)
     return fail(SJ_ERR_INVALID_ARG, "sj_kv_fill: index out of range");
-  sj_status st = reserve(kv, seq, (long)start + n_tokens, nullptr);
+  sj_status st = reserve(kv, seq, (long)start + n_tokens, nullptr, nullptr);
   if (st != SJ_OK) return st;
   cudaError_t e;
   if (kv->t->bf)
@@ -894,8 +922,8 @@ extern "C" sj_status sj_kv_set_len(sj_kv* kv, const int* seq_ids, const int* len
   for (int i = 0; i < B; ++i)
     if (lens[i] < 0 || (size_t)lens[i] > kv->pages[seq_ids[i]].size() * kv->view.page_size)
       return fail(SJ_ERR_STATE, "length %d of sequence %d exceeds its reserved rows", lens[i], seq_ids[i]);
+  CU_TRY(launch(k_edit, dim3(1), dim3(256), 0, kv->t->stream, false, kv->view, edits_of(seq_ids, lens, B, kEditLen)));
   for (int i = 0; i < B; ++i) {
-    CU_TRY(cudaMemcpyAsync(kv->view.kv_len + seq_ids[i], lens + i, sizeof(int), cudaMemcpyHostToDevice, kv->t->stream));
     kv->len_hi[seq_ids[i]] = lens[i];
     kv->exact[seq_ids[i]] = 1;
   }
@@ -909,8 +937,7 @@ extern "C" sj_status sj_kv_set_pending(sj_kv* kv, const int* seq_ids, const int*
   for (int i = 0; i < B; ++i) {
     if (tokens[i] < 0 || tokens[i] >= kv->t->dm.V) return fail(SJ_ERR_INVALID_ARG, "token id out of range");
   }
-  for (int i = 0; i < B; ++i)
-    CU_TRY(cudaMemcpyAsync(kv->view.pending + seq_ids[i], tokens + i, sizeof(int), cudaMemcpyHostToDevice, kv->t->stream));
+  CU_TRY(launch(k_edit, dim3(1), dim3(256), 0, kv->t->stream, false, kv->view, edits_of(seq_ids, tokens, B, kEditPending)));
   return SJ_OK;
 }
 
@@ -939,12 +966,7 @@ extern "C" sj_status sj_rollback_kv(sj_kv* kv, const int* seq_ids, const int* ne
       return fail(SJ_ERR_STATE, "rollback of sequence %d to %d beyond its length (at most %d)", seq_ids[i], new_len[i],
                   kv->len_hi[seq_ids[i]]);
   }
-  int stage[2 * SJ_MAX_BATCH];
-  memcpy(stage, seq_ids, sizeof(int) * B);
-  memcpy(stage + B, new_len, sizeof(int) * B);
-  CU_TRY(cudaMemcpyAsync(kv->d_tmp, stage, sizeof(int) * 2 * B, cudaMemcpyHostToDevice, kv->t->stream));
-  CU_TRY(launch(k_rollback, dim3((B + 127) / 128), dim3(128), 0, kv->t->stream, false, kv->view, (const int*)kv->d_tmp,
-                (const int*)(kv->d_tmp + B), B, kv->t->work.status));
+  CU_TRY(launch(k_rollback, dim3(1), dim3(256), 0, kv->t->stream, false, kv->view, edits_of(seq_ids, new_len, B, kEditLen), kv->t->work.status));
   // Whole pages past the new length go back to the pool.  Everything that still touches them (a verify in
   // flight, this rollback) was enqueued on the target's stream before any later call can hand them out
   // again, and that call's kernels run on the same stream.  If the device refuses the rollback (the live
@@ -1177,7 +1199,6 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
   const size_t ssq_n = (size_t)(dm.d / kTileN) * R;
   auto plan_of = [&](const TcSite& site) { return tc ? SplitPlan{site.d_tile_slots, site.n_tiles} : one; };
 
-  TIMED("plan", launch(k_plan, dim3(1), dim3(256), 0, s, false, args, kv->view, W, chunk_len));
   TIMED("embed_norm", launch(k_embed_norm<T>, dim3(R), dim3(256), row_smem, s, pdl, args, kv->view, W, dm, (const T*)t->embed,
                 (const T*)t->layers[0].na, pair ? W.ssq : (float*)nullptr));
   const int nq = (dm.Hq / dm.Hkv) * (gamma + 1);
@@ -1392,7 +1413,7 @@ static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode
     }
     p.tag0 = t->mega_tag;
     t->mega_tag += 4 * kMegaMaxLayers + 1;   // GEMM phases of a launch
-    CU_TRY(cudaMemsetAsync(t->d_sync, 0, sizeof(unsigned) * 4, s));
+    if (ci > 0) CU_TRY(cudaMemsetAsync(t->d_sync, 0, sizeof(unsigned) * 4, s));   // k_begin did it for the first launch
     cudaEvent_t ea = nullptr, eb = nullptr;
     if (timing) {
       CU_TRY(cudaEventCreate(&ea));
@@ -1523,19 +1544,14 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
   if (group * rows > kAttMaxQ) return fail(SJ_ERR_SHAPE, "(Hq/Hkv)*(gamma+1) = %d exceeds %d", group * rows, kAttMaxQ);
 
   // a0: reserve pages for gamma+1 more rows per sequence; nothing is launched if the pool runs out
-  std::vector<std::pair<int, int>> undo;
+  ReservedPages reserved{kv, {}};
+  KvEdits edits;
+  edits.n = 0;
   long total_keys = 0;
   size_t chunk_need_base = 0;
   for (int i = 0; i < B; ++i) {
     int s = a->seq_ids[i];
-    st = reserve(kv, s, (long)kv->len_hi[s] + rows, &undo);
-    if (st != SJ_OK) {
-      for (auto& u : undo) {
-        std::vector<int>& pg = kv->pages[u.first];
-        while ((int)pg.size() > u.second) { kv->free_pages.push_back(pg.back()); pg.pop_back(); }
-      }
-      return st;
-    }
+    if ((st = reserve(kv, s, (long)kv->len_hi[s] + rows, &reserved.undo, &edits)) != SJ_OK) return st;
     total_keys += kv->len_hi[s] + rows;
   }
   const int chunk_len = pick_chunk_len(t, total_keys);
@@ -1570,7 +1586,7 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
     if ((st = ensure_attn_partials(t, B, rows)) != SJ_OK) return st;
   if (use_logits && (st = ensure_logits(t, R)) != SJ_OK) return st;
 
-  // per-call arguments: one small copy (the driver stages pageable memory before returning)
+  // per-call arguments
   StepArgs h;
   memset(&h, 0, sizeof(h));
   h.draft_ids = a->draft_ids; h.q_tok = a->draft_q_tok; h.q_full = a->draft_q_full; h.uniforms = a->uniforms;
@@ -1588,7 +1604,8 @@ static sj_status verify_step(sj_target* t, sj_kv* kv, const sj_verify_args* a, c
   h.judge_bias = t->judge_bias;
   h.has_judge = t->has_judge ? 1 : 0;
   memcpy(h.seq_ids, a->seq_ids, sizeof(int) * B);
-  CU_TRY(cudaMemcpyAsync(t->d_args, &h, sizeof(h), cudaMemcpyHostToDevice, t->stream));
+  if ((st = begin_step(t, kv, h, edits, use_mega ? nullptr : &t->work, chunk_len, use_mega ? t->d_sync : nullptr)) != SJ_OK) return st;
+  reserved.undo.clear();
 
   // chunk_len shapes only the CUDA-core attention's grid: a growing cache captures no new step elsewhere
   StepKey key{kv, B, gamma, a->mode, simt_attn ? chunk_len : 0, t->opt_gemm, t->opt_attn, t->opt_pdl, h.top_k};
@@ -1772,7 +1789,7 @@ static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* token
   Work W = t->pf_work;
   W.tc_m = t->work.tc_m; W.tc_l = t->work.tc_l; W.tc_o = t->work.tc_o;
   W.status = t->work.status; W.judge_w = t->work.judge_w; W.inv_freq = t->work.inv_freq;
-  if ((st = reserve(kv, seq, (long)kv->len_hi[seq] + n_tokens, nullptr)) != SJ_OK) return st;
+  if ((st = reserve(kv, seq, (long)kv->len_hi[seq] + n_tokens, nullptr, nullptr)) != SJ_OK) return st;
   CU_TRY(cudaMemcpyAsync(t->d_pf_tok, tokens, sizeof(int) * n_tokens, cudaMemcpyHostToDevice, s));
   for (int i0 = 0; i0 < n_tokens; i0 += per) {
     const int n = std::min(per, n_tokens - i0), B = (n + c - 1) / c;
@@ -1783,7 +1800,9 @@ static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* token
     h.n_tok = n; h.pos_step = c; h.kv_rows = n;
     h.B = B; h.gamma = c - 1; h.mode = SJ_MODE_GREEDY; h.inv_temperature = 1.f; h.top_k = 1; h.accept_all = 1;
     for (int b = 0; b < B; ++b) h.seq_ids[b] = seq;
-    CU_TRY(cudaMemcpyAsync(t->d_args, &h, sizeof(h), cudaMemcpyHostToDevice, s));
+    KvEdits none;
+    none.n = 0;
+    if ((st = begin_step(t, kv, h, none, &W, 4096, nullptr)) != SJ_OK) return st;
     if ((st = enqueue_layers<bf16>(t, kv, B, c - 1, 4096, W, 0, true, !last)) != SJ_OK) return st;
     const int n_vtiles = (dm.V + kTileN - 1) / kTileN;
     if (last) {

@@ -24,7 +24,7 @@ template <typename T> __device__ __forceinline__ T from_f(float x);
 template <> __device__ __forceinline__ float from_f<float>(float x) { return x; }
 template <> __device__ __forceinline__ bf16 from_f<bf16>(float x) { return __float2bfloat16_rn(x); }
 
-// Per-call arguments, resident in device memory and rewritten by one small copy per call so
+// Per-call arguments, resident in device memory and rewritten by k_begin at the start of a call so
 // that a captured graph never bakes in a caller's pointer.
 struct StepArgs {
   const int* draft_ids;
@@ -58,7 +58,7 @@ struct StepArgs {
 //   pool[((((layer * n_pages + page) * 2 + kv) * Hkv + head) * page_size + slot) * hd + dim]
 struct KvView {
   void* pool;
-  const int* block_table;  // [max_seqs, max_pages_per_seq]
+  int* block_table;        // [max_seqs, max_pages_per_seq]
   int* kv_len;             // [max_seqs]
   int* pending;            // [max_seqs]
   long n_pages;
@@ -73,6 +73,12 @@ __device__ __forceinline__ T* kv_row(const KvView& kv, int layer, int page, int 
   idx = (idx * kv.page_size + slot) * kv.head_dim;
   return reinterpret_cast<T*>(kv.pool) + idx;
 }
+
+// Changes of a cache's bookkeeping.  They travel as kernel parameters, one launch for all sequences, instead of as a copy
+// from host memory per sequence.
+struct KvEdit { int seq, at, value; };   // at >= 0: entry of the block table; else one of:
+constexpr int kEditLen = -1, kEditPending = -2, kMaxEdits = kMaxBatch;
+struct KvEdits { int n; KvEdit e[kMaxEdits]; };
 
 // How a GEMM's output tile is spread over thread blocks (split along K).  Work is counted in
 // units of (128-feature tile, 64-wide K block); block c owns units [c*U/G, (c+1)*U/G).  A tile's

@@ -110,8 +110,8 @@ class DeviceWorkload:
         return sum(self.kv_lens) * self.shape.kv_bytes_per_token(self.top["embed"].element_size())
 
     def launches_per_step(self, mode: int = binding.MODE_GREEDY, commit: bool = True) -> int:
-        # per stage: set-up and embedding; six kernels a layer; final norm, LM head, acceptance; the draw's two
-        n = 2 + 6 * self.shape.n_layers + 3 + (2 if mode == binding.MODE_SAMPLING else 0)
+        # per stage: pending tokens, set-up and embedding; six kernels a layer; final norm, LM head, acceptance; the draw's two
+        n = 3 + 6 * self.shape.n_layers + 3 + (2 if mode == binding.MODE_SAMPLING else 0)
         return n + (1 if commit else 0)
 
     def close(self) -> None:

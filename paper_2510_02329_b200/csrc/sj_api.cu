@@ -16,6 +16,7 @@
 #include "sj_attn_tc.cuh"
 #include "sj_attn_t5.cuh"
 #include "sj_gemm_tc.cuh"
+#include "sj_gemm_f32.cuh"
 #include "sj_gemm_pair.cuh"
 #include "sj_mega.cuh"
 
@@ -117,11 +118,11 @@ static sj_status make_map(CUtensorMap* tm, const void* base, long rows, long K, 
 // ---------------------------------------------------------------------------------------------
 // tensor-core GEMM sites
 // ---------------------------------------------------------------------------------------------
-struct TcSite {
+struct TcSite {   // (fp32 models: the same plan for k_gemm_f32, in its tiles and K steps)
   // static per site
   int N = 0, K = 0, n_tiles = 0, KB = 0, G = 0, nseg = 0;
   int seg_tile_end[3] = {0, 0, 0};
-  int max_slots = 1;
+  int max_slots = 1, tile_shift = 7;
   int2* d_tile_slots = nullptr;
   bool lm = false;
 };
@@ -282,11 +283,22 @@ static sj_status dev_alloc(sj_target* t, T** p, size_t n) {
   return SJ_OK;
 }
 
+// Block counts and, where tiles are shared between blocks, the table of slots of a site whose tiles and K blocks are set.
+static sj_status deal_site(sj_target* t, TcSite& s, bool lm) {
+  s.lm = lm;
+  s.G = (int)std::min<long long>(lm ? s.n_tiles : (long long)s.n_tiles * s.KB, t->sm_count);
+  if (lm) return SJ_OK;
+  std::vector<int2> slots;
+  build_tile_slots(s.n_tiles, s.KB, s.G, slots, s.max_slots);
+  sj_status st = dev_alloc(t, &s.d_tile_slots, slots.size());
+  if (st != SJ_OK) return st;
+  CU_TRY(cudaMemcpy(s.d_tile_slots, slots.data(), slots.size() * sizeof(int2), cudaMemcpyHostToDevice));
+  return SJ_OK;
+}
 static sj_status setup_site(sj_target* t, TcSite& s, int nseg, const int* seg_rows, int K, bool lm) {
   s.nseg = nseg;
   s.K = K;
   s.KB = K / kBK;
-  s.lm = lm;
   int tiles = 0;
   s.N = 0;
   for (int i = 0; i < 3; ++i) {
@@ -297,15 +309,15 @@ static sj_status setup_site(sj_target* t, TcSite& s, int nseg, const int* seg_ro
     s.seg_tile_end[i] = tiles;
   }
   s.n_tiles = tiles;
-  s.G = std::min(t->sm_count, lm ? tiles : (int)std::min<long long>((long long)tiles * s.KB, t->sm_count));
-  if (!lm) {
-    std::vector<int2> slots;
-    build_tile_slots(tiles, s.KB, s.G, slots, s.max_slots);
-    sj_status st = dev_alloc(t, &s.d_tile_slots, slots.size());
-    if (st != SJ_OK) return st;
-    CU_TRY(cudaMemcpy(s.d_tile_slots, slots.data(), slots.size() * sizeof(int2), cudaMemcpyHostToDevice));
-  }
-  return SJ_OK;
+  return deal_site(t, s, lm);
+}
+static sj_status setup_f32_site(sj_target* t, TcSite& s, int N, int K, bool lm) {
+  s.N = N;
+  s.K = K;
+  s.KB = (K + kF32K - 1) / kF32K;
+  s.n_tiles = (N + kF32Feats - 1) / kF32Feats;
+  s.tile_shift = kF32Shift;
+  return deal_site(t, s, lm);
 }
 
 static bool tc_shapes_ok(const sj_model_config& c) {
@@ -377,7 +389,7 @@ static sj_status alloc_rows(sj_target* t, Work& W, int R) {
 static sj_status alloc_partials(sj_target* t, Work& W, int R) {
   const sj_model_config& c = t->cfg;
   size_t n = (size_t)R * std::max({(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, c.d_model, 2 * c.d_ffn});
-  if (tc_shapes_ok(c)) {
+  if (tc_shapes_ok(c) || !t->bf) {
     n = 0;
     for (TcSite* s : {&t->s_qkv, &t->s_o, &t->s_gu, &t->s_down}) n = std::max(n, (size_t)s->max_slots * R * s->N);
   }
@@ -411,6 +423,9 @@ static sj_status ensure_logits(sj_target* t, size_t R) {
   if (st == SJ_OK) t->logits_cap = need;
   return st;
 }
+
+typedef void (*F32Kernel)(const float*, GemmSegs, float*, size_t, int, int, int, int, int);
+static F32Kernel f32_kernel(int rt) { return rt <= 4 ? k_gemm_f32<4> : (rt <= 8 ? k_gemm_f32<8> : k_gemm_f32<12>); }
 
 typedef void (*PairKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const PairParams, const StepArgs*,
                            const KvView, const Work, const Dims);
@@ -548,6 +563,17 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
       if (cudaOccupancyMaxActiveClusters(&n, pair_kernel(PAIR_RES, c.head_dim), &cfg) != cudaSuccess) { n = 0; cudaGetLastError(); }
       t->pair_clusters[S] = n;
     }
+  }
+  if (!t->bf) {
+    if ((st = setup_f32_site(t, t->s_qkv, qd + 2 * kd, c.d_model, false)) != SJ_OK) return bail(st);
+    if ((st = setup_f32_site(t, t->s_o, c.d_model, qd, false)) != SJ_OK) return bail(st);
+    if ((st = setup_f32_site(t, t->s_gu, 2 * c.d_ffn, c.d_model, false)) != SJ_OK) return bail(st);
+    if ((st = setup_f32_site(t, t->s_down, c.d_model, c.d_ffn, false)) != SJ_OK) return bail(st);
+    if ((st = setup_f32_site(t, t->s_lm, c.vocab, c.d_model, true)) != SJ_OK) return bail(st);
+    cudaError_t e = cudaSuccess;
+    for (int rt = 4; rt <= 12 && e == cudaSuccess; rt += 4)
+      e = cudaFuncSetAttribute(f32_kernel(rt), cudaFuncAttributeMaxDynamicSharedMemorySize, kF32Stages * f32_stage_floats(rt) * (int)sizeof(float));
+    if (e != cudaSuccess) { fail(SJ_ERR_CUDA, "smem opt-in: %s", cudaGetErrorString(e)); return bail(SJ_ERR_CUDA); }
   }
   if ((st = alloc_partials(t, W, R)) != SJ_OK) return bail(st);
   {
@@ -1134,9 +1160,13 @@ static cudaError_t launch_gemm_simt(cudaStream_t s, bool pdl, int sms, const T* 
   if (R <= 8 || (R > 12 && R <= 16)) return launch(k_gemm_simt<T, 8, 4>, grid, block, 0, s, pdl, A, g, Y, R, N, K, planes, ks);
   return launch(k_gemm_simt<T, 12, 4>, grid, block, 0, s, pdl, A, g, Y, R, N, K, planes, ks);
 }
-template <typename T>
-static cudaError_t launch_simt(sj_target* t, const void* A, const GemmSegs& segs, float* Y, int R, int N, int K, bool pdl) {
-  return launch_gemm_simt<T>(t->stream, pdl, t->sm_count, (const T*)A, segs, Y, R, N, K, t->bf ? 2 : 1);
+// A projection of the CUDA-core step: fp32 models k_gemm_f32 with the site's plan; bf16 ones (a cross-check) k_gemm_simt.
+static cudaError_t launch_cudacore(sj_target* t, const TcSite& site, const void* A, const GemmSegs& segs, float* Y, int R, int N, int K, bool pdl) {
+  if (t->bf) return launch_gemm_simt<bf16>(t->stream, pdl, t->sm_count, (const bf16*)A, segs, Y, R, N, K, 2);
+  // rows in passes of about equal size, up to 12: at more, the accumulators leave no registers for the step's weights
+  const int n_pass = (R + 11) / 12, pp = (R + n_pass - 1) / n_pass, rt = round_up(pp, 4);
+  return launch(f32_kernel(rt), dim3(site.G), dim3(kF32Threads), sizeof(float) * kF32Stages * f32_stage_floats(rt), t->stream, pdl, (const float*)A,
+                segs, Y, (size_t)R * N, R, N, K, pp, site.lm ? 1 : 0);
 }
 
 // Launch `expr`; in timing mode bracket it with events filed under `name`.
@@ -1182,7 +1212,6 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
   if (!attn_tc) W.Qb = nullptr, W.KVn = nullptr;
   cudaStream_t s = t->stream;
   const size_t row_smem = sizeof(float) * dm.d;
-  SplitPlan one{nullptr, 0};
   const CUtensorMap *mA_d = nullptr, *mA_q = nullptr, *mA_f = nullptr;
   if (tc) {
     sj_status st;
@@ -1197,7 +1226,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
   // longer shares there (8B-shaped 2.58e-4 against 2.71e-4), and a step on a given cache shows no difference (1.105e-4, 1.109e-4).
   auto seg_kb = [&](int K) { return prefill && K / kBK <= kPairShortKB ? kPairSegKB / 2 : kPairSegKB; };
   const size_t ssq_n = (size_t)(dm.d / kTileN) * R;
-  auto plan_of = [&](const TcSite& site) { return tc ? SplitPlan{site.d_tile_slots, site.n_tiles} : one; };
+  auto plan_of = [&](const TcSite& site) { return tc || !t->bf ? SplitPlan{site.d_tile_slots, site.n_tiles, site.tile_shift} : SplitPlan{nullptr, 0, 0}; };
 
   TIMED("embed_norm", launch(k_embed_norm<T>, dim3(R), dim3(256), row_smem, s, pdl, args, kv->view, W, dm, (const T*)t->embed,
                 (const T*)t->layers[0].na, pair ? W.ssq : (float*)nullptr));
@@ -1219,7 +1248,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
         TIMED("gemm_qkv", launch_tc(t, t->s_qkv, mA_d, &L.m_q, &L.m_k, &L.m_v, R, pdl, true, W));
       } else {
         GemmSegs g{{L.wq, L.wk, L.wv}, {qd, kd, kd}, 3};
-        TIMED("gemm_cudacore", launch_simt<T>(t, W.A, g, W.P, R, qd + 2 * kd, dm.d, pdl));
+        TIMED("gemm_cudacore", launch_cudacore(t, t->s_qkv, W.A, g, W.P, R, qd + 2 * kd, dm.d, pdl));
       }
       TIMED("qkv_rope", launch(k_qkv_rope<T>, dim3(R), dim3(256), 0, s, pdl, args, kv->view, W, dm, plan_of(t->s_qkv),
                     (size_t)R * (qd + 2 * kd), l, (const T*)L.bq, (const T*)L.bk, (const T*)L.bv));
@@ -1267,7 +1296,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
       TIMED("gemm_o", launch_tc(t, t->s_o, mA_q, &L.m_o, nullptr, nullptr, R, pdl, true, W));
     } else {
       GemmSegs g{{L.wo, nullptr, nullptr}, {dm.d, 0, 0}, 1};
-      TIMED("gemm_cudacore", launch_simt<T>(t, W.ATT, g, W.P, R, dm.d, qd, pdl));
+      TIMED("gemm_cudacore", launch_cudacore(t, t->s_o, W.ATT, g, W.P, R, dm.d, qd, pdl));
     }
     TIMED("reduce_norm", launch(k_reduce_norm<T>, dim3(R), dim3(256), row_smem, s, pdl, args, W, dm, plan_of(t->s_o), (size_t)R * dm.d,
                   (const T*)L.nf, 0));
@@ -1276,7 +1305,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
       TIMED("gemm_gateup", launch_tc(t, t->s_gu, mA_d, &L.m_g, &L.m_u, nullptr, R, pdl, true, W));
     } else {
       GemmSegs g{{L.wg, L.wu, nullptr}, {dm.F, dm.F, 0}, 2};
-      TIMED("gemm_cudacore", launch_simt<T>(t, W.A, g, W.P, R, 2 * dm.F, dm.d, pdl));
+      TIMED("gemm_cudacore", launch_cudacore(t, t->s_gu, W.A, g, W.P, R, 2 * dm.F, dm.d, pdl));
     }
     TIMED("swiglu", launch(k_swiglu<T>, dim3((dm.F + 255) / 256, R), dim3(256), 0, s, pdl, W, dm, plan_of(t->s_gu),
                   (size_t)R * 2 * dm.F));
@@ -1285,7 +1314,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
       TIMED("gemm_down", launch_tc(t, t->s_down, mA_f, &L.m_d, nullptr, nullptr, R, pdl, true, W));
     } else {
       GemmSegs g{{L.wd, nullptr, nullptr}, {dm.d, 0, 0}, 1};
-      TIMED("gemm_cudacore", launch_simt<T>(t, W.H, g, W.P, R, dm.d, dm.F, pdl));
+      TIMED("gemm_cudacore", launch_cudacore(t, t->s_down, W.H, g, W.P, R, dm.d, dm.F, pdl));
     }
     const bool last = (l == dm.n_layers - 1);
     const void* gain = last ? t->final_norm : t->layers[l + 1].na;
@@ -1320,7 +1349,7 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
       TIMED("gemm_lm_head", launch_tc(t, t->s_lm, mA_d, &t->m_lm, nullptr, nullptr, R, pdl, true, W));   // stores logits where W has them
   } else {
     GemmSegs g{{t->lm_head, nullptr, nullptr}, {dm.V, 0, 0}, 1};
-    TIMED("gemm_cudacore", launch_simt<T>(t, W.A, g, W.logits, R, dm.V, dm.d, pdl));
+    TIMED("gemm_cudacore", launch_cudacore(t, t->s_lm, W.A, g, W.logits, R, dm.V, dm.d, pdl));
     TIMED("lm_stats", launch(k_lm_stats_from_logits, dim3(n_vtiles, (R + 7) / 8), dim3(256), 0, s, pdl, args, W, dm, R));
   }
   TIMED("finalize", launch(k_finalize, dim3(B), dim3(256), 0, s, pdl, args, kv->view, W, dm, n_vtiles, R));
@@ -1945,7 +1974,7 @@ extern "C" sj_status sj_gemm_skinny(int dtype, int impl, int R, int N, int K, co
   if (e == cudaSuccess) e = launch_tc(&tmp, site, &mA, &mW, nullptr, nullptr, R, false, false, tmp.work);
   if (e == cudaSuccess)
     e = launch(k_sum_slots, dim3((unsigned)(((size_t)R * N + 255) / 256)), dim3(256), 0, s, false, (const float*)P,
-               SplitPlan{site.d_tile_slots, site.n_tiles}, (size_t)R * N, R, N, y);
+               SplitPlan{site.d_tile_slots, site.n_tiles, site.tile_shift}, (size_t)R * N, R, N, y);
   int hstatus = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hstatus, status, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -2048,7 +2077,7 @@ extern "C" sj_status sj_gemm_skinny_noalloc(int R, int N, int K, const void* a, 
   if ((st = make_map(&mW, w, N, K, kTileN)) != SJ_OK) return st;
   CU_TRY(launch_tc(&tmp, site, &mA, &mW, nullptr, nullptr, R, false, false, tmp.work));
   CU_TRY(launch(k_sum_slots, dim3((unsigned)(((size_t)R * N + 255) / 256)), dim3(256), 0, s, false, (const float*)P,
-                SplitPlan{site.d_tile_slots, site.n_tiles}, (size_t)R * N, R, N, y));
+                SplitPlan{site.d_tile_slots, site.n_tiles, site.tile_shift}, (size_t)R * N, R, N, y));
   int hstatus = 0;
   CU_TRY(cudaMemcpyAsync(&hstatus, status, sizeof(int), cudaMemcpyDeviceToHost, s));
   CU_TRY(cudaStreamSynchronize(s));

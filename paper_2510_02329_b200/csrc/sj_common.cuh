@@ -81,12 +81,13 @@ constexpr int kEditLen = -1, kEditPending = -2, kMaxEdits = kMaxBatch;
 struct KvEdits { int n; KvEdit e[kMaxEdits]; };
 
 // How a GEMM's output tile is spread over thread blocks (split along K).  Work is counted in
-// units of (128-feature tile, 64-wide K block); block c owns units [c*U/G, (c+1)*U/G).  A tile's
+// units of (128-feature tile, 64-wide K block) -- fp32 models (64, 128) --; block c owns units [c*U/G, (c+1)*U/G).  A tile's
 // partial sums live in consecutive "slots" of the partial buffer, one per contributing block in
 // block order, so that the consumer adds them in a fixed order (no atomics, bit-reproducible).
 struct SplitPlan {
   const int2* tile_slots;  // per tile: (first contributing block, number of slots); null: one slot
   int n_tiles;
+  int tile_shift;          // log2 of a tile's features
 };
 
 // Partial buffer layout: P[slot][row][N] fp32.
@@ -94,7 +95,7 @@ __device__ __forceinline__ float reduce_partials(const float* __restrict__ P, co
                                                  int N, int r, int n) {
   const float* p = P + (size_t)r * N + n;
   if (sp.tile_slots == nullptr) return *p;
-  int cnt = sp.tile_slots[n / kTileN].y;
+  int cnt = sp.tile_slots[n >> sp.tile_shift].y;
   float s = 0.f;
   for (int i = 0; i < cnt; ++i) s += p[(size_t)i * slot_stride];
   return s;

@@ -628,9 +628,10 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
     if (e != cudaSuccess) { fail(SJ_ERR_CUDA, "smem opt-in: %s", cudaGetErrorString(e)); return bail(SJ_ERR_CUDA); }
   }
   {
-    cudaError_t e;
-    if (t->bf) e = cudaFuncSetAttribute(k_attn_simt<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-    else e = cudaFuncSetAttribute(k_attn_simt<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    const int smem = (int)att_simt_smem(kAttMaxQ, c.head_dim);
+    auto opt_in = [&](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
+    const cudaError_t e = c.head_dim == 128 ? (t->bf ? opt_in(k_attn_simt<bf16, 128>) : opt_in(k_attn_simt<float, 128>))
+                                            : (t->bf ? opt_in(k_attn_simt<bf16, 64>) : opt_in(k_attn_simt<float, 64>));
     if (e != cudaSuccess) { fail(SJ_ERR_CUDA, "smem opt-in: %s", cudaGetErrorString(e)); return bail(SJ_ERR_CUDA); }
   }
   *out = t;
@@ -1231,7 +1232,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
   TIMED("embed_norm", launch(k_embed_norm<T>, dim3(R), dim3(256), row_smem, s, pdl, args, kv->view, W, dm, (const T*)t->embed,
                 (const T*)t->layers[0].na, pair ? W.ssq : (float*)nullptr));
   const int nq = (dm.Hq / dm.Hkv) * (gamma + 1);
-  const size_t att_smem = sizeof(float) * ((size_t)nq * dm.hd + kAttKT * (dm.hd + 1) + kAttKT * dm.hd + (size_t)nq * kAttKT + 3 * nq);
+  const size_t att_smem = att_simt_smem(nq, dm.hd);
   const int att_grid = std::max(1, std::min<int>(t->sm_count * 2, (int)n_chunks_hi * dm.Hkv));
   for (int l = 0; l < dm.n_layers; ++l) {
     const LayerW& L = t->layers[l];
@@ -1275,8 +1276,8 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
         TIMED("attn_combine", launch(k_attn_combine_tc<64>, cgrid, dim3(kCombineThreads), 0, s, pdl, args, W, dm, parts, t->sm_count, aa.n_tail_base, 0, 0));
       }
     } else {
-      TIMED("attn", launch(k_attn_simt<T>, dim3(att_grid), dim3(kAttThreads), att_smem, s, pdl, args, kv->view, W, dm, l, chunk_len));
-      TIMED("attn_combine", launch(k_attn_combine<T>, dim3(R * dm.Hq), dim3(std::min(dm.hd, 128)), 0, s, pdl, args, W, dm));
+      TIMED("attn", launch(dm.hd == 128 ? k_attn_simt<T, 128> : k_attn_simt<T, 64>, dim3(att_grid), dim3(kAttThreads), att_smem, s, pdl, args, kv->view, W, dm, l, chunk_len));
+      TIMED("attn_combine", launch(k_attn_combine<T>, dim3((R * dm.Hq * 32 + kSimtMergeThreads - 1) / kSimtMergeThreads), dim3(kSimtMergeThreads), 0, s, pdl, args, W, dm, R));
     }
     if (pair) {   // O, gate/up and down with their epilogues
       PairOut o, gu, dn;

@@ -403,10 +403,20 @@ k_gemm_simt(const T* __restrict__ A, GemmSegs segs, float* __restrict__ Y, int R
 // a5: causal grouped-query attention over the paged cache, split along the keys.
 // Work item = (chunk of chunk_len keys of one sequence, KV head); all query heads of the group and
 // all gamma+1 rows share the item's K/V.  Each item writes unnormalised partials (m, l, o).
+//
+// What bounds it at the caches it meets (a few hundred to a few thousand keys) is the length of an item's chain: find the
+// item, its pages, its keys; scores; softmax; output.  So a chunk is one tile of 64 keys as a rule, a tile's loads are all
+// in flight together and, where no row of this step is among its keys, requested before the wait for the previous kernel;
+// scores and outputs are blocked in registers (a thread: one key x 6 queries, then one dimension x 6 queries), operands
+// 16 bytes at a time.  1B-shaped cut of 4 layers, 2 sequences of 512 keys, 10 rows: a step 898 -> 763 us (B200).
 // ---------------------------------------------------------------------------------------------
-constexpr int kAttKT = 32;      // keys per inner tile
+constexpr int kAttKT = 64;      // keys per inner tile
 constexpr int kAttMaxQ = 96;    // query vectors per item: (Hq/Hkv) * (gamma+1)
 constexpr int kAttThreads = 256;
+constexpr int kAttQB = 6;       // queries blocked in registers
+__host__ __device__ __forceinline__ size_t att_simt_smem(int nq, int hd) {   // queries, keys, values, scores, (m, l, alpha)
+  return sizeof(float) * ((size_t)nq * hd + kAttKT * (hd + 4) + kAttKT * hd + (size_t)nq * kAttKT + 3 * nq);
+}
 
 __device__ __forceinline__ int find_seq(const int* chunk_start, int B, int chunk) {
   int lo = 0, hi = B - 1;
@@ -417,16 +427,16 @@ __device__ __forceinline__ int find_seq(const int* chunk_start, int B, int chunk
   return lo;
 }
 
-template <typename T>
-__global__ void k_attn_simt(const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, int layer, int chunk_len) {
-  extern __shared__ float sm[];
-  pdl_wait();
-  pdl_launch();
+template <typename T, int hd>
+__global__ void __launch_bounds__(kAttThreads, hd == 64 ? 2 : 1)
+k_attn_simt(const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, int layer, int chunk_len) {
+  extern __shared__ __align__(16) float sm[];
+  // The row positions, the chunk list and the cached rows are the work of kernels before the one that this one waits for.
   const int B = args->B, rows = args->gamma + 1;
-  const int group = dm.Hq / dm.Hkv, nq = group * rows, hd = dm.hd;
+  const int group = dm.Hq / dm.Hkv, nq = group * rows;
   float* qs = sm;                         // [nq][hd]
-  float* ks = qs + nq * hd;               // [KT][hd+1]
-  float* vs = ks + kAttKT * (hd + 1);     // [KT][hd]
+  float* ks = qs + nq * hd;               // [KT][hd + 4]
+  float* vs = ks + kAttKT * (hd + 4);     // [KT][hd]
   float* ss = vs + kAttKT * hd;           // [nq][KT]
   float* m_run = ss + nq * kAttKT;        // [nq]
   float* l_run = m_run + nq;              // [nq]
@@ -434,6 +444,8 @@ __global__ void k_attn_simt(const StepArgs* __restrict__ args, KvView kv, Work w
   const float scale = 1.0f / sqrtf((float)hd);
   const int total = w.chunk_start[B] * dm.Hkv;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int ng = kAttThreads / hd, NA = kAttMaxQ / ng;   // output: thread = dimension, ng groups of queries
+  bool waited = false;
 
   for (int item = blockIdx.x; item < total; item += gridDim.x) {
     const int chunk = item / dm.Hkv, kvh = item % dm.Hkv;
@@ -442,141 +454,200 @@ __global__ void k_attn_simt(const StepArgs* __restrict__ args, KvView kv, Work w
     const int L = w.row_pos[b * rows];  // cached tokens before the block
     const int k_begin = (chunk - w.chunk_start[b]) * chunk_len;
     const int k_end = min(k_begin + chunk_len, L + rows);
-    __syncthreads();
-    // queries of this KV head's group: q index = g * rows + j
-    for (int i = tid; i < nq * hd; i += kAttThreads) {
-      int q = i / hd, dd = i % hd, g = q / rows, j = q % rows;
-      const float* qrow = w.Q + (size_t)(b * rows + j) * (dm.Hq * hd) + (kvh * group + g) * hd;
-      qs[i] = qrow[dd];
-    }
-    for (int q = tid; q < nq; q += kAttThreads) { m_run[q] = -INFINITY; l_run[q] = 0.f; }
-    float acc[48];
+    float acc[NA];   // queries grp + ng * i of this thread's dimension
 #pragma unroll
-    for (int i = 0; i < 48; ++i) acc[i] = 0.f;
+    for (int i = 0; i < NA; ++i) acc[i] = 0.f;
     for (int k0 = k_begin; k0 < k_end; k0 += kAttKT) {
-      __syncthreads();
-      {   // 16-byte loads, all of a thread's requested before any is stored (two to four: hd 64 or 128, fp32 or bf16)
-        constexpr int VN = Vec<T>::n, MAXV = kAttKT * 128 / VN / kAttThreads;
-        typedef typename Vec<T>::type V;
-        V kv4[MAXV], vv4[MAXV];
+      constexpr int VN = Vec<T>::n, MAXV = kAttKT * hd / VN / kAttThreads;
+      typedef typename Vec<T>::type V;
+      V kv4[MAXV], vv4[MAXV];
+      if (!waited && k0 + kAttKT > L) { pdl_wait(); pdl_launch(); waited = true; }   // rows of this step are among the keys
 #pragma unroll
-        for (int u = 0; u < MAXV; ++u) {
-          const int i = (tid + u * kAttThreads) * VN, kk = i / hd, dd = i % hd, key = min(k0 + kk, k_end - 1);
-          if (kk < kAttKT) {
-            const int page = kv.block_table[(size_t)seq * kv.max_pages_per_seq + key / kv.page_size];
-            const T* kr = kv_row<T>(kv, layer, page, 0, kvh, key % kv.page_size) + dd;
-            kv4[u] = *reinterpret_cast<const V*>(kr);
-            vv4[u] = *reinterpret_cast<const V*>(kr + (size_t)kv.n_kv_heads * kv.page_size * kv.head_dim);
+      for (int u = 0; u < MAXV; ++u) {
+        const int i = (tid + u * kAttThreads) * VN, kk = i / hd, dd = i % hd, key = min(k0 + kk, k_end - 1);
+        const int page = kv.block_table[(size_t)seq * kv.max_pages_per_seq + key / kv.page_size];
+        const T* kr = kv_row<T>(kv, layer, page, 0, kvh, key % kv.page_size) + dd;
+        kv4[u] = *reinterpret_cast<const V*>(kr);
+        vv4[u] = *reinterpret_cast<const V*>(kr + (size_t)kv.n_kv_heads * kv.page_size * kv.head_dim);
+      }
+      if (!waited) { pdl_wait(); pdl_launch(); waited = true; }
+      __syncthreads();   // the tile before has been read
+      if (k0 == k_begin) {   // queries of this KV head's group: q index = g * rows + j
+        for (int i = 4 * tid; i < nq * hd; i += 4 * kAttThreads) {
+          const int q = i / hd, dd = i % hd, g = q / rows, j = q % rows;
+          *reinterpret_cast<float4*>(qs + i) = *reinterpret_cast<const float4*>(w.Q + (size_t)(b * rows + j) * (dm.Hq * hd) + (kvh * group + g) * hd + dd);
+        }
+        for (int q = tid; q < nq; q += kAttThreads) { m_run[q] = -INFINITY; l_run[q] = 0.f; }
+      }
+#pragma unroll
+      for (int u = 0; u < MAXV; ++u) {
+        const int i = (tid + u * kAttThreads) * VN, kk = i / hd, dd = i % hd;
+        float kf[VN], vf[VN];
+        unpack(kv4[u], kf);
+        unpack(vv4[u], vf);
+        const bool live = k0 + kk < k_end;
+#pragma unroll
+        for (int e = 0; e < VN; e += 4) {
+          *reinterpret_cast<float4*>(ks + kk * (hd + 4) + dd + e) = live ? make_float4(kf[e], kf[e + 1], kf[e + 2], kf[e + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+          *reinterpret_cast<float4*>(vs + kk * hd + dd + e) = live ? make_float4(vf[e], vf[e + 1], vf[e + 2], vf[e + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+      __syncthreads();
+      // scores: thread = key, four groups of threads take queries tid / 64, + 4, ...
+      {
+        const int kk = tid & (kAttKT - 1), key = k0 + kk, q_first = tid / kAttKT;
+        const float4* kr = reinterpret_cast<const float4*>(ks + kk * (hd + 4));
+        constexpr int QS = kAttThreads / kAttKT;
+        for (int q0 = q_first; q0 < nq; q0 += QS * kAttQB) {
+          float a[kAttQB];
+#pragma unroll
+          for (int i = 0; i < kAttQB; ++i) a[i] = 0.f;
+#pragma unroll 4
+          for (int d4 = 0; d4 < hd / 4; ++d4) {
+            const float4 kx = kr[d4];
+#pragma unroll
+            for (int i = 0; i < kAttQB; ++i) {
+              const float4 qx = *reinterpret_cast<const float4*>(qs + min(q0 + QS * i, nq - 1) * hd + 4 * d4);
+              a[i] = fmaf(qx.w, kx.w, fmaf(qx.z, kx.z, fmaf(qx.y, kx.y, fmaf(qx.x, kx.x, a[i]))));
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < kAttQB; ++i) {
+            const int q = q0 + QS * i;
+            if (q < nq) ss[q * kAttKT + kk] = key < k_end && key <= L + q % rows ? a[i] * scale : -INFINITY;
           }
         }
+      }
+      __syncthreads();
+      // online softmax: a warp per query, three side by side, two keys a lane
+      constexpr int NW = kAttThreads / 32, SQ = 3;
+      for (int q0 = warp; q0 < nq; q0 += NW * SQ) {
+        float s0[SQ], s1[SQ], mx[SQ], sum[SQ], mo[SQ];
 #pragma unroll
-        for (int u = 0; u < MAXV; ++u) {
-          const int i = (tid + u * kAttThreads) * VN, kk = i / hd, dd = i % hd;
-          if (kk < kAttKT) {
-            float kf[VN], vf[VN];
-            unpack(kv4[u], kf);
-            unpack(vv4[u], vf);
-            const bool live = k0 + kk < k_end;
+        for (int i = 0; i < SQ; ++i) {
+          const int q = min(q0 + NW * i, nq - 1);
+          s0[i] = ss[q * kAttKT + lane];
+          s1[i] = ss[q * kAttKT + 32 + lane];
+          mo[i] = m_run[q];
+          mx[i] = fmaxf(s0[i], s1[i]);
+        }
+        __syncwarp();
 #pragma unroll
-            for (int e = 0; e < VN; ++e) {
-              ks[kk * (hd + 1) + dd + e] = live ? kf[e] : 0.f;
-              vs[kk * hd + dd + e] = live ? vf[e] : 0.f;
+        for (int i = 0; i < SQ; ++i) mx[i] = fmaxf(mo[i], warp_max(mx[i]));
+#pragma unroll
+        for (int i = 0; i < SQ; ++i) {
+          s0[i] = s0[i] == -INFINITY ? 0.f : expf(s0[i] - mx[i]);
+          s1[i] = s1[i] == -INFINITY ? 0.f : expf(s1[i] - mx[i]);
+          sum[i] = warp_sum(s0[i] + s1[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < SQ; ++i) {
+          const int q = q0 + NW * i;
+          if (q < nq) {   // warp-uniform
+            ss[q * kAttKT + lane] = s0[i];
+            ss[q * kAttKT + 32 + lane] = s1[i];
+            if (lane == 0) {
+              const float f = mx[i] == -INFINITY ? 1.f : (mo[i] == -INFINITY ? 0.f : expf(mo[i] - mx[i]));
+              alpha[q] = f;
+              l_run[q] = l_run[q] * f + sum[i];
+              m_run[q] = mx[i];
             }
           }
         }
       }
       __syncthreads();
-      // scores: one (q, key) pair per thread-iteration; a warp covers the 32 keys of one q
-      for (int p = tid; p < nq * kAttKT; p += kAttThreads) {
-        int q = p / kAttKT, kk = p % kAttKT, key = k0 + kk, j = q % rows;
-        float s = -INFINITY;
-        if (key < k_end && key <= L + j) {
-          float a = 0.f;
-          const float* qv = qs + q * hd;
-          const float* kvp = ks + kk * (hd + 1);
-          for (int dd = 0; dd < hd; ++dd) a = fmaf(qv[dd], kvp[dd], a);
-          s = a * scale;
-        }
-        ss[p] = s;
-      }
-      __syncthreads();
-      // online softmax, one warp per query vector
-      for (int q = warp; q < nq; q += kAttThreads / 32) {
-        float s = ss[q * kAttKT + lane];
-        float mx = warp_max(s);
-        float m_old = m_run[q];
-        float m_new = fmaxf(m_old, mx);
-        float p = (s == -INFINITY) ? 0.f : expf(s - m_new);
-        float sum = warp_sum(p);
-        ss[q * kAttKT + lane] = p;
-        if (lane == 0) {
-          float a = (m_old == -INFINITY) ? 0.f : expf(m_old - m_new);
-          alpha[q] = (m_new == -INFINITY) ? 1.f : a;
-          l_run[q] = l_run[q] * ((m_new == -INFINITY) ? 1.f : a) + sum;
-          m_run[q] = m_new;
-        }
-      }
-      __syncthreads();
       // o[q][dd] = o * alpha + sum_k p[q][k] v[k][dd]
+      const int dd = tid % hd, grp = tid / hd;
 #pragma unroll
-      for (int i = 0; i < 48; ++i) {
-        int e = tid + i * kAttThreads;
-        if (e < nq * hd) {
-          int q = e / hd, dd = e % hd;
-          float a = acc[i] * alpha[q];
-          const float* pv = ss + q * kAttKT;
-#pragma unroll 8
-          for (int kk = 0; kk < kAttKT; ++kk) a = fmaf(pv[kk], vs[kk * hd + dd], a);
-          acc[i] = a;
+      for (int i0 = 0; i0 < NA; i0 += kAttQB)
+        if (i0 * ng < nq) {   // block-uniform
+          float a[kAttQB];
+          const float* pq[kAttQB];
+#pragma unroll
+          for (int i = 0; i < kAttQB; ++i) {
+            const int q = min(grp + ng * (i0 + i), nq - 1);
+            pq[i] = ss + q * kAttKT;
+            a[i] = acc[i0 + i] * alpha[q];
+          }
+#pragma unroll 4
+          for (int kk = 0; kk < kAttKT; kk += 4) {
+            const float v0 = vs[kk * hd + dd], v1 = vs[(kk + 1) * hd + dd], v2 = vs[(kk + 2) * hd + dd], v3 = vs[(kk + 3) * hd + dd];
+#pragma unroll
+            for (int i = 0; i < kAttQB; ++i) {
+              const float4 p = *reinterpret_cast<const float4*>(pq[i] + kk);
+              a[i] = fmaf(p.w, v3, fmaf(p.z, v2, fmaf(p.y, v1, fmaf(p.x, v0, a[i]))));
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < kAttQB; ++i) acc[i0 + i] = a[i];
         }
-      }
     }
     __syncthreads();
     // partials: index ((chunk * Hq + head) * rows + j)
+    const size_t p0 = ((size_t)chunk * dm.Hq + kvh * group) * rows;   // query q of the group is p0 + q
 #pragma unroll
-    for (int i = 0; i < 48; ++i) {
-      int e = tid + i * kAttThreads;
-      if (e < nq * hd) {
-        int q = e / hd, dd = e % hd, g = q / rows, j = q % rows;
-        size_t pi = ((size_t)chunk * dm.Hq + kvh * group + g) * rows + j;
-        w.att_o[pi * hd + dd] = acc[i];
-      }
+    for (int i = 0; i < NA; ++i) {
+      const int q = tid / hd + ng * i;
+      if (q < nq) w.att_o[(p0 + q) * hd + tid % hd] = acc[i];
     }
     for (int q = tid; q < nq; q += kAttThreads) {
-      int g = q / rows, j = q % rows;
-      size_t pi = ((size_t)chunk * dm.Hq + kvh * group + g) * rows + j;
-      w.att_m[pi] = m_run[q];
-      w.att_l[pi] = l_run[q];
+      w.att_m[p0 + q] = m_run[q];
+      w.att_l[p0 + q] = l_run[q];
     }
   }
+  if (!waited) { pdl_wait(); pdl_launch(); }
 }
 
-// Merge the partials of one (row, head) over its sequence's chunks, in chunk order.
+// Merge the partials of one (row, head) over its sequence's chunks, in chunk order: a warp each, the chunks' maxima and sums
+// one per lane, four chunks' outputs in flight.
+constexpr int kSimtMergeThreads = 128;
 template <typename T>
-__global__ void k_attn_combine(const StepArgs* __restrict__ args, Work w, Dims dm) {
+__global__ void __launch_bounds__(kSimtMergeThreads) k_attn_combine(const StepArgs* __restrict__ args, Work w, Dims dm, int R) {
+  const int rows = args->gamma + 1, lane = threadIdx.x & 31;
+  const int item = blockIdx.x * (kSimtMergeThreads / 32) + (threadIdx.x >> 5), r = item / dm.Hq, h = item % dm.Hq;
+  const int b = min(r, R - 1) / rows, j = r % rows;
+  const int c0 = w.chunk_start[b], c1 = w.chunk_start[b + 1];   // written before the kernel that this one waits for
   pdl_wait();
   pdl_launch();
-  const int rows = args->gamma + 1;
-  const int r = blockIdx.x / dm.Hq, h = blockIdx.x % dm.Hq;
-  const int b = r / rows, j = r % rows;
-  const int c0 = w.chunk_start[b], c1 = w.chunk_start[b + 1];
-  float M = -INFINITY;
-  for (int c = c0; c < c1; ++c) M = fmaxf(M, w.att_m[((size_t)c * dm.Hq + h) * rows + j]);
-  float Lsum = 0.f;
-  for (int c = c0; c < c1; ++c) {
-    size_t pi = ((size_t)c * dm.Hq + h) * rows + j;
-    float m = w.att_m[pi];
-    if (m != -INFINITY) Lsum += w.att_l[pi] * expf(m - M);
-  }
-  for (int dd = threadIdx.x; dd < dm.hd; dd += blockDim.x) {
-    float o = 0.f;
-    for (int c = c0; c < c1; ++c) {
-      size_t pi = ((size_t)c * dm.Hq + h) * rows + j;
-      float m = w.att_m[pi];
-      if (m != -INFINITY) o += w.att_o[pi * dm.hd + dd] * expf(m - M);
+  if (r >= R) return;
+  const int n = c1 - c0, dpl = dm.hd / 32;   // 2 or 4 dimensions per lane
+  const size_t p0 = ((size_t)c0 * dm.Hq + h) * rows + j, step = (size_t)dm.Hq * rows;
+  const float2* o2 = reinterpret_cast<const float2*>(w.att_o + p0 * dm.hd) + lane;
+  const size_t step2 = step * dm.hd / 2;
+  float M = -INFINITY, lsum = 0.f;
+  float2 o[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  for (int k0 = 0; k0 < n; k0 += 32) {
+    const int kn = min(32, n - k0);
+    const bool live = lane < kn;
+    const float m = live ? __ldcg(w.att_m + p0 + (size_t)(k0 + lane) * step) : -INFINITY, l = live ? __ldcg(w.att_l + p0 + (size_t)(k0 + lane) * step) : 0.f;
+    const float Mn = fmaxf(M, warp_max(m)), f = M == -INFINITY ? 0.f : expf(M - Mn);
+    const float wt = m == -INFINITY ? 0.f : expf(m - Mn);
+    lsum = lsum * f + warp_sum(l * wt);
+    M = Mn;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) { o[e].x *= f; o[e].y *= f; }
+    for (int k = 0; k < kn; k += 4) {
+      float2 x[4][2];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (2 * e < dpl) x[u][e] = __ldcg(o2 + (size_t)(k0 + min(k + u, kn - 1)) * step2 + 32 * e);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float wu = __shfl_sync(0xffffffffu, wt, min(k + u, 31));
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (2 * e < dpl && k + u < kn) { o[e].x += x[u][e].x * wu; o[e].y += x[u][e].y * wu; }
+      }
     }
-    store_act<T>(w.ATT, gridDim.x / dm.Hq, dm.Hq * dm.hd, r, h * dm.hd + dd, o / Lsum);
   }
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+    if (2 * e < dpl) {
+      store_act<T>(w.ATT, R, dm.Hq * dm.hd, r, h * dm.hd + 64 * e + 2 * lane, o[e].x / lsum);
+      store_act<T>(w.ATT, R, dm.Hq * dm.hd, r, h * dm.hd + 64 * e + 2 * lane + 1, o[e].y / lsum);
+    }
 }
 
 // Dot product of GEMM-input row r (both bf16 planes) with one weight row, over the whole warp.

@@ -1251,7 +1251,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
         GemmSegs g{{L.wq, L.wk, L.wv}, {qd, kd, kd}, 3};
         TIMED("gemm_cudacore", launch_cudacore(t, t->s_qkv, W.A, g, W.P, R, qd + 2 * kd, dm.d, pdl));
       }
-      TIMED("qkv_rope", launch(k_qkv_rope<T>, dim3(R), dim3(256), 0, s, pdl, args, kv->view, W, dm, plan_of(t->s_qkv),
+      TIMED("qkv_rope", launch(k_qkv_rope<T>, dim3(R, ((dm.Hq + dm.Hkv) * dm.hd / 2 + 255) / 256), dim3(256), 0, s, pdl, args, kv->view, W, dm, plan_of(t->s_qkv),
                     (size_t)R * (qd + 2 * kd), l, (const T*)L.bq, (const T*)L.bk, (const T*)L.bv));
     }
     if (kv_only && l == dm.n_layers - 1) return SJ_OK;
@@ -1299,7 +1299,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
       GemmSegs g{{L.wo, nullptr, nullptr}, {dm.d, 0, 0}, 1};
       TIMED("gemm_cudacore", launch_cudacore(t, t->s_o, W.ATT, g, W.P, R, dm.d, qd, pdl));
     }
-    TIMED("reduce_norm", launch(k_reduce_norm<T>, dim3(R), dim3(256), row_smem, s, pdl, args, W, dm, plan_of(t->s_o), (size_t)R * dm.d,
+    TIMED("reduce_norm", launch(k_reduce_norm<T>, dim3(R), dim3(kNormThreads), row_smem, s, pdl, args, W, dm, plan_of(t->s_o), (size_t)R * dm.d,
                   (const T*)L.nf, 0));
     // gate/up + SwiGLU
     if (tc) {
@@ -1319,7 +1319,7 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
     }
     const bool last = (l == dm.n_layers - 1);
     const void* gain = last ? t->final_norm : t->layers[l + 1].na;
-    TIMED("reduce_norm", launch(k_reduce_norm<T>, dim3(R), dim3(256), row_smem, s, pdl, args, W, dm, plan_of(t->s_down),
+    TIMED("reduce_norm", launch(k_reduce_norm<T>, dim3(R), dim3(kNormThreads), row_smem, s, pdl, args, W, dm, plan_of(t->s_down),
                   (size_t)R * dm.d, (const T*)gain, last ? 1 : 0));
   }
   return SJ_OK;

@@ -95,9 +95,15 @@ __device__ __forceinline__ float reduce_partials(const float* __restrict__ P, co
                                                  int N, int r, int n) {
   const float* p = P + (size_t)r * N + n;
   if (sp.tile_slots == nullptr) return *p;
-  int cnt = sp.tile_slots[n >> sp.tile_shift].y;
+  const int cnt = sp.tile_slots[n >> sp.tile_shift].y;
   float s = 0.f;
-  for (int i = 0; i < cnt; ++i) s += p[(size_t)i * slot_stride];
+  for (int i = 0; i < cnt; i += 4) {   // four slots in flight, added in order
+    float v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = p[(size_t)min(i + u, cnt - 1) * slot_stride];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s += i + u < cnt ? v[u] : 0.f;
+  }
   return s;
 }
 

@@ -180,7 +180,10 @@ __global__ void k_embed_norm(const StepArgs* __restrict__ args, KvView kv, Work 
   norm_row_from_smem<T>(xs, dm.d, gain, dm.eps, w.A, gridDim.x, r, nullptr, nullptr, red);
 }
 
-// a6/a8 tail + a2/a9: X += sum of partials; A = RMSNorm(X) * gain.  final: also fp32 hidden.
+// a6/a8 tail + a2/a9: X += sum of partials; A = RMSNorm(X) * gain.  final: also fp32 hidden.  A row is one block, as wide as
+// blocks get: what bounds it is the chain of loads of a thread's columns.  (This and k_qkv_rope's second grid dimension:
+// 1B-shaped fp32 cut of 4 layers, 10 rows, a step 763 -> 674 us on a B200.)
+constexpr int kNormThreads = 1024;
 template <typename T>
 __global__ void k_reduce_norm(const StepArgs* __restrict__ args, Work w, Dims dm, SplitPlan sp, size_t slot_stride,
                               const T* __restrict__ gain, int final_norm) {
@@ -189,6 +192,7 @@ __global__ void k_reduce_norm(const StepArgs* __restrict__ args, Work w, Dims dm
   pdl_wait();
   pdl_launch();
   const int r = blockIdx.x;
+#pragma unroll 2
   for (int i = threadIdx.x; i < dm.d; i += blockDim.x) {
     float x = w.X[(size_t)r * dm.d + i] + reduce_partials(w.P, sp, slot_stride, dm.d, r, i);
     xs[i] = x;
@@ -214,7 +218,8 @@ __global__ void k_final_norm(const StepArgs* __restrict__ args, Work w, Dims dm,
                         args->dbg_hidden ? args->dbg_hidden + (size_t)r * dm.d : nullptr, red);
 }
 
-// a3 tail + a4: reduce QKV partials, add bias, rotate q and k, store q, append k and v rows.
+// a3 tail + a4: reduce QKV partials, add bias, rotate q and k, store q, append k and v rows.  gridDim.y blocks share a row (with
+// one block per row a thread walked through five pairs of dependent loads while most SMs had nothing to do).
 template <typename T>
 __global__ void k_qkv_rope(const StepArgs* __restrict__ args, KvView kv, Work w, Dims dm, SplitPlan sp,
                            size_t slot_stride, int layer, const T* __restrict__ bq, const T* __restrict__ bk,
@@ -232,7 +237,8 @@ __global__ void k_qkv_rope(const StepArgs* __restrict__ args, KvView kv, Work w,
   const int slot = pos % kv.page_size;
   const float2* rt = w.rope + (size_t)r * half;
   // rotated heads: q heads then k heads
-  for (int p = threadIdx.x; p < (dm.Hq + dm.Hkv) * half; p += blockDim.x) {
+  const int first = blockIdx.y * blockDim.x + threadIdx.x, step = gridDim.y * blockDim.x;
+  for (int p = first; p < (dm.Hq + dm.Hkv) * half; p += step) {
     int head = p / half, i = p % half;
     int n1 = head * dm.hd + i, n2 = n1 + half;
     float x1 = reduce_partials(w.P, sp, slot_stride, N, r, n1);
@@ -273,7 +279,7 @@ __global__ void k_qkv_rope(const StepArgs* __restrict__ args, KvView kv, Work w,
       }
     }
   }
-  for (int p = threadIdx.x; p < kd; p += blockDim.x) {
+  for (int p = first; p < kd; p += step) {
     float x = reduce_partials(w.P, sp, slot_stride, N, r, qd + kd + p);
     if (bv) x += to_f(bv[p]);
     if (store_kv) kv_row<T>(kv, layer, page, 1, p / dm.hd, slot)[p % dm.hd] = from_f<T>(x);

@@ -334,6 +334,19 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     for (int item = g; item < n_items; item += p.n_groups) {
       const int tile = 2 * (item / p.n_rb) + rank, r_lo = item % p.n_rb * p.rb, r_hi = min(r_lo + p.rb, R);
       const bool real = tile < p.n_tiles;   // an odd last tile's partner has no features
+      // per-feature constants, requested beside the MMAs
+      int kind = 0, head = 0, dim = 0;
+      float bias = 0.f, gn = 1.f;
+      if constexpr (SITE == PAIR_QKV) {
+        int fs = tile * kTileN + fl;
+        const bf16* bp = p.bq;
+        if (tile >= p.tile_k) { kind = 2; fs -= p.tile_k * kTileN; bp = p.bv; }
+        else if (tile >= p.tile_q) { kind = 1; fs -= p.tile_q * kTileN; bp = p.bk; }
+        head = fs / HD;
+        dim = fs % HD;
+        if (bp && real) bias = __bfloat162float(bp[fs]);
+      }
+      if constexpr (SITE == PAIR_RES) gn = real ? __bfloat162float(p.gain[tile * kTileN + fl]) : 0.f;
       // residual rows of the first chunk that this split finishes, requested beside the MMAs
       float x_first[16];
       if constexpr (SITE == PAIR_RES) {
@@ -421,26 +434,21 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         cluster_arrive_all();
       }
 
-      // per-feature constants
-      int kind = 0, head = 0, dim = 0;
-      float bias = 0.f, gn = 1.f;
-      if constexpr (SITE == PAIR_QKV) {
-        int fs = tile * kTileN + fl;
-        const bf16* bp = p.bq;
-        if (tile >= p.tile_k) { kind = 2; fs -= p.tile_k * kTileN; bp = p.bv; }
-        else if (tile >= p.tile_q) { kind = 1; fs -= p.tile_q * kTileN; bp = p.bk; }
-        head = fs / HD;
-        dim = fs % HD;
-        if (bp && real) bias = __bfloat162float(bp[fs]);
-      }
-      if constexpr (SITE == PAIR_RES) gn = real ? __bfloat162float(p.gain[tile * kTileN + fl]) : 0.f;
-
-#pragma unroll
+      // Not unrolled: a chunk's own copy of this code would come from L2 when the chunk is reached, and most copies run once a
+      // launch.  The sums move down a chunk each time instead.  (8B-shaped, 44 rows: a score 12602 -> 12395 us; 1B-shaped, 48 rows: a
+      // step 961 -> 946; 8B-shaped prefill of 1000 tokens 32.1 -> 31.5 ms; B200.)
+#pragma unroll 1
       for (int j = 0; j < 4; ++j) {
         const int c0 = r_lo + 16 * grp + 32 * j, nr = min(16, r_hi - c0);
         if (nr <= 0 || !real) break;   // uniform over the group
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          v[i] = sum[0][i];
+#pragma unroll
+          for (int k = 0; k < 3; ++k) sum[k][i] = sum[k + 1][i];
+        }
         if (!(mine >> j & 1u)) continue;
-        float (&v)[16] = sum[j];
         float xs[16];
         if constexpr (SITE == PAIR_RES) {
           if (j == split) {

@@ -1214,13 +1214,13 @@ static sj_status enqueue_layers(sj_target* t, sj_kv* kv, int B, int gamma, int c
   cudaStream_t s = t->stream;
   const size_t row_smem = sizeof(float) * dm.d;
   const CUtensorMap *mA_d = nullptr, *mA_q = nullptr, *mA_f = nullptr;
-  if (tc) {
+  const bool pair = pair_usable(t, kv);
+  if (tc && !pair) {
     sj_status st;
     if ((st = activation_map(t, W.A, R, dm.d, &mA_d)) != SJ_OK) return st;
     if ((st = activation_map(t, W.ATT, R, qd, &mA_q)) != SJ_OK) return st;
     if ((st = activation_map(t, W.H, R, dm.F, &mA_f)) != SJ_OK) return st;
   }
-  const bool pair = pair_usable(t, kv);
   // A prefill's sums of few K blocks (1B-shaped widths: 32) in chains half as long.  The persistent kernel, which runs the
   // narrow blocks, deals such a projection in shares of about five blocks; with chains of 16 the step on a prefilled cache
   // of 400 tokens was off by 1.97e-4 of the hidden state where its was 1.43e-4, with 8 by 1.63e-4 (4 layers).  Wider models have
@@ -1780,9 +1780,9 @@ extern "C" sj_status sj_semantic_score(sj_target* t, sj_kv* kv, int seq, int y_i
 // bf16 pages, so another partition would give slightly other results) over the same sequence -- entry b attends to the stored cache plus the b * c rows before it
 // (its projection has stored them in the pages by the time the attention kernel runs) and to its own rows, which is
 // exactly what B verification steps of c rows one after another would do, at one read of the weights (8B-shaped model,
-// 1000 tokens and a step: 190 ms in blocks of 24 rows, 34 ms in two of 504).  Only the last token's row meets the
+// 1000 tokens and a step: 190 ms in blocks of 24 rows, 34 ms in two of 504, 32 in one of 1008).  Only the last token's row meets the
 // LM head, and a block that is not the last one ends with its key / value rows.
-constexpr int kPrefillRows = SJ_MAX_ROWS;   // rows of a wide block
+constexpr int kPrefillRows = kPairMaxRows;   // rows of a wide block
 
 static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* tokens, int n_tokens, int c, int* d_next, bool* done) {
   const Dims& dm = t->dm;

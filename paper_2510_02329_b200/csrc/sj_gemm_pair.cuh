@@ -46,7 +46,7 @@ namespace sj {
 constexpr int kPairThreads = 384;      // warp 0 TMA, warp 1 MMA (rank 0), warp 2 tensor memory, warps 4..11 epilogue
 constexpr int kPairWorkers = 256;
 constexpr int kPairMaxStages = 10;
-constexpr int kPairMaxRows = kMaxRows;
+constexpr int kPairMaxRows = 1024;     // of a prefill's blocks; a step has at most kMaxRows
 constexpr int kPairSegKB = 16, kPairShortKB = 32;   // K blocks of 64 per accumulation chain; half of them in a prefill's sums of up to kPairShortKB
 constexpr int kPairMaxSplit = 4;        // pairs that share an item's K (a cluster of 8)
 constexpr double kPairHbmBytesPerClk = 3600;   // HBM against the SM clock, for the host's choice of a geometry
@@ -96,10 +96,10 @@ struct PairQkvCtl {
   float exch[2][128][9];
 };
 struct PairGuCtl { float exch[2][128][9]; };
-struct PairResCtl { float sums[4][kPairMaxRows]; };
+struct PairResCtl { float sums[4][128]; };   // by row of the item's block
 struct PairLmCtl {
-  int tok[kPairMaxRows];
-  float pre[kPairMaxRows];
+  int tok[kMaxRows];
+  float pre[kMaxRows];
   RowStat st[2][4][16];
 };
 template <int SITE> struct PairExtra;
@@ -517,7 +517,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             }
           }
           const float t = warp_sum_n<16>(sq, lane);
-          if ((lane & 1) == 0) sm->x.sums[quarter][c0 + (lane >> 1)] = t;
+          if ((lane & 1) == 0) sm->x.sums[quarter][c0 - r_lo + (lane >> 1)] = t;
         } else if constexpr (SITE == PAIR_GU) {
 #pragma unroll
           for (int i = 0; i < 16; ++i) v[i] *= (i < nr ? ctl->inv[c0 + i] : 0.f);
@@ -589,7 +589,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         if (real)
           for (int r = r_lo + wt; r < r_hi; r += kPairWorkers)
             if (mine >> ((r - r_lo) >> 5) & 1u)
-              p.ssq_out[(size_t)tile * R + r] = (sm->x.sums[0][r] + sm->x.sums[1][r]) + (sm->x.sums[2][r] + sm->x.sums[3][r]);
+              p.ssq_out[(size_t)tile * R + r] = (sm->x.sums[0][r - r_lo] + sm->x.sums[1][r - r_lo]) + (sm->x.sums[2][r - r_lo] + sm->x.sums[3][r - r_lo]);
         all_sync();
       }
     }

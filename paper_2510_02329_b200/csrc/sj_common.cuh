@@ -168,6 +168,20 @@ __device__ __forceinline__ void warp_max_n(const float* v, int id, int lane, flo
   arg = b[0];
 }
 
+// Maximum of each of 16 values over the warp: a lane returns that of value lane / 2.
+__device__ __forceinline__ float warp_max16(const float* v, int lane) {
+  float a[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) a[i] = v[i];
+#pragma unroll
+  for (int h = 8; h >= 1; h >>= 1) {
+    const bool up = lane & (2 * h);
+#pragma unroll
+    for (int i = 0; i < h; ++i) a[i] = fmaxf(up ? a[i + h] : a[i], __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + h], 2 * h));
+  }
+  return fmaxf(a[0], __shfl_xor_sync(0xffffffffu, a[0], 1));
+}
+
 // Maximum of each of 8 values over the warp: a lane returns that of value lane / 4.
 __device__ __forceinline__ float warp_max8(const float* v, int lane) {
   float a[8];

@@ -328,6 +328,14 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     }
     all_sync();
     const int n_seg = (kb_hi - kb_lo + p.seg_kb - 1) / p.seg_kb;
+    float invT = 1.f, *dbg = nullptr, *keep = nullptr;
+    bool topk = false;
+    if constexpr (SITE == PAIR_LM) {
+      invT = args->inv_temperature;
+      topk = args->top_k >= 2;
+      dbg = args->dbg_logits;
+      keep = w.logits;
+    }
     int n = 0, n_x = 0;   // segments, exchanges so far
     uint32_t mine = 0;    // the chunks j that this split finishes
     for (int j = split; j < 4; j += S) mine |= 1u << j;
@@ -535,37 +543,53 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           }
           group_sync();
         } else {   // LM head
-          const int n_id = tile * kTileN + fl;
-          const float invT = args->inv_temperature;
-          const bool topk = args->top_k >= 2;
-          float *dbg = args->dbg_logits, *keep = w.logits;   // asked for; sampling mode
+          // What bounds a wide step's LM head is this code's instruction count: two warps on a scheduler issue one instruction in five
+          // clocks each, and at 342 rows an item's epilogue took longer than its MMAs (8B-shaped, 8 layers, top-2 alignment: a step 3607 -> 3559 us, B200).  So what concerns few steps or few
+          // tiles (bounds, stored logits, drafted tokens) is decided once a chunk, and a maximum's token comes from a ballot.
+          const int n_id = tile * kTileN + fl, n_warp = n_id - lane;
           const int own = lane >> 1;   // the chunk's row whose totals this lane ends up with
-          int before = 0;
+          if (nr < 16 || (tile + 1) * kTileN > dm.V) {   // uniform over the group
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int r = min(c0 + i, R - 1);
-            if (topk) {   // uniform
-              const int tg = sm->x.tok[r];
-              const float zd = sm->x.pre[r];
-              const bool bf = i < nr && n_id < dm.V && tg >= 0 && n_id != tg && (v[i] > zd || (v[i] == zd && n_id < tg));
-              const int c = __popc(__ballot_sync(0xffffffffu, bf));
-              if (i == own) before = c;
-            }
-            if (i < nr && n_id < dm.V) {
-              if (dbg) dbg[(size_t)r * dm.V + n_id] = v[i];
-              if (keep) keep[(size_t)r * dm.V + n_id] = v[i];
-              v[i] *= invT;
-              if (n_id == sm->x.tok[r]) w.tgt_logit[r] = v[i];
-            } else {
-              v[i] = -INFINITY;
+            for (int i = 0; i < 16; ++i)
+              if (i >= nr || n_id >= dm.V) v[i] = -INFINITY;
+          }
+          if (dbg || keep) {   // logits asked for; sampling mode
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if (i < nr && n_id < dm.V) {
+                if (dbg) dbg[(size_t)(c0 + i) * dm.V + n_id] = v[i];
+                if (keep) keep[(size_t)(c0 + i) * dm.V + n_id] = v[i];
+              }
+          }
+          // lane i (and i + 16): the drafted token of row i
+          const int tok = (lane & 15) < nr ? sm->x.tok[c0 + (lane & 15)] : -1;
+          int before = 0;
+          if (topk) {   // uniform
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const int tg = __shfl_sync(0xffffffffu, tok, i);
+              const float zd = sm->x.pre[min(c0 + i, R - 1)];
+              const int c = __popc(__ballot_sync(0xffffffffu, n_id != tg && (v[i] > zd || (v[i] == zd && n_id < tg))));
+              if (i == own && tg >= 0) before = c;
             }
           }
-          float m;
-          int arg;
-          warp_max_n<16>(v, n_id, lane, m, arg);
+          if (invT != 1.f) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] *= invT;
+          }
+          const unsigned here = __ballot_sync(0xffffffffu, lane < 16 && tok >= n_warp && tok < min(n_warp + 32, dm.V));
+          if (here) {   // uniform over the warp: some row's drafted token is one of its tokens
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if ((here >> i & 1u) && n_id == __shfl_sync(0xffffffffu, tok, i)) w.tgt_logit[c0 + i] = v[i];
+          }
+          const float m = warp_max16(v, lane);
+          int arg = 0x7fffffff;
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const float mi = __shfl_sync(0xffffffffu, m, 2 * i);
+            const unsigned at = __ballot_sync(0xffffffffu, v[i] == mi);   // the lowest lane has the lowest token
+            if (i == own && at) arg = n_warp + __ffs(at) - 1;
             v[i] = v[i] == -INFINITY ? 0.f : expf(v[i] - mi);
           }
           const float e = warp_sum_n<16>(v, lane);

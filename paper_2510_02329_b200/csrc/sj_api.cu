@@ -429,14 +429,16 @@ static F32Kernel f32_kernel(int rt) { return rt <= 4 ? k_gemm_f32<4> : (rt <= 8 
 
 typedef void (*PairKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const PairParams, const StepArgs*,
                            const KvView, const Work, const Dims);
-static PairKernel pair_kernel(int site, int hd) {
+template <bool NARROW>
+static PairKernel pair_kernel_of(int site, int hd) {
   switch (site) {
-    case PAIR_QKV: return hd == 128 ? k_gemm_pair<PAIR_QKV, 128> : k_gemm_pair<PAIR_QKV, 64>;
-    case PAIR_RES: return k_gemm_pair<PAIR_RES, 0>;
-    case PAIR_GU: return k_gemm_pair<PAIR_GU, 0>;
-    default: return k_gemm_pair<PAIR_LM, 0>;
+    case PAIR_QKV: return hd == 128 ? k_gemm_pair<PAIR_QKV, 128, NARROW> : k_gemm_pair<PAIR_QKV, 64, NARROW>;
+    case PAIR_RES: return k_gemm_pair<PAIR_RES, 0, NARROW>;
+    case PAIR_GU: return k_gemm_pair<PAIR_GU, 0, NARROW>;
+    default: return k_gemm_pair<PAIR_LM, 0, NARROW>;
   }
 }
+static PairKernel pair_kernel(int site, int hd, int rb) { return rb <= 16 ? pair_kernel_of<true>(site, hd) : pair_kernel_of<false>(site, hd); }
 
 extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weights* w, void* cuda_stream,
                                       sj_target** out) {
@@ -543,8 +545,9 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
     }
     if ((st = make_map(&t->m_lm, t->lm_head, c.vocab, c.d_model, kTileN)) != SJ_OK) return bail(st);
     cudaError_t e = cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    for (int site = PAIR_QKV; site <= PAIR_LM && e == cudaSuccess; ++site)
-      e = cudaFuncSetAttribute(pair_kernel(site, c.head_dim), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    for (int site = PAIR_QKV; site <= PAIR_LM; ++site)
+      for (int rb = 16; rb <= 32 && e == cudaSuccess; rb += 16)
+        e = cudaFuncSetAttribute(pair_kernel(site, c.head_dim, rb), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) { fail(SJ_ERR_CUDA, "smem opt-in: %s", cudaGetErrorString(e)); return bail(SJ_ERR_CUDA); }
     // clusters of S pairs, one CTA per SM, that are resident at once (all of a site's kernels take most of an SM)
     t->pair_clusters[1] = t->sm_count / 2;
@@ -560,7 +563,7 @@ extern "C" sj_status sj_create_target(const sj_model_config* cfg, const sj_weigh
       cfg.attrs = &at;
       cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, pair_kernel(PAIR_RES, c.head_dim), &cfg) != cudaSuccess) { n = 0; cudaGetLastError(); }
+      if (cudaOccupancyMaxActiveClusters(&n, pair_kernel(PAIR_RES, c.head_dim, 32), &cfg) != cudaSuccess) { n = 0; cudaGetLastError(); }
       t->pair_clusters[S] = n;
     }
   }
@@ -1073,10 +1076,11 @@ static PairGeom pair_geom(int R, int n_tiles, int KB, const int* clusters, int s
   g.tmem_cols = 32;
   while (g.tmem_cols < (uint32_t)(4 * g.rb)) g.tmem_cols <<= 1;
   g.stage_bytes = kWTileBytes + g.rb * 128;
-  g.xch_js = ((g.rb + 31) / 32 + g.n_split - 1) / g.n_split;
+  const int ch = pair_chunk(g.rb <= 16);
+  g.xch_js = ((g.rb + 2 * ch - 1) / (2 * ch) + g.n_split - 1) / g.n_split;
   const size_t ctl = (site == PAIR_QKV ? sizeof(PairSmem<PAIR_QKV>) : site == PAIR_RES ? sizeof(PairSmem<PAIR_RES>)
                       : site == PAIR_GU ? sizeof(PairSmem<PAIR_GU>) : sizeof(PairSmem<PAIR_LM>)) +
-                     (size_t)(g.n_split - 1) * 2 * g.xch_js * 8192;
+                     (size_t)(g.n_split - 1) * 2 * g.xch_js * 512 * ch;
   g.stages = std::min<int>(kPairMaxStages, (int)((227 * 1024 - 1024 - ctl) / g.stage_bytes));
   g.smem = (size_t)g.stages * g.stage_bytes + ctl + 1024;
   return g;
@@ -1132,7 +1136,7 @@ static sj_status launch_pair(sj_target* t, sj_kv* kv, int site, int n_tiles, int
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 2 : 1;
-  CU_TRY(cudaLaunchKernelEx(&cfg, pair_kernel(site, dm.hd), *mA, *w0, *(w1 ? w1 : w0), *(w2 ? w2 : w0), p, (const StepArgs*)t->d_args,
+  CU_TRY(cudaLaunchKernelEx(&cfg, pair_kernel(site, dm.hd, g.rb), *mA, *w0, *(w1 ? w1 : w0), *(w2 ? w2 : w0), p, (const StepArgs*)t->d_args,
                             kv->view, W, dm));
   return SJ_OK;
 }

@@ -415,7 +415,7 @@ __device__ __forceinline__ bool a5_softmax(const A5Ring& rg, A5Bars* ab, A5Smem*
 #pragma unroll
         for (int c = 0; c < MAXC; ++c)
           if (c < nch) {
-            const float mx = warp_max8(s[c], lane);
+            const float mx = warp_fmax_n<8>(s[c], lane);
             if ((lane & 3) == 0) sh->red[quarter][q0 + 8 * c + (lane >> 2)] = mx;
           }
         bar_sync128(bar_id);

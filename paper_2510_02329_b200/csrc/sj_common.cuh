@@ -168,33 +168,22 @@ __device__ __forceinline__ void warp_max_n(const float* v, int id, int lane, flo
   arg = b[0];
 }
 
-// Maximum of each of 16 values over the warp: a lane returns that of value lane / 2.
-__device__ __forceinline__ float warp_max16(const float* v, int lane) {
-  float a[16];
+// Maximum of each of N values (N = 8 or 16) over the warp: a lane returns that of value lane / (32 / N).
+template <int N>
+__device__ __forceinline__ float warp_fmax_n(const float* v, int lane) {
+  float a[N];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) a[i] = v[i];
+  for (int i = 0; i < N; ++i) a[i] = v[i];
+  int bit = 16;
 #pragma unroll
-  for (int h = 8; h >= 1; h >>= 1) {
-    const bool up = lane & (2 * h);
+  for (int h = N / 2; h >= 1; h >>= 1, bit >>= 1) {
+    const bool up = lane & bit;
 #pragma unroll
-    for (int i = 0; i < h; ++i) a[i] = fmaxf(up ? a[i + h] : a[i], __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + h], 2 * h));
+    for (int i = 0; i < h; ++i) a[i] = fmaxf(up ? a[i + h] : a[i], __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + h], bit));
   }
-  return fmaxf(a[0], __shfl_xor_sync(0xffffffffu, a[0], 1));
-}
-
-// Maximum of each of 8 values over the warp: a lane returns that of value lane / 4.
-__device__ __forceinline__ float warp_max8(const float* v, int lane) {
-  float a[8];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) a[i] = v[i];
-#pragma unroll
-  for (int h = 4; h >= 1; h >>= 1) {
-    const bool up = lane & (4 * h);
-#pragma unroll
-    for (int i = 0; i < h; ++i) a[i] = fmaxf(up ? a[i + h] : a[i], __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + h], 4 * h));
-  }
-  a[0] = fmaxf(a[0], __shfl_xor_sync(0xffffffffu, a[0], 2));
-  return fmaxf(a[0], __shfl_xor_sync(0xffffffffu, a[0], 1));
+  for (; bit >= 1; bit >>= 1) a[0] = fmaxf(a[0], __shfl_xor_sync(0xffffffffu, a[0], bit));
+  return a[0];
 }
 
 // Block-wide sum with a fixed reduction tree (deterministic).  `red` holds >= 32 floats.

@@ -51,6 +51,7 @@ constexpr int kPairSegKB = 16, kPairShortKB = 32;   // K blocks of 64 per accumu
 constexpr int kPairMaxSplit = 4;        // pairs that share an item's K (a cluster of 8)
 constexpr double kPairHbmBytesPerClk = 3600;   // HBM against the SM clock, for the host's choice of a geometry
 constexpr int kPairXchClk = 3000;       // an exchange between the splits
+__host__ __device__ constexpr int pair_chunk(bool narrow) { return narrow ? 8 : 16; }   // rows of an epilogue chunk
 // "My sums have been read" barriers per epilogue group, taken in turn by successive exchanges.  A split that receives
 // nothing in an exchange (all of the row block's chunks belong to others) does not wait for its partners there and may
 // finish it before a partner has looked at the phase of the exchange before; on one barrier that phase would be overtaken,
@@ -171,16 +172,21 @@ __device__ __forceinline__ uint32_t instr_desc_pair(int n) {   // M = 256
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
 }
 
-template <int SITE, int HD>
+// NARROW: row blocks of 16, whose rows the two epilogue groups halve (chunks of 8 rows).  With chunks of 16 the second group had
+// nothing to do and every slot of 16 issued for the 5 rows of a toy step (68.1 -> 52.8 us, two caches in turn; alone 128 -> 114, B200).  Wider blocks keep chunks of 16: with 8
+// a score of 44 rows was 3 % slower.
+template <int SITE, int HD, bool NARROW>
 static __global__ void __launch_bounds__(kPairThreads, 1)
 k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
             const __grid_constant__ CUtensorMap tmW2, const PairParams p, const StepArgs* __restrict__ args, const KvView kv, const Work w,
             const Dims dm) {
+  // rows of an epilogue chunk, chunks of a group, lanes that share a row's totals
+  constexpr int CH = pair_chunk(NARROW), NJ = NARROW ? 1 : 4, LPR = 32 / CH;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  // ring | the other splits' sums [n_split - 1][2 groups][xch_js][4][128 features] of 4 rows each | control
+  // ring | the other splits' sums [n_split - 1][2 groups][xch_js][CH / 4][128 features] of 4 rows each | control
   float4* xch = reinterpret_cast<float4*>(smem + (size_t)p.stages * p.stage_bytes);
-  PairSmem<SITE>* sm = reinterpret_cast<PairSmem<SITE>*>(xch + (size_t)(p.n_split - 1) * 2 * p.xch_js * 512);
+  PairSmem<SITE>* sm = reinterpret_cast<PairSmem<SITE>*>(xch + (size_t)(p.n_split - 1) * 2 * p.xch_js * (32 * CH));
   PairCtl* ctl = &sm->c;
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int S = p.n_split, crank = (int)cluster_rank(), rank = crank & 1, split = crank >> 1, g = blockIdx.x / (2 * S);
@@ -292,7 +298,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     }
   } else if (warp >= 4) {
     // ------------------------------ epilogue (eight warps) ------------------------------
-    // two groups of four warps take alternate 16-row chunks; a warp reads the accumulator lanes 32 * (warp % 4) .. + 31
+    // two groups of four warps take alternate chunks of CH rows; a warp reads the accumulator lanes 32 * (warp % 4) .. + 31
     pdl_wait();
     const int wt = threadIdx.x - 128, grp = wt >> 7, fl = wt & 127, quarter = fl >> 5, bar_id = 2 + grp;
     const int R = p.R, rows = args->gamma + 1;
@@ -338,7 +344,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     }
     int n = 0, n_x = 0;   // segments, exchanges so far
     uint32_t mine = 0;    // the chunks j that this split finishes
-    for (int j = split; j < 4; j += S) mine |= 1u << j;
+    for (int j = split; j < NJ; j += S) mine |= 1u << j;
     for (int item = g; item < n_items; item += p.n_groups) {
       const int tile = 2 * (item / p.n_rb) + rank, r_lo = item % p.n_rb * p.rb, r_hi = min(r_lo + p.rb, R);
       const bool real = tile < p.n_tiles;   // an odd last tile's partner has no features
@@ -356,18 +362,18 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       }
       if constexpr (SITE == PAIR_RES) gn = real ? __bfloat162float(p.gain[tile * kTileN + fl]) : 0.f;
       // residual rows of the first chunk that this split finishes, requested beside the MMAs
-      float x_first[16];
+      float x_first[CH];
       if constexpr (SITE == PAIR_RES) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
-          x_first[i] = __ldcg(w.X + (size_t)min(r_lo + 16 * grp + 32 * split + i, R - 1) * dm.d + min(tile, p.n_tiles - 1) * kTileN + fl);
+        for (int i = 0; i < CH; ++i)
+          x_first[i] = __ldcg(w.X + (size_t)min(r_lo + CH * (grp + 2 * split) + i, R - 1) * dm.d + min(tile, p.n_tiles - 1) * kTileN + fl);
       }
       // the segments' sums: chunk j of this group in registers
-      float sum[4][16];
+      float sum[NJ][CH];
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
+      for (int j = 0; j < NJ; ++j)
 #pragma unroll
-        for (int i = 0; i < 16; ++i) sum[j][i] = 0.f;
+        for (int i = 0; i < CH; ++i) sum[j][i] = 0.f;
 #pragma unroll 1
       for (int sg = 0; sg < n_seg; ++sg, ++n) {
         const int acc = n & 1;
@@ -378,14 +384,19 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         tc_fence_after();
         const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 2 * p.rb);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int c = 16 * grp + 32 * j;   // row of the chunk within the block
-          if (r_lo + c < r_hi) {             // uniform over the group
-            float hi[16], lo[16];
-            tc_ld16(taddr + (uint32_t)c, hi);
-            tc_ld16(taddr + (uint32_t)(p.rb + c), lo);
+        for (int j = 0; j < NJ; ++j) {
+          const int c = CH * (grp + 2 * j);   // row of the chunk within the block
+          if (r_lo + c < r_hi) {              // uniform over the group
+            float hi[CH], lo[CH];
+            if constexpr (NARROW) {
+              tc_ld8(taddr + (uint32_t)c, hi);
+              tc_ld8(taddr + (uint32_t)(p.rb + c), lo);
+            } else {
+              tc_ld16(taddr + (uint32_t)c, hi);
+              tc_ld16(taddr + (uint32_t)(p.rb + c), lo);
+            }
 #pragma unroll
-            for (int i = 0; i < 16; ++i) sum[j][i] += hi[i] + lo[i];
+            for (int i = 0; i < CH; ++i) sum[j][i] += hi[i] + lo[i];
           }
         }
         tc_fence_before();
@@ -400,28 +411,28 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         };
         if (fl == 0) {
           uint32_t bytes = 0;
-          for (int j = split; j < 4; j += S)
-            if (r_lo + 16 * grp + 32 * j < r_hi) bytes += (uint32_t)(S - 1) * 8192u;
+          for (int j = split; j < NJ; j += S)
+            if (r_lo + CH * (grp + 2 * j) < r_hi) bytes += (uint32_t)(S - 1) * (512u * CH);
           mbar_expect_tx(smem_u32(&ctl->xch_full[grp]), bytes);
         }
         if (n_x > 0) xch_wait(&ctl->xch_free[grp][(n_x - 1) % kPairFreeBars], (uint32_t)((n_x - 1) / kPairFreeBars) & 1u);
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (!(mine >> j & 1u) && r_lo + 16 * grp + 32 * j < r_hi) {
+        for (int j = 0; j < NJ; ++j)
+          if (!(mine >> j & 1u) && r_lo + CH * (grp + 2 * j) < r_hi) {
             const int f = j % S, slot = split < f ? split : split - 1;
-            const uint32_t dst = cluster_addr(smem_u32(xch + ((size_t)(slot * 2 + grp) * p.xch_js + j / S) * 512 + fl), 2 * f + rank);
+            const uint32_t dst = cluster_addr(smem_u32(xch + ((size_t)(slot * 2 + grp) * p.xch_js + j / S) * (32 * CH) + fl), 2 * f + rank);
             const uint32_t bar = cluster_addr(smem_u32(&ctl->xch_full[grp]), 2 * f + rank);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) cluster_st4_async(dst + (uint32_t)q * 2048u, &sum[j][4 * q], bar);
+            for (int q = 0; q < CH / 4; ++q) cluster_st4_async(dst + (uint32_t)q * 2048u, &sum[j][4 * q], bar);
           }
         xch_wait(&ctl->xch_full[grp], (uint32_t)n_x & 1u);
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if ((mine >> j & 1u) && r_lo + 16 * grp + 32 * j < r_hi) {
+        for (int j = 0; j < NJ; ++j)
+          if ((mine >> j & 1u) && r_lo + CH * (grp + 2 * j) < r_hi) {
             for (int slot = 0; slot < S - 1; ++slot) {
-              const float4* src = xch + ((size_t)(slot * 2 + grp) * p.xch_js + j / S) * 512 + fl;
+              const float4* src = xch + ((size_t)(slot * 2 + grp) * p.xch_js + j / S) * (32 * CH) + fl;
 #pragma unroll
-              for (int q = 0; q < 4; ++q) {
+              for (int q = 0; q < CH / 4; ++q) {
                 const float4 x = src[q * 128];
                 sum[j][4 * q] += x.x; sum[j][4 * q + 1] += x.y; sum[j][4 * q + 2] += x.z; sum[j][4 * q + 3] += x.w;
               }
@@ -446,33 +457,33 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       // launch.  The sums move down a chunk each time instead.  (8B-shaped, 44 rows: a score 12602 -> 12395 us; 1B-shaped, 48 rows: a
       // step 961 -> 946; 8B-shaped prefill of 1000 tokens 32.1 -> 31.5 ms; B200.)
 #pragma unroll 1
-      for (int j = 0; j < 4; ++j) {
-        const int c0 = r_lo + 16 * grp + 32 * j, nr = min(16, r_hi - c0);
+      for (int j = 0; j < NJ; ++j) {
+        const int c0 = r_lo + CH * (grp + 2 * j), nr = min(CH, r_hi - c0);
         if (nr <= 0 || !real) break;   // uniform over the group
-        float v[16];
+        float v[CH];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
+        for (int i = 0; i < CH; ++i) {
           v[i] = sum[0][i];
 #pragma unroll
-          for (int k = 0; k < 3; ++k) sum[k][i] = sum[k + 1][i];
+          for (int k = 0; k + 1 < NJ; ++k) sum[k][i] = sum[k + 1][i];
         }
         if (!(mine >> j & 1u)) continue;
-        float xs[16];
+        float xs[CH];
         if constexpr (SITE == PAIR_RES) {
           if (j == split) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) xs[i] = x_first[i];
+            for (int i = 0; i < CH; ++i) xs[i] = x_first[i];
           } else
 #pragma unroll
-          for (int i = 0; i < 16; ++i) xs[i] = __ldcg(w.X + (size_t)min(c0 + i, R - 1) * dm.d + tile * kTileN + fl);
+          for (int i = 0; i < CH; ++i) xs[i] = __ldcg(w.X + (size_t)min(c0 + i, R - 1) * dm.d + tile * kTileN + fl);
         }
         if constexpr (SITE == PAIR_QKV) {
           constexpr int half = HD / 2;
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] = v[i] * (i < nr ? ctl->inv[c0 + i] : 0.f) + bias;
+          for (int i = 0; i < CH; ++i) v[i] = v[i] * (i < nr ? ctl->inv[c0 + i] : 0.f) + bias;
           if (kind < 2) {   // uniform over the CTA
 #pragma unroll
-            for (int h8 = 0; h8 < 16; h8 += 8) {
+            for (int h8 = 0; h8 < CH; h8 += 8) {
               float2 cs[8];
 #pragma unroll
               for (int i = 0; i < 8; ++i) cs[i] = __ldcg(w.rope + (size_t)min(c0 + h8 + i, R - 1) * half + (dim & (half - 1)));
@@ -493,7 +504,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             __half* qb = w.Qb + (size_t)head * rows * HD + dim;
             __half* ql = w.Qlo + (size_t)head * rows * HD + dim;
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
+            for (int i = 0; i < CH; ++i)
               if (i < nr) {
                 const float qv = v[i] * qscale;
                 const __half hq = __float2half_rn(qv);
@@ -505,7 +516,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                         ((size_t)p.layer * kv.n_pages * 2 * dm.Hkv + (size_t)(kind - 1) * dm.Hkv + head) * kv.page_size * HD + dim;
             __half* kn = w.KVn + (size_t)(head * 2 + kind - 1) * rows * HD + dim;
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
+            for (int i = 0; i < CH; ++i)
               if (i < nr) {
                 if (sm->x.kvoff[c0 + i] >= 0) kvb[sm->x.kvoff[c0 + i]] = __float2bfloat16_rn(v[i]);
                 kn[sm->x.nkvoff[c0 + i]] = __float2half_rn(v[i]);
@@ -513,9 +524,9 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           }
         } else if constexpr (SITE == PAIR_RES) {
           const int f = tile * kTileN + fl;
-          float sq[16];
+          float sq[CH];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
+          for (int i = 0; i < CH; ++i) {
             sq[i] = 0.f;
             if (i < nr) {
               const float x = xs[i] + v[i];
@@ -524,21 +535,22 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
               sq[i] = x * x;
             }
           }
-          const float t = warp_sum_n<16>(sq, lane);
-          if ((lane & 1) == 0) sm->x.sums[quarter][c0 - r_lo + (lane >> 1)] = t;
+          const float t = warp_sum_n<CH>(sq, lane);
+          if (lane % LPR == 0) sm->x.sums[quarter][c0 - r_lo + lane / LPR] = t;
         } else if constexpr (SITE == PAIR_GU) {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] *= (i < nr ? ctl->inv[c0 + i] : 0.f);
-          // gate threads finish the chunk's rows 0..7, up threads rows 8..15: each hands over its other eight values
+          for (int i = 0; i < CH; ++i) v[i] *= (i < nr ? ctl->inv[c0 + i] : 0.f);
+          // gate threads finish the chunk's first half, up threads the second: each hands over its other values
+          constexpr int H = CH / 2;
           const bool is_gate = fl < 64;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) sm->x.exch[grp][fl][i] = is_gate ? v[8 + i] : v[i];
+          for (int i = 0; i < H; ++i) sm->x.exch[grp][fl][i] = is_gate ? v[H + i] : v[i];
           group_sync();
-          const int f = tile * 64 + (fl & 63), h8 = is_gate ? 0 : 8;
+          const int f = tile * 64 + (fl & 63), h8 = is_gate ? 0 : H;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
+          for (int i = 0; i < H; ++i) {
             const float other = sm->x.exch[grp][fl ^ 64][i];
-            const float gt = is_gate ? v[i] : other, up = is_gate ? other : v[8 + i];
+            const float gt = is_gate ? v[i] : other, up = is_gate ? other : v[H + i];
             if (h8 + i < nr) store_act<bf16>(p.planes_out, R, p.K_out, c0 + h8 + i, f, gt / (1.0f + expf(-gt)) * up);
           }
           group_sync();
@@ -547,26 +559,26 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           // clocks each, and at 342 rows an item's epilogue took longer than its MMAs (8B-shaped, 8 layers, top-2 alignment: a step 3607 -> 3559 us, B200).  So what concerns few steps or few
           // tiles (bounds, stored logits, drafted tokens) is decided once a chunk, and a maximum's token comes from a ballot.
           const int n_id = tile * kTileN + fl, n_warp = n_id - lane;
-          const int own = lane >> 1;   // the chunk's row whose totals this lane ends up with
-          if (nr < 16 || (tile + 1) * kTileN > dm.V) {   // uniform over the group
+          const int own = lane / LPR;   // the chunk's row whose totals this lane ends up with
+          if (nr < CH || (tile + 1) * kTileN > dm.V) {   // uniform over the group
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
+            for (int i = 0; i < CH; ++i)
               if (i >= nr || n_id >= dm.V) v[i] = -INFINITY;
           }
           if (dbg || keep) {   // logits asked for; sampling mode
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
+            for (int i = 0; i < CH; ++i)
               if (i < nr && n_id < dm.V) {
                 if (dbg) dbg[(size_t)(c0 + i) * dm.V + n_id] = v[i];
                 if (keep) keep[(size_t)(c0 + i) * dm.V + n_id] = v[i];
               }
           }
-          // lane i (and i + 16): the drafted token of row i
-          const int tok = (lane & 15) < nr ? sm->x.tok[c0 + (lane & 15)] : -1;
+          // lane i (and i + CH ..): the drafted token of row i
+          const int tok = lane % CH < nr ? sm->x.tok[c0 + lane % CH] : -1;
           int before = 0;
           if (topk) {   // uniform
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
+            for (int i = 0; i < CH; ++i) {
               const int tg = __shfl_sync(0xffffffffu, tok, i);
               const float zd = sm->x.pre[min(c0 + i, R - 1)];
               const int c = __popc(__ballot_sync(0xffffffffu, n_id != tg && (v[i] > zd || (v[i] == zd && n_id < tg))));
@@ -575,25 +587,25 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
           }
           if (invT != 1.f) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] *= invT;
+            for (int i = 0; i < CH; ++i) v[i] *= invT;
           }
-          const unsigned here = __ballot_sync(0xffffffffu, lane < 16 && tok >= n_warp && tok < min(n_warp + 32, dm.V));
+          const unsigned here = __ballot_sync(0xffffffffu, lane < CH && tok >= n_warp && tok < min(n_warp + 32, dm.V));
           if (here) {   // uniform over the warp: some row's drafted token is one of its tokens
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
+            for (int i = 0; i < CH; ++i)
               if ((here >> i & 1u) && n_id == __shfl_sync(0xffffffffu, tok, i)) w.tgt_logit[c0 + i] = v[i];
           }
-          const float m = warp_max16(v, lane);
+          const float m = warp_fmax_n<CH>(v, lane);
           int arg = 0x7fffffff;
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float mi = __shfl_sync(0xffffffffu, m, 2 * i);
+          for (int i = 0; i < CH; ++i) {
+            const float mi = __shfl_sync(0xffffffffu, m, LPR * i);
             const unsigned at = __ballot_sync(0xffffffffu, v[i] == mi);   // the lowest lane has the lowest token
             if (i == own && at) arg = n_warp + __ffs(at) - 1;
             v[i] = v[i] == -INFINITY ? 0.f : expf(v[i] - mi);
           }
-          const float e = warp_sum_n<16>(v, lane);
-          if ((lane & 1) == 0) {
+          const float e = warp_sum_n<CH>(v, lane);
+          if (lane % LPR == 0) {
             RowStat st; st.m = m; st.s = e; st.arg = arg; st.pad = before;
             sm->x.st[grp][quarter][own] = st;
           }
@@ -612,7 +624,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         all_sync();
         if (real)
           for (int r = r_lo + wt; r < r_hi; r += kPairWorkers)
-            if (mine >> ((r - r_lo) >> 5) & 1u)
+            if (mine >> ((r - r_lo) / (2 * CH)) & 1u)
               p.ssq_out[(size_t)tile * R + r] = (sm->x.sums[0][r - r_lo] + sm->x.sums[1][r - r_lo]) + (sm->x.sums[2][r - r_lo] + sm->x.sums[3][r - r_lo]);
         all_sync();
       }

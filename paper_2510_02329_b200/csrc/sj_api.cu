@@ -1372,17 +1372,18 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
 //   widths: a phase has to stream for longer than its barrier takes: ten 16 KiB units of gate/up for every block, 3.6 us at the
 //     copy rate.  One sequence, 9 rows, 24 layers: d 512, ffn 2048 (1.7 units) 1419 / 1054; d 1024, ffn 4096 (6.9) 1232 / 1161; d 1536,
 //     ffn 6144 (15.6) 1197 / 1257; 1B-shaped (27.7, 16 layers) 1012 / 1274.
-//   rows: its barriers cost less than launches, the paired projections are the better GEMM, and the per-stage attention kernels
-//     spread several sequences better.  8B-shaped, 16 layers, 1024 / 4000 keys a sequence: one sequence, 12 rows 1895 / 2000 and
-//     2029 / 2114, 16 rows 2049 / 2005 and 2189 / 2116, 17 rows 2102 / 2191 and 2322 / 2318, 24 rows 2233 / 2233 and 2475 / 2390; two
-//     sequences, 12 rows 1903 / 2024 and 2083 / 2065, 16 rows 1997 / 2033 and 2233 / 2075, 18 rows 2094 / 2103 and 2364 / 2154; four, 12 rows
-//     1956 / 1993, 16 rows 2056 / 2007; eight, 16 rows 2166 / 2016.  32B-shaped, 12 layers: one sequence, 9 rows 2470 / 2543, 16 rows
-//     2654 / 2680, 17 rows 2773 / 2754; two, 12 rows 2542 / 2608, 16 rows 2649 / 2608; four, 12 rows 2588 / 2592, 16 rows 2664 / 2594.
-//     (Between 12 and 24 rows of one sequence the two are within 4 % of each other, either way: the line is the last row count
-//     at which neither key count is slower.)
-//     1B-shaped (head dimension 64; no per-stage tcgen05 attention): one sequence, 20 rows 1196 / 1224, 24 rows 1232 / 1222; two, 24 rows
-//     1254 / 1260; four, 16 rows 1158 / 1214, 24 rows 1287 / 1287, 36 rows 1470 / 1296; six, 18 rows 1234 / 1220; eight, 16 rows
-//     1201 / 1187, 24 rows 1289 / 1239.
+//   rows and keys: its barriers cost less than launches, the paired projections are the better GEMM, and the per-stage attention
+//     spreads several sequences and long caches better.  One stream, steps back to back (steps on several streams overlap
+//     per stage and do not here: 8B-shaped, 9 rows, 4096 keys, two streams 3753 / 2851 a step).
+//     8B-shaped, 16 layers, one sequence: 9 rows 1813 / 1840 at 300 keys, 1856 / 1851 at 600, 1866 / 1855 at 1024, 1985 / 1975 at 4000;
+//     5 rows 1819 / 1837 at 1024, 1906 / 1938 at 4000; 12 rows 1851 / 1849 at 300, 1905 / 1872 at 1024, 2036 / 1980 at 4000; 16 rows 2059 / 1880,
+//     2184 / 1985; 17 rows 2028 / 2054 at 300, 2097 / 2063 at 600, 2113 / 2085, 2328 / 2197.  Two, 1024 keys: 10 rows 1886 / 1893, 12 rows
+//     1907 / 1894; four, 12 rows 1884 / 1840 at 300, 1960 / 1864 at 1024.
+//     32B-shaped (233 units of gate/up a block against 97: phases long enough to hide more), 8 layers, 2000 keys: 9 rows 1793 / 1836,
+//     12 rows 1848 / 1842, 13 rows 1870 / 1890, 16 rows 1899 / 1890, 17 rows 2030 / 2004.
+//     1B-shaped (head dimension 64; no per-stage tcgen05 attention), one sequence: 9 rows 1076 / 1155 at 2048 keys, 13 rows 1118 / 1165 at
+//     1024, 16 rows 1132 / 1060 at 600, 1240 / 1222 at 2048, 24 rows 1341 / 1245; two, 1024 keys: 12 rows 1112 / 1166, 16 rows 1197 / 1191; three, 12
+//     rows 1096 / 1076; four, 8 rows 991 / 983, 12 rows 1106 / 1029; six, 12 rows 1123 / 1017.
 // Caches of several 128-key tiles per SM (and head dimension 128): its mma.sync attention takes about three times as long a
 // key as the tcgen05 kernel (8B-shaped, 9 rows: 8000 keys, 3.4 tiles, 2156 / 2159).
 static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma, long total_keys) {
@@ -1390,8 +1391,11 @@ static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma, l
   if (t->opt_step == 0 || t->opt_gemm != 1 || !t->mega_shapes || !kv->has_tm_pool || R > kMegaMaxRows || group * rows > 16 * 6 || !t->stream)
     return false;
   if (t->dm.hd == 128 && t->opt_attn == 2 && total_keys * t->dm.Hkv / kT5Keys / t->sm_count >= t->opt_a5_min_tiles) return false;
-  const int most = t->dm.hd == 128 ? (B == 1 ? 17 : 12) : (B <= 4 ? 24 : 12);
-  return t->opt_step == 1 || t->opt_attn == 0 || (R <= most && (long)(t->dm.F / 64) * (t->dm.d / kBK) >= 10L * t->sm_count);
+  const long units = (long)(t->dm.F / 64) * (t->dm.d / kBK), keys = total_keys / B;
+  int most;   // rows; caches shorter than these keep the older lines
+  if (t->dm.hd == 128) most = keys < 512 ? (B == 1 ? 17 : 12) : (units >= 150L * t->sm_count ? 15 : 8);
+  else most = keys < 256 ? (B <= 4 ? 24 : 12) : (B <= 2 ? 15 : 8);
+  return t->opt_step == 1 || t->opt_attn == 0 || (R <= most && units >= 10L * t->sm_count);
 }
 
 static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode, bool use_logits) {

@@ -1373,17 +1373,21 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
 //     copy rate.  One sequence, 9 rows, 24 layers: d 512, ffn 2048 (1.7 units) 1419 / 1054; d 1024, ffn 4096 (6.9) 1232 / 1161; d 1536,
 //     ffn 6144 (15.6) 1197 / 1257; 1B-shaped (27.7, 16 layers) 1012 / 1274.
 //   rows and keys: its barriers cost less than launches, the paired projections are the better GEMM, and the per-stage attention
-//     spreads several sequences and long caches better.  One stream, steps back to back (steps on several streams overlap
-//     per stage and do not here: 8B-shaped, 9 rows, 4096 keys, two streams 3753 / 2851 a step).
-//     8B-shaped, 16 layers, one sequence: 9 rows 1813 / 1840 at 300 keys, 1856 / 1851 at 600, 1866 / 1855 at 1024, 1985 / 1975 at 4000;
-//     5 rows 1819 / 1837 at 1024, 1906 / 1938 at 4000; 12 rows 1851 / 1849 at 300, 1905 / 1872 at 1024, 2036 / 1980 at 4000; 16 rows 2059 / 1880,
-//     2184 / 1985; 17 rows 2028 / 2054 at 300, 2097 / 2063 at 600, 2113 / 2085, 2328 / 2197.  Two, 1024 keys: 10 rows 1886 / 1893, 12 rows
-//     1907 / 1894; four, 12 rows 1884 / 1840 at 300, 1960 / 1864 at 1024.
-//     32B-shaped (233 units of gate/up a block against 97: phases long enough to hide more), 8 layers, 2000 keys: 9 rows 1793 / 1836,
-//     12 rows 1848 / 1842, 13 rows 1870 / 1890, 16 rows 1899 / 1890, 17 rows 2030 / 2004.
-//     1B-shaped (head dimension 64; no per-stage tcgen05 attention), one sequence: 9 rows 1076 / 1155 at 2048 keys, 13 rows 1118 / 1165 at
-//     1024, 16 rows 1132 / 1060 at 600, 1240 / 1222 at 2048, 24 rows 1341 / 1245; two, 1024 keys: 12 rows 1112 / 1166, 16 rows 1197 / 1191; three, 12
-//     rows 1096 / 1076; four, 8 rows 991 / 983, 12 rows 1106 / 1029; six, 12 rows 1123 / 1017.
+//     spreads several sequences and long caches better.  Steps of one target back to back, all layers (one at a time they compare alike).
+//     The first step on a new cache is what capturing costs the per-stage path on top (8B-shaped 0.7 to 0.9 ms), so a tie stays here.
+//     8B-shaped, one sequence: 5 rows 3439 / 3458 at 1024 keys; 9 rows 3413 / 3502 at 300, 3534 / 3499 at 1024, 3772 / 3726 at 4096
+//     (sampling, 3001 keys: 3729 / 3744); 10 rows 3579 / 3501, 12 rows 3605 / 3518; 13 rows (its instantiation for 16) 3853 / 3522; 16 rows
+//     3906 / 3539, 4141 / 3755 at 4000; 17 rows (row blocks of 32 per stage) 3991 / 3937, 4278 / 4152 at 3001 (sampling 4308 / 4165).
+//     1024 keys: two sequences, 8 rows 3522 / 3560, 12 rows 3629 / 3588, 14 rows 3784 / 3600 (16 layers, 10 rows 1886 / 1893); three, 9 rows
+//     3625 / 3515; four, 12 rows 3751 / 3526; five, 10 rows 3760 / 3515.
+//     32B-shaped, 16 layers, 2000 keys: one, 9 rows 3261 / 3308, 12 rows 3382 / 3311, 16 rows 3488 / 3457, 17 rows 3742 / 3655; two, 12 rows
+//     3360 / 3276, 14 rows 3444 / 3285; three, 9 rows 3348 / 3228; four, 12 rows 3470 / 3273; five, 10 rows 3293 / 3299.
+//     1B-shaped (head dimension 64; no per-stage tcgen05 attention): one, 9 rows 1078 / 1159 at 2048 keys, 16 rows 1142 / 1064 at 600, 1147 / 1166
+//     at 1024, 24 rows 1272 / 1186; two, 1024 keys, 12 rows 1114 / 1166, 16 rows 1197 / 1192; three, 600 keys, 9 rows 1045 / 1007, 12 rows
+//     1083 / 1048; four, 8 rows 991 / 983 at 1024, 12 rows 1092 / 1005; six, 12 rows 1127 / 1018.
+//     Shorter caches keep lines that were drawn when the per-stage path was slower.  It is the faster one now in part of what they leave to
+//     this kernel: 8B-shaped, 300 keys, 13 rows 3636 / 3490, 16 rows 3678 / 3499 (17 rows 3846 / 3868); 1B-shaped, 40 keys, 16 rows 1129 / 918, 24
+//     rows 1245 / 1082, four sequences, 16 rows 1095 / 911.
 // Caches of several 128-key tiles per SM (and head dimension 128): its mma.sync attention takes about three times as long a
 // key as the tcgen05 kernel (8B-shaped, 9 rows: 8000 keys, 3.4 tiles, 2156 / 2159).
 static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma, long total_keys) {
@@ -1391,11 +1395,11 @@ static bool mega_usable(const sj_target* t, const sj_kv* kv, int B, int gamma, l
   if (t->opt_step == 0 || t->opt_gemm != 1 || !t->mega_shapes || !kv->has_tm_pool || R > kMegaMaxRows || group * rows > 16 * 6 || !t->stream)
     return false;
   if (t->dm.hd == 128 && t->opt_attn == 2 && total_keys * t->dm.Hkv / kT5Keys / t->sm_count >= t->opt_a5_min_tiles) return false;
-  const long units = (long)(t->dm.F / 64) * (t->dm.d / kBK), keys = total_keys / B;
+  const long keys = total_keys / B;
   int most;   // rows; caches shorter than these keep the older lines
-  if (t->dm.hd == 128) most = keys < 512 ? (B == 1 ? 17 : 12) : (units >= 150L * t->sm_count ? 15 : 8);
+  if (t->dm.hd == 128) most = keys < 512 ? (B == 1 ? 17 : 12) : (B == 1 ? 9 : (B == 2 ? 10 : 8));
   else most = keys < 256 ? (B <= 4 ? 24 : 12) : (B <= 2 ? 15 : 8);
-  return t->opt_step == 1 || t->opt_attn == 0 || (R <= most && units >= 10L * t->sm_count);
+  return t->opt_step == 1 || t->opt_attn == 0 || (R <= most && (long)(t->dm.F / 64) * (t->dm.d / kBK) >= 10L * t->sm_count);
 }
 
 static sj_status launch_mega(sj_target* t, sj_kv* kv, int B, int gamma, int mode, bool use_logits) {

@@ -9,8 +9,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("shape,n,gamma,keys,persistent", [
-    (synth.LLAMA_8B, 1, 7, 900, True), (synth.LLAMA_8B, 1, 8, 900, False), (synth.LLAMA_8B, 1, 8, 500, True), (synth.LLAMA_8B, 1, 8, 503, False),
-    (synth.QWEN_32B, 1, 14, 900, True), (synth.QWEN_32B, 1, 15, 900, False),
+    (synth.LLAMA_8B, 1, 8, 900, True), (synth.LLAMA_8B, 1, 8, 4096, True), (synth.LLAMA_8B, 1, 9, 900, False), (synth.LLAMA_8B, 1, 9, 500, True),
+    (synth.LLAMA_8B, 1, 9, 503, False), (synth.LLAMA_8B, 2, 4, 900, True), (synth.LLAMA_8B, 2, 5, 900, False), (synth.LLAMA_8B, 3, 2, 900, False),
+    (synth.LLAMA_8B, 4, 1, 900, True), (synth.QWEN_32B, 1, 8, 900, True), (synth.QWEN_32B, 1, 9, 900, False), (synth.QWEN_32B, 2, 4, 900, True),
+    (synth.QWEN_32B, 2, 6, 900, False), (synth.QWEN_32B, 3, 3, 900, False),
     (synth.LLAMA_1B, 1, 14, 900, True), (synth.LLAMA_1B, 1, 15, 900, False), (synth.LLAMA_1B, 1, 15, 239, True), (synth.LLAMA_1B, 1, 15, 240, False),
     (synth.LLAMA_1B, 3, 3, 300, False), (synth.LLAMA_1B, 4, 1, 300, True)], ids=lambda x: x.name if hasattr(x, "name") else str(x))
 def test_default_route_by_keys(shape, n, gamma, keys, persistent):

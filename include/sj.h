@@ -212,7 +212,7 @@ sj_status sj_verify(sj_target *t, sj_kv *kv, const sj_verify_args *args, const s
  * min(32, 96 / (Hq/Hkv), max_rows) tokens: each block runs as a verification step whose first row is the
  * block's first token and whose "drafts" are the following ones, every position accepted and committed
  * (accept_all), so the cache receives exactly the K/V rows a verification step would read.  bf16 models with
- * tensor-core options take up to 1024 tokens' blocks through the layers at once (a workspace for them is
+ * tensor-core options take up to SJ_MAX_ROWS tokens' blocks through the layers at once (a workspace for them is
  * allocated by the first such call; without memory for it the blocks run one by one).  On return (the
  * work is queued on the target's stream) the sequence is n_tokens longer and its pending token is the target's
  * greedy token after the last appended one; with next_token != NULL (host) that token is also copied out,

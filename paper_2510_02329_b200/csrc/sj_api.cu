@@ -1792,9 +1792,9 @@ extern "C" sj_status sj_semantic_score(sj_target* t, sj_kv* kv, int seq, int y_i
 // bf16 pages, so another partition would give slightly other results) over the same sequence -- entry b attends to the stored cache plus the b * c rows before it
 // (its projection has stored them in the pages by the time the attention kernel runs) and to its own rows, which is
 // exactly what B verification steps of c rows one after another would do, at one read of the weights (8B-shaped model,
-// 1000 tokens and a step: 190 ms in blocks of 24 rows, 34 ms in two of 504, 32 in one of 1008).  Only the last token's row meets the
+// 1000 tokens and a step: 190 ms in blocks of 24 rows, 34 ms in two of 504).  Only the last token's row meets the
 // LM head, and a block that is not the last one ends with its key / value rows.
-constexpr int kPrefillRows = kPairMaxRows;   // rows of a wide block
+constexpr int kPrefillRows = SJ_MAX_ROWS;   // rows of a wide block
 
 static sj_status prefill_wide(sj_target* t, sj_kv* kv, int seq, const int* tokens, int n_tokens, int c, int* d_next, bool* done) {
   const Dims& dm = t->dm;

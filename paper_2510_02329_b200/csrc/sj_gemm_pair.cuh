@@ -46,7 +46,7 @@ namespace sj {
 constexpr int kPairThreads = 384;      // warp 0 TMA, warp 1 MMA (rank 0), warp 2 tensor memory, warps 4..11 epilogue
 constexpr int kPairWorkers = 256;
 constexpr int kPairMaxStages = 10;
-constexpr int kPairMaxRows = 1024;     // of a prefill's blocks; a step has at most kMaxRows
+constexpr int kPairMaxRows = kMaxRows;
 constexpr int kPairSegKB = 16, kPairShortKB = 32;   // K blocks of 64 per accumulation chain; half of them in a prefill's sums of up to kPairShortKB
 constexpr int kPairMaxSplit = 4;        // pairs that share an item's K (a cluster of 8)
 constexpr double kPairHbmBytesPerClk = 3600;   // HBM against the SM clock, for the host's choice of a geometry
@@ -99,8 +99,8 @@ struct PairQkvCtl {
 struct PairGuCtl { float exch[2][128][9]; };
 struct PairResCtl { float sums[4][128]; };   // by row of the item's block
 struct PairLmCtl {
-  int tok[kMaxRows];
-  float pre[kMaxRows];
+  int tok[kPairMaxRows];
+  float pre[kPairMaxRows];
   RowStat st[2][4][16];
 };
 template <int SITE> struct PairExtra;

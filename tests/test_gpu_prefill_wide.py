@@ -6,7 +6,8 @@ import torch
 import harness
 import helpers
 from oracle import sj_oracle as orc
-from paper_2510_02329_b200 import synth
+from paper_2510_02329_b200 import binding, synth
+from perf import cases
 from test_gpu_extensions import _empty_case
 
 pytestmark = pytest.mark.gpu
@@ -46,9 +47,27 @@ def test_wide_prefill(shape, before, n):
         case.close()
 
 
+@pytest.mark.parametrize("shape,n,block", [(synth.LLAMA_8B.cut(2, vocab=2048), 1000, 504), (synth.LLAMA_1B.cut(2, vocab=2048), 700, 360)],
+                         ids=lambda x: x.name if hasattr(x, "name") else str(x))
+def test_a_long_prompt_leaves_the_bits_of_its_blocks(shape, n, block):
+    """At most 512 rows go through the layers at once, in blocks of equal size: the same calls by hand leave the same cache."""
+    target = cases.make_model(shape, torch.bfloat16, 53, 64)
+    kv = binding.KVCache(target, 1, n // 16 + 2)
+    prompt = synth.token_ids(shape.vocab, n, seed=53, stream=9).tolist()
+    stored = []
+    for piece in (n, block):
+        kv.rollback([0], [0])
+        for i in range(0, n, piece):
+            kv.prefill(0, prompt[i:i + piece], want_next=False)
+        stored.append([kv.read(0, l, 0, n) for l in range(shape.n_layers)])
+    for whole, parts in zip(*stored):
+        assert torch.equal(whole[0], parts[0]) and torch.equal(whole[1], parts[1])
+    kv.close()
+    target.close()
+
+
 def _verify(case, si, shape):
-    from paper_2510_02329_b200 import binding as b
-    out = b.VerifyBuffers(1, 3, shape.d_model, shape.vocab, debug=True)
-    b.verify(case.target, case.kv, [0], torch.from_numpy(si.draft_ids).cuda(), out, commit=False)
+    out = binding.VerifyBuffers(1, 3, shape.d_model, shape.vocab, debug=True)
+    binding.verify(case.target, case.kv, [0], torch.from_numpy(si.draft_ids).cuda(), out, commit=False)
     case.target.sync()
     return out.dbg_logits.cpu().numpy()[0]

@@ -160,9 +160,9 @@ sj_status sj_kv_fill(sj_kv *kv, int seq, int layer, int start, int n_tokens, con
 /* Read rows back (same layout); synchronises the stream.  For tests. */
 sj_status sj_kv_read(sj_kv *kv, int seq, int layer, int start, int n_tokens, void *k_out, void *v_out);
 /* Set the length of sequences (tokens [0,len) are live).  len must not exceed the rows reserved
- * by fills/verifies.  seq_ids, lens: host [B]. */
+ * by fills/verifies.  seq_ids, lens: host [B]; of a sequence named more than once the last entry counts. */
 sj_status sj_kv_set_len(sj_kv *kv, const int *seq_ids, const int *lens, int B);
-/* Set the pending token x_t of sequences (fed at row 0 of the next block).  host [B]. */
+/* Set the pending token x_t of sequences (fed at row 0 of the next block).  host [B]; the last entry of a sequence counts. */
 sj_status sj_kv_set_pending(sj_kv *kv, const int *seq_ids, const int *tokens, int B);
 /* Current lengths (host out[B]); synchronises the stream and returns unused pages to the pool. */
 sj_status sj_kv_len(sj_kv *kv, const int *seq_ids, int *out_len, int B);
@@ -234,6 +234,7 @@ sj_status sj_semantic_score(sj_target *t, sj_kv *kv, int seq, int y_i, int z_i, 
 
 /* Truncate sequences to new_len <= current length (host arrays [B]) and return the whole pages
  * past new_len to the pool (the KV-length rollback that follows the first-rejection scan, Sec. 3.1).
+ * Of a sequence named more than once the shortest length counts.
  * Asynchronous; if new_len exceeds the true length the device leaves the sequence unchanged and
  * sj_sync() returns SJ_ERR_STATE.  new_len above what the host knows could be live fails at once
  * with STATE. */

@@ -884,11 +884,16 @@ static sj_status begin_step(sj_target* t, sj_kv* kv, const StepArgs& h, const Kv
   CU_TRY(launch(k_begin, dim3(1), dim3(256), 0, t->stream, false, h, edits, t->d_args, kv->view, W ? *W : Work{}, chunk_len, W ? 1 : 0, sync));
   return SJ_OK;
 }
-// One kind of bookkeeping entry of B sequences.
+// One kind of bookkeeping entry of B sequences.  The kernels' threads take the entries in no order, so a sequence that is named
+// more than once gets one entry, its last.
 static KvEdits edits_of(const int* seq_ids, const int* values, int B, int at) {
   KvEdits x;
-  x.n = B;
-  for (int i = 0; i < B; ++i) x.e[i] = {seq_ids[i], at, values[i]};
+  x.n = 0;
+  for (int i = B - 1; i >= 0; --i) {
+    bool later = false;
+    for (int k = 0; k < x.n && !later; ++k) later = x.e[k].seq == seq_ids[i];
+    if (!later) x.e[x.n++] = {seq_ids[i], at, values[i]};
+  }
   return x;
 }
 
@@ -996,14 +1001,18 @@ extern "C" sj_status sj_rollback_kv(sj_kv* kv, const int* seq_ids, const int* ne
       return fail(SJ_ERR_STATE, "rollback of sequence %d to %d beyond its length (at most %d)", seq_ids[i], new_len[i],
                   kv->len_hi[seq_ids[i]]);
   }
-  CU_TRY(launch(k_rollback, dim3(1), dim3(256), 0, kv->t->stream, false, kv->view, edits_of(seq_ids, new_len, B, kEditLen), kv->t->work.status));
+  KvEdits to;   // all entries: the device looks at each, and the shortest of a sequence counts
+  to.n = B;
+  for (int i = 0; i < B; ++i) to.e[i] = {seq_ids[i], kEditLen, new_len[i]};
+  CU_TRY(launch(k_rollback, dim3(1), dim3(kMaxEdits), 0, kv->t->stream, false, kv->view, to, kv->t->work.status));
   // Whole pages past the new length go back to the pool.  Everything that still touches them (a verify in
   // flight, this rollback) was enqueued on the target's stream before any later call can hand them out
   // again, and that call's kernels run on the same stream.  If the device refuses the rollback (the live
   // length turned out shorter than new_len) the pages kept for new_len still cover it.
   for (int i = 0; i < B; ++i) {
-    kv->len_hi[seq_ids[i]] = new_len[i];
-    release_beyond(kv, seq_ids[i], new_len[i]);
+    int& hi = kv->len_hi[seq_ids[i]];
+    hi = std::min(hi, new_len[i]);
+    release_beyond(kv, seq_ids[i], hi);
   }
   return SJ_OK;
 }

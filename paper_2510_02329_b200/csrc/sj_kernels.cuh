@@ -987,13 +987,15 @@ static __global__ void k_prefill_commit(KvView kv, int seq, int n, const RowStat
   }
 }
 
-// Rollback: kv_len <- new_len where new_len <= kv_len, else flag the error and leave it.
-static __global__ void k_rollback(KvView kv, const __grid_constant__ KvEdits to, int* status) {
-  for (int i = threadIdx.x; i < to.n; i += blockDim.x) {
-    const int s = to.e[i].seq, n = to.e[i].value;
-    if (n >= 0 && n <= kv.kv_len[s]) kv.kv_len[s] = n;
-    else atomicCAS(status, DEV_OK, DEV_STATE);
-  }
+// Rollback: kv_len <- new_len where new_len <= kv_len, else flag the error and leave it; a sequence named more than once ends at the
+// shortest.  One thread per entry, one block.
+static __global__ void __launch_bounds__(kMaxEdits) k_rollback(KvView kv, const __grid_constant__ KvEdits to, int* status) {
+  const bool live = (int)threadIdx.x < to.n;
+  const int s = to.e[live ? threadIdx.x : 0].seq, n = to.e[live ? threadIdx.x : 0].value;
+  const bool ok = live && n >= 0 && n <= kv.kv_len[s];
+  __syncthreads();   // every entry is held against the length before the call
+  if (ok) atomicMin(&kv.kv_len[s], n);
+  else if (live) atomicCAS(status, DEV_OK, DEV_STATE);
 }
 
 // Copy rows between a contiguous [n, Hkv, hd] buffer and the paged pool (fill: to_pool = 1).

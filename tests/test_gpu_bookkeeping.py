@@ -1,5 +1,7 @@
 """Pending tokens, page numbers, lengths and roll-backs of many sequences at once: each travels as the parameters of one
-kernel, up to the largest batch."""
+kernel, up to the largest batch.  A sequence named twice in one call ends as if its entries came one after another."""
+import random
+
 import pytest
 import torch
 
@@ -51,4 +53,45 @@ def test_a_large_batch_equals_its_parts(B, step_impl):
     assert clear.sum() >= B // 4
     for n in ("accepted_len", "next_token"):
         assert torch.equal(whole[n][clear], parts[n][clear])
+    c.close()
+
+
+@pytest.mark.parametrize("n_seqs", [1, 5, 40])
+def test_a_sequence_named_twice_ends_with_its_last_entry(n_seqs):
+    """The largest batch of entries over a few sequences; roll-backs end at the shortest, the host's page count with them."""
+    room, shape, ids = 96, synth.TINY, list(range(n_seqs))
+    c = harness.Case(shape, torch.bfloat16, [16], 2, seed=5, cache="fill").gpu_setup(max_rows=256)
+    kv = binding.KVCache(c.target, n_seqs, n_seqs * (room // 16) + 8)
+    rows = torch.randn(room, shape.n_kv_heads, shape.head_dim, device="cuda").bfloat16()
+    for s in ids:
+        for l in range(shape.n_layers):
+            kv.fill(s, l, 0, rows, rows)
+    r = random.Random(n_seqs)
+    drafts = torch.randint(0, shape.vocab, (n_seqs, 2), dtype=torch.int32, device="cuda")
+
+    def logits():
+        out = binding.VerifyBuffers(n_seqs, 2, shape.d_model, shape.vocab, debug=True)
+        binding.verify(c.target, kv, ids, drafts, out, commit=False)
+        c.target.sync()
+        return out.dbg_logits
+
+    for _ in range(20):
+        named = ids + [r.randrange(n_seqs) for _ in range(256 - n_seqs)]
+        r.shuffle(named)
+        lens, tokens = [r.randrange(1, room - 3) for _ in named], [r.randrange(shape.vocab) for _ in named]
+        last = dict(zip(named, zip(lens, tokens)))
+        kv.set_len(named, lens)
+        kv.set_pending(named, tokens)
+        assert kv.lengths(ids) == [last[s][0] for s in ids]
+        got = logits()
+        kv.set_pending(ids, [last[s][1] for s in ids])
+        assert torch.equal(got, logits())
+        for s in ids:      # lengths() has given the pages beyond a sequence's length back
+            kv.fill(s, 0, 0, rows, rows)
+        kv.set_len(ids, [room] * n_seqs)
+        kv.rollback(named, lens)
+        assert kv.lengths(ids) == [min(n for s, n in zip(named, lens) if s == i) for i in ids]
+        for s in ids:
+            kv.fill(s, 0, 0, rows, rows)
+    kv.close()
     c.close()

@@ -446,7 +446,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       }
       // The kernel's last cluster barrier, reported to as soon as this warp is done with the other CTAs' memory and with its
       // accumulators: nobody waits for it behind the epilogue (at the kernel's end it was 0.7 us of each: 8B-shaped 44 rows, 32 layers
-      // 4.37 -> 4.26 ms a step, 1B-shaped 48 rows 1024 -> 964 us, B200).
+      // 4.37 -> 4.26 ms a step, 1B-shaped 48 rows 1024 -> 964 us, B200).  A wait that runs out holds its warp's report back itself.
       if (item + p.n_groups >= n_items) {
         tc_fence_before();
         __syncwarp();
@@ -637,7 +637,6 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     tc_fence_before();
     cluster_arrive_all();
   }
-  if (*abort_flag) __nanosleep(20000);   // let copies still in flight land before the pair retires
   cluster_wait_all();   // nothing of the pair touches the other CTA's memory after this
   if (warp == 2) {
     tc_fence_after();

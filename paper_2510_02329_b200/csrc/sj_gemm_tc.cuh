@@ -86,7 +86,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Bounded wait: gives up after `limit` polls or when another thread of the block gave up.
+// Bounded wait: gives up after `limit` polls or when another thread of the block gave up.  The thread whose wait has run out stays for
+// another 20 us: copies in flight land before its warp lets the block, or at a cluster's last barrier any of its blocks, retire.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
                                           uint32_t limit = kSpinLimit) {
 #pragma unroll 1
@@ -99,6 +100,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
   *abort_flag = 1;
   atomicCAS(status, DEV_OK, DEV_TIMEOUT);
+  __nanosleep(20000);
   return false;
 }
 __device__ __forceinline__ uint64_t l2_policy_evict_first() {
@@ -420,7 +422,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
-    if (*abort_flag) __nanosleep(20000);  // let copies still in flight land before the block retires
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");
   }

@@ -198,7 +198,8 @@ __device__ __forceinline__ bool a5_produce(const A5Ring& rg, A5Pos& pos, const C
           if (*rg.abort_flag) return false;
           __nanosleep(20);
         }
-        if (i >= kAttSpin) { *rg.abort_flag = 1; atomicCAS(rg.status, DEV_OK, DEV_TIMEOUT); return false; }
+        if (i >= 16 * kAttSpin) {   // polls of shared memory, far shorter than those of a barrier
+          *rg.abort_flag = 1; atomicCAS(rg.status, DEV_OK, DEV_TIMEOUT); return false; }
       }
       __syncwarp();
     }

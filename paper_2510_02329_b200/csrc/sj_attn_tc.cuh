@@ -31,7 +31,7 @@ namespace sj {
 constexpr int kAttStageBytes = 16384;     // one ring tile: K part then V part, 8 KiB each
 constexpr int kAttMaxWarps = 8;           // consumer warps per block
 constexpr int kAttMaxSub = 4;             // sub-partials per segment (key shares)
-constexpr uint32_t kAttSpin = 1u << 22;
+constexpr uint32_t kAttSpin = 1u << 18;        // polls of a bounded wait, 4.1 us each (B200)
 
 __device__ __forceinline__ uint32_t att_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 

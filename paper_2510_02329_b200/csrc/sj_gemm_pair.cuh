@@ -58,7 +58,7 @@ __host__ __device__ constexpr int pair_chunk(bool narrow) { return narrow ? 8 : 
 // and a wait that knows only its parity would see it as not yet complete.  To finish the second exchange after, a split
 // needs its partners' arrivals of the first, which they give after their look: two barriers are never overtaken.
 constexpr int kPairFreeBars = 2;
-constexpr uint32_t kPairSpin = 1u << 22;
+constexpr uint32_t kPairSpin = kSpinLimit;
 
 enum PairSite { PAIR_QKV = 0, PAIR_RES = 1, PAIR_GU = 2, PAIR_LM = 3 };
 

@@ -464,7 +464,7 @@ def main():
                 dw.step(mode)
             dw.target.sync()
             tot = 0.0
-            for name in ("embed_norm", "gemm_qkv", "gemm_o", "gemm_gateup", "gemm_down", "gemm_lm_head",
+            for name in ("plan", "embed_norm", "gemm_qkv", "gemm_o", "gemm_gateup", "gemm_down", "gemm_lm_head",
                          "qkv_rope", "attn_combine", "reduce_norm", "swiglu", "finalize", "resample"):
                 ms, n = dw.target.kernel_time(name)
                 if n:

@@ -878,12 +878,6 @@ struct ReservedPages {
   }
 };
 
-// The launch that starts a step: arguments and page numbers to the device (k_begin).  W: workspace to plan a per-stage
-// step in, or null.
-static sj_status begin_step(sj_target* t, sj_kv* kv, const StepArgs& h, const KvEdits& edits, const Work* W, int chunk_len, unsigned* sync) {
-  CU_TRY(launch(k_begin, dim3(1), dim3(256), 0, t->stream, false, h, edits, t->d_args, kv->view, W ? *W : Work{}, chunk_len, W ? 1 : 0, sync));
-  return SJ_OK;
-}
 // One kind of bookkeeping entry of B sequences.  The kernels' threads take the entries in no order, so a sequence that is named
 // more than once gets one entry, its last.
 static KvEdits edits_of(const int* seq_ids, const int* values, int B, int at) {
@@ -1210,6 +1204,15 @@ static cudaError_t launch_cudacore(sj_target* t, const TcSite& site, const void*
     if (st_ != SJ_OK) return st_;                                                \
     TIMED_END(name)                                                              \
   } while (0)
+
+// The launch that starts a step: arguments and page numbers to the device (k_begin).  W: workspace to plan a per-stage
+// step in (filed as "plan"), or null.
+static sj_status begin_step(sj_target* t, sj_kv* kv, const StepArgs& h, const KvEdits& edits, const Work* W, int chunk_len, unsigned* sync) {
+  cudaStream_t s = t->stream;
+  const bool timing = t->opt_timing != 0 && !t->opt_graph && W;
+  TIMED("plan", launch(k_begin, dim3(1), dim3(256), 0, s, false, h, edits, t->d_args, kv->view, W ? *W : Work{}, chunk_len, W ? 1 : 0, sync));
+  return SJ_OK;
+}
 
 // The decoder layers of a step (set-up and embedding included): from the step's arguments to the GEMM input planes of
 // the final norm.  prefill: a wide block of known tokens; kv_only: its key / value rows are all that is wanted (blocks

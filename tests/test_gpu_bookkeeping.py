@@ -95,3 +95,14 @@ def test_a_sequence_named_twice_ends_with_its_last_entry(n_seqs):
             kv.fill(s, 0, 0, rows, rows)
     kv.close()
     c.close()
+
+
+def test_a_timed_step_files_every_launch_of_its_own():
+    """One record per kernel of a per-stage step: set-up, embedding, six a layer, final norm, LM head, acceptance."""
+    c = harness.Case(synth.TINY, torch.bfloat16, [40, 17], 3, seed=5, cache="fill").gpu_setup()
+    for name, value in (("step_impl", 0), ("graph", 0), ("timing", 1)):
+        c.target.set_option(name, value)
+    c.run_gpu(0, debug=False)
+    assert c.target.kernel_time("plan")[1] == c.target.kernel_time("embed_norm")[1] == 1
+    assert c.target.kernel_time("")[1] == 2 + 6 * synth.TINY.n_layers + 3
+    c.close()

@@ -60,7 +60,7 @@ class ClockSampler:
          "clocks_event_reasons.sw_thermal_slowdown,clocks_event_reasons.sw_power_cap")
 
     def __init__(self, index: int):
-        self.index, self.rows, self.proc = index, [], None
+        self.index, self.rows, self.proc, self.first = index, [], None, threading.Event()
 
     def __enter__(self):
         try:
@@ -68,6 +68,8 @@ class ClockSampler:
                                           "-lms", "50", "-i", str(self.index)], stdout=subprocess.PIPE, text=True)
             self.thread = threading.Thread(target=self._read, daemon=True)
             self.thread.start()
+            self.first.wait(timeout=5)      # nvidia-smi may take longer to start than the timed steps do
+            self.rows.clear()               # of an idle GPU
         except Exception:
             self.proc = None
         return self
@@ -75,6 +77,7 @@ class ClockSampler:
     def _read(self):
         for line in self.proc.stdout:
             self.rows.append([x.strip() for x in line.split(",")])
+            self.first.set()
 
     def __exit__(self, *a):
         if self.proc:
@@ -373,10 +376,10 @@ def main():
 
     # ---------------- device-resident timing ----------------
     with torch.cuda.stream(stream):
-        for _ in range(args.warmup):
-            dw.step(mode)
-        dw.target.sync()
         with ClockSampler(local_rank) as clk:
+            for _ in range(args.warmup):
+                dw.step(mode)
+            dw.target.sync()
             barrier()
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             e0.record(stream)

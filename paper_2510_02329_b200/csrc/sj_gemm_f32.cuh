@@ -9,9 +9,13 @@
 // weights at 12 rows.  Loading straight into registers a step ahead (k_gemm_simt) kept 32 KiB on the way and read each
 // activation once per four features from L1.  Work is dealt in units (tile, K step), evenly to one block per SM, so that
 // every SM streams the same bytes whatever N is; a tile that several blocks share leaves a slot of sums per block, added in
-// block order by the kernel that reads them (SplitPlan).  Rows beyond RT take another pass over a block's share of the
-// tile, which L2 still holds.  1B-shaped cut of 4 layers, 2 sequences of 512 keys, 10 rows, one cache replayed back to back: a step
-// 1159 -> 898 us (B200).
+// block order by the kernel that reads them (SplitPlan).  1B-shaped cut of 4 layers, 2 sequences of 512 keys, 10 rows, one cache
+// replayed back to back: a step 1159 -> 898 us (B200).
+//
+// Rows beyond RT take another pass over a block's share of the tile, at most 256 K bytes: from L2 where 148 shares fit it (K = 2048: 78
+// MB), from HBM again where they do not (K above 3300 or so where a tile is one block's, as in the LM head).  A step of 200 keys with
+// k_gemm_simt and the attention and row kernels of its time, and now: 1B-shaped, 4 layers, 12 rows 1239 -> 718 us, 24 rows 2439 -> 1180, 96 rows
+// 8824 -> 4035; 8B-shaped, 2 layers (K 4096 and 14336), 12 rows 1659 -> 665, 24 rows 3199 -> 1148, 512 rows 66455 -> 21704.
 #pragma once
 
 #include "sj_kernels.cuh"

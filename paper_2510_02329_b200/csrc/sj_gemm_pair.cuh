@@ -20,8 +20,8 @@
 //
 // Where the items (tile, row block) leave pairs idle (down has 16 to 20 tiles of 256 features), a cluster of n_split <= 4
 // pairs shares an item's K.  Every pair sends its sums of the rows that another one finishes into that one's shared
-// memory and finishes its own: chunk j (32 rows) belongs to split j % n_split, so all of them work on the epilogue and
-// no sum crosses L2.  A cluster is scheduled as a whole, so its pairs can wait for one another.
+// memory and finishes its own: the rows [32 j, 32 j + 32) of a block belong to split j % n_split, so all of them work on the
+// epilogue (split 0 does all of a block of 16 rows) and no sum crosses L2.  A cluster is scheduled as a whole, so its pairs can wait for one another.
 // The sums go as st.async: their arrival is the signal.  (A release after plain stores is one more trip: 1B-shaped 48 rows
 // 954 -> 934 us a step, 8B-shaped 44 rows 4459 -> 4377, with the residual rows requested beside the MMAs.)
 // Down at 72 rows (20 tiles, K 27648, 283 MB): 94.5 us with row blocks of 32 on 60 pairs, 60.4 as 80 rows on 40 pairs;
@@ -68,7 +68,7 @@ struct PairParams {
   int n_groups;           // clusters
   int n_split;            // pairs of a cluster: they share an item's K blocks
   int seg_kb;             // K blocks per accumulation chain
-  int xch_js;             // 32-row chunks of a row block that one split finishes, at most
+  int xch_js;             // epilogue chunks of a group that one split finishes, at most
   int R, rb, n_rb;        // rows, rows per block (a multiple of 16, at most 128: an M = 256 MMA takes N = 32, 64 .. 256), row blocks
   int plane_rows;         // row of the lo plane in the activation matrix
   int stages, stage_bytes;

@@ -185,7 +185,7 @@ __global__ void k_embed_norm(const StepArgs* __restrict__ args, KvView kv, Work 
 // 1B-shaped fp32 cut of 4 layers, 10 rows, a step 763 -> 674 us on a B200.)
 constexpr int kNormThreads = 1024;
 template <typename T>
-__global__ void k_reduce_norm(const StepArgs* __restrict__ args, Work w, Dims dm, SplitPlan sp, size_t slot_stride,
+__global__ void __launch_bounds__(kNormThreads) k_reduce_norm(const StepArgs* __restrict__ args, Work w, Dims dm, SplitPlan sp, size_t slot_stride,
                               const T* __restrict__ gain, int final_norm) {
   extern __shared__ float xs[];
   __shared__ float red[32];
@@ -332,6 +332,7 @@ __device__ __forceinline__ void unpack(const uint4& v, float* f) {
   }
 }
 
+// Projections on the CUDA cores where k_gemm_f32 does not go: bf16 models without tensor-core options, and sj_gemm_skinny.
 // `planes` = 2: the input is a hi/lo pair of bf16 planes (see Work); the two are added before use.
 template <typename T, int RT, int NF>
 __global__ void __launch_bounds__(256)

@@ -563,7 +563,6 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   extern __shared__ uint8_t t5_smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(t5_smem_raw) + 1023) & ~(uintptr_t)1023);
   const int warp = warp_index(), lane = threadIdx.x & 31;
-  pdl_launch();
   const int B = args->B, rows = args->gamma + 1, Hkv = dm.Hkv, group = dm.Hq / dm.Hkv, nq = group * rows;
   const int G = gridDim.x, c = blockIdx.x;
   uint8_t* p_area = sm + (size_t)stages * kT5Part;
@@ -592,6 +591,7 @@ k_attn_t5(const __grid_constant__ CUtensorMap tmKV, const StepArgs* __restrict__
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_launch();   // with this block's tensor memory in hand: a dependent that got there first would wait for this kernel, and this for it
   const AttPlan& pl = ctl->plan;
   const long long t_lo = att_first_tile(c, pl.T, G), t_hi = att_first_tile(c + 1, pl.T, G);
   att_fill_pages(ctl->pages, pl, kv, args, B, kT5Keys, t_lo, t_hi, threadIdx.x, blockDim.x);

@@ -107,8 +107,8 @@ sj_status sj_load_judge_head(sj_target *t, const float *w_host, float bias, floa
  *   "attn_tcgen05_min_tiles"  n >= 0 (default 4; 0 = always): with "attn_impl" 2, a step whose caches hold at least this
  *                many 128-key tiles per SM runs as one kernel per stage, with the tcgen05 attention, whatever "step_impl"
  *   "step_impl"  1 = the whole step as one persistent cooperative kernel (bf16, tcgen05 GEMMs, at most 48
- *                block rows), 0 = one kernel per stage, 2 = whichever is the faster for the step's rows and sequences and
- *                the model's widths (default when the shape allows)
+ *                block rows), 0 = one kernel per stage, 2 = one or the other by the step's rows and sequences, the caches'
+ *                lengths and the model's widths, along lines that were measured (default when the shape allows)
  *   "attn_two_term_layers"  n >= 0 (default 1): in layers [0, n) the tensor-core attention carries queries and
  *                probabilities as a sum of two fp16 terms (twice the MMAs).  Where the residual stream is still
  *                small (the first layer: an embedding row), the attention output is most of what the next

@@ -1380,7 +1380,7 @@ static sj_status enqueue_step(sj_target* t, sj_kv* kv, int B, int gamma, int mod
 #undef TIMED_END
 
 // The whole step as one cooperative launch per chunk of kMegaMaxLayers layers.  "step_impl" 1 takes it up to kMegaMaxRows
-// rows; the default (2) where it is the faster of the two (B200, us a step, persistent / per stage):
+// rows; the default (2) along these lines (B200, us a step, persistent / per stage):
 //   widths: a phase has to stream for longer than its barrier takes: ten 16 KiB units of gate/up for every block, 3.6 us at the
 //     copy rate.  One sequence, 9 rows, 24 layers: d 512, ffn 2048 (1.7 units) 1419 / 1054; d 1024, ffn 4096 (6.9) 1232 / 1161; d 1536,
 //     ffn 6144 (15.6) 1197 / 1257; 1B-shaped (27.7, 16 layers) 1012 / 1274.

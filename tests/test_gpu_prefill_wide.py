@@ -19,7 +19,8 @@ HD128_G4 = synth.ModelShape("hd128-group4", 2, 512, 4, 1, 128, 256, 640)
 @pytest.mark.parametrize("shape", [synth.TINY, HD128, HD128_G4], ids=lambda s: s.name)
 @pytest.mark.parametrize("before,n", [(0, 33), (0, 64), (7, 512), (21, 513), (0, 1025)])
 def test_wide_prefill(shape, before, n):
-    """One block, a full one, a full and a tiny one, three; `before` tokens in the cache already (a page's middle)."""
+    """One block, one of 512 rows (entries of 32; two of 264 where they are 24), a token more (two blocks of equal size), three blocks;
+    `before` tokens in the cache already (a page's middle)."""
     case = _empty_case(shape, torch.bfloat16, room=1100)
     try:
         prompt = synth.token_ids(shape.vocab, before + n, seed=51, stream=9)
